@@ -94,6 +94,7 @@ struct esp_ctx {
     int32_t *s_jmap = nullptr;
     // Gamma term (esp_set_penalties): the loaded values, kept once penalties are first set
     double *values0 = nullptr;
+    unsigned char *pen_in = nullptr;   // device copies of its inputs (current configurations, slowdowns, thresholds)
     // the pass table tile by tile (units then values of each tile; one bulk copy per tile), when every
     // tile of the per-warp plan allows it; n_tiles: tiles of that plan
     unsigned char *il = nullptr;
@@ -298,6 +299,7 @@ void release_table(esp_ctx *ctx, bool keep = false)
     ctx->s_off = nullptr;
     ctx->s_jmap = nullptr;
     ctx->values0 = nullptr;
+    ctx->pen_in = nullptr;
     ctx->il = nullptr;
     ctx->il_f32 = false;
     ctx->persist_grid = 0;
@@ -1829,76 +1831,44 @@ esp_status esp_set_penalties(esp_ctx *ctx, double gamma0, const int32_t *c_cur, 
         return ESP_ERR_INVALID_ARG;
     ESP_CUDA(cudaSetDevice(ctx->device));
     const size_t n_jobs = (size_t)ctx->S * ctx->J, n_opt = (size_t)ctx->n_opt;
+    // The loaded values and the inputs' device copies, allocated by the first call and kept with the table
+    // (a cudaMalloc and cudaFree per call took 60 to 180 us of a 0.5 ms outer round of the ESP-IAC loop,
+    // depending on whether the driver had to map memory for them).
+    const size_t cur_b = (n_jobs * sizeof(int32_t) + 255) & ~size_t(255), sh_b = (n_opt * sizeof(double) + 255) & ~size_t(255),
+                 tau_b = n_jobs * sizeof(double);
     if (!ctx->values0) {
-        void *q = nullptr;
-        cudaError_t e = cudaMalloc(&q, n_opt * sizeof(double) + 64);
-        if (e == cudaErrorMemoryAllocation) {
-            cudaGetLastError();
-            return ESP_ERR_OOM;
-        }
-        ESP_CUDA(e);
-        ctx->table_bufs.emplace_back(q, n_opt * sizeof(double) + 64);
-        ctx->values0 = static_cast<double *>(q);
-        ESP_CUDA(cudaMemcpyAsync(ctx->values0, ctx->values, n_opt * sizeof(double), cudaMemcpyDeviceToDevice,
-                                 ctx->stream));
+        double *v0 = nullptr;
+        if ((st = dev_alloc(ctx, &v0, n_opt, 64, false)) != ESP_OK)
+            return st;
+        ESP_CUDA(cudaMemcpyAsync(v0, ctx->values, n_opt * sizeof(double), cudaMemcpyDeviceToDevice, ctx->stream));
+        ctx->values0 = v0;
     }
-    // inputs on the device, for this call only
-    void *buf = nullptr;
-    const size_t cur_b = c_cur ? n_jobs * sizeof(int32_t) : 0, sh_b = s_hat ? n_opt * sizeof(double) : 0,
-                 tau_b = s_hat ? n_jobs * sizeof(double) : 0;
-    const size_t a1 = (cur_b + 255) & ~size_t(255), a2 = (sh_b + 255) & ~size_t(255);
-    if (cur_b + sh_b + tau_b > 0) {
-        cudaError_t e = cudaMalloc(&buf, a1 + a2 + tau_b + 64);
-        if (e == cudaErrorMemoryAllocation) {
-            cudaGetLastError();
-            return ESP_ERR_OOM;
-        }
-        ESP_CUDA(e);
-    }
-    unsigned char *b = static_cast<unsigned char *>(buf);
-    int32_t *d_cur = c_cur ? reinterpret_cast<int32_t *>(b) : nullptr;
-    double *d_sh = s_hat ? reinterpret_cast<double *>(b + a1) : nullptr;
-    double *d_tau = s_hat ? reinterpret_cast<double *>(b + a1 + a2) : nullptr;
-    auto done = [&](esp_status r) {
-        if (buf) {
-            cudaStreamSynchronize(ctx->stream);
-            cudaFree(buf);
-        }
-        return r;
-    };
-#define ESP_PEN_CUDA(call)                          \
-    do {                                            \
-        cudaError_t e_ = (call);                    \
-        if (e_ != cudaSuccess) {                    \
-            cudaGetLastError();                     \
-            return done(cuda_fail(ctx, e_));        \
-        }                                           \
-    } while (0)
+    if (!ctx->pen_in && (c_cur || s_hat) && (st = dev_alloc(ctx, &ctx->pen_in, cur_b + sh_b + tau_b, 64, false)) != ESP_OK)
+        return st;
+    unsigned char *buf = ctx->pen_in;
+    int32_t *d_cur = c_cur ? reinterpret_cast<int32_t *>(buf) : nullptr;
+    double *d_sh = s_hat ? reinterpret_cast<double *>(buf + cur_b) : nullptr;
+    double *d_tau = s_hat ? reinterpret_cast<double *>(buf + cur_b + sh_b) : nullptr;
     if (c_cur)
-        ESP_PEN_CUDA(cudaMemcpyAsync(d_cur, c_cur, cur_b, cudaMemcpyHostToDevice, ctx->stream));
+        ESP_CUDA(cudaMemcpyAsync(d_cur, c_cur, n_jobs * sizeof(int32_t), cudaMemcpyHostToDevice, ctx->stream));
     if (s_hat) {
-        ESP_PEN_CUDA(cudaMemcpyAsync(d_sh, s_hat, sh_b, cudaMemcpyHostToDevice, ctx->stream));
-        ESP_PEN_CUDA(cudaMemcpyAsync(d_tau, tau, tau_b, cudaMemcpyHostToDevice, ctx->stream));
+        ESP_CUDA(cudaMemcpyAsync(d_sh, s_hat, n_opt * sizeof(double), cudaMemcpyHostToDevice, ctx->stream));
+        ESP_CUDA(cudaMemcpyAsync(d_tau, tau, tau_b, cudaMemcpyHostToDevice, ctx->stream));
     }
-    ESP_PEN_CUDA(cudaMemsetAsync(ctx->valflags, 0, sizeof(unsigned int), ctx->stream));
-    ESP_PEN_CUDA(launch_apply_penalties(dev_table(ctx), ctx->values0, d_cur, d_sh, d_tau, gamma0, alpha, ctx->values,
-                                        ctx->valflags, ctx->stream));
+    ESP_CUDA(cudaMemsetAsync(ctx->valflags, 0, sizeof(unsigned int), ctx->stream));
+    ESP_CUDA(launch_apply_penalties(dev_table(ctx), ctx->values0, d_cur, d_sh, d_tau, gamma0, alpha, ctx->values,
+                                    ctx->valflags, ctx->stream));
     unsigned int pflags = 0;
-    ESP_PEN_CUDA(cudaMemcpyAsync(&pflags, ctx->valflags, sizeof(unsigned int), cudaMemcpyDeviceToHost, ctx->stream));
-    ESP_PEN_CUDA(cudaStreamSynchronize(ctx->stream));
-#undef ESP_PEN_CUDA
-    if (pflags) {   // back to the loaded values
-        cudaError_t e = cudaMemcpyAsync(ctx->values, ctx->values0, n_opt * sizeof(double), cudaMemcpyDeviceToDevice,
-                                        ctx->stream);
-        if (e != cudaSuccess)
-            return done(cuda_fail(ctx, e));
-    }
+    ESP_CUDA(cudaMemcpyAsync(&pflags, ctx->valflags, sizeof(unsigned int), cudaMemcpyDeviceToHost, ctx->stream));
+    ESP_CUDA(cudaStreamSynchronize(ctx->stream));
+    if (pflags)   // back to the loaded values
+        ESP_CUDA(cudaMemcpyAsync(ctx->values, ctx->values0, n_opt * sizeof(double), cudaMemcpyDeviceToDevice,
+                                 ctx->stream));
     unsigned int vflags = 0;
-    st = refresh_after_values(ctx, &vflags);
-    if (st != ESP_OK)
-        return done(st);
+    if ((st = refresh_after_values(ctx, &vflags)) != ESP_OK)
+        return st;
     ctx->solved = false;
-    return done((pflags || vflags) ? ESP_ERR_INVALID_ARG : ESP_OK);
+    return (pflags || vflags) ? ESP_ERR_INVALID_ARG : ESP_OK;
 }
 
 esp_status esp_last_launch_count(esp_ctx *ctx, int64_t *out)
