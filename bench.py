@@ -116,8 +116,8 @@ def measured_peak():
         return 6800.0, "fallback"
 
 
-PASS_KERNEL_SOURCES = ("esp_kernels.cu", "esp_kernels_f32.cu", "esp_pass.cuh", "esp_tile.cuh", "esp_ptx.cuh", "esp_warp.cuh", "esp_device.cuh",
-                       "esp_common.h", "esp_kernels.h")
+PASS_KERNEL_SOURCES = ("esp_packed.cu", "esp_packed.h", "esp_kernels.cu", "esp_pass.cuh", "esp_tile.cuh", "esp_ptx.cuh", "esp_warp.cuh",
+                       "esp_device.cuh", "esp_common.h", "esp_kernels.h")
 
 
 def pass_kernel_sha256() -> str:
@@ -413,13 +413,13 @@ def time_streaming(esp, solver, w, T, args, dist, barrier, stream, clk=None):
     ev_avg_ms = pass_ms / max(n_pass, 1)
     ev_achieved = bytes_pass / (ev_avg_ms / 1e3) / 1e9 if n_pass else None
     kind = {0: "k_pass (per-warp pass, two bulk copies per tile)",
-            1: "k_pass (per-warp pass, one bulk copy per tile from the tile-interleaved table)",
-            3: "k_pass (per-warp pass, one bulk copy per tile, fp32 units)"}.get(
+            1: "k_packed or k_pass (a private copy in the order of its tiles, one bulk copy per step or tile)",
+            3: "k_packed (packed screen copy, one bulk copy per 256 options)"}.get(
         esp.esp_debug_pass_kernel(ctx), "k_place (factored placement pass)")
     persist = esp.esp_debug_persistent(ctx) > 0
     if persist:
-        kind = ("k_pass_persist (rounds 0..T-1 in one cooperative launch, scenarios released by their price "
-                "updates; one bulk copy per tile, fp32 units) + k_pass (final pass)")
+        kind = ("k_packed_persist (rounds 0..T-1 in one cooperative launch, scenarios released by their price "
+                "updates; packed screen copy) + k_packed (final pass)")
     roofline = {"bound": "hbm", "kernel": kind + ": best response + demand aggregation + fused price update",
                 "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                 "traffic": kernel_traffic(w.name, t.n_opt),

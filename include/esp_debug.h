@@ -96,17 +96,18 @@ esp_status esp_debug_hold_stage(esp_ctx *ctx);
  * very next) reports ESP_ERR_OOM as a failed cudaMalloc would; n < 0 disarms it. */
 esp_status esp_debug_fail_alloc(esp_ctx *ctx, int64_t n);
 
-/* *kind receives how the loaded table is evaluated: 0 the per-warp pass with two bulk copies per tile
- * (units and values apart), 1 the per-warp pass with one bulk copy per tile (tile-interleaved table),
- * 2 the factored placement pass, 3 as 1 with the units of the interleaved table stored as fp32 (every
- * unit below 2^23, so each is exact; the screen then needs no conversion per unit). */
+/* *kind receives how the loaded table is evaluated: 0 the staged pass with two bulk copies per tile (units
+ * and values apart), 1 a private copy of the table in the order of its tiles, one launch per round (the
+ * packed screen copy, or the tile-interleaved table of the staged pass), 2 the factored placement pass, 3
+ * the packed screen copy where the persistent pass is available too. */
 esp_status esp_debug_pass_kernel(esp_ctx *ctx, int32_t *kind);
 
 /* Persistent pass: every round of a solve in one cooperative launch, each scenario's next round
- * released by its price update instead of a kernel boundary (tables whose interleaved tiles hold fp32
- * units; solves without per-pass events, fingerprint or dual trace). mode -1 (the default) uses it on
- * uniform tables with at least 16 tiles per warp of its launch, 0 never, 1 wherever the table can take
- * it; later solves of this context follow the mode. Results are identical either way.
+ * released by its price update instead of a kernel boundary (packed tables of R = 4, 6 or 8, or large
+ * enough to use it by default; solves without per-pass events, fingerprint or dual trace). mode -1 (the
+ * default) uses it on tables with at least 5 steps of 256 options per warp of its launch, 0 never, 1
+ * wherever the table can take it; later solves of this context follow the mode. Results are identical
+ * either way.
  * esp_debug_persistent: *grid receives the CTAs of the persistent launch that a plain solve of the
  * loaded table uses under the current mode (0: one launch per round). */
 esp_status esp_debug_set_persistent(esp_ctx *ctx, int32_t mode);
@@ -117,22 +118,22 @@ esp_status esp_debug_persistent(esp_ctx *ctx, int32_t *grid);
 esp_status esp_debug_persist_waits(esp_ctx *ctx, int64_t *ns, int64_t *waits, int32_t reset);
 
 /* Profile of the last esp_load_options / esp_load_options_device of this context: ms[0..6] the host
- * milliseconds from its start until its uploads and validation were queued, until the sorted layout
- * was queued, until the occupancy of the pass kernels was known, until the pass was planned, until
- * the uploads, validation and duplicate marks were done, until the tiles, interleaved table and solve
+ * milliseconds from its start until its uploads and validation were queued, until the duplicate marks
+ * were queued, until the packed passes were planned, until that plan was stored, until the uploads,
+ * validation and duplicate marks were done, until the private copy of the table and the solve
  * state were queued, and until it returned; *mallocs and *frees the cudaMalloc and cudaFree calls it
  * made (a reload of a table of the same shape makes none). */
 esp_status esp_debug_load_profile(esp_ctx *ctx, double *ms, int64_t *mallocs, int64_t *frees);
 
-/* enable = 0 makes later loads keep integer units in the tile-interleaved table; 1 restores the
- * default (fp32 units where every unit is below 2^23 and the table has no group column, R = 4, 6 or 8,
- * uniform or sorted). Results are identical either way. */
+/* enable = 0 makes later loads use the staged pass (integer units in the tile-interleaved table); 1
+ * restores the default, the packed passes where every unit is below 2^23, the table has no group column
+ * and its unit fields fit 8 words per option. Results are identical either way. */
 esp_status esp_debug_set_stage_f32(esp_ctx *ctx, int32_t enable);
 
-/* enable = 0 makes later loads keep the per-warp pass's table as separate unit and value arrays (two
- * bulk copies per tile); 1 restores the default, a tile-interleaved copy (each tile's units then its
- * values, one bulk copy per tile) wherever every tile allows it (esp_debug_pass_kernel then reports
- * 1). Results are identical either way. */
+/* enable = 0 makes later loads use the staged pass with separate unit and value arrays (two bulk copies
+ * per tile); 1 restores the default, a private copy in the order of its tiles: packed, or else interleaved
+ * (each tile's units then its values, one bulk copy per tile) wherever every tile allows it. Results are
+ * identical either way. */
 esp_status esp_debug_set_interleave(esp_ctx *ctx, int32_t enable);
 
 /* Failure-detection hooks of the IAC predictor's tensor-core kernel (esp_iac.h). limit_ms bounds each

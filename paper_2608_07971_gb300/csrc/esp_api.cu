@@ -56,9 +56,13 @@ struct PlanCache {
     bool grouped = false, sorted_enabled = false;
     std::vector<int64_t> off;
     int64_t min_k = 0, max_k = 0;
-    bool sorted = false;
+    bool has_lay = false, sorted = false;   // lay: the sorted layout of the staged pass
     esp::SortedLayout lay;
+    bool has_plan = false;         // plan: the staged pass's tiles
     esp::Plan plan;
+    bool has_pack = false;         // pack: the packed passes' tiles
+    int32_t pack_warps = 0;
+    esp::PackPlan pack;
 };
 
 struct esp_ctx {
@@ -99,7 +103,12 @@ struct esp_ctx {
     // tile of the per-warp plan allows it; n_tiles: tiles of that plan
     unsigned char *il = nullptr;
     int64_t n_tiles = 0;
-    bool il_f32 = false;             // il holds the units as fp32 bit patterns (every unit below 2^23)
+
+    // the packed screen copy and its plan (esp_packed.h): what the passes of an ungrouped table with
+    // units below 2^23 read
+    bool packed = false;
+    DevPack pack = {};
+    uint4 *pk_data = nullptr;
 
     // factored placement table (esp_load_placement): no stored option table
     bool placement = false;
@@ -115,8 +124,8 @@ struct esp_ctx {
 
     TileDesc *tiles = nullptr;
     int32_t *warp_begin = nullptr;
-    bool il_enabled = true;          // later loads may interleave the pass table (esp_debug_set_interleave)
-    bool il_f32_enabled = true;      // ... with fp32 units where exact (esp_debug_set_stage_f32)
+    bool il_enabled = true;          // later loads may pack or interleave the table (esp_debug_set_interleave)
+    bool il_f32_enabled = true;      // ... pack it (esp_debug_set_stage_f32)
     // failure-detection hooks (esp_debug.h): limit of a bounded wait of the evaluation passes in ms
     // (0: the default, 4 s), extra bytes announced on the next solve's first stage, allocations left
     // before an injected failure (-1: none)
@@ -124,8 +133,6 @@ struct esp_ctx {
     uint32_t hold_tx = 0;
     int64_t fail_alloc_in = -1;
     int32_t *scen_warps = nullptr;   // warps owning tiles of each scenario
-    int32_t *scen_tiles = nullptr;   // tiles of each scenario
-    int32_t *item_order = nullptr;   // the plan's ranges by the scenario of their first tile
     unsigned int *arrive = nullptr;  // per-scenario arrivals of the round pass in flight
     unsigned int *ver = nullptr;     // per-scenario price versions of the persistent pass
     unsigned int *work = nullptr;    // work items the persistent pass has handed out
@@ -301,7 +308,12 @@ void release_table(esp_ctx *ctx, bool keep = false)
     ctx->values0 = nullptr;
     ctx->pen_in = nullptr;
     ctx->il = nullptr;
-    ctx->il_f32 = false;
+    ctx->packed = false;
+    ctx->pack = DevPack{};
+    ctx->pk_data = nullptr;
+    ctx->tiles = nullptr;
+    ctx->warp_begin = nullptr;
+    ctx->scen_warps = nullptr;
     ctx->persist_grid = 0;
     ctx->persist_auto = false;
     ctx->n_tiles = 0;
@@ -356,7 +368,6 @@ DevTable dev_table(const esp_ctx *c)
     t.small_units = c->small_units;
     t.jmap = nullptr;
     t.il = nullptr;
-    t.il_f32 = 0;
     return t;
 }
 
@@ -372,7 +383,6 @@ DevTable pass_table(const esp_ctx *c)
         t.jmap = c->s_jmap;
     }
     t.il = c->il;
-    t.il_f32 = (c->il != nullptr && c->il_f32) ? 1 : 0;
     return t;
 }
 
@@ -531,6 +541,186 @@ private:
     bool active_ = false;
 };
 
+// Uploads the packed passes' plan (pc.pack) and fills the packed copy of the table.
+esp_status load_packed(esp_ctx *ctx, const PackFormat &fmt)
+{
+    const PackPlan &p = ctx->pc.pack;
+    PackTile *tiles = nullptr;
+    int32_t *jb = nullptr, *job = nullptr, *wb = nullptr, *scen_tiles = nullptr;
+    esp_status st = ESP_OK;
+    auto up = [&](auto **ptr, const auto &src) {   // the host arrays stay in the plan cache
+        if (st == ESP_OK)
+            st = dev_alloc(ctx, ptr, src.size(), 64, false);
+        if (st == ESP_OK &&
+            cudaMemcpyAsync(*ptr, src.data(), src.size() * sizeof(src[0]), cudaMemcpyHostToDevice, ctx->stream) != cudaSuccess)
+            st = cuda_fail(ctx, cudaGetLastError());
+    };
+    up(&tiles, p.tiles);
+    up(&jb, p.job_begin);
+    if (!p.job.empty())
+        up(&job, p.job);
+    up(&wb, p.warp_begin);
+    up(&scen_tiles, p.scen_tiles);
+    if (st == ESP_OK)
+        st = dev_alloc(ctx, &ctx->pk_data, (size_t)p.vecs * (size_t)(fmt.nw + 1), 64, false);
+    if (st != ESP_OK)
+        return st;
+    DevPack &d = ctx->pack;
+    d.data = ctx->pk_data;
+    d.tiles = tiles;
+    d.job_begin = jb;
+    d.job = job;
+    d.warp_begin = wb;
+    d.scen_tiles = scen_tiles;
+    d.n_tiles = (int32_t)p.tiles.size();
+    d.n_warps = p.n_warps;
+    d.fmt = fmt;
+    ESP_CUDA(launch_pack(dev_table(ctx), d, ctx->pk_data, ctx->stream));
+    ctx->packed = true;
+    ctx->grid = (p.n_warps + kWarpsPerCta - 1) / kWarpsPerCta;
+    // The persistent pass: every CTA of its launch co-resident, no more warps than tiles. By default on
+    // tables with at least kPersistMinSteps steps per warp of its launch. Measured per round (one launch
+    // per round against persistent): what-if batch at 64 / 128 / 256 / 1024 scenarios (2.7 / 5.4 / 10.8 / 43
+    // steps per warp) 23.6 / 34.2 / 55.1 / 144 us against 33.0 / 30.9 / 41.0 / 90.2, heavy-tailed table at
+    // 2 / 4 / 16 scenarios 50 / 91 / 247 against 48 / 63 / 170: below, the waits for prices cost more than
+    // the launches; above, static tile ranges leave the GPU waiting for its slowest warps. Smaller
+    // tables of R = 4, 6, 8 take it on request.
+    const int per_sm = packed_ctas_per_sm(fmt.nw);
+    if (per_sm > 0 && d.n_tiles > 0) {
+        ctx->persist_auto = p.steps >= (int64_t)kPersistMinSteps * per_sm * ctx->sm_count * kWarpsPerCta;
+        if (ctx->persist_auto || ctx->R == 4 || ctx->R == 6 || ctx->R == 8)
+            ctx->persist_grid = (int32_t)std::min<int64_t>((int64_t)per_sm * ctx->sm_count,
+                                                           ((int64_t)d.n_tiles + kWarpsPerCta - 1) / kWarpsPerCta);
+    }
+    return ESP_OK;
+}
+
+// Builds the sorted layout of a general table without a group column for the staged pass (a table that
+// the packed passes do not take): runs of equal-size jobs take its uniform paths. Jobs keep their
+// option order, so the copy inherits the duplicate marks of the original; its padding is marked as it is
+// written.
+esp_status load_sorted(esp_ctx *ctx)
+{
+    PlanCache &pc = ctx->pc;
+    if (!pc.has_lay) {
+        pc.sorted = sort_layout(pc.off.data(), ctx->S, ctx->J, pc.lay, kRunMaxK);
+        pc.has_lay = true;
+    }
+    if (!pc.sorted)
+        return ESP_OK;
+    const SortedLayout &lay = pc.lay;
+    const size_t n_jobs = (size_t)ctx->S * ctx->J;
+    const int64_t sn = lay.off.back();
+    esp_status st = ESP_OK;
+    auto al = [&](auto **ptr, size_t n) {
+        if (st == ESP_OK)
+            st = dev_alloc(ctx, ptr, n, 64, false);
+    };
+    al(&ctx->s_units, (size_t)sn * ctx->R);   // every option of the layout, padding included
+    al(&ctx->s_values, (size_t)sn);
+    al(&ctx->s_off, n_jobs + 1);
+    al(&ctx->s_jmap, n_jobs);
+    if (st != ESP_OK)
+        return st;
+    ESP_CUDA(cudaMemcpyAsync(ctx->s_off, lay.off.data(), lay.off.size() * sizeof(int64_t), cudaMemcpyHostToDevice,
+                             ctx->stream));
+    ESP_CUDA(cudaMemcpyAsync(ctx->s_jmap, lay.jmap.data(), lay.jmap.size() * sizeof(int32_t), cudaMemcpyHostToDevice,
+                             ctx->stream));
+    ctx->s_n_opt = sn;
+    ctx->sorted = true;
+    ESP_CUDA(launch_gather_sorted(dev_table(ctx), pass_table(ctx), ctx->s_units, ctx->s_values, ctx->stream));
+    return ESP_OK;
+}
+
+// Plans the staged pass (tiles through shared memory) from the cached host offsets, uploads its plan
+// and, where every tile allows it, the tile-interleaved copy.
+esp_status load_staged(esp_ctx *ctx)
+{
+    PlanCache &pc = ctx->pc;
+    const int32_t S = ctx->S, J = ctx->J, R = ctx->R;
+    const bool grouped = ctx->group != nullptr;
+    const int64_t *plan_off = ctx->sorted ? pc.lay.off.data() : pc.off.data();
+    const int32_t *plan_scen = ctx->sorted ? pc.lay.scen.data() : nullptr;
+    const int32_t *plan_runk = ctx->sorted ? pc.lay.runk.data() : nullptr;
+    const int tile_opt = tile_options_for(R, grouped, ctx->max_k, ctx->uniform_k >= 4);
+    // a sorted layout's tiles are runs and chunks only (the sorted layout exists only without a group
+    // column): the runs-only instantiation
+    const int mode = ctx->uniform_k > 0 ? kModeUniform : (ctx->sorted && !grouped) ? kModeRuns : kModeGeneral;
+    const int per_sm = pass_ctas_per_sm(R, grouped, mode, ctx->P, tile_opt);
+    if (per_sm < 1)
+        return ESP_ERR_UNSUPPORTED;
+    // Ranges of the plan as waves of resident CTAs: two by default (CTAs that finish early take the
+    // second wave's ranges), one for a sorted layout (measured 2% faster there).
+    const int waves = ctx->plan_waves > 0 ? ctx->plan_waves : (mode == kModeRuns) ? 1 : 2;
+    const int max_warps = ctx->sm_count * per_sm * kWarpsPerCta * waves;
+    if (!(pc.has_plan && pc.max_warps == max_warps && pc.tile_opt == tile_opt)) {
+        pc.has_plan = false;
+        if (!plan_tiles(plan_off, S, J, tile_opt, max_warps, pc.plan, plan_scen, plan_runk) ||
+            !check_plan(plan_off, S, J, pc.plan, plan_scen, plan_runk))
+            return ESP_ERR_INVALID_ARG;
+        pc.has_plan = true;
+        pc.max_warps = max_warps;
+        pc.tile_opt = tile_opt;
+    }
+    const Plan &plan = pc.plan;
+    // the runs-only instantiation has no path for a general tile
+    if (mode == kModeRuns)
+        for (const TileDesc &d : plan.tiles)
+            if (!(d.flags & (TILE_RUN | TILE_BIG)))
+                return ESP_ERR_INVALID_ARG;
+    esp_status st = ESP_OK;
+    auto al = [&](auto **ptr, size_t n) {
+        if (st == ESP_OK)
+            st = dev_alloc(ctx, ptr, n);
+    };
+    al(&ctx->scen_warps, (size_t)S);
+    al(&ctx->tiles, plan.tiles.size() + 1);
+    al(&ctx->warp_begin, plan.warp_begin.size());
+    if (st != ESP_OK)
+        return st;
+    ctx->n_warps = plan.n_warps;
+    ctx->tile_opt = plan.tile_opt;
+    ctx->grid = (plan.n_warps + kWarpsPerCta - 1) / kWarpsPerCta;
+    std::vector<int32_t> sw((size_t)S, 0);
+    for (int32_t w = 0; w < plan.n_warps; ++w) {
+        int32_t last = -1;
+        for (int32_t k = plan.warp_begin[w]; k < plan.warp_begin[w + 1]; ++k)
+            if (plan.tiles[k].scenario != last) {
+                last = plan.tiles[k].scenario;
+                ++sw[last];
+            }
+    }
+    ESP_CUDA(cudaMemcpyAsync(ctx->scen_warps, sw.data(), sw.size() * sizeof(int32_t), cudaMemcpyHostToDevice,
+                             ctx->stream));
+    ESP_CUDA(cudaStreamSynchronize(ctx->stream));
+    if (!plan.tiles.empty())
+        ESP_CUDA(cudaMemcpyAsync(ctx->tiles, plan.tiles.data(), plan.tiles.size() * sizeof(TileDesc),
+                                 cudaMemcpyHostToDevice, ctx->stream));
+    ESP_CUDA(cudaMemcpyAsync(ctx->warp_begin, plan.warp_begin.data(), plan.warp_begin.size() * sizeof(int32_t),
+                             cudaMemcpyHostToDevice, ctx->stream));
+    // one bulk copy per tile when every tile can take it: no job offsets needed (uniform tables,
+    // runs and chunks of the sorted layout), every tile 16-byte aligned in the interleaved copy,
+    // and its values aligned in the stage for the loads of its path (16 bytes for the paths of
+    // four options per lane, 8 otherwise)
+    const int64_t W = 4 * (int64_t)R + 8;
+    bool il_ok = ctx->il_enabled && !grouped && (ctx->uniform_k > 0 || ctx->sorted) && !plan.tiles.empty();
+    for (size_t k = 0; il_ok && k < plan.tiles.size(); ++k) {
+        const TileDesc &d = plan.tiles[k];
+        const int kk = (d.flags & TILE_RUN) ? tile_run_k(d.flags) : ctx->uniform_k;
+        const bool vec = (d.flags & TILE_BIG) ? ((d.opt_begin | (int64_t)d.n_opt) & 3) == 0 : kk >= 4;
+        il_ok = (d.opt_begin * W) % 16 == 0 && ((int64_t)d.n_opt * R * 4) % (vec ? 16 : 8) == 0 &&
+                ((d.flags & (TILE_BIG | TILE_RUN)) || ctx->uniform_k > 0);
+    }
+    if (il_ok) {
+        const int64_t pass_opt = ctx->sorted ? ctx->s_n_opt : ctx->n_opt;
+        if ((st = dev_alloc(ctx, &ctx->il, (size_t)(pass_opt * W), 64, false)) != ESP_OK)   // the tiles cover every option
+            return st;
+        ctx->n_tiles = (int64_t)plan.tiles.size();
+        ESP_CUDA(launch_interleave(pass_table(ctx), ctx->tiles, ctx->n_tiles, ctx->il, ctx->stream));
+    }
+    return ESP_OK;
+}
+
 // Upload (host or device source), validate on the device, plan, allocate the solve state.
 esp_status load_common(esp_ctx *ctx, int32_t S, int32_t J, int32_t R, int32_t P, int32_t rg, const int64_t *job_off,
                        const int32_t *units, const double *values, const uint16_t *group, const int64_t *capacity,
@@ -672,79 +862,48 @@ esp_status load_common(esp_ctx *ctx, int32_t S, int32_t J, int32_t R, int32_t P,
     // plan the evaluation pass
     ctx->uniform_k = (!grouped && min_k == max_k && max_k <= 32 && (max_k & (max_k - 1)) == 0) ? (int32_t)max_k : 0;
 
-    // general tables without a group column: the evaluation pass reads the sorted layout (runs of
-    // equal-size jobs take the uniform paths). Jobs keep their option order, so the copy inherits
-    // the duplicate marks of the original; its padding is marked as it is written.
-    SortedLayout lay_new;
-    bool use_sorted = false;
-    if (cached)
-        use_sorted = pc.sorted;
-    else
-        use_sorted = ctx->sorted_enabled && !grouped && ctx->uniform_k == 0 && J >= 1 &&
-                     sort_layout(off_host, S, J, lay_new, kRunMaxK);
-    const SortedLayout &lay = cached ? pc.lay : lay_new;
-    if (use_sorted) {
-        const int64_t sn = lay.off.back();
-        ALLOC_FILLED(ctx->s_units, (size_t)sn * R);   // every option of the layout, padding included
-        ALLOC_FILLED(ctx->s_values, (size_t)sn);
-        ALLOC_FILLED(ctx->s_off, (size_t)n_jobs + 1);
-        ALLOC_FILLED(ctx->s_jmap, (size_t)n_jobs);
-        ESP_CUDA(cudaMemcpyAsync(ctx->s_off, lay.off.data(), lay.off.size() * sizeof(int64_t), cudaMemcpyHostToDevice,
-                                 ctx->stream));
-        ESP_CUDA(cudaMemcpyAsync(ctx->s_jmap, lay.jmap.data(), lay.jmap.size() * sizeof(int32_t),
-                                 cudaMemcpyHostToDevice, ctx->stream));
-        ctx->s_n_opt = sn;
-        ctx->sorted = true;
-        ESP_CUDA(launch_gather_sorted(dev_table(ctx), pass_table(ctx), ctx->s_units, ctx->s_values, ctx->stream));
+    // the packed passes (esp_packed.h) take a table without a group column whose units are below 2^23;
+    // the last is known after the validation, so the plan for them is made meanwhile, for the unit
+    // words that pairs of columns need. Tables they do not take are evaluated by the staged pass, general
+    // ones without a group column in the sorted layout.
+    const bool may_sort = ctx->sorted_enabled && !grouped && ctx->uniform_k == 0 && J >= 1;
+    const bool may_pack = ctx->il_enabled && ctx->il_f32_enabled && !grouped && (ctx->uniform_k > 0 || may_sort) &&
+                          n_jobs > 0;
+    ctx->load_ms[1] = since();
+    PackPlan pack_new;
+    int32_t pack_warps = 0;
+    bool pack_cached = false, pack_ok = false;
+    if (may_pack) {
+        const int per_sm = packed_ctas_per_sm(R <= 4 ? 2 : R <= 6 ? 3 : R <= 8 ? 4 : R <= 12 ? 6 : 8);
+        const int waves = ctx->plan_waves > 0 ? ctx->plan_waves : 1;
+        pack_warps = ctx->sm_count * std::max(per_sm, 1) * kWarpsPerCta * waves;
+        pack_cached = cached && pc.has_pack && pc.pack_warps == pack_warps;
+        const int64_t all_k = min_k == max_k ? max_k : 0;
+        pack_ok = per_sm > 0 && (pack_cached || (plan_packed(off_host, S, J, pack_warps, pack_new, all_k) &&
+                                                 check_packed(off_host, S, J, pack_new, all_k)));
     }
-    ctx->load_ms[1] = since();   // sorted layout queued
-    const int64_t *plan_off = ctx->sorted ? lay.off.data() : off_host;
-    const int32_t *plan_scen = ctx->sorted ? lay.scen.data() : nullptr;
-    const int32_t *plan_runk = ctx->sorted ? lay.runk.data() : nullptr;
-
-    Plan plan_new;
-    const int tile_opt = tile_options_for(R, grouped, max_k, ctx->uniform_k >= 4);
-    // a sorted layout's tiles are runs and chunks only (the sorted layout exists only without a group
-    // column): the runs-only instantiation
-    const int mode = ctx->uniform_k > 0 ? kModeUniform : (use_sorted && !grouped) ? kModeRuns : kModeGeneral;
-    int per_sm = pass_ctas_per_sm(R, grouped, mode, P, tile_opt);
-    // a table that may take the persistent pass is planned for its co-resident CTAs, so that each of
-    // its physical warps runs exactly `waves` ranges (its fp32 stage units are decided after the
-    // validation; a table that turns out not to qualify runs the same plan with per-round launches)
-    const int per_sm_persist = (ctx->il_enabled && ctx->il_f32_enabled && pass_f32_shape(R, grouped, mode))
-                                   ? pass_persist_ctas_per_sm(R, mode, P, tile_opt)
-                                   : 0;
-    if (per_sm_persist > 0 && per_sm_persist < per_sm)
-        per_sm = per_sm_persist;
-    ctx->load_ms[2] = since();   // occupancy of the pass kernels
-    if (per_sm < 1) {
-        cudaStreamSynchronize(ctx->stream);
-        release_table(ctx);
-        return ESP_ERR_UNSUPPORTED;
+    ctx->load_ms[2] = since();   // packed passes planned
+    // keep this load's layout (and below its plan) for the next load of the same offsets
+    if (!cached) {
+        pc.valid = true;
+        pc.S = S;
+        pc.J = J;
+        pc.R = R;
+        pc.P = P;
+        pc.grouped = grouped;
+        pc.sorted_enabled = ctx->sorted_enabled;
+        pc.off.assign(off_host, off_host + n_jobs + 1);
+        pc.min_k = min_k;
+        pc.max_k = max_k;
+        pc.has_lay = pc.has_plan = pc.has_pack = false;
     }
-    // Ranges of the plan as waves of resident CTAs: two by default (with per-round launches, CTAs that
-    // finish early take the second wave's ranges; the persistent pass hands them out as work items,
-    // two per warp and round), one for a sorted layout (measured 2% faster there).
-    const int waves = ctx->plan_waves > 0 ? ctx->plan_waves : (mode == kModeRuns) ? 1 : 2;
-    const int max_warps = ctx->sm_count * per_sm * kWarpsPerCta * waves;
-    const bool plan_cached = cached && pc.max_warps == max_warps && pc.tile_opt == tile_opt;
-    if (!plan_cached && (!plan_tiles(plan_off, S, J, tile_opt, max_warps, plan_new, plan_scen, plan_runk) ||
-                         !check_plan(plan_off, S, J, plan_new, plan_scen, plan_runk))) {
-        cudaStreamSynchronize(ctx->stream);
-        release_table(ctx);
-        return ESP_ERR_INVALID_ARG;
+    if (pack_ok && !pack_cached) {
+        pc.has_pack = true;
+        pc.pack_warps = pack_warps;
+        pc.pack = std::move(pack_new);
     }
-    const Plan &plan = plan_cached ? pc.plan : plan_new;
-    // the runs-only instantiation has no path for a general tile
-    if (mode == kModeRuns)
-        for (const TileDesc &d : plan.tiles)
-            if (!(d.flags & (TILE_RUN | TILE_BIG))) {
-                cudaStreamSynchronize(ctx->stream);
-                release_table(ctx);
-                return ESP_ERR_INVALID_ARG;
-            }
-    // the validation result (the copies, validation and duplicate marking ran during the planning)
     ctx->load_ms[3] = since();   // planned
+    // the validation result (the copies, validation and duplicate marking ran during the planning)
     ESP_CUDA(cudaStreamSynchronize(ctx->stream));
     ctx->load_ms[4] = since();   // uploads, validation and marks done
     const unsigned int vflags = *h_vflags;
@@ -753,88 +912,27 @@ esp_status load_common(esp_ctx *ctx, int32_t S, int32_t J, int32_t R, int32_t P,
         return ESP_ERR_INVALID_ARG;
     }
     ctx->small_units = 1;
-    for (size_t i = 0; i < (size_t)S * R; ++i)
+    std::vector<int32_t> col_max((size_t)R, 0);
+    for (size_t i = 0; i < (size_t)S * R; ++i) {
+        col_max[i % R] = std::max(col_max[i % R], h_umax[i]);
         if (h_umax[i] >= (1 << 23))
             ctx->small_units = 0;
-    ALLOC(ctx->scen_warps, (size_t)S);
-    ALLOC(ctx->scen_tiles, (size_t)S);
-    ALLOC(ctx->item_order, (size_t)std::max<int32_t>(plan.n_warps, 1));
+    }
     ALLOC(ctx->arrive, (size_t)S);
-    {
-        ctx->n_warps = plan.n_warps;
-        ctx->tile_opt = plan.tile_opt;
-        ctx->grid = (plan.n_warps + kWarpsPerCta - 1) / kWarpsPerCta;
-        ALLOC(ctx->tiles, plan.tiles.size() + 1);
-        ALLOC(ctx->warp_begin, plan.warp_begin.size());
-        std::vector<int32_t> sw((size_t)S, 0);
-        for (int32_t w = 0; w < plan.n_warps; ++w) {
-            int32_t last = -1;
-            for (int32_t k = plan.warp_begin[w]; k < plan.warp_begin[w + 1]; ++k)
-                if (plan.tiles[k].scenario != last) {
-                    last = plan.tiles[k].scenario;
-                    ++sw[last];
-                }
+    PackFormat fmt;
+    if (pack_ok && pack_format(col_max.data(), R, fmt)) {
+        if ((st = load_packed(ctx, fmt)) != ESP_OK) {
+            release_table(ctx);
+            return st;
         }
-        std::vector<int32_t> stl((size_t)S, 0);
-        for (const TileDesc &d : plan.tiles)
-            ++stl[d.scenario];
-        ESP_CUDA(cudaMemcpyAsync(ctx->scen_warps, sw.data(), sw.size() * sizeof(int32_t), cudaMemcpyHostToDevice,
-                                 ctx->stream));
-        ESP_CUDA(cudaMemcpyAsync(ctx->scen_tiles, stl.data(), stl.size() * sizeof(int32_t), cudaMemcpyHostToDevice,
-                                 ctx->stream));
-        // the ranges by the scenario of their first tile, in table order within a scenario (a sorted
-        // layout keeps each scenario's runs, large jobs and one- and two-option jobs apart)
-        std::vector<int32_t> order((size_t)plan.n_warps);
-        for (int32_t w = 0; w < plan.n_warps; ++w)
-            order[w] = w;
-        auto first_scen = [&](int32_t w) {
-            const int32_t k = plan.warp_begin[w];
-            return k < (int32_t)plan.tiles.size() ? plan.tiles[k].scenario : S;
-        };
-        std::stable_sort(order.begin(), order.end(),
-                         [&](int32_t x, int32_t y) { return first_scen(x) < first_scen(y); });
-        if (!order.empty())
-            ESP_CUDA(cudaMemcpyAsync(ctx->item_order, order.data(), order.size() * sizeof(int32_t),
-                                     cudaMemcpyHostToDevice, ctx->stream));
-        ESP_CUDA(cudaStreamSynchronize(ctx->stream));
-        if (!plan.tiles.empty())
-            ESP_CUDA(cudaMemcpyAsync(ctx->tiles, plan.tiles.data(), plan.tiles.size() * sizeof(TileDesc),
-                                     cudaMemcpyHostToDevice, ctx->stream));
-        ESP_CUDA(cudaMemcpyAsync(ctx->warp_begin, plan.warp_begin.data(), plan.warp_begin.size() * sizeof(int32_t),
-                                 cudaMemcpyHostToDevice, ctx->stream));
-        // one bulk copy per tile when every tile can take it: no job offsets needed (uniform tables,
-        // runs and chunks of the sorted layout), every tile 16-byte aligned in the interleaved copy,
-        // and its values aligned in the stage for the loads of its path (16 bytes for the paths of
-        // four options per lane, 8 otherwise)
-        const int64_t W = 4 * (int64_t)R + 8;
-        bool il_ok = ctx->il_enabled && !grouped && (ctx->uniform_k > 0 || ctx->sorted) && !plan.tiles.empty();
-        for (size_t k = 0; il_ok && k < plan.tiles.size(); ++k) {
-            const TileDesc &d = plan.tiles[k];
-            const int kk = (d.flags & TILE_RUN) ? tile_run_k(d.flags) : ctx->uniform_k;
-            const bool vec = (d.flags & TILE_BIG) ? ((d.opt_begin | (int64_t)d.n_opt) & 3) == 0 : kk >= 4;
-            il_ok = (d.opt_begin * W) % 16 == 0 && ((int64_t)d.n_opt * R * 4) % (vec ? 16 : 8) == 0 &&
-                    ((d.flags & (TILE_BIG | TILE_RUN)) || ctx->uniform_k > 0);
-        }
-        if (il_ok) {
-            const int64_t pass_opt = ctx->sorted ? ctx->s_n_opt : n_opt;
-            ALLOC_FILLED(ctx->il, (size_t)(pass_opt * W));   // the tiles cover every option
-            ctx->n_tiles = (int64_t)plan.tiles.size();
-            // units as fp32 where every unit converts exactly and the shape has that instantiation
-            ctx->il_f32 = ctx->il_f32_enabled && ctx->small_units && pass_f32_shape(R, grouped, mode);
-            ESP_CUDA(launch_interleave(pass_table(ctx), ctx->tiles, ctx->n_tiles, ctx->il, ctx->il_f32,
-                                       ctx->stream));
-            // the persistent pass: every CTA of its launch co-resident, no more warps than ranges. Used
-            // by default on uniform tables with at least kPersistMinTiles tiles per warp of its launch
-            // (measured on the what-if batch at 1024 and 256 scenarios: 16% and 19% faster per solve;
-            // at 64 scenarios, 4.5 tiles per warp, 5% slower; sorted layouts measured faster with
-            // per-round launches)
-            if (ctx->il_f32 && per_sm_persist > 0 && plan.n_warps > 0) {
-                const int64_t cap_ctas = (int64_t)per_sm_persist * ctx->sm_count;
-                const int64_t need_ctas = ((int64_t)plan.n_warps + kWarpsPerCta - 1) / kWarpsPerCta;
-                ctx->persist_grid = (int32_t)std::min(cap_ctas, need_ctas);
-                ctx->persist_auto = mode == kModeUniform &&
-                                    ctx->n_tiles >= (int64_t)kPersistMinTiles * ctx->persist_grid * kWarpsPerCta;
-            }
+    } else {
+        if (may_sort)
+            st = load_sorted(ctx);
+        if (st == ESP_OK)
+            st = load_staged(ctx);
+        if (st != ESP_OK) {
+            release_table(ctx);
+            return st;
         }
     }
 
@@ -848,25 +946,6 @@ esp_status load_common(esp_ctx *ctx, int32_t S, int32_t J, int32_t R, int32_t P,
         return st;
     }
     ESP_CUDA(cudaStreamSynchronize(ctx->stream));
-    if (!plan_cached) {   // keep this load's plan for the next load of the same offsets
-        pc.valid = true;
-        pc.S = S;
-        pc.J = J;
-        pc.R = R;
-        pc.P = P;
-        pc.grouped = grouped;
-        pc.sorted_enabled = ctx->sorted_enabled;
-        if (!cached) {
-            pc.off.assign(off_host, off_host + n_jobs + 1);
-            pc.min_k = min_k;
-            pc.max_k = max_k;
-            pc.sorted = use_sorted;
-            pc.lay = std::move(lay_new);
-        }
-        pc.max_warps = max_warps;
-        pc.tile_opt = tile_opt;
-        pc.plan = std::move(plan_new);
-    }
     ctx->load_ms[5] = since();   // tiles, interleaved table and solve state queued
     trim_pool(ctx);
     ctx->load_ms[6] = since();
@@ -907,14 +986,18 @@ bool state_ready(const esp_ctx *c)
     const void *need[] = {c->lam, c->p64, c->p32, c->ebound, c->U, c->U_final, c->hash, c->sel, c->job_val,
                           c->job_min, c->rounds_run, c->converged, c->status, c->frozen, c->feasible,
                           c->best_dual, c->primal, c->dual, c->lambda0, c->err, c->vmax, c->umax, c->stats,
-                          c->arrive, c->ver, c->work, c->cap, c->scen_warps};
+                          c->arrive, c->ver, c->work, c->cap};
     for (const void *p : need)
         if (!p)
             return false;
     if (c->placement)
         return c->place.cfg_units && c->place.cfg_values && c->place.sens && c->place.job_type &&
-               c->place.node_type && c->place.D && c->place.cfg_dup && c->place.warp_job && c->place.n_warps > 0;
-    return c->grid == 0 || (c->tiles && c->warp_begin && c->units && c->values && c->off);
+               c->place.node_type && c->place.D && c->place.cfg_dup && c->place.warp_job && c->place.n_warps > 0 &&
+               c->scen_warps;
+    if (c->packed)
+        return c->pack.data && c->pack.tiles && c->pack.job_begin && c->pack.warp_begin && c->pack.scen_tiles && c->units &&
+               c->values && c->off;
+    return c->grid == 0 || (c->scen_warps && c->tiles && c->warp_begin && c->units && c->values && c->off);
 }
 
 // The plan of the evaluation pass as the kernels take it.
@@ -928,8 +1011,6 @@ DevPlan dev_plan(const esp_ctx *c, bool fused)
     pl.uniform_k = c->uniform_k;
     pl.runs_only = (c->sorted && c->group == nullptr) ? 1 : 0;
     pl.scen_warps = fused ? c->scen_warps : nullptr;
-    pl.scen_tiles = c->scen_tiles;
-    pl.item_order = c->item_order;
     return pl;
 }
 
@@ -1039,11 +1120,16 @@ esp_status plan_resident_options(esp_ctx *ctx)
     return ESP_OK;
 }
 
-// Whether the passes of this table are launched as programmatic dependents by default: measured
-// on GB300 it pays for large uniform tables (what-if batch: -1.2% per solve) and costs on others
-// (one 2048-job scenario: +10%; the ragged 16-scenario table: +12%), so only the former use it.
+// Whether the passes of this table are launched as programmatic dependents by default. Packed passes: where
+// every warp has one tile at most, so that its step is on chip before the pass before it ends (measured
+// per round: tiny cluster 7.9 -> 6.7 us, one 2048-job cluster 11.0 -> 10.7, a ragged batch of seven
+// 1777-job clusters 14.7 -> 13.4; with several tiles per warp, heavy-tailed at 1 and 16 scenarios, 28.3 ->
+// 29.0 and 232 -> 238). Staged passes: large uniform tables (what-if batch: -1.2% per solve; one 2048-job
+// scenario: +10%, the ragged 16-scenario table: +12%).
 bool pdl_default(const esp_ctx *c)
 {
+    if (c->packed)
+        return c->pack.n_tiles <= c->pack.n_warps;
     return !c->placement && c->uniform_k > 0 && (int64_t)c->S * c->J >= (1 << 16);
 }
 
@@ -1072,6 +1158,8 @@ esp_status enqueue_solve(esp_ctx *ctx, const esp_params *p, const DevState &st, 
     const DevPlan pl = dev_plan(ctx, fused);
     const SolveArgs a = solve_args(ctx, p->eta0, p->step, p->mode, p->max_rounds, p->tol, p->flags);
     ctx->hold_tx = 0;   // the hook holds one solve only
+    DevPack pk = ctx->pack;
+    pk.fused = fused ? 1 : 0;
     const int T = p->max_rounds;
 
     const bool timed = (p->flags & ESP_FLAG_PASS_EVENTS) != 0;
@@ -1092,12 +1180,12 @@ esp_status enqueue_solve(esp_ctx *ctx, const esp_params *p, const DevState &st, 
                            st.hash_trace == nullptr && st.dual_trace == nullptr;
     const bool hold = place_res && ctx->hold_barrier;
     ctx->hold_barrier = false;
-    // rounds 0 .. T-1 in one persistent launch (fused updates, fp32 stage units, no per-pass events,
+    // rounds 0 .. T-1 in one persistent launch (fused updates, the packed copy, no per-pass events,
     // no fingerprint or dual trace: those are written by the round passes)
     const bool persist = ctx->persist_grid > 0 && (ctx->persist_mode > 0 || (ctx->persist_mode < 0 && ctx->persist_auto)) &&
                          !ctx->placement && ri < 0 && fused &&
-                         !timed && t.il_f32 && T > 0 && st.hash_trace == nullptr && st.dual_trace == nullptr &&
-                         (int64_t)T * ctx->n_tiles < (int64_t)INT32_MAX;   // items and a warp's tiles below 2^31
+                         !timed && ctx->packed && T > 0 && st.hash_trace == nullptr && st.dual_trace == nullptr &&
+                         (int64_t)T * pk.n_tiles < (int64_t)INT32_MAX - (1 << 20);   // item indices below 2^31
     auto timed_launch = [&](auto &&launch) -> cudaError_t {
         if (!timed)
             return launch();
@@ -1129,7 +1217,10 @@ esp_status enqueue_solve(esp_ctx *ctx, const esp_params *p, const DevState &st, 
             return timed_launch([&]() { return launch_place(t, st, pp, a, r, kind, ctx->place_grid, ctx->stream); });
         // without per-pass events the previous operation is always a kernel: the pass overlaps its
         // start with that kernel's tail (programmatic dependent launch)
-        return timed_launch([&]() { return launch_pass(t, st, pl, a, r, kind, ctx->grid, ctx->stream, pdl); });
+        return timed_launch([&]() {
+            return ctx->packed ? launch_packed(t, st, pk, a, r, kind, ctx->stream, pdl)
+                               : launch_pass(t, st, pl, a, r, kind, ctx->grid, ctx->stream, pdl);
+        });
     };
     auto issue = [&]() -> cudaError_t {
         cudaError_t e = launch_init(t, st, a, has_l0 ? ctx->lambda0 : nullptr, ctx->stream);
@@ -1155,10 +1246,10 @@ esp_status enqueue_solve(esp_ctx *ctx, const esp_params *p, const DevState &st, 
         }
         if (persist) {
             if (e == cudaSuccess)
-                e = launch_pass_persist(t, st, pl, a, T, ctx->persist_grid, ctx->stream);
+                e = launch_packed_persist(t, st, pk, a, T, ctx->persist_grid, ctx->stream);
             // after the cooperative launch the final pass starts as an ordinary launch
             if (e == cudaSuccess)
-                e = launch_pass(t, st, pl, a, T, PASS_FINAL, ctx->grid, ctx->stream, false);
+                e = launch_packed(t, st, pk, a, T, PASS_FINAL, ctx->stream, false);
             if (e == cudaSuccess)
                 e = launch_objectives(t, st, a, ctx->stream);
             return e;
@@ -1213,6 +1304,7 @@ esp_status enqueue_solve(esp_ctx *ctx, const esp_params *p, const DevState &st, 
         mix(&t_orig, sizeof(t_orig));
         mix(&st, sizeof(st));
         mix(&pl, sizeof(pl));
+        mix(&pk, sizeof(pk));
         mix(&a, sizeof(a));
         mix(&pp, sizeof(pp));
         mix(&ctx->lambda0, sizeof(ctx->lambda0));
@@ -1404,7 +1496,13 @@ esp_status esp_load_options(esp_ctx *ctx, int32_t S, int32_t J, int32_t R, int32
     LoadStreamScope scope(ctx);
     if ((st = scope.begin()) != ESP_OK)
         return st;
-    return load_common(ctx, S, J, R, P, r_global, job_offsets, units, values, group, capacity, false);
+    try {
+        return load_common(ctx, S, J, R, P, r_global, job_offsets, units, values, group, capacity, false);
+    } catch (const std::bad_alloc &) {   // host memory for the plan; no exception crosses the C boundary
+        cudaStreamSynchronize(ctx->stream);
+        release_table(ctx);
+        return ESP_ERR_OOM;
+    }
 }
 
 esp_status esp_load_options_device(esp_ctx *ctx, int32_t S, int32_t J, int32_t R, int32_t P, int32_t r_global,
@@ -1417,7 +1515,13 @@ esp_status esp_load_options_device(esp_ctx *ctx, int32_t S, int32_t J, int32_t R
     LoadStreamScope scope(ctx);
     if ((st = scope.begin()) != ESP_OK)
         return st;
-    return load_common(ctx, S, J, R, P, r_global, job_offsets, units, values, group, capacity, true);
+    try {
+        return load_common(ctx, S, J, R, P, r_global, job_offsets, units, values, group, capacity, true);
+    } catch (const std::bad_alloc &) {   // host memory for the plan; no exception crosses the C boundary
+        cudaStreamSynchronize(ctx->stream);
+        release_table(ctx);
+        return ESP_ERR_OOM;
+    }
 }
 
 esp_status esp_solve_async(esp_ctx *ctx, const esp_params *params)
@@ -1593,6 +1697,8 @@ esp_status esp_evaluate(esp_ctx *ctx, const double *lambda, int32_t mode, uint32
     ESP_CUDA(launch_init(t, ds, a, ctx->lambda0, ctx->stream));
     if (ctx->placement)
         ESP_CUDA(launch_place(t, ds, ctx->place, a, 0, PASS_FINAL, ctx->place_grid, ctx->stream));
+    else if (ctx->packed)
+        ESP_CUDA(launch_packed(t, ds, ctx->pack, a, 0, PASS_FINAL, ctx->stream, false));
     else if (ctx->grid > 0)
         ESP_CUDA(launch_pass(t, ds, pl, a, 0, PASS_FINAL, ctx->grid, ctx->stream));
     ESP_CUDA(launch_objectives(t, ds, a, ctx->stream));
@@ -1809,7 +1915,9 @@ esp_status refresh_after_values(esp_ctx *ctx, unsigned int *vflags)
     if (ctx->sorted)
         ESP_CUDA(launch_gather_sorted(t, pass_table(ctx), ctx->s_units, ctx->s_values, ctx->stream));
     if (ctx->il)
-        ESP_CUDA(launch_interleave(pass_table(ctx), ctx->tiles, ctx->n_tiles, ctx->il, ctx->il_f32, ctx->stream));
+        ESP_CUDA(launch_interleave(pass_table(ctx), ctx->tiles, ctx->n_tiles, ctx->il, ctx->stream));
+    if (ctx->packed)
+        ESP_CUDA(launch_pack(t, ctx->pack, ctx->pk_data, ctx->stream));
     ESP_CUDA(cudaMemcpyAsync(vflags, ctx->valflags, sizeof(unsigned int), cudaMemcpyDeviceToHost, ctx->stream));
     ESP_CUDA(cudaStreamSynchronize(ctx->stream));
     return ESP_OK;
@@ -2174,7 +2282,7 @@ esp_status esp_debug_pass_kernel(esp_ctx *ctx, int32_t *kind)
         return ESP_ERR_INVALID_ARG;
     if (!ctx->loaded)
         return ESP_ERR_NOT_LOADED;
-    *kind = ctx->placement ? 2 : ctx->il ? (ctx->il_f32 ? 3 : 1) : 0;
+    *kind = ctx->placement ? 2 : ctx->persist_grid > 0 ? 3 : (ctx->packed || ctx->il) ? 1 : 0;   // 3 only when packed
     return ESP_OK;
 }
 

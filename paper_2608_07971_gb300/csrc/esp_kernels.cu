@@ -167,14 +167,8 @@ int pass_smem_bytes(int R, bool grouped, int mode, int P, int tile_opt)
 int pass_ctas_per_sm(int R, bool grouped, int mode, int P, int tile_opt)
 {
     const int smem = pass_smem_bytes(R, grouped, mode, P, tile_opt);
-    int n = dispatch_shape(R, grouped, mode,
-                           [&](auto k) -> int { return pass_kernels_ctas_per_sm<decltype(k)>(smem); });
-    if (n > 0 && pass_f32_shape(R, grouped, mode)) {
-        // the plan must also suit the instantiation that reads fp32 stage units
-        const int m = pass_ctas_per_sm_f32(R, mode, smem);
-        n = m < n ? m : n;
-    }
-    return n;
+    return dispatch_shape(R, grouped, mode,
+                          [&](auto k) -> int { return pass_kernels_ctas_per_sm<decltype(k)>(smem); });
 }
 
 cudaError_t launch_init(const DevTable &t, const DevState &st, const SolveArgs &a, const double *lambda0,
@@ -192,8 +186,6 @@ cudaError_t launch_pass(const DevTable &t, const DevState &st, const DevPlan &pl
     const int mode = pass_mode(pl);
     const int smem = pass_smem_bytes(t.R, grouped, mode, t.P, pl.tile_opt);
     const bool plain = kind == PASS_ROUND && st.hash_trace == nullptr && st.dual_trace == nullptr;
-    if (t.il_f32)
-        return launch_pass_f32(t, st, pl, a, round, kind, grid, smem, stream, pdl);
     dispatch_shape(t.R, grouped, mode, [&](auto k) -> int {
         decltype(k)::launch(plain, grid, smem, stream, t, st, pl, a, round, kind, pdl);
         return 0;

@@ -1,0 +1,1070 @@
+// Evaluation passes over the packed screen copy (esp_packed.h) of the ESP tatonnement (Sec. 3.2.2 and
+// 3.2.3) for sm_103a: one launch per round with the price update fused in, and every round of a solve
+// in one cooperative launch.
+//
+// What bounds them: a table larger than L2 streams from HBM every round. The passes this design
+// replaced staged 4R + 8 bytes per option through shared memory, 128 options at a time; the what-if batch
+// (R = 6, 32 bytes per option) ran at 0.995 of the copy bandwidth with 88% of the issue slots taken (668
+// warp instructions per 128 options), so neither fewer bytes nor fewer instructions alone would have
+// helped. Here an option takes 16 bytes, a warp screens 256 options per step, eight per lane, and a step is
+// one bulk copy into one of the warp's two slots, two steps ahead.
+//
+// Screen. A lane screens eight consecutive options of a job. Unit fields become floats by inserting the
+// exponent of 2^23 (one logic op for a low field, one funnel shift for a high field) and subtracting
+// 2^23, exactly; the two fields of a word run as one packed fp32 pair (add.rn.f32x2, fma.rn.f32x2), the
+// low fields accumulating from -v, the high fields from 0, and q is the sum of both chains. Against the
+// exact score each chain has at most R roundings and the last sum one more, each within 2^-24 of
+// M = |v| + sum_r p_r u_r, so |q - s| <= (R + 4) u M (1 + small) + 2^-99 holds as for the chain in column
+// order, and the decision rule and its proof are those of esp_kernels.cu.
+//
+// The winner's units come from the words in the slot. Values in fp64 and int32 units are read from
+// the table itself, only to rescore the survivors of ambiguous jobs and for the outputs of the final
+// pass.
+
+#include <algorithm>
+#include <cmath>
+#include <cstdint>
+#include <cuda_runtime.h>
+
+#include "esp_device.cuh"
+#include "esp_kernels.h"
+#include "esp_ptx.cuh"
+#include "esp_warp.cuh"
+
+namespace esp {
+
+namespace {
+
+#ifndef ESP_PACK_CTAS
+#define ESP_PACK_CTAS 5
+#endif
+constexpr int kPackWarps = 4;        // warps per CTA
+constexpr int kPackSlots = 2;        // steps a warp holds: the one being screened and one on its way
+// Winners a lane's 32-bit sums may take between flushes: each is below 2^23, so 511 fit; a tile adds at
+// most 8 per step and kPackTileSteps (8) steps (a job of more steps counts once).
+constexpr uint32_t kPackSpill = 511 - 8 * 8;
+
+// Resident CTAs the register budget must allow.
+constexpr int pack_min_ctas(int nw)
+{
+    return nw <= 3 ? ESP_PACK_CTAS : nw == 4 ? 5 : 4;
+}
+
+// Shared memory of a warp: the slots, then their barriers.
+__host__ __device__ constexpr int pack_slot_bytes(int nw)
+{
+    return (nw + 1) * kPackStepVecs * 16;
+}
+__host__ __device__ constexpr int pack_warp_bytes(int nw)
+{
+    return kPackSlots * pack_slot_bytes(nw) + 16;
+}
+
+__device__ __forceinline__ unsigned long long pack2(float lo, float hi)
+{
+    unsigned long long r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+
+__device__ __forceinline__ float2 unpack2(unsigned long long v)
+{
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+}
+
+__device__ __forceinline__ unsigned long long add2(unsigned long long a, unsigned long long b)
+{
+    unsigned long long r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+
+__device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigned long long b, unsigned long long c)
+{
+    unsigned long long r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+
+// Smallest value over the warp (one hardware reduction).
+__device__ __forceinline__ float warp_min_f32(float x)
+{
+    float r;
+    asm volatile("redux.sync.min.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(x));
+    return r;
+}
+
+// The warp's state for the scenario it is in.
+template <int NW>
+struct Ctx {
+    unsigned long long price[NW];   // fp32 prices of word k's (low, high) fields
+    uint32_t lo[NW], hi[NW];        // the lane's demand since the last flush, per field
+    uint32_t wins;                  // upper bound of the winners in them
+    unsigned long long hash;
+    const double *p64;              // fp64 prices of the scenario
+    float e2;                       // 2E, +inf: exact evaluation
+    bool exact, skip;
+    int s;                          // scenario, -1: none
+    int tiles;                      // tiles evaluated since the last arrival
+    unsigned int resolved;
+};
+
+// Scores of the four options of vector `v` of plane 0; the other planes follow `plane` vectors apart.
+template <int NW>
+__device__ __forceinline__ void screen4(const uint4 *v, int plane, const PackFormat &f, const Ctx<NW> &c, float *q)
+{
+    const unsigned long long bias = pack2(-8388608.0f, -8388608.0f);
+    const uint4 n = v[0];
+    unsigned long long acc[4] = {pack2(__uint_as_float(n.x), 0.0f), pack2(__uint_as_float(n.y), 0.0f),
+                                 pack2(__uint_as_float(n.z), 0.0f), pack2(__uint_as_float(n.w), 0.0f)};
+#pragma unroll
+    for (int k = 0; k < NW; ++k) {
+        const uint4 y = v[(k + 1) * plane];
+        const uint32_t x[4] = {y.x, y.y, y.z, y.w};
+#pragma unroll
+        for (int o = 0; o < 4; ++o) {
+            const uint32_t lo = (x[o] & f.mask[k]) | 0x4b000000u;
+            const uint32_t hi = __funnelshift_r(x[o], f.magic[k], f.shift[k]);
+            acc[o] = fma2(c.price[k], add2(pack2(__uint_as_float(lo), __uint_as_float(hi)), bias), acc[o]);
+        }
+    }
+#pragma unroll
+    for (int o = 0; o < 4; ++o) {
+        const float2 t = unpack2(acc[o]);
+        q[o] = t.x + t.y;
+    }
+}
+
+// Smallest and second smallest of four.
+__device__ __forceinline__ void two_smallest(const float *q, float &m1, float &m2)
+{
+    const float a0 = fminf(q[0], q[1]), a1 = fmaxf(q[0], q[1]);
+    const float b0 = fminf(q[2], q[3]), b1 = fmaxf(q[2], q[3]);
+    m1 = fminf(a0, b0);
+    m2 = fminf(fmaxf(a0, b0), fminf(a1, b1));
+}
+
+// Adds the units in the word at w (plane 0) to the lane's demand.
+template <int NW>
+__device__ __forceinline__ void add_option(Ctx<NW> &c, const PackFormat &f, const uint32_t *w, int plane)
+{
+#pragma unroll
+    for (int k = 0; k < NW; ++k) {
+        const uint32_t x = w[(k + 1) * plane * 4];
+        c.lo[k] += x & f.mask[k];
+        c.hi[k] += x >> f.shift[k];
+    }
+}
+
+// Everything a pass needs beyond the warp's own state.
+struct Pass {
+    const DevTable &t;
+    const DevState &st;
+    const DevPack &pk;
+    const SolveArgs &a;
+    int round, kind, lane;
+    bool want_min, want_hash;   // minimal reduced costs; selection fingerprints
+};
+
+// The exact score of option o of the pass table (the chain of Eq. esp_score in column order).
+__device__ __forceinline__ double exact_option(const int32_t *units, const double *values, int R, const double *p64,
+                                               int64_t o)
+{
+    const int32_t *u = units + o * R;
+    double s = -__ldg(values + o);
+    for (int r = 0; r < R; ++r) {
+        const int32_t x = __ldg(u + r);
+        // prices through L2: a persistent pass sees them change between rounds
+        s = __fma_rn(__ldcg(p64 + r), __int2double_rn(r == 0 ? (x & 0x7fffffff) : x), s);
+    }
+    return s;
+}
+
+struct Exact {
+    long long key;
+    int idx;
+};
+
+// The lexicographic minimum of (s, index) over the options first + i, i in the bits of `mask`, in fp64;
+// their indices are loc + i. (Ambiguous jobs only; out of line it made the row loops spill around the call.)
+__device__ __forceinline__ Exact rescore(const int32_t *units, const double *values, int R, const double *p64,
+                                      int64_t first, uint32_t mask, int loc)
+{
+    Exact x{0x7fffffffffffffffLL, kIdxNone};
+    while (mask != 0u) {
+        const int i = __ffs((int)mask) - 1;
+        mask &= mask - 1;
+        const long long k = order_key(exact_option(units, values, R, p64, first + i));
+        if (k < x.key) {   // increasing index: the first of equal scores stays
+            x.key = k;
+            x.idx = loc + i;
+        }
+    }
+    return x;
+}
+
+// The minimum of (key, idx) over aligned groups of `lanes` lanes.
+__device__ __forceinline__ Exact group_min(Exact x, int lanes)
+{
+    for (int d = 1; d < lanes; d <<= 1) {
+        const long long ok = __shfl_xor_sync(FULL, x.key, d);
+        const int oi = __shfl_xor_sync(FULL, x.idx, d);
+        if (ok < x.key || (ok == x.key && oi < x.idx)) {
+            x.key = ok;
+            x.idx = oi;
+        }
+    }
+    return x;
+}
+
+// Options of a vector that survive the screen (q <= thr; in exact mode every option but duplicates and
+// padding); n: their -v32 words.
+__device__ __forceinline__ uint32_t survivors(const uint4 &n, const float *q, bool exact, float thr)
+{
+    return ((n.x != kPackInf && (exact || q[0] <= thr)) ? 1u : 0u) |
+           ((n.y != kPackInf && (exact || q[1] <= thr)) ? 2u : 0u) |
+           ((n.z != kPackInf && (exact || q[2] <= thr)) ? 4u : 0u) |
+           ((n.w != kPackInf && (exact || q[3] <= thr)) ? 8u : 0u);
+}
+
+// Table job and first option of job jl of tile k.
+struct JobAt {
+    int64_t job, opt0;
+};
+
+__device__ __forceinline__ JobAt job_at(const Pass &ps, int k, int jl)
+{
+    const int i = __ldg(ps.pk.job_begin + k) + jl;
+    JobAt x;
+    x.job = ps.pk.job ? __ldg(ps.pk.job + i) : i;
+    x.opt0 = __ldg(ps.t.job_off + x.job);
+    return x;
+}
+
+// Outputs of a winner beyond its demand: its job, local index and, when known, exact score.
+template <int NW>
+__device__ __forceinline__ void extras(const Pass &ps, Ctx<NW> &c, const JobAt &at, int local, bool have_s, long long key)
+{
+    if (ps.want_hash)
+        c.hash += splitmix64_mix(((uint64_t)(uint32_t)(at.job - (int64_t)c.s * ps.t.J) << 32) | (uint32_t)local);
+    if (ps.kind == PASS_FINAL) {
+        ps.st.sel[at.job] = local;
+        ps.st.job_val[at.job] = __ldg(ps.t.values + at.opt0 + local);
+    }
+    if (ps.want_min)
+        ps.st.job_min[at.job] = have_s ? key_value(key)
+                                       : exact_option(ps.t.units, ps.t.values, ps.t.R, c.p64, at.opt0 + local);
+}
+
+// Adds the lane's demand to the scenario's totals: every sum across the warp by two hardware reductions
+// of 16-bit halves (each below 2^21), then one atomic per field, all fields in one instruction.
+template <int NW>
+__device__ __forceinline__ void add_demand(const Pass &ps, Ctx<NW> &c)
+{
+    unsigned long long *dst = (ps.kind == PASS_ROUND ? ps.st.U : ps.st.U_final) + (size_t)c.s * ps.t.P;
+    unsigned long long mine = 0ull;
+    int col = -1;
+#pragma unroll
+    for (int i = 0; i < 2 * NW; ++i) {
+        const uint32_t v = (i & 1) ? c.hi[i >> 1] : c.lo[i >> 1];
+        const unsigned long long x = (unsigned long long)__reduce_add_sync(FULL, v & 0xffffu) +
+                                     ((unsigned long long)__reduce_add_sync(FULL, v >> 16) << 16);
+        if (ps.lane == i) {
+            mine = x;
+            col = (i & 1) ? ps.pk.fmt.col_hi[i >> 1] : ps.pk.fmt.col_lo[i >> 1];
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < NW; ++k)
+        c.lo[k] = c.hi[k] = 0u;
+    if (col >= 0 && mine != 0ull)
+        atomicAdd(dst + col, mine);
+    c.wins = 0;
+}
+
+// Eq. price_update for scenario s of a table without a group column after round `round` (one warp, lane k
+// holds price k: P = R <= 16), as update_scenario does it, with every input loaded at once and the new
+// prices and bound computed from registers. The chain of dependent trips to L2 is what this costs (it
+// is the serial end of every round): one here, three when the new prices went through memory
+// between the update, the effective prices and the bound.
+__device__ __forceinline__ void update_flat(const DevTable &t, const DevState &st, const SolveArgs &a, int s, int round,
+                                            int lane)
+{
+    const int P = t.P, J = t.J, T = a.T;
+    const size_t sp = (size_t)s * P;
+    const bool mine = lane < P;
+    long long U = 0, C = 1;
+    double lam = 0.0;
+    int umax = 0;
+    if (mine) {
+        U = (long long)__ldcg(st.U + sp + lane);
+        C = __ldg(t.cap + sp + lane);
+        lam = __ldcg(st.lam + sp + lane);
+        umax = __ldg(st.umax + sp + lane);   // R = P
+    }
+    const double vmax = __ldg(st.vmax + s);
+    const double Cd = (double)C;
+
+    if (st.dual_trace) {   // g(lambda^t) from the minimal reduced costs of round t
+        double part = 0.0;
+        for (int j = lane; j < J; j += 32)
+            part += -__ldcg(st.job_min + (size_t)s * J + j);
+        const double lc = mine ? ((a.mode == 1) ? lam : lam * Cd) : 0.0;
+        const double g = warp_sum_fixed(part) + warp_sum_fixed(lc);
+        if (lane == 0) {
+            st.dual_trace[(size_t)s * (T + 1) + round] = g;
+            if (g < st.best_dual[s])
+                st.best_dual[s] = g;
+        }
+    }
+    if (st.hash_trace && lane == 0) {
+        st.hash_trace[(size_t)s * T + round] = __ldcg(st.hash + s);
+        st.hash[s] = 0ull;
+    }
+    if (st.dem_trace && mine)
+        st.dem_trace[((size_t)s * T + round) * P + lane] = U;
+    if (mine)
+        st.U[sp + lane] = 0ull;
+
+    const double nl = mine ? price_step(lam, U, C, Cd, step_size(a.eta0, a.step, round), a.mode) : 0.0;
+    if (__any_sync(FULL, mine && !isfinite(nl))) {
+        if (lane == 0) {
+            st.status[s] = 2;
+            st.frozen[s] = 1;
+        }
+        return;
+    }
+    const double p = mine ? effective_price(nl, Cd, a.mode) : 0.0;
+    if (mine) {
+        st.lam[sp + lane] = nl;
+        st.p64[sp + lane] = p;
+        st.p32[sp + lane] = __double2float_rn(p);
+        if (st.lam_trace)
+            st.lam_trace[((size_t)s * (T + 1) + round + 1) * P + lane] = nl;
+    }
+    const bool huge = __any_sync(FULL, mine && !(p <= 0x1p100));
+    const double M = vmax + warp_sum_fixed(mine ? p * (double)umax : 0.0);
+    bool conv = false;
+    if (a.tol > 0.0) {
+        const double dmax = warp_max(mine ? fabs(nl - lam) : 0.0), amax = warp_max(mine ? fabs(lam) : 0.0);
+        conv = dmax <= a.tol * fmax(1.0, amax);
+    }
+    if (lane == 0) {
+        st.ebound[s] = screen_bound(M, t.R, a.exact_only || huge);
+        if (st.time_trace)
+            st.time_trace[(size_t)s * T + round] = global_ns();
+        st.rounds_run[s] = round + 1;
+        if (conv) {
+            st.converged[s] = 1;
+            st.frozen[s] = 1;
+        }
+    }
+}
+
+// The update of scenario s after `round`, by the warp whose arrival completed it; persist: then its
+// version, which releases the scenario's next round (a stopped scenario releases every later one).
+__device__ __forceinline__ void finish_scenario(const DevTable &t, const DevState &st, const SolveArgs &a, int s, int round,
+                                             int lane, bool persist)
+{
+    asm volatile("fence.acq_rel.gpu;" ::: "memory");
+    update_flat(t, st, a, s, round, lane);
+    if (lane == 0)
+        st.arrive[s] = 0u;   // every tile of the round has arrived
+    if (persist) {
+        // every lane's writes (prices, bound, cleared demand) before the version
+        __threadfence();
+        __syncwarp();
+        if (lane == 0) {
+            const unsigned int v = st.frozen[s] ? kVerStopped : (unsigned int)(round + 1);
+            asm volatile("st.release.gpu.u32 [%0], %1;" ::"l"(st.ver + s), "r"(v) : "memory");
+        }
+    }
+}
+
+// The end of the warp's work on its scenario for now: demand and fingerprint, then (round passes with
+// fused updates) the arrival of the tiles evaluated; the arrival that completes the scenario applies
+// Eq. price_update. Every lane may have issued demand atomics or written reduced costs: the warp barrier
+// orders them before lane 0's release-ordered (cumulative) arrival, which publishes them.
+template <int NW, bool PERSIST>
+__device__ __forceinline__ void leave(const Pass &ps, Ctx<NW> &c)
+{
+    if (c.s < 0 || c.skip)
+        return;
+    add_demand(ps, c);
+    if (ps.want_hash) {
+        unsigned long long h = c.hash;
+#pragma unroll
+        for (int d = 16; d >= 1; d >>= 1)
+            h += __shfl_xor_sync(FULL, h, d);
+        if (ps.lane == 0)
+            atomicAdd(ps.st.hash + c.s, h);
+        c.hash = 0ull;
+    }
+    if (ps.kind != PASS_ROUND || !ps.pk.fused)
+        return;
+    __syncwarp();
+    unsigned int old = 0;
+    if (ps.lane == 0)
+        asm volatile("atom.add.release.gpu.u32 %0, [%1], %2;"
+                     : "=r"(old)
+                     : "l"(ps.st.arrive + c.s), "r"((unsigned int)c.tiles)
+                     : "memory");
+    old = __shfl_sync(FULL, old, 0);
+    if (old + (unsigned int)c.tiles == (unsigned int)__ldg(ps.pk.scen_tiles + c.s))
+        finish_scenario(ps.t, ps.st, ps.a, c.s, ps.round, ps.lane, PERSIST);
+}
+
+// Prices, bound and state of scenario s (through L2: another warp of this launch may have written them).
+template <int NW>
+__device__ __forceinline__ void enter(const Pass &ps, Ctx<NW> &c, int s)
+{
+    const DevState &st = ps.st;
+    const size_t sp = (size_t)s * ps.t.P;
+    const PackFormat &f = ps.pk.fmt;
+    c.s = s;
+    c.tiles = 0;
+    const int frozen = __ldcg(st.frozen + s);
+    const float e = __ldcg(st.ebound + s);
+#pragma unroll
+    for (int k = 0; k < NW; ++k) {
+        const float pl = f.col_lo[k] >= 0 ? __ldcg(st.p32 + sp + f.col_lo[k]) : 0.0f;
+        const float ph = f.col_hi[k] >= 0 ? __ldcg(st.p32 + sp + f.col_hi[k]) : 0.0f;
+        c.price[k] = pack2(pl, ph);
+    }
+    c.skip = ps.kind == PASS_ROUND && frozen != 0;
+    c.exact = !(e < INFINITY);
+    c.e2 = c.exact ? INFINITY : 2.0f * e;
+    c.p64 = st.p64 + sp;
+}
+
+// A step of whole jobs of 3 .. 256 options: each job has 2^code lanes, its lane sub the options
+// sub << per .. (per = 3: eight, per = 2: four) as vectors ia and ib of the slot (has_a, has_b: they exist; +inf past a job's end and in the
+// jobs missing from a tile's last step). The lane's job is job jl of tile k, which has n_job. An
+// unambiguous job's winner is the one option that holds the smallest score.
+template <int NW, bool PLAIN>
+__device__ __forceinline__ void step_jobs(const Pass &ps, Ctx<NW> &c, const uint4 *slot, int V, int ia, int ib, bool has_a,
+                                          bool has_b, bool any_b, int code, int per, int k, int jl, int n_job)
+{
+    float qa[4], qb[4] = {INFINITY, INFINITY, INFINITY, INFINITY};
+    float a1, a2, b1 = INFINITY, b2 = INFINITY;
+    screen4<NW>(slot + ia, V, ps.pk.fmt, c, qa);
+    two_smallest(qa, a1, a2);
+    if (any_b) {
+        screen4<NW>(slot + ib, V, ps.pk.fmt, c, qb);
+        two_smallest(qb, b1, b2);
+    }
+    a1 = has_a ? a1 : INFINITY;
+    a2 = has_a ? a2 : INFINITY;
+    b1 = has_b ? b1 : INFINITY;
+    b2 = has_b ? b2 : INFINITY;
+    const float l1 = fminf(a1, b1);
+    float m1 = l1, m2 = fminf(fmaxf(a1, b1), fminf(a2, b2));
+    if (code == 5) {
+        // one job on all lanes: the lane that holds the smallest offers its second smallest, the others
+        // their smallest; two lanes with the same smallest make both equal
+        m1 = warp_min_f32(l1);
+        const uint32_t holders = __ballot_sync(FULL, l1 == m1);
+        const float o = warp_min_f32(l1 == m1 ? m2 : l1);
+        m2 = (holders & (holders - 1u)) ? m1 : o;
+    } else {
+        for (int d = 1; d < (1 << code); d <<= 1) {
+            const float o1 = __shfl_xor_sync(FULL, m1, d);
+            const float o2 = __shfl_xor_sync(FULL, m2, d);
+            m2 = fminf(fminf(m2, o2), fmaxf(m1, o1));
+            m1 = fminf(m1, o1);
+        }
+    }
+    const float thr = __fadd_ru(m1, c.e2);
+    const bool amb = c.exact ? jl < n_job : (m1 < INFINITY && !(m2 > thr));
+    bool mine = !amb && m1 < INFINITY && l1 == m1;   // held by one option only: a tie would make m2 = m1
+    int o = a1 == m1 ? (qa[0] == m1 ? 0 : qa[1] == m1 ? 1 : qa[2] == m1 ? 2 : 3)
+                     : (qb[0] == m1 ? 4 : qb[1] == m1 ? 5 : qb[2] == m1 ? 6 : 7);
+    bool have_s = false;
+    long long key = 0;
+    if (__any_sync(FULL, amb)) {
+        const int loc = (ps.lane & ((1 << code) - 1)) << per;
+        Exact x{0x7fffffffffffffffLL, kIdxNone};
+        if (amb) {
+            const uint32_t sv = (has_a ? survivors(slot[ia], qa, c.exact, thr) : 0u) |
+                                (has_b ? survivors(slot[ib], qb, c.exact, thr) << 4 : 0u);
+            if (sv != 0u)
+                x = rescore(ps.t.units, ps.t.values, ps.t.R, c.p64, job_at(ps, k, jl).opt0 + loc, sv, loc);
+        }
+        x = group_min(x, 1 << code);
+        if (amb && x.idx >= loc && x.idx < loc + (1 << per)) {
+            mine = have_s = true;
+            o = x.idx - loc;
+            key = x.key;
+            ++c.resolved;
+        }
+    }
+    if (mine) {
+        add_option<NW>(c, ps.pk.fmt, reinterpret_cast<const uint32_t *>(slot + (o < 4 ? ia : ib)) + (o & 3), V);
+        if (!PLAIN)
+            extras<NW>(ps, c, job_at(ps, k, jl), ((ps.lane & ((1 << code) - 1)) << per) + o, have_s, key);
+    }
+}
+
+// Four consecutive options of a tile whose jobs have one or two: jobs j0 .. of tile k, `n` of them left in
+// it. v: the vector.
+template <int NW, bool PLAIN>
+__device__ __forceinline__ void step_tiny(const Pass &ps, Ctx<NW> &c, const uint4 *v, int V, int K, int k, int j0, int n)
+{
+    float q[4];
+    screen4<NW>(v, V, ps.pk.fmt, c, q);
+    const uint32_t *w = reinterpret_cast<const uint32_t *>(v);
+#pragma unroll
+    for (int h = 0; h < 4; ++h) {
+        if (K == 2 && (h & 1))
+            continue;
+        const int jl = K == 2 ? h >> 1 : h;
+        if (jl >= n)
+            continue;
+        int o = h;
+        bool have_s = false;
+        long long key = 0;
+        if (K == 2) {
+            const float qa = q[h], qb = q[(h + 1) & 3];
+            const float thr = __fadd_ru(fminf(qa, qb), c.e2);
+            o = qb < qa ? h + 1 : h;
+            if (c.exact || !(fmaxf(qa, qb) > thr)) {   // ambiguous
+                const uint32_t sv = (survivors(v[0], q, c.exact, thr) >> h) & 3u;
+                const Exact x = rescore(ps.t.units, ps.t.values, ps.t.R, c.p64, job_at(ps, k, j0 + jl).opt0, sv, h);
+                o = x.idx;
+                key = x.key;
+                have_s = true;
+                ++c.resolved;
+            }
+        }
+        add_option<NW>(c, ps.pk.fmt, w + o, V);
+        if (!PLAIN)
+            extras<NW>(ps, c, job_at(ps, k, j0 + jl), o - h, have_s, key);
+    }
+}
+
+// A job of more than 256 options, step by step: each lane keeps the best of its own options; the job's
+// last step reduces across the warp, and the winner's words, read again from the packed copy, are added
+// when the next job closes (or the tile ends), so that no job waits for them.
+template <int NW>
+struct Large {
+    float m1, m2;
+    int idx;
+    uint32_t x[NW];   // words of the previous job's winner, zero on the other lanes
+};
+
+template <int NW>
+__device__ __forceinline__ void add_pending(Ctx<NW> &c, const PackFormat &f, Large<NW> &b)
+{
+#pragma unroll
+    for (int k = 0; k < NW; ++k) {
+        c.lo[k] += b.x[k] & f.mask[k];
+        c.hi[k] += b.x[k] >> f.shift[k];
+        b.x[k] = 0u;
+    }
+}
+
+// The packed vector (plane 0) that holds vector `vec` of a large job whose data start at `base`.
+template <int NW>
+__device__ __forceinline__ const uint4 *large_vec(const uint4 *base, const PackShape &sh, int vec)
+{
+    const int step = vec / sh.v, x = vec - step * sh.v;
+    return base + (int64_t)step * sh.v * (NW + 1) + ((x & 1) ? sh.ca + (x >> 1) : x >> 1);
+}
+
+// Survivors of a large job in fp64 when a lane may hold several: its packed vectors are screened again (the
+// same instructions give the same q).
+template <int NW>
+__device__ __forceinline__ Exact rescan_large(const Pass &ps, const Ctx<NW> &c, const uint4 *base, const PackShape &sh,
+                                              int64_t opt0, float thr)
+{
+    Exact x{0x7fffffffffffffffLL, kIdxNone};
+    for (int g = ps.lane; g < sh.m; g += 32) {
+        const uint4 *v = large_vec<NW>(base, sh, g);
+        float q[4];
+        screen4<NW>(v, sh.v, ps.pk.fmt, c, q);
+        const Exact y = rescore(ps.t.units, ps.t.values, ps.t.R, c.p64, opt0 + 4 * g, survivors(v[0], q, c.exact, thr), 4 * g);
+        if (y.key < x.key)
+            x = y;
+    }
+    return x;
+}
+
+template <int NW, bool PLAIN>
+__device__ __forceinline__ void close_large(const Pass &ps, Ctx<NW> &c, const uint4 *base, const PackShape &sh, int k,
+                                            int jl, Large<NW> &b)
+{
+    add_pending(c, ps.pk.fmt, b);
+    const float m1 = warp_min_f32(b.m1);
+    const bool first = b.m1 == m1;
+    const uint32_t holders = __ballot_sync(FULL, first);
+    const float o2 = warp_min_f32(first ? b.m2 : b.m1);
+    const float m2 = (holders & (holders - 1u)) ? m1 : o2;
+    const float thr = __fadd_ru(m1, c.e2);
+    bool mine = first, have_s = false;
+    int win = b.idx;
+    long long key = 0;
+    if (c.exact || !(m2 > thr)) {
+        const int64_t opt0 = job_at(ps, k, jl).opt0;
+        Exact x{0x7fffffffffffffffLL, kIdxNone};
+        if (!c.exact && !__any_sync(FULL, b.m2 <= thr)) {   // every lane's own best at most
+            if (b.m1 <= thr)
+                x = rescore(ps.t.units, ps.t.values, ps.t.R, c.p64, opt0 + b.idx, 1u, b.idx);
+        } else {
+            x = rescan_large<NW>(ps, c, base, sh, opt0, thr);
+        }
+        const int own = x.idx;
+        x = group_min(x, 32);
+        win = x.idx;
+        key = x.key;
+        have_s = true;
+        mine = own == win;
+        if (mine)
+            ++c.resolved;
+    }
+    if (mine) {
+        const uint32_t *w = reinterpret_cast<const uint32_t *>(large_vec<NW>(base, sh, win >> 2)) + (win & 3);
+#pragma unroll
+        for (int i = 0; i < NW; ++i)
+            b.x[i] = __ldg(w + (i + 1) * sh.v * 4);
+        if (!PLAIN)
+            extras<NW>(ps, c, job_at(ps, k, jl), win, have_s, key);
+    }
+    b.m1 = b.m2 = INFINITY;
+    b.idx = kIdxNone;
+}
+
+template <int NW>
+__device__ __forceinline__ void reset(Ctx<NW> &c)
+{
+    c.s = -1;
+    c.skip = false;
+    c.tiles = 0;
+    c.wins = 0;
+    c.hash = 0ull;
+    c.resolved = 0;
+#pragma unroll
+    for (int k = 0; k < NW; ++k)
+        c.lo[k] = c.hi[k] = 0u;
+}
+
+// One warp's work: the tiles `next` hands out (its index, its round in *round; -1 when there are no
+// more), evaluated in order. Lane 0 copies the step after the one in flight as soon as its slot is free,
+// across tiles; a tile's record is loaded while the tile before it is evaluated. hold_tx: see SolveArgs.
+template <int NW, bool PLAIN, bool PERSIST, typename Next>
+__device__ __forceinline__ void run_warp(const DevTable &t, const DevState &st, const DevPack &pk, const SolveArgs &a,
+                                         int round, int kind, unsigned char *smem, uint32_t hold_tx, Next &&next)
+{
+    const int lane = threadIdx.x & 31;
+    Pass ps{t, st, pk, a, round, PLAIN ? (int)PASS_ROUND : kind, lane,
+            PLAIN ? false : (kind == PASS_FINAL || st.dual_trace != nullptr),
+            PLAIN ? false : (kind == PASS_ROUND && st.hash_trace != nullptr)};
+    constexpr int kSlot = pack_slot_bytes(NW);
+    const uint32_t slots_s = smem_u32(smem), bars = slots_s + kPackSlots * kSlot;
+    int rt = 0, rn = 0;
+    int kt = next(&rt);          // the tile being evaluated, its round, and the next tile
+    if (kt < 0)
+        return;
+    int kn = next(&rn);
+    auto load = [&](int k) {
+        const uint4 x = __ldg(reinterpret_cast<const uint4 *>(pk.tiles + k));
+        return PackTile{x.x, x.y, x.z, x.w};
+    };
+    PackTile T = load(kt), N = T;
+    if (kn >= 0)
+        N = load(kn);
+    if (lane == 0) {
+        for (int s = 0; s < kPackSlots; ++s)
+            mbar_init(bars + 8 * s, 1);
+        fence_barrier_init();
+    }
+    __syncwarp();
+    // the copies: source of the next step, its bytes, steps left in its tile; steps in flight
+    const unsigned char *src;
+    uint32_t bytes;
+    int left, flying = 0, to = 0;
+    bool in_next = false;
+    auto start = [&](const PackTile &x) {
+        const PackShape sh = pack_shape(x);
+        src = reinterpret_cast<const unsigned char *>(pk.data) + (uint64_t)x.base * (16 * (NW + 1));
+        bytes = (uint32_t)sh.v * (16 * (NW + 1));
+        left = sh.steps;
+    };
+    auto issue = [&]() {
+        if (left == 0) {
+            if (in_next || kn < 0)
+                return;
+            start(N);
+            in_next = true;
+        }
+        if (lane == 0) {
+            fence_proxy_async();
+            mbar_arrive_expect_tx(bars + 8 * to, bytes + hold_tx);
+            bulk_g2s(slots_s + to * kSlot, src, bytes, bars + 8 * to);
+        }
+        hold_tx = 0u;
+        src += bytes;
+        --left;
+        ++flying;
+        to ^= 1;
+    };
+    start(T);
+    issue();
+    issue();
+    // everything above reads only the packed table and the plan; prices, flags and the demand
+    // accumulators were written by the previous kernel on the stream (a no-op for an ordinary launch)
+    if (!PERSIST)
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+    Ctx<NW> c;
+    reset(c);
+    int at = 0;                  // slot of the step to be screened
+    uint32_t phases = 0;         // parity of each slot's next completion
+    // the step in slot `at` has landed (bounded; warp-uniform)
+    auto landed = [&]() {
+        const bool ok = __all_sync(FULL, wait_stage(bars + 8 * at, (phases >> at) & 1u, st.err, a.wait_ms));
+        if (ok) {
+            phases ^= 1u << at;
+            --flying;
+        }
+        return ok;
+    };
+    auto release = [&]() {       // every lane is done with slot `at`
+        __syncwarp();
+        at ^= 1;
+        issue();
+    };
+    // an earlier launch's wait gave up: this warp does nothing (looked at after the first loads of prices)
+    const unsigned int gave_up = __ldcg(st.err);
+    bool ok = true;
+    while (ok) {
+        if (flying < kPackSlots)
+            issue();             // a tile of one step left the copies waiting for this tile's successor
+        const PackShape sh = pack_shape(T);
+        if (PERSIST) {
+            leave<NW, true>(ps, c);
+            c.s = -1;
+            if (!wait_version(st.ver, (int)T.scenario, rt, st.err, a.wait_ms, st.stats)) {
+                ok = false;
+                break;
+            }
+            ps.round = rt;
+            enter(ps, c, (int)T.scenario);
+        } else if ((int)T.scenario != c.s) {
+            leave<NW, false>(ps, c);
+            enter(ps, c, (int)T.scenario);
+        }
+        if (__any_sync(FULL, (gave_up & DEV_ERR_TIMEOUT) != 0u)) {
+            ok = false;
+            break;
+        }
+        if (c.wins >= kPackSpill)
+            add_demand(ps, c);
+        const int n_job = (int)T.n_job, steps = sh.steps;
+        if (sh.code < (int)kPackTiny) {
+            const int code = sh.code, sub = lane & ((1 << code) - 1), jl = lane >> code;
+            const bool has_a = sub < sh.ca, has_b = sub < sh.cb, any_b = sh.cb > 0;
+            const int ia = has_a ? jl * sh.ca + sub : 0, ib = has_b ? sh.per_step * sh.ca + jl * sh.cb + sub : 0;
+            for (int st_i = 0; st_i < steps; ++st_i) {
+                if (!(ok = landed()))
+                    break;
+                if (!c.skip)
+                    step_jobs<NW, PLAIN>(ps, c, reinterpret_cast<const uint4 *>(smem + at * kSlot), sh.v, ia, ib, has_a, has_b,
+                                         any_b, code, sh.narrow ? 2 : 3, kt, st_i * sh.per_step + jl, n_job);
+                release();
+            }
+            c.wins += steps;
+        } else if (sh.code == (int)kPackLarge) {
+            Large<NW> big;
+            big.m1 = big.m2 = INFINITY;
+            big.idx = kIdxNone;
+#pragma unroll
+            for (int k = 0; k < NW; ++k)
+                big.x[k] = 0u;
+            int job = 0, ch = 0;
+            for (int st_i = 0; st_i < steps; ++st_i) {
+                if (!(ok = landed()))
+                    break;
+                if (!c.skip) {
+                    const uint4 *slot = reinterpret_cast<const uint4 *>(smem + at * kSlot);
+#pragma unroll 1
+                    for (int h = 0; h < 2; ++h) {
+                        if (lane >= (h ? sh.cb : sh.ca))
+                            break;
+                        float q[4], r1, r2;
+                        screen4<NW>(slot + (h ? sh.ca : 0) + lane, sh.v, pk.fmt, c, q);
+                        two_smallest(q, r1, r2);
+                        if (r1 < big.m1) {   // increasing index: earlier options keep ties
+                            big.m2 = fminf(big.m1, r2);
+                            big.idx = 4 * (ch * sh.v + 2 * lane + h) + (q[0] == r1 ? 0 : q[1] == r1 ? 1 : q[2] == r1 ? 2 : 3);
+                            big.m1 = r1;
+                        } else {
+                            big.m2 = fminf(big.m2, r1);
+                        }
+                    }
+                    __syncwarp();
+                    if (++ch == sh.nch) {
+                        close_large<NW, PLAIN>(ps, c,
+                                               pk.data + ((uint64_t)T.base + (uint64_t)job * sh.nch * sh.v) * (NW + 1), sh, kt,
+                                               job, big);
+                        ch = 0;
+                        ++job;
+                    }
+                }
+                release();
+            }
+            add_pending(c, pk.fmt, big);
+            c.wins += n_job;
+        } else {
+            for (int st_i = 0; st_i < steps; ++st_i) {
+                if (!(ok = landed()))
+                    break;
+                if (!c.skip) {
+                    const uint4 *slot = reinterpret_cast<const uint4 *>(smem + at * kSlot);
+#pragma unroll 1
+                    for (int h = 0; h < 2; ++h) {
+                        const int o0 = 4 * (64 * st_i + 32 * h + lane), j0 = o0 / sh.m;   // m = 1 or 2
+                        if (j0 < n_job)
+                            step_tiny<NW, PLAIN>(ps, c, slot + 32 * h + lane, 64, sh.m, kt, j0, n_job - j0);
+                    }
+                }
+                release();
+            }
+            c.wins += 8 * steps;
+        }
+        if (!ok)
+            break;
+        ++c.tiles;
+        if (kn < 0) {
+            leave<NW, PERSIST>(ps, c);
+            break;
+        }
+        T = N;
+        kt = kn;
+        rt = rn;
+        in_next = false;
+        kn = next(&rn);
+        if (kn >= 0)
+            N = load(kn);
+    }
+    if (!ok) {   // a wait gave up: wait (bounded) for every copy still in flight, then leave
+        for (; flying > 0; --flying, at ^= 1) {
+            wait_stage(bars + 8 * at, (phases >> at) & 1u, st.err, a.wait_ms);
+            phases ^= 1u << at;
+        }
+    }
+    const unsigned int n = __reduce_add_sync(FULL, c.resolved);
+    if (lane == 0 && n != 0u)
+        atomicAdd(st.stats, (unsigned long long)n);
+}
+
+// One pass: warp w evaluates the tiles of its range. PLAIN: a round pass without traces.
+template <int NW, bool PLAIN>
+__global__ void __launch_bounds__(kPackWarps * 32, pack_min_ctas(NW))
+    k_packed(const __grid_constant__ DevTable t, const __grid_constant__ DevState st, const __grid_constant__ DevPack pk,
+             const __grid_constant__ SolveArgs a, int round, int kind)
+{
+    extern __shared__ __align__(128) unsigned char smem[];
+    // a pass launched as a programmatic dependent of this one may start its CTAs as slots free up; it
+    // waits for this grid's completion before it reads state
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const int wid = threadIdx.x >> 5, w = blockIdx.x * kPackWarps + wid;
+    if (w >= pk.n_warps)
+        return;
+    int k = w, end = w + 1;
+    if (pk.n_warps != pk.n_tiles) {
+        k = __ldg(pk.warp_begin + w);
+        end = __ldg(pk.warp_begin + w + 1);
+    }
+    run_warp<NW, PLAIN, false>(t, st, pk, a, round, kind, smem + (size_t)wid * pack_warp_bytes(NW),
+                               (w == 0 && round == 0 && kind == PASS_ROUND) ? a.hold_tx : 0u,
+                               [&](int *) { return k < end ? k++ : -1; });
+}
+
+// Rounds 0 .. n_rounds - 1 in one cooperative launch. Between two round passes a kernel boundary costs
+// the whole GPU the slowest warp's tail, the next pass's ramp-up and the launch gap. Here the only
+// dependence left is the true one: scenario s may be evaluated in round r once its r-th price update is
+// done, published as ver[s] >= r by the warp whose arrival completed the round before.
+// Work items are (round, tile) pairs, q = round * n_tiles + i, taken from one counter in increasing
+// order by whichever warp is free; the tiles are listed by scenario, so a scenario's next-round items are
+// handed out about a round after its current ones.
+// Lane 0 asks the counter one item ahead of the one it hands out.
+// Deadlock-free: every CTA is co-resident (cooperative launch); an item depends only on items of smaller
+// index, a warp evaluates its items in the order it took them and publishes one before it waits for the
+// next one's scenario, so the smallest unfinished item waits only for published work. Every wait is
+// bounded.
+template <int NW>
+__global__ void __launch_bounds__(kPackWarps * 32, pack_min_ctas(NW))
+    k_packed_persist(const __grid_constant__ DevTable t, const __grid_constant__ DevState st,
+                     const __grid_constant__ DevPack pk, const __grid_constant__ SolveArgs a, int n_rounds)
+{
+    extern __shared__ __align__(128) unsigned char smem[];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const unsigned int Q = (unsigned int)n_rounds * (unsigned int)pk.n_tiles;   // below 2^31 (host)
+    unsigned int pend = 0;
+    if (lane == 0)
+        pend = atomicAdd(st.work, 1u);
+    run_warp<NW, true, true>(t, st, pk, a, 0, (int)PASS_ROUND, smem + (size_t)wid * pack_warp_bytes(NW),
+                             blockIdx.x == 0 && wid == 0 ? a.hold_tx : 0u,
+                             [&](int *round) {
+                                 const unsigned int q = __shfl_sync(FULL, pend, 0);
+                                 if (q >= Q)
+                                     return -1;
+                                 if (lane == 0)
+                                     pend = atomicAdd(st.work, 1u);
+                                 const unsigned int r = q / (unsigned int)pk.n_tiles;
+                                 *round = (int)r;
+                                 return (int)(q - r * (unsigned int)pk.n_tiles);
+                             });
+}
+
+// The words of the packed copy (esp_packed.h): one block per step, one thread per option.
+__global__ void __launch_bounds__(4 * kPackStepVecs) k_pack(DevTable t, const __grid_constant__ DevPack pk, uint32_t *data)
+{
+    const int R = t.R, words = pk.fmt.nw + 1;
+    const PackTile T = pk.tiles[blockIdx.x];
+    const PackShape sh = pack_shape(T);
+    const int w = threadIdx.x;
+    if (w >= 4 * sh.v)
+        return;
+    const int j0 = pk.job_begin[blockIdx.x], n_job = (int)T.n_job;
+    // the job of word w of a plane and the option of it
+    const int x = w >> 2, o = w & 3;
+    for (int step = blockIdx.y; step < sh.steps; step += gridDim.y) {
+        int jl, opt;
+        if (sh.code == (int)kPackTiny) {
+            const int at = 4 * (64 * step + x) + o;
+            jl = at / sh.m;
+            opt = at - jl * sh.m;
+        } else if (sh.code == (int)kPackLarge) {
+            jl = step / sh.nch;
+            const int vec = x < sh.ca ? 2 * x : 2 * (x - sh.ca) + 1;
+            opt = 4 * ((step - jl * sh.nch) * sh.v + vec) + o;
+        } else {
+            const int na = sh.per_step * sh.ca;
+            const bool first = x < na;
+            const int y = first ? x : x - na, per = first ? sh.ca : sh.cb;
+            const int q = y / per, sub = y - q * per;
+            jl = step * sh.per_step + q;
+            opt = 4 * (sh.narrow ? sub : 2 * sub + (first ? 0 : 1)) + o;
+        }
+        uint32_t v = kPackInf, f[kPackMaxWords];
+#pragma unroll
+        for (int k = 0; k < kPackMaxWords; ++k)
+            f[k] = 0u;
+        if (jl < n_job) {
+            const int64_t job = pk.job ? pk.job[j0 + jl] : j0 + jl;
+            const int64_t a = t.job_off[job];
+            if (opt < t.job_off[job + 1] - a) {
+                const int32_t *u = t.units + (a + opt) * R;
+                if (u[0] >= 0) {   // not a duplicate
+                    v = __float_as_uint(-screen_value(t.values[a + opt]));
+                    if (v == kPackInf)   // beyond the screen's range (evaluated exactly): not padding
+                        v = 0x7f7fffffu;
+                }
+#pragma unroll
+                for (int k = 0; k < kPackMaxWords; ++k) {
+                    if (k < pk.fmt.nw && pk.fmt.col_lo[k] >= 0)
+                        f[k] = (uint32_t)(u[pk.fmt.col_lo[k]] & 0x7fffffff);
+                    if (k < pk.fmt.nw && pk.fmt.col_hi[k] >= 0)
+                        f[k] |= (uint32_t)(u[pk.fmt.col_hi[k]] & 0x7fffffff) << pk.fmt.shift[k];
+                }
+            }
+        }
+        uint32_t *out = data + ((uint64_t)T.base + (uint64_t)step * sh.v) * words * 4;
+        out[w] = v;
+#pragma unroll
+        for (int k = 0; k < kPackMaxWords; ++k)
+            if (k < pk.fmt.nw)
+                out[(k + 1) * sh.v * 4 + w] = f[k];
+    }
+}
+
+template <int NW>
+struct PackKernels {
+    static const void *fn(int which)
+    {
+        return which == 0   ? reinterpret_cast<const void *>(&k_packed<NW, true>)
+               : which == 1 ? reinterpret_cast<const void *>(&k_packed<NW, false>)
+                            : reinterpret_cast<const void *>(&k_packed_persist<NW>);
+    }
+};
+
+template <typename F>
+auto pack_dispatch(int nw, F &&f)
+{
+    switch (nw) {
+    case 2: return f(PackKernels<2>());
+    case 3: return f(PackKernels<3>());
+    case 4: return f(PackKernels<4>());
+    case 6: return f(PackKernels<6>());
+    default: return f(PackKernels<8>());
+    }
+}
+
+}  // namespace
+
+int packed_ctas_per_sm(int nw)
+{
+    return pack_dispatch(nw, [&](auto k) -> int {
+        int best = 0;
+        const int smem = kPackWarps * pack_warp_bytes(nw);
+        for (int i = 0; i < 3; ++i) {
+            int n = 0;
+            if (cudaFuncSetAttribute(decltype(k)::fn(i), cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
+                cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, decltype(k)::fn(i), kPackWarps * 32, smem) !=
+                    cudaSuccess) {
+                cudaGetLastError();
+                return 0;
+            }
+            best = i == 0 ? n : std::min(best, n);
+        }
+        return best;
+    });
+}
+
+cudaError_t launch_pack(const DevTable &t, const DevPack &pk, uint4 *data, cudaStream_t stream)
+{
+    if (pk.n_tiles <= 0)
+        return cudaSuccess;
+    k_pack<<<dim3((unsigned)pk.n_tiles, 8), 4 * kPackStepVecs, 0, stream>>>(t, pk, reinterpret_cast<uint32_t *>(data));
+    return cudaGetLastError();
+}
+
+cudaError_t launch_packed(const DevTable &t, const DevState &st, const DevPack &pk, const SolveArgs &a, int round,
+                          PassKind kind, cudaStream_t stream, bool pdl)
+{
+    const bool plain = kind == PASS_ROUND && st.hash_trace == nullptr && st.dual_trace == nullptr;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)((pk.n_warps + kPackWarps - 1) / kPackWarps));
+    cfg.blockDim = dim3(kPackWarps * 32);
+    cfg.dynamicSmemBytes = (size_t)(kPackWarps * pack_warp_bytes(pk.fmt.nw));
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = pdl ? 1 : 0;
+    int k = kind;
+    void *args[] = {(void *)&t, (void *)&st, (void *)&pk, (void *)&a, (void *)&round, (void *)&k};
+    return pack_dispatch(pk.fmt.nw, [&](auto kk) { return cudaLaunchKernelExC(&cfg, decltype(kk)::fn(plain ? 0 : 1), args); });
+}
+
+cudaError_t launch_packed_persist(const DevTable &t, const DevState &st, const DevPack &pk, const SolveArgs &a,
+                                  int n_rounds, int grid, cudaStream_t stream)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3(kPackWarps * 32);
+    cfg.dynamicSmemBytes = (size_t)(kPackWarps * pack_warp_bytes(pk.fmt.nw));
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeCooperative;   // every CTA co-resident: the version waits can end
+    attr[0].val.cooperative = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    void *args[] = {(void *)&t, (void *)&st, (void *)&pk, (void *)&a, (void *)&n_rounds};
+    return pack_dispatch(pk.fmt.nw, [&](auto kk) { return cudaLaunchKernelExC(&cfg, decltype(kk)::fn(2), args); });
+}
+
+}  // namespace esp

@@ -2,6 +2,8 @@
 #include "esp_plan.h"
 
 #include <algorithm>
+#include <climits>
+#include <cstdint>
 
 namespace esp {
 
@@ -276,6 +278,238 @@ bool sort_layout(const int64_t *off, int32_t S, int32_t J, SortedLayout &out, in
                 if (off[j + 1] - off[j] == k)
                     push(j, s, k, (int32_t)k);
     return (int64_t)out.jmap.size() == n_jobs;
+}
+
+bool pack_format(const int32_t *umax, int32_t R, PackFormat &out)
+{
+    out = PackFormat{};
+    if (R < 1 || R > kMaxR)
+        return false;
+    struct Col {
+        int bits, col;
+    };
+    std::vector<Col> cols;
+    for (int32_t r = 0; r < R; ++r) {
+        int b = 0;
+        while (b < 31 && (umax[r] >> b) != 0)
+            ++b;
+        if (umax[r] < 0 || b > 23)
+            return false;
+        cols.push_back({std::max(b, 1), r});
+    }
+    std::stable_sort(cols.begin(), cols.end(), [](const Col &x, const Col &y) { return x.bits > y.bits; });
+    std::vector<char> used(cols.size(), 0);
+    int nw = 0;
+    for (int k = 0; k < kPackMaxWords; ++k) {   // empty words: nothing low, one bit high
+        out.mask[k] = 0u;
+        out.shift[k] = 31;
+        out.magic[k] = 0x4b000000u >> 1;
+        out.col_lo[k] = out.col_hi[k] = -1;
+    }
+    for (size_t i = 0; i < cols.size(); ++i) {
+        if (used[i])
+            continue;
+        if (nw == kPackMaxWords)
+            return false;
+        out.mask[nw] = (1u << cols[i].bits) - 1u;
+        out.col_lo[nw] = (int8_t)cols[i].col;
+        for (size_t j = i + 1; j < cols.size(); ++j)
+            if (!used[j] && cols[i].bits + cols[j].bits <= 32) {
+                used[j] = 1;
+                out.shift[nw] = 32 - cols[j].bits;
+                out.magic[nw] = 0x4b000000u >> cols[j].bits;   // exact: its low 24 bits are zero
+                out.col_hi[nw] = (int8_t)cols[j].col;
+                break;
+            }
+        ++nw;
+    }
+    for (int n : {2, 3, 4, 6, 8})
+        if (nw <= n) {
+            out.nw = n;
+            return true;
+        }
+    return false;
+}
+
+// Kind and vector count of a job of k options, as a tile's mk. narrow: four options per lane (jobs of up to
+// 128 options).
+static uint32_t pack_kind(int64_t k, bool narrow)
+{
+    if (k <= 2)
+        return (uint32_t)k << 3 | kPackTiny;
+    const int64_t m = (k + 3) / 4;
+    if (m > 64)
+        return (uint32_t)m << 3 | kPackLarge;
+    const int64_t lanes = narrow && m <= 32 ? m : (m + 1) / 2;
+    uint32_t code = 0;
+    while ((1 << code) < lanes)
+        ++code;
+    return (uint32_t)m << 3 | code;
+}
+
+bool plan_packed(const int64_t *off, int32_t S, int32_t J, int32_t max_warps, PackPlan &out, int64_t all_k)
+{
+    out = PackPlan();
+    out.scen_tiles.assign((size_t)std::max(S, 1), 0);
+    const int64_t n_jobs = (int64_t)S * J;
+    if (S < 1 || J < 0 || max_warps < 1 || n_jobs >= INT32_MAX || off[0] != 0)
+        return false;
+    // 1. the order: within a scenario by kind and vector count (a counting sort over the kinds of at most
+    //    256 options keeps the table's order inside each; larger jobs are sorted by vector count)
+    struct Seg {
+        int32_t job, n, scen;
+        uint32_t mk;
+    };
+    std::vector<Seg> segs;
+    bool same = true;
+    if (all_k >= (int64_t)1 << 30)
+        return false;
+    if (all_k > 0)
+        for (int32_t s = 0; s < S && J > 0; ++s)
+            segs.push_back({s * J, J, s, pack_kind(all_k, false)});
+    std::vector<int32_t> count(67), at(67), order(all_k > 0 ? 0 : (size_t)J), big;
+    auto cls = [](uint32_t mk) { return (mk & 7u) == kPackTiny ? (int)(mk >> 3) - 1 : (int)(mk >> 3) + 1; };   // 0, 1, 2 .. 65
+    std::vector<int32_t> perm;
+    perm.reserve(all_k > 0 ? 0 : (size_t)n_jobs);
+    std::vector<uint32_t> kind(order.size());
+    for (int32_t s = 0; s < S && all_k == 0; ++s) {
+        const int64_t j0 = (int64_t)s * J;
+        std::fill(count.begin(), count.end(), 0);
+        big.clear();
+        for (int32_t j = 0; j < J; ++j) {
+            const int64_t k = off[j0 + j + 1] - off[j0 + j];
+            if (k < 1 || k >= (int64_t)1 << 30)
+                return false;
+            kind[(size_t)j] = pack_kind(k, false);
+            if ((kind[(size_t)j] & 7u) == kPackLarge)
+                big.push_back(j);
+            else
+                ++count[(size_t)cls(kind[(size_t)j])];
+        }
+        int32_t sum = 0;
+        for (int c = 66; c >= 0; --c) {   // large vector counts first
+            at[(size_t)c] = sum;
+            sum += count[(size_t)c];
+        }
+        for (int32_t j = 0; j < J; ++j)
+            if ((kind[(size_t)j] & 7u) != kPackLarge)
+                order[(size_t)at[(size_t)cls(kind[(size_t)j])]++] = j;
+        std::stable_sort(big.begin(), big.end(), [&](int32_t x, int32_t y) { return kind[(size_t)x] > kind[(size_t)y]; });
+        std::copy(big.begin(), big.end(), order.begin() + sum);
+        for (int32_t i = 0; i < J; ++i) {
+            const int32_t j = order[(size_t)i];
+            same = same && j == i;
+            if (i == 0 || kind[(size_t)j] != segs.back().mk)
+                segs.push_back({(int32_t)perm.size(), 0, s, kind[(size_t)j]});
+            ++segs.back().n;
+            perm.push_back((int32_t)(j0 + j));
+        }
+    }
+    if (!same)
+        out.job = std::move(perm);
+    // 2. tiles: about three per warp where the table has the steps, else single steps
+    for (const Seg &g : segs)
+        out.steps += pack_shape(PackTile{0, 0, g.mk, (uint32_t)g.n}).steps;
+    // a table of at most half a step per warp: four options per lane, twice the steps and each shorter
+    // (one 2048-job cluster of 16 options per job: 128 steps of eight options per lane took 12.8 us per
+    // round, 256 of four 12.2)
+    out.narrow = 2 * out.steps <= max_warps;
+    if (out.narrow) {
+        out.steps = 0;
+        for (Seg &g : segs) {
+            const int64_t m = g.mk >> 3;
+            if ((g.mk & 7u) < kPackTiny)
+                g.mk = pack_kind(4 * m, true);
+            out.steps += pack_shape(PackTile{0, 0, g.mk, (uint32_t)g.n}).steps;
+        }
+    }
+    const int64_t steps_max = std::min<int64_t>(kPackTileSteps, std::max<int64_t>(1, out.steps / (3LL * max_warps)));
+    for (const Seg &g : segs) {
+        const PackShape one = pack_shape(PackTile{0, 0, g.mk, 1});
+        const int64_t jobs_max = std::max<int64_t>(1, steps_max / one.nch) * one.per_step;
+        for (int64_t a = 0; a < g.n; a += jobs_max) {
+            PackTile t;
+            t.base = (uint32_t)out.vecs;
+            t.scenario = (uint32_t)g.scen;
+            t.mk = g.mk;
+            t.n_job = (uint32_t)std::min<int64_t>(jobs_max, g.n - a);
+            const PackShape sh = pack_shape(t);
+            out.job_begin.push_back((int32_t)(g.job + a));
+            out.vecs += (int64_t)sh.steps * sh.v;
+            if (out.vecs > (int64_t)UINT32_MAX)
+                return false;
+            ++out.scen_tiles[(size_t)g.scen];
+            out.tiles.push_back(t);
+        }
+    }
+    out.job_begin.push_back((int32_t)n_jobs);
+    if (out.tiles.size() >= (size_t)INT32_MAX)
+        return false;
+    // 3. the round pass's ranges: contiguous tiles of about equal cost (in tenths of a step)
+    const int64_t n_tiles = (int64_t)out.tiles.size();
+    std::vector<int64_t> pre((size_t)n_tiles + 1, 0);
+    for (int64_t i = 0; i < n_tiles; ++i)
+        pre[i + 1] = pre[i] + 5 + 10LL * pack_shape(out.tiles[i]).steps;
+    const int32_t W = (int32_t)std::min<int64_t>(max_warps, n_tiles);
+    out.n_warps = W;
+    out.warp_begin.assign((size_t)W + 1, 0);
+    for (int32_t w = 1; w < W; ++w) {
+        const int64_t target = (int64_t)((__int128)pre[n_tiles] * w / W);
+        int64_t i = std::lower_bound(pre.begin(), pre.end(), target) - pre.begin();
+        if (i > 0 && target - pre[i - 1] < pre[i] - target)
+            --i;
+        out.warp_begin[w] = (int32_t)std::min<int64_t>(std::max<int64_t>(i, out.warp_begin[w - 1]), n_tiles);
+    }
+    out.warp_begin[W] = (int32_t)n_tiles;
+    return true;
+}
+
+bool check_packed(const int64_t *off, int32_t S, int32_t J, const PackPlan &p, int64_t all_k)
+{
+    const int64_t n_jobs = (int64_t)S * J, n_tiles = (int64_t)p.tiles.size();
+    if ((int64_t)p.job_begin.size() != n_tiles + 1 || p.job_begin.front() != 0 || p.job_begin.back() != n_jobs ||
+        (!p.job.empty() && (int64_t)p.job.size() != n_jobs))
+        return false;
+    std::vector<char> seen(p.job.empty() ? 0 : (size_t)n_jobs, 0);
+    std::vector<int32_t> count((size_t)S, 0);
+    int64_t vecs = 0;
+    int32_t last = 0;
+    for (int64_t i = 0; i < n_tiles; ++i) {
+        const PackTile &t = p.tiles[(size_t)i];
+        if (t.base != (uint64_t)vecs || t.n_job < 1 || (int64_t)p.job_begin[i] + t.n_job != p.job_begin[i + 1] ||
+            (int32_t)t.scenario < last || (int32_t)t.scenario >= S)
+            return false;
+        last = (int32_t)t.scenario;
+        if (all_k > 0) {   // every job alike, in the table's order: the ends tell
+            if (!p.job.empty() || p.job_begin[i] / J != (int32_t)t.scenario || (p.job_begin[i + 1] - 1) / J != (int32_t)t.scenario ||
+                pack_kind(all_k, p.narrow) != t.mk)
+                return false;
+        }
+        for (int64_t q = p.job_begin[i]; q < p.job_begin[i + 1] && all_k == 0; ++q) {
+            const int64_t j = p.job.empty() ? q : p.job[(size_t)q];
+            if (j < (int64_t)t.scenario * J || j >= (int64_t)(t.scenario + 1) * J || pack_kind(off[j + 1] - off[j], p.narrow) != t.mk)
+                return false;
+            if (!p.job.empty()) {
+                if (seen[(size_t)j])
+                    return false;
+                seen[(size_t)j] = 1;
+            }
+        }
+        const PackShape sh = pack_shape(t);
+        if (sh.v < 1 || sh.v > kPackStepVecs || sh.steps < 1 ||
+            (sh.code < (int)kPackTiny && (sh.code > 5 || sh.ca > (1 << sh.code))))
+            return false;
+        ++count[(size_t)t.scenario];
+        vecs += (int64_t)sh.steps * sh.v;
+    }
+    if (vecs != p.vecs || count != p.scen_tiles)
+        return false;
+    if ((int32_t)p.warp_begin.size() != p.n_warps + 1 || p.warp_begin.front() != 0 || p.warp_begin.back() != n_tiles)
+        return false;
+    for (int32_t w = 0; w < p.n_warps; ++w)
+        if (p.warp_begin[w] > p.warp_begin[w + 1])
+            return false;
+    return true;
 }
 
 }  // namespace esp

@@ -5,6 +5,7 @@
 #include <vector>
 
 #include "esp_common.h"
+#include "esp_packed.h"
 
 namespace esp {
 
@@ -49,6 +50,33 @@ struct SortedLayout {
 bool sort_layout(const int64_t *job_off, int32_t S, int32_t J, SortedLayout &out, int32_t run_max_k = kRunMaxK);
 
 
+// Plan of the packed passes over a table (esp_packed.h).
+struct PackPlan {
+    std::vector<int32_t> job;          // table job of each job in the packed order; empty: the same order
+    std::vector<int32_t> job_begin;    // n_tiles + 1: first job (packed order) of each tile
+    std::vector<PackTile> tiles;       // by scenario
+    std::vector<int32_t> warp_begin;   // n_warps + 1: the round pass's ranges of about equal cost
+    std::vector<int32_t> scen_tiles;   // S: tiles of each scenario
+    int64_t vecs = 0;                  // vectors per plane of the whole copy
+    int64_t steps = 0;
+    bool narrow = false;               // four options per lane (small tables)
+    int32_t n_warps = 0;
+};
+
+// Word layout of the unit fields for the largest unit of each column over the table (each below
+// 2^23): columns paired so that two fit 32 bits, the widest with the widest that still fits. False when
+// the table needs more words than the passes have (kPackMaxWords) or a unit is 2^23 or more.
+bool pack_format(const int32_t *umax, int32_t R, PackFormat &out);
+
+// Packed order (per scenario, jobs of the same kind and vector count together), tiles of at most
+// kPackTileSteps steps (fewer where the table is small, so that every warp has work; a job of more steps
+// is a tile by itself) and ranges for at most max_warps warps. False on inconsistent offsets or a table
+// beyond the tile records' 32-bit fields. all_k > 0: every job is known to have that many options.
+constexpr int kPackTileSteps = 8;
+bool plan_packed(const int64_t *off, int32_t S, int32_t J, int32_t max_warps, PackPlan &out, int64_t all_k = 0);
+// Checks a packed plan against the table: every job once, every tile's jobs of its scenario, kind and
+// vector count, the tiles' data contiguous, the ranges covering every tile once and in order.
+bool check_packed(const int64_t *off, int32_t S, int32_t J, const PackPlan &p, int64_t all_k = 0);
 
 // Slices of the cluster-resident kernel: every scenario's jobs split into cs contiguous runs of about
 // equal option counts, run c starting at the first job whose first option lies at least

@@ -16,7 +16,7 @@ namespace esp {
 
 namespace {
 
-template <int RT, bool G, bool F>
+template <int RT, bool G>
 __device__ __forceinline__ bool load_option(const WarpCtx<RT, G> &c, bool in_smem, const int32_t *units_s,
                                             const double *vals_s, const uint16_t *grp_s, int o, int64_t gfirst,
                                             int32_t *u, double &v, int &g)
@@ -25,7 +25,7 @@ __device__ __forceinline__ bool load_option(const WarpCtx<RT, G> &c, bool in_sme
     bool dup;
     g = 0;
     if (in_smem) {
-        dup = load_units_stage<RT, F>(units_s + (size_t)o * R, u, R);
+        dup = load_units_smem<RT>(units_s + (size_t)o * R, u, R);
         v = vals_s[o];
         if (G)
             g = grp_s[o];
@@ -46,7 +46,7 @@ __device__ __forceinline__ bool load_option(const WarpCtx<RT, G> &c, bool in_sme
 // load-time marking did not cover) is skipped for the same reason, so only survivors that differ
 // from c0 are rescored in fp64. q is recomputed with the same instructions as the screen.
 // Returns the job-local index; s_out is set when has_s is true (always when need_s).
-template <int RT, bool G, bool F>
+template <int RT, bool G>
 __device__ void resolve_job(WarpCtx<RT, G> &c, int lane, bool in_smem, const int32_t *units_s, const double *vals_s,
                             const uint16_t *grp_s, int jstart, int jend, int64_t gfirst, float thr, bool need_s,
                             double &s_out, bool &has_s, int &local_out)
@@ -57,7 +57,7 @@ __device__ void resolve_job(WarpCtx<RT, G> &c, int lane, bool in_smem, const int
     int g;
     int first = kIdxNone;
     for (int o = jstart + lane; o < jend; o += 32) {
-        if (load_option<RT, G, F>(c, in_smem, units_s, vals_s, grp_s, o, gfirst, u, v, g))
+        if (load_option<RT, G>(c, in_smem, units_s, vals_s, grp_s, o, gfirst, u, v, g))
             continue;
         if (c.sp.exact || screen_score<RT, G>(u, v, g, c.sp, R, c.rg) <= thr) {
             first = o;
@@ -68,7 +68,7 @@ __device__ void resolve_job(WarpCtx<RT, G> &c, int lane, bool in_smem, const int
     int32_t u0[Cols<RT>::N];
     double v0;
     int g0;
-    load_option<RT, G, F>(c, in_smem, units_s, vals_s, grp_s, first, gfirst, u0, v0, g0);
+    load_option<RT, G>(c, in_smem, units_s, vals_s, grp_s, first, gfirst, u0, v0, g0);
 
     long long best_key = 0x7fffffffffffffffLL;
     int best_i = kIdxNone;
@@ -76,7 +76,7 @@ __device__ void resolve_job(WarpCtx<RT, G> &c, int lane, bool in_smem, const int
     for (int o = jstart + lane; o < jend; o += 32) {
         if (o <= first)
             continue;
-        if (load_option<RT, G, F>(c, in_smem, units_s, vals_s, grp_s, o, gfirst, u, v, g))
+        if (load_option<RT, G>(c, in_smem, units_s, vals_s, grp_s, o, gfirst, u, v, g))
             continue;
         if (!(c.sp.exact || screen_score<RT, G>(u, v, g, c.sp, R, c.rg) <= thr))
             continue;
@@ -124,7 +124,7 @@ __device__ void resolve_job(WarpCtx<RT, G> &c, int lane, bool in_smem, const int
 
 // Resolves, one after the other, the ambiguous jobs whose closing lanes are set in amask, and records
 // each winner (lane 0). big: the job is chunked and read from global memory.
-template <int RT, bool G, bool F>
+template <int RT, bool G>
 __device__ __forceinline__ void resolve_row(WarpCtx<RT, G> &c, int lane, uint32_t amask, bool big,
                                             const int32_t *units_s, const double *vals_s, const uint16_t *grp_s,
                                             int jstart, int jend, float thr, int64_t job, int64_t big_first)
@@ -139,14 +139,14 @@ __device__ __forceinline__ void resolve_row(WarpCtx<RT, G> &c, int lane, uint32_
         double s_w = 0.0;
         bool has_s = false;
         int li;
-        resolve_job<RT, G, F>(c, lane, !big, units_s, vals_s, grp_s, js, je, big ? big_first : 0, th, c.want_min,
+        resolve_job<RT, G>(c, lane, !big, units_s, vals_s, grp_s, js, je, big ? big_first : 0, th, c.want_min,
                            s_w, has_s, li);
         if (lane == 0) {
             atomicAdd(c.st.stats, 1ull);
             int32_t uw[Cols<RT>::N];
             double vw;
             int gw;
-            load_option<RT, G, F>(c, !big, units_s, vals_s, grp_s, js + li, big ? big_first : 0, uw, vw, gw);
+            load_option<RT, G>(c, !big, units_s, vals_s, grp_s, js + li, big ? big_first : 0, uw, vw, gw);
             take_winner<RT, G>(c, jb, li, uw, vw, gw, has_s, s_w);
         }
     }
@@ -189,7 +189,7 @@ __device__ __forceinline__ StagePtrs stage_ptrs_il(const TileDesc &d, const unsi
 // butterfly gives every lane of the group the smallest and second-smallest screen value; when the
 // job is unambiguous the unique lane holding the smallest value is the winner and records it from
 // its own registers.
-template <int RT, bool G, bool F>
+template <int RT, bool G>
 __device__ void process_tile_uniform(WarpCtx<RT, G> &c, const TileDesc &d, const StagePtrs &sp, int lane, int K,
                                      int log2_k)
 {
@@ -208,7 +208,7 @@ __device__ void process_tile_uniform(WarpCtx<RT, G> &c, const TileDesc &d, const
             if (G)
                 g = sp.grp[i];
             if (!dup)
-                q = screen_score_st<RT, G, F>(u, v, g, c.sp, R, c.rg);
+                q = screen_score<RT, G>(u, v, g, c.sp, R, c.rg);
         }
         float m1 = q, m2 = INFINITY;
         for (int dd = 1; dd < K; dd <<= 1) {
@@ -221,12 +221,11 @@ __device__ void process_tile_uniform(WarpCtx<RT, G> &c, const TileDesc &d, const
         const bool amb = c.sp.exact || !(m2 > thr);
         const int64_t job = d.job_begin + (i >> log2_k);
         if (valid && !amb && q == m1) {
-            stage_units_to_int<RT, F>(u, R);
             take_winner<RT, G>(c, job, i & (K - 1), u, v, g, false, 0.0);
         }
         const uint32_t amask = __ballot_sync(FULL, valid && amb && (i & (K - 1)) == 0);
         if (amask)
-            resolve_row<RT, G, F>(c, lane, amask, false, sp.units, sp.vals, sp.grp, i, i + K, thr, job, 0);
+            resolve_row<RT, G>(c, lane, amask, false, sp.units, sp.vals, sp.grp, i, i + K, thr, job, 0);
     }
 }
 
@@ -301,7 +300,7 @@ __device__ __forceinline__ void load_units4_smem(const int32_t *p, int32_t (*u)[
 // lexicographic minimum of (s, job-local index), and the lane holding that option records it.
 // The options are still in the stage, so no option is read twice from memory. base: tile-local
 // index of the lane's first option; loc0: its job-local index; lamb: the lane's job is ambiguous.
-template <int RT, bool G, bool F>
+template <int RT, bool G>
 __device__ __forceinline__ void resolve4_in_row(WarpCtx<RT, G> &c, const StagePtrs &sp, bool lamb, const float *q,
                                                 uint32_t dupmask, float thr, int base, int loc0, int64_t job, int L,
                                                 int rot)
@@ -316,7 +315,7 @@ __device__ __forceinline__ void resolve4_in_row(WarpCtx<RT, G> &c, const StagePt
                 continue;
             const int o = s ^ (rot << 1);
             int32_t u[Cols<RT>::N];
-            load_units_stage<RT, F>(sp.units + (size_t)(base + o) * c.R, u, c.R);
+            load_units_smem<RT>(sp.units + (size_t)(base + o) * c.R, u, c.R);
             const long long k = order_key(exact_score<RT, G>(u, sp.vals[base + o], 0, c.sp, c.R, c.rg));
             if (k < key || (k == key && loc0 + o < bi)) {
                 key = k;
@@ -335,7 +334,7 @@ __device__ __forceinline__ void resolve4_in_row(WarpCtx<RT, G> &c, const StagePt
     if (lamb && bi >= loc0 && bi < loc0 + 4) {
         const int i = base + (bi - loc0);
         int32_t uw[Cols<RT>::N];
-        load_units_stage<RT, F>(sp.units + (size_t)i * c.R, uw, c.R);
+        load_units_smem<RT>(sp.units + (size_t)i * c.R, uw, c.R);
         take_winner<RT, G>(c, job, bi, uw, sp.vals[i], 0, true, key_value(key));
         atomicAdd(c.st.stats, 1ull);
     }
@@ -345,7 +344,7 @@ __device__ __forceinline__ void resolve4_in_row(WarpCtx<RT, G> &c, const StagePt
 // consecutive options of one job (a tile row block is 128 options), keeps their smallest and
 // second-smallest screen values, and a log2(K / 4)-step xor butterfly over the job's K / 4 lanes
 // completes the job. An unambiguous job's winner is the unique option holding the smallest value.
-template <int RT, bool G, bool F>
+template <int RT, bool G>
 __device__ void process_tile_uniform4(WarpCtx<RT, G> &c, const TileDesc &d, const StagePtrs &sp, int lane)
 {
     const int R = c.R;
@@ -369,7 +368,7 @@ __device__ void process_tile_uniform4(WarpCtx<RT, G> &c, const TileDesc &d, cons
             for (int o = 0; o < 4; ++o) {
                 dupmask |= dup[o] ? (1u << o) : 0u;
                 if (!dup[o])
-                    q[o] = screen_score_st<RT, G, F>(u[o], v[o], 0, c.sp, R, c.rg);
+                    q[o] = screen_score<RT, G>(u[o], v[o], 0, c.sp, R, c.rg);
             }
         }
         // smallest and second smallest of the lane's four values
@@ -395,13 +394,13 @@ __device__ void process_tile_uniform4(WarpCtx<RT, G> &c, const TileDesc &d, cons
             if (w >= 0) {
                 const int i = base + w;
                 int32_t uw[Cols<RT>::N];
-                load_units_stage<RT, F>(sp.units + (size_t)i * R, uw, R);
+                load_units_smem<RT>(sp.units + (size_t)i * R, uw, R);
                 take_winner<RT, G>(c, d.job_begin + (i >> c.log2_k), i & (K - 1), uw, sp.vals[i], 0, false, 0.0);
             }
         }
         const bool lamb = valid && amb;
         if (__any_sync(FULL, lamb))
-            resolve4_in_row<RT, G, F>(c, sp, lamb, q, dupmask, thr, base, base & (K - 1),
+            resolve4_in_row<RT, G>(c, sp, lamb, q, dupmask, thr, base, base & (K - 1),
                                    d.job_begin + (base >> c.log2_k), KL, rot);
     }
 }
@@ -412,7 +411,7 @@ __device__ void process_tile_uniform4(WarpCtx<RT, G> &c, const TileDesc &d, cons
 // lanes keeps the lexicographic minimum of (s, job-local index), and the lane holding that option
 // records it. base: tile-local index of the lane's first option; loc: its job-local index; lamb: the
 // lane's job is ambiguous.
-template <int RT, bool G, bool F>
+template <int RT, bool G>
 __device__ __forceinline__ void resolve_run_row(WarpCtx<RT, G> &c, const StagePtrs &sp, bool lamb, float thr,
                                                 int base, int loc, int64_t job, int L)
 {
@@ -421,7 +420,7 @@ __device__ __forceinline__ void resolve_run_row(WarpCtx<RT, G> &c, const StagePt
     if (lamb) {
         for (int o = 0; o < 4; ++o) {
             int32_t u[Cols<RT>::N];
-            if (load_units_stage<RT, F>(sp.units + (size_t)(base + o) * c.R, u, c.R))
+            if (load_units_smem<RT>(sp.units + (size_t)(base + o) * c.R, u, c.R))
                 continue;
             const double v = sp.vals[base + o];
             if (!c.sp.exact && !(screen_score<RT, G>(u, v, 0, c.sp, c.R, c.rg) <= thr))
@@ -444,7 +443,7 @@ __device__ __forceinline__ void resolve_run_row(WarpCtx<RT, G> &c, const StagePt
     if (lamb && bi >= loc && bi < loc + 4) {
         const int i = base + (bi - loc);
         int32_t uw[Cols<RT>::N];
-        load_units_stage<RT, F>(sp.units + (size_t)i * c.R, uw, c.R);
+        load_units_smem<RT>(sp.units + (size_t)i * c.R, uw, c.R);
         take_winner<RT, G>(c, job, bi, uw, sp.vals[i], 0, true, key_value(key));
         atomicAdd(c.st.stats, 1ull);
     }
@@ -456,7 +455,7 @@ __device__ __forceinline__ void resolve_run_row(WarpCtx<RT, G> &c, const StagePt
 // index) and second-smallest value; lanes past the job's end idle. A log2(L)-step xor butterfly of
 // (smallest, second smallest) completes the job as in the uniform path; an unambiguous job's winner
 // is the unique option holding the smallest value, recorded by the lane that holds it.
-template <int RT, bool G, bool F>
+template <int RT, bool G>
 __device__ void process_tile_run4(WarpCtx<RT, G> &c, const TileDesc &d, const StagePtrs &sp, int lane, int K)
 {
     const int R = c.R;
@@ -485,7 +484,7 @@ __device__ void process_tile_run4(WarpCtx<RT, G> &c, const TileDesc &d, const St
             // smallest value is held by one slot (otherwise m2 = m1 and the job is ambiguous)
 #pragma unroll
             for (int o = 0; o < 4; ++o) {
-                const float q = dup[o] ? INFINITY : screen_score_st<RT, G, F>(u[o], v[o], 0, c.sp, R, c.rg);
+                const float q = dup[o] ? INFINITY : screen_score<RT, G>(u[o], v[o], 0, c.sp, R, c.rg);
                 const bool better = q < m1;
                 m2 = better ? m1 : fminf(m2, q);
                 i1 = better ? loc + (o ^ (rot << 1)) : i1;
@@ -505,12 +504,12 @@ __device__ void process_tile_run4(WarpCtx<RT, G> &c, const TileDesc &d, const St
         if (valid && !amb && lm1 == m1) {
             const int i = jl * K + i1;
             int32_t uw[Cols<RT>::N];
-            load_units_stage<RT, F>(sp.units + (size_t)i * R, uw, R);
+            load_units_smem<RT>(sp.units + (size_t)i * R, uw, R);
             take_winner<RT, G>(c, job, i1, uw, sp.vals[i], 0, false, 0.0);
         }
         const bool lamb = valid && amb;
         if (__any_sync(FULL, lamb))
-            resolve_run_row<RT, G, F>(c, sp, lamb, thr, base, loc, job, L);
+            resolve_run_row<RT, G>(c, sp, lamb, thr, base, loc, job, L);
     }
 }
 
@@ -519,7 +518,7 @@ __device__ void process_tile_run4(WarpCtx<RT, G> &c, const TileDesc &d, const St
 // offsets; a job continuing from the previous row enters as a carry; rows entirely inside one job
 // only fold per lane. A job larger than a tile arrives as consecutive chunk tiles of this warp
 // (big_first / big_carry carry its state across them) and is resolved from global memory.
-template <int RT, bool G, bool F>
+template <int RT, bool G>
 __device__ void process_tile_general(WarpCtx<RT, G> &c, const TileDesc &d, const StagePtrs &sp, int64_t &big_first,
                                      Best &big_carry, int lane)
 {
@@ -548,7 +547,7 @@ __device__ void process_tile_general(WarpCtx<RT, G> &c, const TileDesc &d, const
         int32_t u[Cols<RT>::N];
         float q = INFINITY;
         if (valid) {
-            const bool dup = load_units_stage<RT, F>(sp.units + (size_t)i * R, u, R);
+            const bool dup = load_units_smem<RT>(sp.units + (size_t)i * R, u, R);
             const double v = sp.vals[i];
             const int g = G ? (int)sp.grp[i] : 0;
             if (!dup)
@@ -621,13 +620,13 @@ __device__ void process_tile_general(WarpCtx<RT, G> &c, const TileDesc &d, const
             int32_t uw[Cols<RT>::N];
             double vw;
             int gw;
-            load_option<RT, G, F>(c, !big, sp.units, sp.vals, sp.grp, big ? x.idx : x.idx, big ? big_first : 0, uw, vw,
+            load_option<RT, G>(c, !big, sp.units, sp.vals, sp.grp, big ? x.idx : x.idx, big ? big_first : 0, uw, vw,
                                gw);
             take_winner<RT, G>(c, job, li, uw, vw, gw, false, 0.0);
         }
         const uint32_t amask = __ballot_sync(FULL, amb);
         if (amask)
-            resolve_row<RT, G, F>(c, lane, amask, big, sp.units, sp.vals, sp.grp, jstart, jend, thr, job, big_first);
+            resolve_row<RT, G>(c, lane, amask, big, sp.units, sp.vals, sp.grp, jstart, jend, thr, job, big_first);
     }
     if (big) {
         if (priv_dirty)
@@ -638,7 +637,7 @@ __device__ void process_tile_general(WarpCtx<RT, G> &c, const TileDesc &d, const
 // needed. Each lane folds the options it owns (lane-strided: conflict-free shared loads) into a
 // lane-private state carried across the job's chunks; the job's last chunk reduces the states across
 // the warp once and records the winner (exact resolution from global memory when ambiguous).
-template <int RT, bool G, bool F>
+template <int RT, bool G>
 __device__ void process_tile_bigchunk(WarpCtx<RT, G> &c, const TileDesc &d, const StagePtrs &sp, int64_t &big_first,
                                       Best &big_priv, int lane)
 {
@@ -665,7 +664,7 @@ __device__ void process_tile_bigchunk(WarpCtx<RT, G> &c, const TileDesc &d, cons
                 const double v = sp.vals[i];
                 const int g = G ? (int)sp.grp[i] : 0;
                 if (!dup)
-                    q[o] = screen_score_st<RT, G, F>(u, v, g, c.sp, R, c.rg);
+                    q[o] = screen_score<RT, G>(u, v, g, c.sp, R, c.rg);
             }
         }
 #pragma unroll
@@ -682,7 +681,7 @@ __device__ void process_tile_bigchunk(WarpCtx<RT, G> &c, const TileDesc &d, cons
         const bool dup = load_units_smem<RT>(sp.units + (size_t)i * R, u, R);
         const double v = sp.vals[i];
         const int g = G ? (int)sp.grp[i] : 0;
-        const float q = dup ? INFINITY : screen_score_st<RT, G, F>(u, v, g, c.sp, R, c.rg);
+        const float q = dup ? INFINITY : screen_score<RT, G>(u, v, g, c.sp, R, c.rg);
         big_priv = combine(big_priv, Best{q, dup ? kIdxNone : chunk_base + i, INFINITY});
     }
 #endif
@@ -700,7 +699,7 @@ __device__ void process_tile_bigchunk(WarpCtx<RT, G> &c, const TileDesc &d, cons
             double vw;
             int gw;
             const bool here = x.idx >= chunk_base;
-            load_option<RT, G, F>(c, here, sp.units, sp.vals, sp.grp, here ? x.idx - chunk_base : x.idx, big_first, uw,
+            load_option<RT, G>(c, here, sp.units, sp.vals, sp.grp, here ? x.idx - chunk_base : x.idx, big_first, uw,
                                vw, gw);
             take_winner<RT, G>(c, d.job_begin, x.idx, uw, vw, gw, false, 0.0);
         }
@@ -713,7 +712,7 @@ __device__ void process_tile_bigchunk(WarpCtx<RT, G> &c, const TileDesc &d, cons
             int32_t u[Cols<RT>::N];
             double v;
             int g;
-            load_option<RT, G, F>(c, false, sp.units, sp.vals, sp.grp, big_priv.idx, big_first, u, v, g);
+            load_option<RT, G>(c, false, sp.units, sp.vals, sp.grp, big_priv.idx, big_first, u, v, g);
             key = order_key(exact_score<RT, G>(u, v, g, c.sp, c.R, c.rg));
             bi = big_priv.idx;
         }
@@ -730,12 +729,12 @@ __device__ void process_tile_bigchunk(WarpCtx<RT, G> &c, const TileDesc &d, cons
             int32_t uw[Cols<RT>::N];
             double vw;
             int gw;
-            load_option<RT, G, F>(c, false, sp.units, sp.vals, sp.grp, bi, big_first, uw, vw, gw);
+            load_option<RT, G>(c, false, sp.units, sp.vals, sp.grp, bi, big_first, uw, vw, gw);
             take_winner<RT, G>(c, d.job_begin, bi, uw, vw, gw, true, key_value(key));
             atomicAdd(c.st.stats, 1ull);
         }
     } else {
-        resolve_row<RT, G, F>(c, lane, 1u, true, sp.units, sp.vals, sp.grp, 0, K, thr, d.job_begin, big_first);
+        resolve_row<RT, G>(c, lane, 1u, true, sp.units, sp.vals, sp.grp, 0, K, thr, d.job_begin, big_first);
     }
 }
 }  // namespace

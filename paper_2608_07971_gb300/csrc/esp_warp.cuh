@@ -60,7 +60,6 @@ __device__ __forceinline__ double exact_score(const int32_t *u, double v, int g,
     for (int r = 0; r < Cols<RT>::N; ++r) {
         if (RT == 0 && r >= R)
             break;
-        // through L2: a persistent pass sees the prices change between rounds
         const double price = __ldcg(sp.p64g + ((G && r >= rg) ? rg + (R - rg) * g + (r - rg) : r));
         s = __fma_rn(price, __int2double_rn(u[r]), s);
     }
@@ -91,49 +90,6 @@ __device__ __forceinline__ bool load_units_smem(const int32_t *p, int32_t *u, in
     }
     const bool dup = u[0] < 0;
     u[0] &= 0x7fffffff;
-    return dup;
-}
-
-// Units staged as fp32 bit patterns (F: the tile-interleaved copy of a table whose units are all
-// below 2^23, each converted exactly at load; the duplicate mark stays the sign bit of column 0). The
-// screen takes them as they are: the same fp32 values the conversion of the integers gives, so the
-// same q, without a conversion per unit. Every other use converts them back to the integers.
-template <int RT, bool G, bool F>
-__device__ __forceinline__ float screen_score_st(const int32_t *u, double v, int g, const ScenarioPrices &sp, int R,
-                                                 int rg)
-{
-    if constexpr (F) {
-        static_assert(!G, "fp32 stage units only for tables without a group column");
-        float q = -screen_value(v);
-#pragma unroll
-        for (int r = 0; r < Cols<RT>::N; ++r) {
-            if (RT == 0 && r >= R)
-                break;
-            q = __fmaf_rn(sp.pf[r], __int_as_float(u[r]), q);
-        }
-        return q;
-    } else {
-        return screen_score<RT, G>(u, v, g, sp, R, rg);
-    }
-}
-
-template <int RT, bool F>
-__device__ __forceinline__ void stage_units_to_int(int32_t *u, int R)
-{
-    if constexpr (F) {
-#pragma unroll
-        for (int r = 0; r < Cols<RT>::N; ++r)
-            if (RT != 0 || r < R)
-                u[r] = __float2int_rn(__int_as_float(u[r]));
-    }
-}
-
-// Units of one staged option as integers (duplicate mark removed and returned).
-template <int RT, bool F>
-__device__ __forceinline__ bool load_units_stage(const int32_t *p, int32_t *u, int R)
-{
-    const bool dup = load_units_smem<RT>(p, u, R);
-    stage_units_to_int<RT, F>(u, R);
     return dup;
 }
 
@@ -307,6 +263,56 @@ __device__ void update_scenario(const DevTable &t, const DevState &st, const Sol
 
 
 
+// Bounded wait of a warp until scenario s has had `round` price updates (ver[s] >= round). Every lane
+// polls the word with relaxed loads (one transaction per poll) and, once all see it, reads it once
+// more with acquire semantics, so that each lane's later reads of the scenario's prices and bound are
+// ordered after the update that released them. The poll spins (each load is an L2 round trip) and
+// sleeps only after a long spin: a sleep can last far longer than asked, and a woken waiter would
+// then lag its scenario by that much. Gives up when another wait flagged a timeout, or after
+// limit_ms of the global timer (flagging one). The result is warp-uniform.
+__device__ __forceinline__ bool wait_version(const unsigned int *ver, int s, int round, unsigned int *err,
+                                             uint32_t limit_ms, unsigned long long *stats)
+{
+    auto seen = [&](bool acquire) {
+        unsigned int v;
+        if (acquire)
+            asm volatile("ld.acquire.gpu.u32 %0, [%1];" : "=r"(v) : "l"(ver + s) : "memory");
+        else
+            asm volatile("ld.relaxed.gpu.u32 %0, [%1];" : "=r"(v) : "l"(ver + s) : "memory");
+        return __all_sync(FULL, v >= (unsigned int)round);
+    };
+    if (seen(true))
+        return true;
+    const uint64_t t0 = __shfl_sync(FULL, global_ns(), 0);
+    const uint64_t limit = (uint64_t)limit_ms * 1000000ull;
+    bool ok = false;
+    for (uint32_t it = 1;; ++it) {
+        if (seen(false)) {
+            ok = seen(true);   // the value only grows: the acquire read sees it too
+            if (ok)
+                break;
+        }
+        if ((it & 63) == 0) {
+            unsigned int e;
+            asm volatile("ld.relaxed.gpu.u32 %0, [%1];" : "=r"(e) : "l"(err) : "memory");
+            if (__any_sync(FULL, (e & DEV_ERR_TIMEOUT) != 0))
+                break;
+            if (__shfl_sync(FULL, (global_ns() - t0 > limit) ? 1 : 0, 0)) {
+                if ((threadIdx.x & 31) == 0)
+                    atomicOr(err, DEV_ERR_TIMEOUT);
+                break;
+            }
+            if (it >= 4096)
+                __nanosleep(256);
+        }
+    }
+    if ((threadIdx.x & 31) == 0) {   // the time this wait polled (esp_debug_persist_waits)
+        atomicAdd(stats + 2, (unsigned long long)(global_ns() - t0));
+        atomicAdd(stats + 3, 1ull);
+    }
+    return ok;
+}
+
 // ---------------------------------------------------------------------------------------------
 // The warp's evaluation context.
 
@@ -324,9 +330,6 @@ struct WarpCtx {
     int uniform_k;            // > 0: every job has this many options (a power of two <= 32)
     int log2_k;
     int s;                    // current scenario
-    bool persist;             // persistent pass: the update publishes the scenario's price version
-    const int32_t *scen_tiles;  // persistent pass: tiles of each scenario (arrivals count tiles)
-    int ntiles;               // persistent pass: tiles of the current scenario evaluated since the last flush
     ScenarioPrices sp;
     long long acc[Cols<RT>::N];   // per-lane demand of the globally priced columns
     unsigned long long hacc;
@@ -368,32 +371,16 @@ __device__ void flush(WarpCtx<RT, G> &c, int lane)
             __syncwarp();
             __threadfence();
         }
-        // the persistent pass counts tiles (a warp flushes when its scenario or round changes, whatever
-        // the plan's ranges); the round pass counts the plan's warps
-        const unsigned int add = c.persist ? (unsigned int)c.ntiles : 1u;
-        const unsigned int need = (unsigned int)__ldg((c.persist ? c.scen_tiles : c.scen_warps) + c.s);
-        c.ntiles = 0;
+        const unsigned int need = (unsigned int)__ldg(c.scen_warps + c.s);
         unsigned int old = 0;
         if (lane == 0)
-            asm volatile("atom.add.release.gpu.u32 %0, [%1], %2;" : "=r"(old) : "l"(c.st.arrive + c.s), "r"(add)
-                         : "memory");
+            asm volatile("atom.add.release.gpu.u32 %0, [%1], 1;" : "=r"(old) : "l"(c.st.arrive + c.s) : "memory");
         old = __shfl_sync(FULL, old, 0);
-        if (old + add == need) {
+        if (old + 1u == need) {
             asm volatile("fence.acq_rel.gpu;" ::: "memory");
             update_scenario<G ? 8 : 1>(c.t, c.st, c.a, c.s, c.round, lane);
             if (lane == 0)
                 c.st.arrive[c.s] = 0u;     // every warp of this pass has arrived
-            if (c.persist) {
-                // publish the scenario's next round: every lane's writes (prices, bound, cleared
-                // demand) are fenced before lane 0's release of the version; a stopped scenario
-                // releases every later round at once (its warps then skip it)
-                __threadfence();
-                __syncwarp();
-                if (lane == 0) {
-                    const unsigned int v = c.st.frozen[c.s] ? kVerStopped : (unsigned int)(c.round + 1);
-                    asm volatile("st.release.gpu.u32 [%0], %1;" ::"l"(c.st.ver + c.s), "r"(v) : "memory");
-                }
-            }
         }
     }
 }

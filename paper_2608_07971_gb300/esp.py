@@ -491,13 +491,13 @@ def esp_debug_fail_alloc(ctx: int, n: int) -> None:
 
 
 def esp_debug_set_interleave(ctx: int, enable: bool) -> None:
-    """Later loads interleave the per-warp pass's table tile by tile (True, the default) or not."""
+    """Later loads keep a private copy of the table in the order of its tiles (True, the default) or not."""
     _check(load_library().esp_debug_set_interleave(ctx, 1 if enable else 0), "esp_debug_set_interleave")
 
 
 def esp_debug_set_stage_f32(ctx: int, enable: bool) -> None:
-    """Later loads store the units of the tile-interleaved table as fp32 where every unit is below 2^23
-    (True, the default) or keep them as integers."""
+    """Later loads use the packed passes where every unit is below 2^23 (True, the default) or the staged pass
+    with integer units."""
     _check(load_library().esp_debug_set_stage_f32(ctx, 1 if enable else 0), "esp_debug_set_stage_f32")
 
 
@@ -532,8 +532,8 @@ def esp_debug_load_profile(ctx: int):
 
 
 def esp_debug_pass_kernel(ctx: int) -> int:
-    """How the loaded table is evaluated: 0 per-warp pass, two copies per tile; 1 per-warp pass on the
-    tile-interleaved table, one copy per tile; 2 factored placement; 3 as 1 with fp32 units."""
+    """How the loaded table is evaluated: 0 staged pass, two copies per tile; 1 a private copy in the order of
+    its tiles, one launch per round; 2 factored placement; 3 packed, persistent pass available."""
     k = ctypes.c_int32()
     _check(load_library().esp_debug_pass_kernel(ctx, ctypes.byref(k)), "esp_debug_pass_kernel")
     return k.value
