@@ -157,7 +157,7 @@ struct esp_ctx {
     bool res_slower = false;   // the automatic choice is predicted slower than streaming: streaming runs
     int res_force = -1;    // index forced through esp_debug_resident (-1: automatic)
 
-    double *lam = nullptr, *p64 = nullptr, *job_val = nullptr, *job_min = nullptr;
+    double *lam = nullptr, *rcp = nullptr, *p64 = nullptr, *job_val = nullptr, *job_min = nullptr;
     double *best_dual = nullptr, *primal = nullptr, *dual = nullptr, *lambda0 = nullptr;
     float *p32 = nullptr, *ebound = nullptr;
     unsigned long long *U = nullptr, *U_final = nullptr, *hash = nullptr;
@@ -390,6 +390,7 @@ DevState dev_state(const esp_ctx *c)
 {
     DevState s{};
     s.lam = c->lam;
+    s.rcp = c->rcp;
     s.p64 = c->p64;
     s.p32 = c->p32;
     s.ebound = c->ebound;
@@ -463,6 +464,7 @@ esp_status alloc_solve_state(esp_ctx *ctx)
             a = dev_alloc(ctx, p, n);
     };
     al(&ctx->lam, SP);
+    al(&ctx->rcp, SP);
     al(&ctx->p64, SP);
     al(&ctx->p32, SP);
     al(&ctx->ebound, S);
@@ -983,7 +985,7 @@ esp_status check_params(const esp_ctx *ctx, const esp_params *p)
 // host instead of reaching a kernel as a null pointer).
 bool state_ready(const esp_ctx *c)
 {
-    const void *need[] = {c->lam, c->p64, c->p32, c->ebound, c->U, c->U_final, c->hash, c->sel, c->job_val,
+    const void *need[] = {c->lam, c->rcp, c->p64, c->p32, c->ebound, c->U, c->U_final, c->hash, c->sel, c->job_val,
                           c->job_min, c->rounds_run, c->converged, c->status, c->frozen, c->feasible,
                           c->best_dual, c->primal, c->dual, c->lambda0, c->err, c->vmax, c->umax, c->stats,
                           c->arrive, c->ver, c->work, c->cap};
@@ -1057,7 +1059,16 @@ esp_status plan_resident_options(esp_ctx *ctx)
             esp_ctx::ResOption o;
             o.plan.cs = cs;
             o.plan.k = rk;
-            o.plan.m_pad = (sh.m_max + 31) & ~31;
+            // lanes per job: as many as the CTA has for its jobs, up to one per option. The lanes of one
+            // option read 32 / lanes consecutive jobs; an odd multiple of that as the pitch keeps the
+            // options of a warp's lanes in different banks
+            o.plan.lanes = 1;
+            while (o.plan.lanes < 8 && 2 * o.plan.lanes * sh.m_max <= kResWarps * 32 && 2 * o.plan.lanes <= ctx->pc.max_k)
+                o.plan.lanes *= 2;
+            const int32_t unit = 32 / o.plan.lanes;
+            o.plan.m_pad = std::max(1, (sh.m_max + unit - 1) / unit) * unit;
+            if (o.plan.lanes > 1 && (o.plan.m_pad / unit) % 2 == 0)
+                o.plan.m_pad += unit;
             o.plan.n_cap = (sh.n_max + 1) & ~1LL;
             o.smem = res_smem_bytes(R, o.plan);
             o.n_max = sh.n_max;
@@ -1088,31 +1099,36 @@ esp_status plan_resident_options(esp_ctx *ctx)
                 at += shapes[i].cuts.size();
             }
             ESP_CUDA(cudaStreamSynchronize(ctx->stream));
-            // automatic size: most scenario-rounds per microsecond under a simple cost model, a fixed
-            // cost per round (barriers and the price update; smaller without a cluster) plus the
-            // slice's options at the SM's screening rate; ties keep the smaller cluster
+            // automatic size: most scenario-rounds per microsecond under a simple cost model, fitted to
+            // rounds measured on GB300: 2.0 us (prices and barriers), 0.3 + 0.02 cs us for the exchange in a
+            // cluster, and 0.09 us per option a lane screens one after the other (a 2048-job cluster
+            // of 16 options per job: 3.60 us with 16 CTAs, 4.0 with 8; 500 jobs of 8: 3.07, 2.77, 2.66
+            // and 2.77 with 1, 2, 4 and 16; tiny cluster: 2.16 with 1, 2.4 with 16). Slices in CSR order
+            // and widths without an instantiation cost about twice that per option, each (seven ragged
+            // 1777-job clusters of 5 columns: 19.5 us). Ties keep the smaller cluster
+            const double per_option = 0.09 * (ctx->pc.min_k == ctx->pc.max_k ? 1.0 : 2.0) *
+                                      (R == 4 || R == 6 || R == 8 ? 1.0 : 2.0);
+            auto round_us = [&](const esp_ctx::ResOption &o) {
+                const double serial = std::max((double)o.n_max / (kResWarps * 32), (double)ctx->pc.max_k / o.plan.lanes);
+                return 2.0 + (o.plan.cs == 1 ? 0.0 : 0.3 + 0.02 * o.plan.cs) + per_option * serial;
+            };
             double best = -1.0;
             for (size_t i = 0; i < ctx->res.size(); ++i) {
-                const esp_ctx::ResOption &o = ctx->res[i];
-                const double round_us = (o.plan.cs == 1 ? 0.6 : 1.0) + 7.8e-5 * (double)o.n_max;
-                const double rate = (double)std::min<int64_t>(S, o.clusters) / round_us;
+                const double rate = (double)std::min<int64_t>(S, ctx->res[i].clusters) / round_us(ctx->res[i]);
                 if (rate > best * 1.02) {
                     best = rate;
                     ctx->res_auto = (int)i;
                 }
             }
-            // the automatic choice runs only where it is predicted faster than streaming. Absolute
-            // times per round measured on GB300: a resident round of one wave of clusters costs about
-            // 2.6 + 0.135 cs + 7.8e-5 n_max us (2.7 us at 1 CTA, 4.75 us at 16 CTAs), and S scenarios
-            // take ceil(S / clusters) waves; a streaming round reads the table at about 5.6 TB/s
-            // plus 3 us, and no streaming round takes less than about 9 us (launch and update latency)
+            // the automatic choice runs only where it is predicted faster than streaming: S scenarios take
+            // ceil(S / clusters) waves of clusters; a streaming round takes about 12 us plus its table (half of
+            // it, packed) at 6 TB/s, and 6.5 us (launch and update latency) where it is a few steps
             if (ctx->res_auto >= 0) {
                 const esp_ctx::ResOption &o = ctx->res[ctx->res_auto];
                 const double waves = std::ceil((double)S / (double)o.clusters);
-                const double res_us = waves * (2.6 + 0.135 * o.plan.cs + 7.8e-5 * (double)o.n_max);
                 const double bytes = (double)ctx->n_opt * (4.0 * R + 8.0);
-                const double stream_us = std::max(9.0, 3.0 + bytes / 5.6e6);
-                ctx->res_slower = res_us > stream_us;
+                const double stream_us = bytes < 1e5 ? 6.5 : 12.0 + bytes / 12e6;
+                ctx->res_slower = waves * round_us(o) > stream_us;
             }
         }
     }

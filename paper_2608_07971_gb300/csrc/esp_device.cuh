@@ -9,6 +9,7 @@
 #include <cuda_runtime.h>
 
 #include "esp_common.h"
+#include "esp_div.h"
 
 namespace esp {
 
@@ -113,6 +114,29 @@ __device__ __forceinline__ double price_step(double lam, long long U, long long 
 __device__ __forceinline__ double effective_price(double lam, double Cd, int mode)
 {
     return mode == 1 ? lam / Cd : lam;
+}
+
+// The same two with rcp = 1 / Cd (correctly rounded) at hand: the same bits without a divide (div_by;
+// prices outside its range take the divide). A fp64 operation waits about 65 cycles for the one
+// before it, so the two divides were most of the serial end of a round. moved is never a NaN (a fused
+// multiply-add of finite operands): its sign bit decides the projection.
+__device__ __forceinline__ double price_step_rcp(double lam, long long U, long long C, double Cd, double rcp, double eta,
+                                                 int mode)
+{
+    double excess = (double)(U - C);
+    if (mode == 1)
+        excess = div_by(excess, Cd, rcp);
+    const double moved = __fma_rn(eta, excess, lam);
+    return __double2hiint(moved) < 0 ? 0.0 : moved;
+}
+
+__device__ __forceinline__ double effective_price_rcp(double lam, double Cd, double rcp, int mode)
+{
+    if (mode != 1)
+        return lam;
+    if (!div_safe(__double_as_longlong(lam)))
+        return lam / Cd;
+    return div_by(lam, Cd, rcp);
 }
 
 // Screen bound E of a scenario (fp32, rounded up) from M = max|v| + sum_r max p_r * max u_r, or

@@ -53,6 +53,7 @@ __global__ void k_init(DevTable t, DevState st, SolveArgs a, const double *lambd
     for (int k = lane; k < P; k += 32) {
         const double l0 = lambda0 ? lambda0[(size_t)s * P + k] : 0.0;
         st.lam[(size_t)s * P + k] = l0;
+        st.rcp[(size_t)s * P + k] = 1.0 / (double)t.cap[(size_t)s * P + k];
         st.U[(size_t)s * P + k] = 0ull;
         st.U_final[(size_t)s * P + k] = 0ull;
         if (st.lam_trace)

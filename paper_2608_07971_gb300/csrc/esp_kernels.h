@@ -26,6 +26,7 @@ struct DevTable {
 
 struct DevState {
     double *lam;              // S*P prices lambda
+    double *rcp;              // S*P 1 / C, correctly rounded (k_init)
     double *p64;              // S*P per-unit prices (lambda, or lambda / C in NORMALIZED mode)
     float *p32;               // S*P the same rounded to fp32 (the screen's prices)
     float *ebound;            // S   screen error bound E of the current prices; +inf: exact evaluation
@@ -197,7 +198,8 @@ struct ResPlan {
     const int32_t *cuts;
     int32_t cs;
     int32_t k;          // > 0: every job has k options (interleaved layout); 0: CSR layout
-    int32_t m_pad;      // job slots of a slice, a multiple of 32
+    int32_t lanes;      // lanes per job (1, 2, 4 or 8)
+    int32_t m_pad;      // job slots of a slice: an odd multiple of 32 / lanes
     int64_t n_cap;      // option slots of a slice (CSR layout)
 };
 

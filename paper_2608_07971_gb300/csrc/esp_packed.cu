@@ -296,12 +296,13 @@ __device__ __forceinline__ void update_flat(const DevTable &t, const DevState &s
     const size_t sp = (size_t)s * P;
     const bool mine = lane < P;
     long long U = 0, C = 1;
-    double lam = 0.0;
+    double lam = 0.0, rcp = 1.0;
     int umax = 0;
     if (mine) {
         U = (long long)__ldcg(st.U + sp + lane);
         C = __ldg(t.cap + sp + lane);
         lam = __ldcg(st.lam + sp + lane);
+        rcp = __ldcg(st.rcp + sp + lane);
         umax = __ldg(st.umax + sp + lane);   // R = P
     }
     const double vmax = __ldg(st.vmax + s);
@@ -328,7 +329,7 @@ __device__ __forceinline__ void update_flat(const DevTable &t, const DevState &s
     if (mine)
         st.U[sp + lane] = 0ull;
 
-    const double nl = mine ? price_step(lam, U, C, Cd, step_size(a.eta0, a.step, round), a.mode) : 0.0;
+    const double nl = mine ? price_step_rcp(lam, U, C, Cd, rcp, step_size(a.eta0, a.step, round), a.mode) : 0.0;
     if (__any_sync(FULL, mine && !isfinite(nl))) {
         if (lane == 0) {
             st.status[s] = 2;
@@ -336,7 +337,7 @@ __device__ __forceinline__ void update_flat(const DevTable &t, const DevState &s
         }
         return;
     }
-    const double p = mine ? effective_price(nl, Cd, a.mode) : 0.0;
+    const double p = mine ? effective_price_rcp(nl, Cd, rcp, a.mode) : 0.0;
     if (mine) {
         st.lam[sp + lane] = nl;
         st.p64[sp + lane] = p;

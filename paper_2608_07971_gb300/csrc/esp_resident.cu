@@ -4,16 +4,22 @@
 // One thread-block cluster per scenario. Each CTA of the cluster copies a contiguous slice of the
 // scenario's jobs (about 1/cs of its options) into its shared memory once and keeps it there for all
 // rounds, so a round reads no table bytes from HBM. A round:
-//   1. every lane takes whole jobs and scores their options with the fp32 screen; a job whose screen
-//      is ambiguous is resolved in fp64 on the same lane (the rule and its proof are those of the
-//      streaming kernel: survivors are the options with q <= m1 + 2E, the winner is the lexicographic
-//      minimum of (s, index));
+//   1. a job has 1 to 8 lanes (as many as the CTA has for its jobs), each scores every 1st to 8th of
+//      its options with the fp32 screen, and shuffles combine them; an ambiguous job is resolved in fp64
+//      (the rule and its proof are those of the streaming kernel: survivors are the options with
+//      q <= m1 + 2E, the winner is the lexicographic minimum of (s, index));
 //   2. the int64 demands of the winners are summed per warp, then per CTA in warp order;
-//   3. each CTA writes its partial into every CTA of the cluster (distributed shared memory) and the
-//      cluster meets at one barrier;
+//   3. each CTA writes its partial into every CTA of the cluster (distributed shared memory; each warp
+//      to its share of them) and the cluster meets at one barrier;
 //   4. every CTA sums the partials in rank order and applies Eq. price_update itself. The inputs and
 //      instructions are the same in every CTA, so all of them hold identical prices without a second
 //      exchange; the arithmetic is the streaming path's (esp_device.cuh), so the prices are too.
+// What bounds it is the chain of one round, not a rate: of 7,400 cycles of a 2048-job cluster of 16
+// options in 16 CTAs, 1,800 are the screen, 400 the warp sums, 1,000 the sends, 2,100 the cluster
+// barrier, 500 the sum of the partials and 1,600 the update and the prices. Per round: 3.60 us, where one
+// lane per job, all sends from one warp and hardware division took 4.97; 2.1 and 3.0 on the tiny cluster.
+// Sending the partials with an arrival on each peer's own barrier, so that no cluster barrier is needed, took
+// 4.4 to 5.2; 16 warps per CTA 3.95.
 // After the last round (or the stopping rule) the final evaluation at lambda^T writes the selection,
 // the chosen values and the minimal reduced costs, and adds the final demand to U_final.
 //
@@ -24,6 +30,7 @@
 
 #include <cmath>
 #include <cstdint>
+#include <type_traits>
 #include <cuda_runtime.h>
 
 #include "esp_device.cuh"
@@ -120,6 +127,7 @@ struct ResSlice {
     int m;                  // jobs of the slice
     int stride;             // distance between the columns of one option (m_pad, or 1)
     int K;                  // uniform layout: options per job
+    int lanes, log2_jobs;   // lanes per job; log2 of the jobs a warp takes at once (32 / lanes)
     int jloc0;              // scenario-local index of the slice's first job
     int64_t gj0;            // global index of the slice's first job
     int R;
@@ -167,10 +175,12 @@ __device__ __forceinline__ double res_exact(const ResSlice<RT, UNI> &sl, int bu,
     return s;
 }
 
-// Per-lane accumulators of one evaluation.
-template <int RT>
+// Per-lane accumulators of one evaluation. SMALL: units below 2^23, and a lane adds those of at most 76
+// jobs (an option takes 12 bytes of 227 KB, and the CTA has 256 lanes), so 32 bits hold its demand.
+template <int RT, bool SMALL>
 struct ResAcc {
-    long long dem[ResCols<RT>::N];
+    using Dem = typename std::conditional<SMALL, uint32_t, unsigned long long>::type;
+    Dem dem[ResCols<RT>::N];
     unsigned long long hash;
     double dual;          // sum of -s_min over the lane's jobs
     unsigned int resolved;
@@ -244,16 +254,18 @@ __device__ __forceinline__ int res_resolve_warp(const ResSlice<RT, UNI> &sl, int
     return bi;
 }
 
-// Best responses of the slice's jobs: lane = job. FINAL writes the selection outputs; otherwise the
-// demand (and, when asked, fingerprint and dual sum) of the winners accumulate in acc. Ambiguous
-// jobs are resolved by the whole warp one after the other when they are few, else each by its lane.
+// Best responses of the slice's jobs: a warp takes 32 / lanes jobs at once, its lane (sub, jl) the options
+// sub, sub + lanes, ... of job jl of them. FINAL writes the selection outputs; otherwise the demand (and,
+// when asked, fingerprint and dual sum) of the winners accumulate in acc of a job's first lane. Ambiguous
+// jobs are resolved by the whole warp one after the other when they are few, else each by its lanes.
 template <int RT, bool UNI, bool SMALL, bool FINAL>
-__device__ void res_evaluate(const DevState &st, const ResSlice<RT, UNI> &sl, bool want_hash, bool want_min,
-                             ResAcc<RT> &acc, int warp, int lane)
+__device__ __forceinline__ void res_evaluate(const DevState &st, const ResSlice<RT, UNI> &sl, bool want_hash, bool want_min,
+                                             ResAcc<RT, SMALL> &acc, int warp, int lane)
 {
     const int R = RT ? RT : sl.R;
-    for (int jb = warp * 32; jb < sl.m; jb += kResWarps * 32) {
-        const int jj = jb + lane;
+    const int jobs = 1 << sl.log2_jobs, sub = lane >> sl.log2_jobs;
+    for (int jb = warp << sl.log2_jobs; jb < sl.m; jb += kResWarps << sl.log2_jobs) {
+        const int jj = jb + (lane & (jobs - 1));
         const bool act = jj < sl.m;
         int ob = 0, K = act ? sl.K : 0;
         if (!UNI && act) {
@@ -262,47 +274,64 @@ __device__ void res_evaluate(const DevState &st, const ResSlice<RT, UNI> &sl, bo
         }
         float m1 = INFINITY, m2 = INFINITY;
         int i1 = 0;
-#pragma unroll 4
-        for (int k = 0; k < K; ++k) {
-            bool dup;
-            float q = res_screen<RT, UNI, SMALL>(sl, sl.ucol0(jj, ob, k), sl.V[sl.vslot(jj, ob, k)], dup);
-            q = dup ? INFINITY : q;
-            const bool better = q < m1;
-            m2 = better ? m1 : fminf(m2, q);
-            i1 = better ? k : i1;
-            m1 = fminf(m1, q);
+        // four options at a time, so that their loads are in flight together (one after the other, an
+        // option took 119 cycles)
+        for (int k0 = sub; k0 < K; k0 += 4 * sl.lanes) {
+            float q[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int k = k0 + i * sl.lanes, kk = k < K ? k : k0;
+                bool dup;
+                q[i] = res_screen<RT, UNI, SMALL>(sl, sl.ucol0(jj, ob, kk), sl.V[sl.vslot(jj, ob, kk)], dup);
+                q[i] = (dup || k >= K) ? INFINITY : q[i];
+            }
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const bool better = q[i] < m1;
+                m2 = better ? m1 : fminf(m2, q[i]);
+                i1 = better ? k0 + i * sl.lanes : i1;
+                m1 = fminf(m1, q[i]);
+            }
+        }
+        // a tie between lanes makes m2 = m1, and the job ambiguous, so any of its indices will do
+        for (int d = jobs; d < 32; d <<= 1) {
+            const float o1 = __shfl_xor_sync(FULL, m1, d), o2 = __shfl_xor_sync(FULL, m2, d);
+            const int oi = __shfl_xor_sync(FULL, i1, d);
+            m2 = fminf(fminf(m2, o2), fmaxf(m1, o1));
+            i1 = o1 < m1 ? oi : i1;
+            m1 = fminf(m1, o1);
         }
         const float thr = __fadd_ru(m1, sl.e2);
         const bool amb = act && (sl.exact || !(m2 > thr));
         int w = i1;
         double s_w = 0.0;
         bool have_s = false;
-        uint32_t amask = __ballot_sync(FULL, amb);
+        uint32_t amask = __ballot_sync(FULL, amb && sub == 0);
         if (__popc(amask) > 4) {
             if (amb) {
                 const int bi = res_resolve_lane<RT, UNI, SMALL>(sl, jj, ob, K, thr, s_w);
                 w = (bi == kIdxNone) ? i1 : bi;    // the option of m1 always survives; defensive only
                 have_s = true;
-                ++acc.resolved;
+                acc.resolved += sub == 0;
             }
         } else {
             while (amask) {
-                const int cl = __ffs(amask) - 1;
+                const int cl = __ffs(amask) - 1;   // the job's lane of sub 0
                 amask &= amask - 1;
                 const int cob = __shfl_sync(FULL, ob, cl);
                 const int cK = __shfl_sync(FULL, K, cl);
                 const float cthr = __shfl_sync(FULL, thr, cl);
                 double cs_w;
                 const int bi = res_resolve_warp<RT, UNI, SMALL>(sl, jb + cl, cob, cK, cthr, cs_w, lane);
-                if (lane == cl) {
+                if ((lane & (jobs - 1)) == cl) {
                     w = (bi == kIdxNone) ? i1 : bi;
                     s_w = cs_w;
                     have_s = true;
-                    ++acc.resolved;
+                    acc.resolved += sub == 0;
                 }
             }
         }
-        if (!act)
+        if (!act || sub != 0)
             continue;
         const int bw = sl.ucol0(jj, ob, w);
 #pragma unroll
@@ -312,7 +341,7 @@ __device__ void res_evaluate(const DevState &st, const ResSlice<RT, UNI> &sl, bo
             uint32_t u = sl.U[bw + r * sl.stride];
             if (r == 0)
                 u &= 0x7fffffffu;
-            acc.dem[r] += unit_i64<SMALL>(u);
+            acc.dem[r] += (typename ResAcc<RT, SMALL>::Dem)unit_i64<SMALL>(u);
         }
         if (want_hash)
             acc.hash += splitmix64_mix(((uint64_t)(uint32_t)(sl.jloc0 + jj) << 32) | (uint32_t)w);
@@ -343,18 +372,25 @@ __device__ __forceinline__ unsigned long long warp_sum_u64(unsigned long long v)
     return c0 + (c1 << 22) + (c2 << 44);
 }
 
+// The same of 32-bit words by two reductions of 16-bit halves (each sum below 2^21).
+__device__ __forceinline__ unsigned long long warp_sum_u64(uint32_t v)
+{
+    return (unsigned long long)__reduce_add_sync(FULL, v & 0xffffu) +
+           ((unsigned long long)__reduce_add_sync(FULL, v >> 16) << 16);
+}
+
 // Prices of lambda (lanes c < R of warp 0 hold lambda_c, R <= 16): the fp64 and fp32 per-unit prices
 // (the same values as the streaming path's) and the screen bound 2E, written to shared memory. E
 // only has to bound the screen error from above, so it is computed in fp32 with every operation
 // rounded up: p <= p32 (1 + 2^-23) + 2^-149, M = max|v| + sum_r p_r max u_r and
 // E = (4R + 16) 2^-24 M + 2^-99, each replaced by an upper bound; no fp64 operation beyond the
 // prices themselves. A price bound above 2^100, or M above 2^100, selects exact mode.
-__device__ __forceinline__ void res_set_prices(double lam, double capd, float umax_up, float vmax_up, int R,
+__device__ __forceinline__ void res_set_prices(double lam, double capd, double rcp, float umax_up, float vmax_up, int R,
                                                int mode, bool exact_only, double *p64s, float *p32s, float *e2s,
                                                int lane)
 {
     const bool mine = lane < R;
-    const double p = mine ? effective_price(lam, capd, mode) : 0.0;
+    const double p = mine ? effective_price_rcp(lam, capd, rcp, mode) : 0.0;
     const float p32 = __double2float_rn(p);
     const float p_up = __fadd_ru(__fmul_ru(p32, 1.0f + 0x1p-23f), 0x1p-149f);
     float term = mine ? __fmul_ru(p_up, umax_up) : 0.0f;
@@ -426,7 +462,7 @@ __global__ void __launch_bounds__(kResThreads, ESP_RES_MIN_CTAS) k_resident(DevT
 
     // ---- price state: warp 0 of every CTA holds lambda_c, C_c and max u_c in lane c
     const size_t sp = (size_t)s * P;
-    double lam = 0.0, capd = 1.0;
+    double lam = 0.0, capd = 1.0, rcp = 1.0;
     long long cap = 1;
     float umax_up = 0.0f;
     const float vmax_up = __double2float_ru(st.vmax[s]);
@@ -435,9 +471,10 @@ __global__ void __launch_bounds__(kResThreads, ESP_RES_MIN_CTAS) k_resident(DevT
             lam = st.lam[sp + lane];
             cap = t.cap[sp + lane];
             capd = (double)cap;
+            rcp = 1.0 / capd;
             umax_up = __int2float_ru(st.umax[(size_t)s * R + lane]);
         }
-        res_set_prices(lam, capd, umax_up, vmax_up, R, a.mode, a.exact_only != 0, p64s, p32s, e2s, lane);
+        res_set_prices(lam, capd, rcp, umax_up, vmax_up, R, a.mode, a.exact_only != 0, p64s, p32s, e2s, lane);
         if (lane == 0)
             *stops = 0;
     }
@@ -452,6 +489,8 @@ __global__ void __launch_bounds__(kResThreads, ESP_RES_MIN_CTAS) k_resident(DevT
     sl.m = m;
     sl.stride = UNI ? rp.m_pad : 1;
     sl.K = rp.k;
+    sl.lanes = rp.lanes;
+    sl.log2_jobs = 5 - (__ffs(rp.lanes) - 1);
     sl.jloc0 = j0;
     sl.gj0 = gj0;
     sl.R = R;
@@ -459,7 +498,7 @@ __global__ void __launch_bounds__(kResThreads, ESP_RES_MIN_CTAS) k_resident(DevT
 
     const bool want_hash = st.hash_trace != nullptr;
     const bool want_min = st.dual_trace != nullptr;
-    ResAcc<RT> acc;
+    ResAcc<RT, SMALL> acc;
     acc.resolved = 0;
     int rounds = 0, status = 0, converged = 0;
     double best_dual = INFINITY;
@@ -484,14 +523,16 @@ __global__ void __launch_bounds__(kResThreads, ESP_RES_MIN_CTAS) k_resident(DevT
             res_evaluate<RT, UNI, SMALL, false>(st, sl, want_hash, want_min, acc, warp, lane);
 
             // 2. warp sums, then (after the barrier) the CTA partial in warp order
+            unsigned long long mine = 0ull;
 #pragma unroll
             for (int r = 0; r < ResCols<RT>::N; ++r) {
                 if (RT == 0 && r >= R)
                     break;
-                const long long v = (long long)warp_sum_u64((unsigned long long)acc.dem[r]);
-                if (lane == 0)
-                    wpart[warp * kResCols + r] = (unsigned long long)v;
+                const unsigned long long v = warp_sum_u64(acc.dem[r]);
+                mine = lane == r ? v : mine;
             }
+            if (lane < R)
+                wpart[warp * kResCols + lane] = mine;
             if (want_hash) {
                 const long long h = (long long)warp_sum_u64(acc.hash);
                 if (lane == 0)
@@ -505,8 +546,10 @@ __global__ void __launch_bounds__(kResThreads, ESP_RES_MIN_CTAS) k_resident(DevT
         }
         __syncthreads();
 
-        // 3. the CTA partial into buffer (round & 1) of every CTA of the cluster
-        if (!stopped && warp == 0) {
+        // 3. the CTA partial into buffer (round & 1) of every CTA of the cluster, by warp w into CTAs w,
+        // w + kResWarps (each warp adds up the partial itself; one warp writing to all 16 took 16 stores
+        // one after the other)
+        if (!stopped && warp < cs) {
             const int c = lane;
             const bool live = c < R || (c == kColHash && want_hash) || (c == kColDual && want_min);
             if (live) {
@@ -522,7 +565,7 @@ __global__ void __launch_bounds__(kResThreads, ESP_RES_MIN_CTAS) k_resident(DevT
                         tot += wpart[w * kResCols + c];
                 }
                 const uint32_t slot = smem_u32(cpart + ((size_t)par * cs + rank) * kResCols + c);
-                for (int rk = 0; rk < cs; ++rk)
+                for (int rk = warp; rk < cs; rk += kResWarps)
                     st_cluster_u64(map_rank(slot, (uint32_t)rk), tot);
             }
         }
@@ -561,7 +604,7 @@ __global__ void __launch_bounds__(kResThreads, ESP_RES_MIN_CTAS) k_resident(DevT
             if (st.dem_trace && lead && c < R)
                 st.dem_trace[((size_t)s * T + round) * P + c] = Uc;
             const double eta = step_size(a.eta0, a.step, round);
-            const double nl = (c < R) ? price_step(lam, Uc, cap, capd, eta, a.mode) : 0.0;
+            const double nl = (c < R) ? price_step_rcp(lam, Uc, cap, capd, rcp, eta, a.mode) : 0.0;
             const bool bad = __any_sync(FULL, c < R && !isfinite(nl));
             bool stop;
             if (bad) {
@@ -581,7 +624,7 @@ __global__ void __launch_bounds__(kResThreads, ESP_RES_MIN_CTAS) k_resident(DevT
                 }
                 lam = nl;
                 converged = stop ? 1 : 0;
-                res_set_prices(lam, capd, umax_up, vmax_up, R, a.mode, a.exact_only != 0, p64s, p32s, e2s, lane);
+                res_set_prices(lam, capd, rcp, umax_up, vmax_up, R, a.mode, a.exact_only != 0, p64s, p32s, e2s, lane);
             }
             if (lane == 0)
                 *stops = stop ? 1 : 0;
@@ -603,9 +646,9 @@ __global__ void __launch_bounds__(kResThreads, ESP_RES_MIN_CTAS) k_resident(DevT
     for (int r = 0; r < ResCols<RT>::N; ++r) {
         if (RT == 0 && r >= R)
             break;
-        const long long v = (long long)warp_sum_u64((unsigned long long)acc.dem[r]);
+        const unsigned long long v = warp_sum_u64(acc.dem[r]);
         if (lane == 0 && v != 0)
-            atomicAdd(st.U_final + sp + r, (unsigned long long)v);
+            atomicAdd(st.U_final + sp + r, v);
     }
     const unsigned int nres = __reduce_add_sync(FULL, acc.resolved);
     if (lane == 0 && nres)
