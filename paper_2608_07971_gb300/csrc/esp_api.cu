@@ -104,7 +104,7 @@ struct esp_ctx {
     unsigned char *il = nullptr;
     int64_t n_tiles = 0;
 
-    // the packed screen copy and its plan (esp_packed.h): what the passes of an ungrouped table with
+    // the packed screen copy and its plan (esp_packed.h): what the passes of a table with
     // units below 2^23 read
     bool packed = false;
     DevPack pack = {};
@@ -568,6 +568,9 @@ esp_status load_packed(esp_ctx *ctx, const PackFormat &fmt)
     if (st != ESP_OK)
         return st;
     DevPack &d = ctx->pack;
+    d.all_k = ctx->pc.min_k == ctx->pc.max_k && p.job.empty() && ctx->pc.max_k <= INT32_MAX ? (int32_t)ctx->pc.max_k : 0;
+    if (d.all_k == 0 && (st = dev_alloc(ctx, &d.opt0, (size_t)ctx->S * ctx->J, 64, false)) != ESP_OK)
+        return st;
     d.data = ctx->pk_data;
     d.tiles = tiles;
     d.job_begin = jb;
@@ -587,8 +590,9 @@ esp_status load_packed(esp_ctx *ctx, const PackFormat &fmt)
     // 2 / 4 / 16 scenarios 50 / 91 / 247 against 48 / 63 / 170: below, the waits for prices cost more than
     // the launches; above, static tile ranges leave the GPU waiting for its slowest warps. Smaller
     // tables of R = 4, 6, 8 take it on request.
-    const int per_sm = packed_ctas_per_sm(fmt.nw);
-    if (per_sm > 0 && d.n_tiles > 0) {
+    // A table with a group column has no persistent pass.
+    const int per_sm = packed_ctas_per_sm(fmt.nw, fmt.g_bytes);
+    if (per_sm > 0 && d.n_tiles > 0 && !ctx->group) {
         ctx->persist_auto = p.steps >= (int64_t)kPersistMinSteps * per_sm * ctx->sm_count * kWarpsPerCta;
         if (ctx->persist_auto || ctx->R == 4 || ctx->R == 6 || ctx->R == 8)
             ctx->persist_grid = (int32_t)std::min<int64_t>((int64_t)per_sm * ctx->sm_count,
@@ -864,19 +868,21 @@ esp_status load_common(esp_ctx *ctx, int32_t S, int32_t J, int32_t R, int32_t P,
     // plan the evaluation pass
     ctx->uniform_k = (!grouped && min_k == max_k && max_k <= 32 && (max_k & (max_k - 1)) == 0) ? (int32_t)max_k : 0;
 
-    // the packed passes (esp_packed.h) take a table without a group column whose units are below 2^23;
-    // the last is known after the validation, so the plan for them is made meanwhile, for the unit
-    // words that pairs of columns need. Tables they do not take are evaluated by the staged pass, general
-    // ones without a group column in the sorted layout.
+    // the packed passes (esp_packed.h) take a table whose units are below 2^23, grouped ones where
+    // pack_groups_fit; the first is known after the validation, so the plan for them is made meanwhile, for
+    // the unit words that pairs of columns need. Tables they do not take are evaluated by the staged pass,
+    // general ones without a group column in the sorted layout.
     const bool may_sort = ctx->sorted_enabled && !grouped && ctx->uniform_k == 0 && J >= 1;
-    const bool may_pack = ctx->il_enabled && ctx->il_f32_enabled && !grouped && (ctx->uniform_k > 0 || may_sort) &&
-                          n_jobs > 0;
+    const bool may_pack = ctx->il_enabled && ctx->il_f32_enabled && n_jobs > 0 &&
+                          (grouped ? pack_groups_fit(R, rg, P) : ctx->uniform_k > 0 || may_sort);
+    const int group_bytes = grouped ? pack_group_bytes(P, n_groups) : 0;
     ctx->load_ms[1] = since();
     PackPlan pack_new;
     int32_t pack_warps = 0;
     bool pack_cached = false, pack_ok = false;
     if (may_pack) {
-        const int per_sm = packed_ctas_per_sm(R <= 4 ? 2 : R <= 6 ? 3 : R <= 8 ? 4 : R <= 12 ? 6 : 8);
+        const int per_sm = grouped ? packed_ctas_per_sm(R <= 6 ? 3 : R <= 8 ? 4 : 6, group_bytes)
+                                   : packed_ctas_per_sm(R <= 4 ? 2 : R <= 6 ? 3 : R <= 8 ? 4 : R <= 12 ? 6 : 8);
         const int waves = ctx->plan_waves > 0 ? ctx->plan_waves : 1;
         pack_warps = ctx->sm_count * std::max(per_sm, 1) * kWarpsPerCta * waves;
         pack_cached = cached && pc.has_pack && pc.pack_warps == pack_warps;
@@ -922,7 +928,8 @@ esp_status load_common(esp_ctx *ctx, int32_t S, int32_t J, int32_t R, int32_t P,
     }
     ALLOC(ctx->arrive, (size_t)S);
     PackFormat fmt;
-    if (pack_ok && pack_format(col_max.data(), R, fmt)) {
+    if (pack_ok && pack_format(col_max.data(), R, fmt, rg, n_groups)) {
+        fmt.g_bytes = group_bytes;
         if ((st = load_packed(ctx, fmt)) != ESP_OK) {
             release_table(ctx);
             return st;
@@ -997,7 +1004,7 @@ bool state_ready(const esp_ctx *c)
                c->place.node_type && c->place.D && c->place.cfg_dup && c->place.warp_job && c->place.n_warps > 0 &&
                c->scen_warps;
     if (c->packed)
-        return c->pack.data && c->pack.tiles && c->pack.job_begin && c->pack.warp_begin && c->pack.scen_tiles && c->units &&
+        return c->pack.data && (c->pack.all_k > 0 || c->pack.opt0) && c->pack.tiles && c->pack.job_begin && c->pack.warp_begin && c->pack.scen_tiles && c->units &&
                c->values && c->off;
     return c->grid == 0 || (c->scen_warps && c->tiles && c->warp_begin && c->units && c->values && c->off);
 }

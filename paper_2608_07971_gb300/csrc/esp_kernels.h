@@ -87,15 +87,18 @@ struct DevPack {
     const PackTile *tiles;       // n_tiles
     const int32_t *job_begin;    // n_tiles: first job (packed order) of each tile
     const int32_t *job;          // table job of each job in the packed order; nullptr: the same
+    int64_t *opt0;               // first option of each job in the packed order (k_pack); nullptr when all_k > 0
     const int32_t *warp_begin;   // n_warps + 1: the round pass's tile ranges
     const int32_t *scen_tiles;   // S: tiles of each scenario (arrivals count tiles)
     int32_t n_tiles, n_warps;
+    int32_t all_k;               // options of every job where all have the same, in the table's order; else 0
     int32_t fused;               // the last arrival of a scenario in a round updates its prices
     PackFormat fmt;
 };
 
 // Resident CTAs per SM of the packed passes (round and persistent) for nw unit words; 0: no such kernel.
-int packed_ctas_per_sm(int nw);
+// group_bytes > 0: of the round passes of a table with a group column (PackFormat::g_bytes).
+int packed_ctas_per_sm(int nw, int group_bytes = 0);
 // Fills the packed copy of table t (duplicate marks included) for the tiles of pk.
 cudaError_t launch_pack(const DevTable &t, const DevPack &pk, uint4 *data, cudaStream_t stream);
 // One evaluation pass over the packed copy (round passes with fused updates when pk.fused).

@@ -17,6 +17,12 @@
 // M = |v| + sum_r p_r u_r, so |q - s| <= (R + 4) u M (1 + small) + 2^-99 holds as for the chain in column
 // order, and the decision rule and its proof are those of esp_kernels.cu.
 //
+// Tables with a group column (G): the option's group slot is a field of one of its words, the columns priced
+// per group are its last word, and their two prices come from a table in the warp's shared memory. The
+// placement table of 4096 jobs x 768 options (R = 8, 64 groups; 20 bytes per option instead of 42) takes 29.1 us
+// per round where the staged pass took 77.4; of the 29, 19 are the screen (63 MB, which L2 holds), the rest the
+// chain of the slowest ambiguous job and of the update of 134 prices.
+//
 // The winner's units come from the words in the slot. Values in fp64 and int32 units are read from
 // the table itself, only to rescore the survivors of ambiguous jobs and for the outputs of the final
 // pass.
@@ -44,10 +50,11 @@ constexpr int kPackSlots = 2;        // steps a warp holds: the one being screen
 // most 8 per step and kPackTileSteps (8) steps (a job of more steps counts once).
 constexpr uint32_t kPackSpill = 511 - 8 * 8;
 
-// Resident CTAs the register budget must allow.
-constexpr int pack_min_ctas(int nw)
+// Resident CTAs the register budget must allow (grouped with five: 44.1 us per round of the placement table
+// of 4096 jobs x 768 options against 38.7, for the spills).
+constexpr int pack_min_ctas(int nw, bool grouped = false)
 {
-    return nw <= 3 ? ESP_PACK_CTAS : nw == 4 ? 5 : 4;
+    return grouped ? 4 : nw <= 3 ? ESP_PACK_CTAS : nw == 4 ? 5 : 4;
 }
 
 // Shared memory of a warp: the slots, then their barriers.
@@ -104,6 +111,7 @@ struct Ctx {
     uint32_t wins;                  // upper bound of the winners in them
     unsigned long long hash;
     const double *p64;              // fp64 prices of the scenario
+    unsigned char *groups;          // grouped tables: shared memory, the two fp32 prices of each group slot
     float e2;                       // 2E, +inf: exact evaluation
     bool exact, skip;
     int s;                          // scenario, -1: none
@@ -112,13 +120,22 @@ struct Ctx {
 };
 
 // Scores of the four options of vector `v` of plane 0; the other planes follow `plane` vectors apart.
-template <int NW>
+template <int NW, bool G>
 __device__ __forceinline__ void screen4(const uint4 *v, int plane, const PackFormat &f, const Ctx<NW> &c, float *q)
 {
     const unsigned long long bias = pack2(-8388608.0f, -8388608.0f);
     const uint4 n = v[0];
     unsigned long long acc[4] = {pack2(__uint_as_float(n.x), 0.0f), pack2(__uint_as_float(n.y), 0.0f),
                                  pack2(__uint_as_float(n.z), 0.0f), pack2(__uint_as_float(n.w), 0.0f)};
+    // the last word's prices are those of the option's group
+    unsigned long long own[4];
+    if (G) {
+        const uint4 y = v[(f.g_word + 1) * plane];
+        const uint32_t x[4] = {y.x, y.y, y.z, y.w};
+#pragma unroll
+        for (int o = 0; o < 4; ++o)
+            own[o] = *reinterpret_cast<const unsigned long long *>(c.groups + 8 * ((x[o] >> f.g_shift) & f.g_mask));
+    }
 #pragma unroll
     for (int k = 0; k < NW; ++k) {
         const uint4 y = v[(k + 1) * plane];
@@ -127,7 +144,7 @@ __device__ __forceinline__ void screen4(const uint4 *v, int plane, const PackFor
         for (int o = 0; o < 4; ++o) {
             const uint32_t lo = (x[o] & f.mask[k]) | 0x4b000000u;
             const uint32_t hi = __funnelshift_r(x[o], f.magic[k], f.shift[k]);
-            acc[o] = fma2(c.price[k], add2(pack2(__uint_as_float(lo), __uint_as_float(hi)), bias), acc[o]);
+            acc[o] = fma2(G && k == NW - 1 ? own[o] : c.price[k], add2(pack2(__uint_as_float(lo), __uint_as_float(hi)), bias), acc[o]);
         }
     }
 #pragma unroll
@@ -146,18 +163,6 @@ __device__ __forceinline__ void two_smallest(const float *q, float &m1, float &m
     m2 = fminf(fmaxf(a0, b0), fminf(a1, b1));
 }
 
-// Adds the units in the word at w (plane 0) to the lane's demand.
-template <int NW>
-__device__ __forceinline__ void add_option(Ctx<NW> &c, const PackFormat &f, const uint32_t *w, int plane)
-{
-#pragma unroll
-    for (int k = 0; k < NW; ++k) {
-        const uint32_t x = w[(k + 1) * plane * 4];
-        c.lo[k] += x & f.mask[k];
-        c.hi[k] += x >> f.shift[k];
-    }
-}
-
 // Everything a pass needs beyond the warp's own state.
 struct Pass {
     const DevTable &t;
@@ -168,16 +173,74 @@ struct Pass {
     bool want_min, want_hash;   // minimal reduced costs; selection fingerprints
 };
 
-// The exact score of option o of the pass table (the chain of Eq. esp_score in column order).
-__device__ __forceinline__ double exact_option(const int32_t *units, const double *values, int R, const double *p64,
-                                               int64_t o)
+// The scenario's demand totals.
+template <int NW>
+__device__ __forceinline__ unsigned long long *totals(const Pass &ps, const Ctx<NW> &c)
 {
-    const int32_t *u = units + o * R;
-    double s = -__ldg(values + o);
-    for (int r = 0; r < R; ++r) {
-        const int32_t x = __ldg(u + r);
-        // prices through L2: a persistent pass sees them change between rounds
-        s = __fma_rn(__ldcg(p64 + r), __int2double_rn(r == 0 ? (x & 0x7fffffff) : x), s);
+    return (ps.kind == PASS_ROUND ? ps.st.U : ps.st.U_final) + (size_t)c.s * ps.t.P;
+}
+
+// Group columns of a winner: straight to the totals of its group (a scenario's winners spread over its groups).
+template <int NW>
+__device__ __forceinline__ void add_group(const Pass &ps, const Ctx<NW> &c, uint32_t x, uint32_t slot_word)
+{
+    const PackFormat &f = ps.pk.fmt;
+    const uint32_t lo = x & f.mask[NW - 1], hi = f.col_hi[NW - 1] >= 0 ? x >> f.shift[NW - 1] : 0u;
+    const int rg = ps.t.r_global;
+    unsigned long long *dst =
+        totals(ps, c) + rg + (ps.t.R - rg) * (int)pack_slot_group((slot_word >> f.g_shift) & f.g_mask);
+    if (lo != 0u)
+        atomicAdd(dst, (unsigned long long)lo);
+    if (hi != 0u)
+        atomicAdd(dst + 1, (unsigned long long)hi);
+}
+
+// Adds the units in the word at w (plane 0) to the lane's demand.
+template <int NW, bool G>
+__device__ __forceinline__ void add_option(const Pass &ps, Ctx<NW> &c, const uint32_t *w, int plane)
+{
+    const PackFormat &f = ps.pk.fmt;
+#pragma unroll
+    for (int k = 0; k < (G ? NW - 1 : NW); ++k) {
+        const uint32_t x = w[(k + 1) * plane * 4];
+        c.lo[k] += x & f.mask[k];
+        c.hi[k] += x >> f.shift[k];
+    }
+    if (G)
+        add_group(ps, c, w[NW * plane * 4], w[(f.g_word + 1) * plane * 4]);
+}
+
+// The exact score of option o of the pass table (the chain of Eq. esp_score in column order).
+template <bool G>
+__device__ __forceinline__ double exact_option(const DevTable &t, const double *p64, int64_t o)
+{
+    const int R = t.R, rg = t.r_global;
+    const int32_t *u = t.units + o * R;
+    double s = -__ldg(t.values + o);
+    if (!G) {
+        for (int r = 0; r < R; ++r) {
+            const int32_t x = __ldg(u + r);
+            // prices through L2: a persistent pass sees them change between rounds
+            s = __fma_rn(__ldcg(p64 + r), __int2double_rn(r == 0 ? (x & 0x7fffffff) : x), s);
+        }
+        return s;
+    }
+    // four columns' units and prices on their way together (placement table of 4096 jobs: 38.7 -> 37.0 us per
+    // round; without groups the plain loop is the faster one, 10.3 against 10.7 on a 2048-job cluster)
+    const int own = (R - rg) * (int)__ldg(t.group + o);
+    for (int r0 = 0; r0 < R; r0 += 4) {
+        double p[4];
+        int32_t x[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int r = r0 + i < R ? r0 + i : r0;
+            x[i] = __ldg(u + r);
+            p[i] = __ldcg(p64 + (r >= rg ? r + own : r));
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            if (r0 + i < R)
+                s = __fma_rn(p[i], __int2double_rn(x[i] & 0x7fffffff), s);
     }
     return s;
 }
@@ -189,14 +252,14 @@ struct Exact {
 
 // The lexicographic minimum of (s, index) over the options first + i, i in the bits of `mask`, in fp64;
 // their indices are loc + i. (Ambiguous jobs only; out of line it made the row loops spill around the call.)
-__device__ __forceinline__ Exact rescore(const int32_t *units, const double *values, int R, const double *p64,
-                                      int64_t first, uint32_t mask, int loc)
+template <bool G>
+__device__ __forceinline__ Exact rescore(const DevTable &t, const double *p64, int64_t first, uint32_t mask, int loc)
 {
     Exact x{0x7fffffffffffffffLL, kIdxNone};
     while (mask != 0u) {
         const int i = __ffs((int)mask) - 1;
         mask &= mask - 1;
-        const long long k = order_key(exact_option(units, values, R, p64, first + i));
+        const long long k = order_key(exact_option<G>(t, p64, first + i));
         if (k < x.key) {   // increasing index: the first of equal scores stays
             x.key = k;
             x.idx = loc + i;
@@ -229,45 +292,39 @@ __device__ __forceinline__ uint32_t survivors(const uint4 &n, const float *q, bo
            ((n.w != kPackInf && (exact || q[3] <= thr)) ? 8u : 0u);
 }
 
-// Table job and first option of job jl of tile k.
-struct JobAt {
-    int64_t job, opt0;
-};
-
-__device__ __forceinline__ JobAt job_at(const Pass &ps, int k, int jl)
+// First option of packed job i. Of a table whose jobs have all the same number of options it is known without
+// a load, else with one: an ambiguous job is a chain of trips to memory, and the round waits for the slowest.
+__device__ __forceinline__ int64_t first_option(const Pass &ps, int i)
 {
-    const int i = __ldg(ps.pk.job_begin + k) + jl;
-    JobAt x;
-    x.job = ps.pk.job ? __ldg(ps.pk.job + i) : i;
-    x.opt0 = __ldg(ps.t.job_off + x.job);
-    return x;
+    return ps.pk.all_k > 0 ? (int64_t)i * ps.pk.all_k : __ldg(ps.pk.opt0 + i);
 }
 
-// Outputs of a winner beyond its demand: its job, local index and, when known, exact score.
-template <int NW>
-__device__ __forceinline__ void extras(const Pass &ps, Ctx<NW> &c, const JobAt &at, int local, bool have_s, long long key)
+// Outputs of a winner beyond its demand: its packed job, local index and, when known, exact score.
+template <int NW, bool G>
+__device__ __forceinline__ void extras(const Pass &ps, Ctx<NW> &c, int i, int local, bool have_s, long long key)
 {
+    const int64_t job = ps.pk.job ? __ldg(ps.pk.job + i) : i;
     if (ps.want_hash)
-        c.hash += splitmix64_mix(((uint64_t)(uint32_t)(at.job - (int64_t)c.s * ps.t.J) << 32) | (uint32_t)local);
+        c.hash += splitmix64_mix(((uint64_t)(uint32_t)(job - (int64_t)c.s * ps.t.J) << 32) | (uint32_t)local);
     if (ps.kind == PASS_FINAL) {
-        ps.st.sel[at.job] = local;
-        ps.st.job_val[at.job] = __ldg(ps.t.values + at.opt0 + local);
+        ps.st.sel[job] = local;
+        ps.st.job_val[job] = __ldg(ps.t.values + first_option(ps, i) + local);
     }
     if (ps.want_min)
-        ps.st.job_min[at.job] = have_s ? key_value(key)
-                                       : exact_option(ps.t.units, ps.t.values, ps.t.R, c.p64, at.opt0 + local);
+        ps.st.job_min[job] = have_s ? key_value(key) : exact_option<G>(ps.t, c.p64, first_option(ps, i) + local);
 }
 
 // Adds the lane's demand to the scenario's totals: every sum across the warp by two hardware reductions
 // of 16-bit halves (each below 2^21), then one atomic per field, all fields in one instruction.
-template <int NW>
+template <int NW, bool G>
 __device__ __forceinline__ void add_demand(const Pass &ps, Ctx<NW> &c)
 {
-    unsigned long long *dst = (ps.kind == PASS_ROUND ? ps.st.U : ps.st.U_final) + (size_t)c.s * ps.t.P;
+    constexpr int NU = G ? NW - 1 : NW;   // words of columns without groups
+    unsigned long long *dst = totals(ps, c);
     unsigned long long mine = 0ull;
     int col = -1;
 #pragma unroll
-    for (int i = 0; i < 2 * NW; ++i) {
+    for (int i = 0; i < 2 * NU; ++i) {
         const uint32_t v = (i & 1) ? c.hi[i >> 1] : c.lo[i >> 1];
         const unsigned long long x = (unsigned long long)__reduce_add_sync(FULL, v & 0xffffu) +
                                      ((unsigned long long)__reduce_add_sync(FULL, v >> 16) << 16);
@@ -284,6 +341,41 @@ __device__ __forceinline__ void add_demand(const Pass &ps, Ctx<NW> &c)
     c.wins = 0;
 }
 
+// What an update records before the prices move: the dual value of the round, the fingerprint.
+__device__ __forceinline__ void trace_round(const DevTable &t, const DevState &st, const SolveArgs &a, int s, int round,
+                                            double lam_part, int lane)
+{
+    if (st.dual_trace) {   // g(lambda^t) from the minimal reduced costs of round t
+        double part = 0.0;
+        for (int j = lane; j < t.J; j += 32)
+            part += -__ldcg(st.job_min + (size_t)s * t.J + j);
+        const double g = warp_sum_fixed(part) + warp_sum_fixed(lam_part);
+        if (lane == 0) {
+            st.dual_trace[(size_t)s * (a.T + 1) + round] = g;
+            if (g < st.best_dual[s])
+                st.best_dual[s] = g;
+        }
+    }
+    if (st.hash_trace && lane == 0) {
+        st.hash_trace[(size_t)s * a.T + round] = __ldcg(st.hash + s);
+        st.hash[s] = 0ull;
+    }
+}
+
+// The end of an update (lane 0): the new prices' bound, the round's time and the stopping rule.
+__device__ __forceinline__ void close_round(const DevTable &t, const DevState &st, const SolveArgs &a, int s, int round,
+                                            double M, bool huge, bool conv)
+{
+    st.ebound[s] = screen_bound(M, t.R, a.exact_only || huge);
+    if (st.time_trace)
+        st.time_trace[(size_t)s * a.T + round] = global_ns();
+    st.rounds_run[s] = round + 1;
+    if (conv) {
+        st.converged[s] = 1;
+        st.frozen[s] = 1;
+    }
+}
+
 // Eq. price_update for scenario s of a table without a group column after round `round` (one warp, lane k
 // holds price k: P = R <= 16), as update_scenario does it, with every input loaded at once and the new
 // prices and bound computed from registers. The chain of dependent trips to L2 is what this costs (it
@@ -292,7 +384,7 @@ __device__ __forceinline__ void add_demand(const Pass &ps, Ctx<NW> &c)
 __device__ __forceinline__ void update_flat(const DevTable &t, const DevState &st, const SolveArgs &a, int s, int round,
                                             int lane)
 {
-    const int P = t.P, J = t.J, T = a.T;
+    const int P = t.P, T = a.T;
     const size_t sp = (size_t)s * P;
     const bool mine = lane < P;
     long long U = 0, C = 1;
@@ -308,22 +400,7 @@ __device__ __forceinline__ void update_flat(const DevTable &t, const DevState &s
     const double vmax = __ldg(st.vmax + s);
     const double Cd = (double)C;
 
-    if (st.dual_trace) {   // g(lambda^t) from the minimal reduced costs of round t
-        double part = 0.0;
-        for (int j = lane; j < J; j += 32)
-            part += -__ldcg(st.job_min + (size_t)s * J + j);
-        const double lc = mine ? ((a.mode == 1) ? lam : lam * Cd) : 0.0;
-        const double g = warp_sum_fixed(part) + warp_sum_fixed(lc);
-        if (lane == 0) {
-            st.dual_trace[(size_t)s * (T + 1) + round] = g;
-            if (g < st.best_dual[s])
-                st.best_dual[s] = g;
-        }
-    }
-    if (st.hash_trace && lane == 0) {
-        st.hash_trace[(size_t)s * T + round] = __ldcg(st.hash + s);
-        st.hash[s] = 0ull;
-    }
+    trace_round(t, st, a, s, round, mine ? ((a.mode == 1) ? lam : lam * Cd) : 0.0, lane);
     if (st.dem_trace && mine)
         st.dem_trace[((size_t)s * T + round) * P + lane] = U;
     if (mine)
@@ -352,25 +429,124 @@ __device__ __forceinline__ void update_flat(const DevTable &t, const DevState &s
         const double dmax = warp_max(mine ? fabs(nl - lam) : 0.0), amax = warp_max(mine ? fabs(lam) : 0.0);
         conv = dmax <= a.tol * fmax(1.0, amax);
     }
-    if (lane == 0) {
-        st.ebound[s] = screen_bound(M, t.R, a.exact_only || huge);
-        if (st.time_trace)
-            st.time_trace[(size_t)s * T + round] = global_ns();
-        st.rounds_run[s] = round + 1;
-        if (conv) {
-            st.converged[s] = 1;
-            st.frozen[s] = 1;
+    if (lane == 0)
+        close_round(t, st, a, s, round, M, huge, conv);
+}
+
+constexpr int kKeepAtOnce = 5;
+
+// The same for a table with a group column: P prices, new ones kept in `keep` (P doubles of the warp's shared
+// memory) until all are known to be finite.
+__device__ __forceinline__ void update_grouped(const DevTable &t, const DevState &st, const SolveArgs &a, int s, int round,
+                                               double *keep, int lane)
+{
+    const int P = t.P, T = a.T, R = t.R, rg = t.r_global, own = R - rg;   // own: 1 or 2 columns per group
+    const size_t sp = (size_t)s * P;
+    double lc = 0.0;
+    if (st.dual_trace)
+        for (int k = lane; k < P; k += 32) {
+            const double lam = __ldcg(st.lam + sp + k);
+            lc += (a.mode == 1) ? lam : lam * (double)__ldg(t.cap + sp + k);
+        }
+    trace_round(t, st, a, s, round, lc, lane);
+    const double eta = step_size(a.eta0, a.step, round);
+    const double vmax = __ldg(st.vmax + s);
+    const int umax = lane < R ? __ldg(st.umax + (size_t)s * R + lane) : 0;
+    bool bad = false;
+    double dmax = 0.0, amax = 0.0;
+    __syncwarp();   // every lane is done with the group prices in the same memory
+    // five of a lane's prices at a time, their loads together (a loop whose last turn only some lanes take
+    // ran one price after the other: 10 us for 134 prices)
+    for (int k0 = lane; k0 < P + lane; k0 += 32 * kKeepAtOnce) {
+        long long U[kKeepAtOnce], C[kKeepAtOnce];
+        double lam[kKeepAtOnce], rcp[kKeepAtOnce];
+#pragma unroll
+        for (int i = 0; i < kKeepAtOnce; ++i) {
+            const int k = k0 + 32 * i < P ? k0 + 32 * i : 0;
+            U[i] = (long long)__ldcg(st.U + sp + k);
+            C[i] = __ldg(t.cap + sp + k);
+            lam[i] = __ldcg(st.lam + sp + k);
+            rcp[i] = __ldg(st.rcp + sp + k);
+        }
+#pragma unroll
+        for (int i = 0; i < kKeepAtOnce; ++i) {
+            const int k = k0 + 32 * i;
+            const double nl = price_step_rcp(lam[i], U[i], C[i], (double)C[i], rcp[i], eta, a.mode);
+            if (k >= P)
+                continue;
+            if (st.dem_trace)
+                st.dem_trace[((size_t)s * T + round) * P + k] = U[i];
+            keep[k] = nl;
+            bad |= !isfinite(nl);
+            dmax = fmax(dmax, fabs(nl - lam[i]));
+            amax = fmax(amax, fabs(lam[i]));
         }
     }
+    __syncwarp();
+    bad = __any_sync(FULL, bad);
+    bool huge = false;
+    double flat = 0.0, pm0 = 0.0, pm1 = 0.0;   // the lane's global price, its largest price of each group column
+    for (int k0 = lane; k0 < P + lane; k0 += 32 * kKeepAtOnce) {
+        double nl[kKeepAtOnce], p[kKeepAtOnce];
+#pragma unroll
+        for (int i = 0; i < kKeepAtOnce; ++i) {
+            const int k = k0 + 32 * i < P ? k0 + 32 * i : lane < P ? lane : 0;
+            nl[i] = keep[k];
+            p[i] = effective_price_rcp(nl[i], (double)__ldg(t.cap + sp + k), __ldg(st.rcp + sp + k), a.mode);
+        }
+#pragma unroll
+        for (int i = 0; i < kKeepAtOnce; ++i) {
+            const int k = k0 + 32 * i;
+            if (k >= P)
+                continue;
+            st.U[sp + k] = 0ull;
+            if (bad)
+                continue;
+            st.lam[sp + k] = nl[i];
+            st.p64[sp + k] = p[i];
+            st.p32[sp + k] = __double2float_rn(p[i]);
+            if (st.lam_trace)
+                st.lam_trace[((size_t)s * (T + 1) + round + 1) * P + k] = nl[i];
+            huge |= !(p[i] <= 0x1p100);
+            if (k < rg)
+                flat = p[i];   // k = lane
+            else if (own == 1 || ((k - rg) & 1) == 0)
+                pm0 = fmax(pm0, p[i]);
+            else
+                pm1 = fmax(pm1, p[i]);
+        }
+    }
+    if (bad) {
+        if (lane == 0) {
+            st.status[s] = 2;
+            st.frozen[s] = 1;
+        }
+        return;
+    }
+    huge = __any_sync(FULL, huge);
+    pm0 = warp_max(pm0);
+    if (own == 2)
+        pm1 = warp_max(pm1);
+    const double term = (lane < rg ? flat : lane == rg ? pm0 : pm1) * (double)umax;   // umax: 0 beyond column R - 1
+    const double M = vmax + warp_sum_fixed(lane < R ? term : 0.0);
+    bool conv = false;
+    if (a.tol > 0.0)
+        conv = warp_max(dmax) <= a.tol * fmax(1.0, warp_max(amax));
+    if (lane == 0)
+        close_round(t, st, a, s, round, M, huge, conv);
 }
 
 // The update of scenario s after `round`, by the warp whose arrival completed it; persist: then its
 // version, which releases the scenario's next round (a stopped scenario releases every later one).
+template <bool G>
 __device__ __forceinline__ void finish_scenario(const DevTable &t, const DevState &st, const SolveArgs &a, int s, int round,
-                                             int lane, bool persist)
+                                             unsigned char *groups, int lane, bool persist)
 {
     asm volatile("fence.acq_rel.gpu;" ::: "memory");
-    update_flat(t, st, a, s, round, lane);
+    if (G)
+        update_grouped(t, st, a, s, round, reinterpret_cast<double *>(groups), lane);
+    else
+        update_flat(t, st, a, s, round, lane);
     if (lane == 0)
         st.arrive[s] = 0u;   // every tile of the round has arrived
     if (persist) {
@@ -388,12 +564,12 @@ __device__ __forceinline__ void finish_scenario(const DevTable &t, const DevStat
 // fused updates) the arrival of the tiles evaluated; the arrival that completes the scenario applies
 // Eq. price_update. Every lane may have issued demand atomics or written reduced costs: the warp barrier
 // orders them before lane 0's release-ordered (cumulative) arrival, which publishes them.
-template <int NW, bool PERSIST>
+template <int NW, bool G, bool PERSIST>
 __device__ __forceinline__ void leave(const Pass &ps, Ctx<NW> &c)
 {
     if (c.s < 0 || c.skip)
         return;
-    add_demand(ps, c);
+    add_demand<NW, G>(ps, c);
     if (ps.want_hash) {
         unsigned long long h = c.hash;
 #pragma unroll
@@ -414,11 +590,11 @@ __device__ __forceinline__ void leave(const Pass &ps, Ctx<NW> &c)
                      : "memory");
     old = __shfl_sync(FULL, old, 0);
     if (old + (unsigned int)c.tiles == (unsigned int)__ldg(ps.pk.scen_tiles + c.s))
-        finish_scenario(ps.t, ps.st, ps.a, c.s, ps.round, ps.lane, PERSIST);
+        finish_scenario<G>(ps.t, ps.st, ps.a, c.s, ps.round, c.groups, ps.lane, PERSIST);
 }
 
 // Prices, bound and state of scenario s (through L2: another warp of this launch may have written them).
-template <int NW>
+template <int NW, bool G>
 __device__ __forceinline__ void enter(const Pass &ps, Ctx<NW> &c, int s)
 {
     const DevState &st = ps.st;
@@ -429,10 +605,20 @@ __device__ __forceinline__ void enter(const Pass &ps, Ctx<NW> &c, int s)
     const int frozen = __ldcg(st.frozen + s);
     const float e = __ldcg(st.ebound + s);
 #pragma unroll
-    for (int k = 0; k < NW; ++k) {
+    for (int k = 0; k < (G ? NW - 1 : NW); ++k) {
         const float pl = f.col_lo[k] >= 0 ? __ldcg(st.p32 + sp + f.col_lo[k]) : 0.0f;
         const float ph = f.col_hi[k] >= 0 ? __ldcg(st.p32 + sp + f.col_hi[k]) : 0.0f;
         c.price[k] = pack2(pl, ph);
+    }
+    if (G) {   // the slots' prices; an update of the scenario before may have used the memory
+        const int rg = ps.t.r_global, own = ps.t.R - rg;
+        __syncwarp();
+        for (int g = ps.lane; g < ps.t.n_groups; g += 32) {
+            const float *p = st.p32 + sp + rg + own * g;
+            const float a = __ldcg(p), b = own == 2 ? __ldcg(p + 1) : 0.0f;
+            *reinterpret_cast<unsigned long long *>(c.groups + 8 * pack_slot((uint32_t)g)) = pack2(a, b);
+        }
+        __syncwarp();
     }
     c.skip = ps.kind == PASS_ROUND && frozen != 0;
     c.exact = !(e < INFINITY);
@@ -442,18 +628,18 @@ __device__ __forceinline__ void enter(const Pass &ps, Ctx<NW> &c, int s)
 
 // A step of whole jobs of 3 .. 256 options: each job has 2^code lanes, its lane sub the options
 // sub << per .. (per = 3: eight, per = 2: four) as vectors ia and ib of the slot (has_a, has_b: they exist; +inf past a job's end and in the
-// jobs missing from a tile's last step). The lane's job is job jl of tile k, which has n_job. An
+// jobs missing from a tile's last step). The lane's job is job jl of a tile of n_job jobs from packed job job0 on. An
 // unambiguous job's winner is the one option that holds the smallest score.
-template <int NW, bool PLAIN>
+template <int NW, bool G, bool PLAIN>
 __device__ __forceinline__ void step_jobs(const Pass &ps, Ctx<NW> &c, const uint4 *slot, int V, int ia, int ib, bool has_a,
-                                          bool has_b, bool any_b, int code, int per, int k, int jl, int n_job)
+                                          bool has_b, bool any_b, int code, int per, int job0, int jl, int n_job)
 {
     float qa[4], qb[4] = {INFINITY, INFINITY, INFINITY, INFINITY};
     float a1, a2, b1 = INFINITY, b2 = INFINITY;
-    screen4<NW>(slot + ia, V, ps.pk.fmt, c, qa);
+    screen4<NW, G>(slot + ia, V, ps.pk.fmt, c, qa);
     two_smallest(qa, a1, a2);
     if (any_b) {
-        screen4<NW>(slot + ib, V, ps.pk.fmt, c, qb);
+        screen4<NW, G>(slot + ib, V, ps.pk.fmt, c, qb);
         two_smallest(qb, b1, b2);
     }
     a1 = has_a ? a1 : INFINITY;
@@ -491,7 +677,7 @@ __device__ __forceinline__ void step_jobs(const Pass &ps, Ctx<NW> &c, const uint
             const uint32_t sv = (has_a ? survivors(slot[ia], qa, c.exact, thr) : 0u) |
                                 (has_b ? survivors(slot[ib], qb, c.exact, thr) << 4 : 0u);
             if (sv != 0u)
-                x = rescore(ps.t.units, ps.t.values, ps.t.R, c.p64, job_at(ps, k, jl).opt0 + loc, sv, loc);
+                x = rescore<G>(ps.t, c.p64, first_option(ps, job0 + jl) + loc, sv, loc);
         }
         x = group_min(x, 1 << code);
         if (amb && x.idx >= loc && x.idx < loc + (1 << per)) {
@@ -502,19 +688,19 @@ __device__ __forceinline__ void step_jobs(const Pass &ps, Ctx<NW> &c, const uint
         }
     }
     if (mine) {
-        add_option<NW>(c, ps.pk.fmt, reinterpret_cast<const uint32_t *>(slot + (o < 4 ? ia : ib)) + (o & 3), V);
+        add_option<NW, G>(ps, c, reinterpret_cast<const uint32_t *>(slot + (o < 4 ? ia : ib)) + (o & 3), V);
         if (!PLAIN)
-            extras<NW>(ps, c, job_at(ps, k, jl), ((ps.lane & ((1 << code) - 1)) << per) + o, have_s, key);
+            extras<NW, G>(ps, c, job0 + jl, ((ps.lane & ((1 << code) - 1)) << per) + o, have_s, key);
     }
 }
 
-// Four consecutive options of a tile whose jobs have one or two: jobs j0 .. of tile k, `n` of them left in
+// Four consecutive options of a tile whose jobs have one or two: jobs job0 + j0 .., `n` of them left in
 // it. v: the vector.
-template <int NW, bool PLAIN>
-__device__ __forceinline__ void step_tiny(const Pass &ps, Ctx<NW> &c, const uint4 *v, int V, int K, int k, int j0, int n)
+template <int NW, bool G, bool PLAIN>
+__device__ __forceinline__ void step_tiny(const Pass &ps, Ctx<NW> &c, const uint4 *v, int V, int K, int job0, int j0, int n)
 {
     float q[4];
-    screen4<NW>(v, V, ps.pk.fmt, c, q);
+    screen4<NW, G>(v, V, ps.pk.fmt, c, q);
     const uint32_t *w = reinterpret_cast<const uint32_t *>(v);
 #pragma unroll
     for (int h = 0; h < 4; ++h) {
@@ -532,16 +718,16 @@ __device__ __forceinline__ void step_tiny(const Pass &ps, Ctx<NW> &c, const uint
             o = qb < qa ? h + 1 : h;
             if (c.exact || !(fmaxf(qa, qb) > thr)) {   // ambiguous
                 const uint32_t sv = (survivors(v[0], q, c.exact, thr) >> h) & 3u;
-                const Exact x = rescore(ps.t.units, ps.t.values, ps.t.R, c.p64, job_at(ps, k, j0 + jl).opt0, sv, h);
+                const Exact x = rescore<G>(ps.t, c.p64, first_option(ps, job0 + j0 + jl), sv, h);
                 o = x.idx;
                 key = x.key;
                 have_s = true;
                 ++c.resolved;
             }
         }
-        add_option<NW>(c, ps.pk.fmt, w + o, V);
+        add_option<NW, G>(ps, c, w + o, V);
         if (!PLAIN)
-            extras<NW>(ps, c, job_at(ps, k, j0 + jl), o - h, have_s, key);
+            extras<NW, G>(ps, c, job0 + j0 + jl, o - h, have_s, key);
     }
 }
 
@@ -553,13 +739,19 @@ struct Large {
     float m1, m2;
     int idx;
     uint32_t x[NW];   // words of the previous job's winner, zero on the other lanes
+    uint32_t slot;    // the one of them that holds its group slot
 };
 
-template <int NW>
-__device__ __forceinline__ void add_pending(Ctx<NW> &c, const PackFormat &f, Large<NW> &b)
+template <int NW, bool G>
+__device__ __forceinline__ void add_pending(const Pass &ps, Ctx<NW> &c, Large<NW> &b)
 {
+    const PackFormat &f = ps.pk.fmt;
+    if (G && b.x[NW - 1] != 0u) {
+        add_group(ps, c, b.x[NW - 1], b.slot);
+        b.x[NW - 1] = 0u;
+    }
 #pragma unroll
-    for (int k = 0; k < NW; ++k) {
+    for (int k = 0; k < (G ? NW - 1 : NW); ++k) {
         c.lo[k] += b.x[k] & f.mask[k];
         c.hi[k] += b.x[k] >> f.shift[k];
         b.x[k] = 0u;
@@ -576,7 +768,7 @@ __device__ __forceinline__ const uint4 *large_vec(const uint4 *base, const PackS
 
 // Survivors of a large job in fp64 when a lane may hold several: its packed vectors are screened again (the
 // same instructions give the same q).
-template <int NW>
+template <int NW, bool G>
 __device__ __forceinline__ Exact rescan_large(const Pass &ps, const Ctx<NW> &c, const uint4 *base, const PackShape &sh,
                                               int64_t opt0, float thr)
 {
@@ -584,19 +776,38 @@ __device__ __forceinline__ Exact rescan_large(const Pass &ps, const Ctx<NW> &c, 
     for (int g = ps.lane; g < sh.m; g += 32) {
         const uint4 *v = large_vec<NW>(base, sh, g);
         float q[4];
-        screen4<NW>(v, sh.v, ps.pk.fmt, c, q);
-        const Exact y = rescore(ps.t.units, ps.t.values, ps.t.R, c.p64, opt0 + 4 * g, survivors(v[0], q, c.exact, thr), 4 * g);
+        screen4<NW, G>(v, sh.v, ps.pk.fmt, c, q);
+        const Exact y = rescore<G>(ps.t, c.p64, opt0 + 4 * g, survivors(v[0], q, c.exact, thr), 4 * g);
         if (y.key < x.key)
             x = y;
     }
     return x;
 }
 
-template <int NW, bool PLAIN>
-__device__ __forceinline__ void close_large(const Pass &ps, Ctx<NW> &c, const uint4 *base, const PackShape &sh, int k,
+// The same of one lane's options, its vectors spread over the warp: one trip to memory, where rescan_large makes
+// one per step of the job.
+template <int NW, bool G>
+__device__ __forceinline__ void rescan_lane(const Pass &ps, const Ctx<NW> &c, const uint4 *base, const PackShape &sh,
+                                            int64_t opt0, float thr, int of, Exact &x)
+{
+    for (int i = ps.lane; i < 2 * sh.nch; i += 32) {
+        const int step = i >> 1, at = 2 * of + (i & 1), g = step * sh.v + at;
+        if (at >= sh.v || g >= sh.m)
+            continue;
+        const uint4 *v = large_vec<NW>(base, sh, g);
+        float q[4];
+        screen4<NW, G>(v, sh.v, ps.pk.fmt, c, q);
+        const Exact y = rescore<G>(ps.t, c.p64, opt0 + 4 * g, survivors(v[0], q, c.exact, thr), 4 * g);
+        if (y.key < x.key || (y.key == x.key && y.idx < x.idx))
+            x = y;
+    }
+}
+
+template <int NW, bool G, bool PLAIN>
+__device__ __forceinline__ void close_large(const Pass &ps, Ctx<NW> &c, const uint4 *base, const PackShape &sh, int job0,
                                             int jl, Large<NW> &b)
 {
-    add_pending(c, ps.pk.fmt, b);
+    add_pending<NW, G>(ps, c, b);
     const float m1 = warp_min_f32(b.m1);
     const bool first = b.m1 == m1;
     const uint32_t holders = __ballot_sync(FULL, first);
@@ -607,13 +818,21 @@ __device__ __forceinline__ void close_large(const Pass &ps, Ctx<NW> &c, const ui
     int win = b.idx;
     long long key = 0;
     if (c.exact || !(m2 > thr)) {
-        const int64_t opt0 = job_at(ps, k, jl).opt0;
+        const int64_t opt0 = first_option(ps, job0 + jl);
         Exact x{0x7fffffffffffffffLL, kIdxNone};
         if (!c.exact && !__any_sync(FULL, b.m2 <= thr)) {   // every lane's own best at most
             if (b.m1 <= thr)
-                x = rescore(ps.t.units, ps.t.values, ps.t.R, c.p64, opt0 + b.idx, 1u, b.idx);
+                x = rescore<G>(ps.t, c.p64, opt0 + b.idx, 1u, b.idx);
         } else {
-            x = rescan_large<NW>(ps, c, base, sh, opt0, thr);
+            const uint32_t several = __ballot_sync(FULL, b.m2 <= thr);   // lanes with more than their own best
+            if (!c.exact && __popc(several) <= sh.nch) {
+                if (b.m1 <= thr && !(b.m2 <= thr))
+                    x = rescore<G>(ps.t, c.p64, opt0 + b.idx, 1u, b.idx);
+                for (uint32_t l = several; l != 0u; l &= l - 1u)
+                    rescan_lane<NW, G>(ps, c, base, sh, opt0, thr, __ffs((int)l) - 1, x);
+            } else {
+                x = rescan_large<NW, G>(ps, c, base, sh, opt0, thr);
+            }
         }
         const int own = x.idx;
         x = group_min(x, 32);
@@ -629,8 +848,10 @@ __device__ __forceinline__ void close_large(const Pass &ps, Ctx<NW> &c, const ui
 #pragma unroll
         for (int i = 0; i < NW; ++i)
             b.x[i] = __ldg(w + (i + 1) * sh.v * 4);
+        if (G)
+            b.slot = __ldg(w + (ps.pk.fmt.g_word + 1) * sh.v * 4);
         if (!PLAIN)
-            extras<NW>(ps, c, job_at(ps, k, jl), win, have_s, key);
+            extras<NW, G>(ps, c, job0 + jl, win, have_s, key);
     }
     b.m1 = b.m2 = INFINITY;
     b.idx = kIdxNone;
@@ -653,7 +874,7 @@ __device__ __forceinline__ void reset(Ctx<NW> &c)
 // One warp's work: the tiles `next` hands out (its index, its round in *round; -1 when there are no
 // more), evaluated in order. Lane 0 copies the step after the one in flight as soon as its slot is free,
 // across tiles; a tile's record is loaded while the tile before it is evaluated. hold_tx: see SolveArgs.
-template <int NW, bool PLAIN, bool PERSIST, typename Next>
+template <int NW, bool G, bool PLAIN, bool PERSIST, typename Next>
 __device__ __forceinline__ void run_warp(const DevTable &t, const DevState &st, const DevPack &pk, const SolveArgs &a,
                                          int round, int kind, unsigned char *smem, uint32_t hold_tx, Next &&next)
 {
@@ -673,8 +894,11 @@ __device__ __forceinline__ void run_warp(const DevTable &t, const DevState &st, 
         return PackTile{x.x, x.y, x.z, x.w};
     };
     PackTile T = load(kt), N = T;
-    if (kn >= 0)
+    int job0 = __ldg(pk.job_begin + kt), jobn = 0;   // their first jobs
+    if (kn >= 0) {
         N = load(kn);
+        jobn = __ldg(pk.job_begin + kn);
+    }
     if (lane == 0) {
         for (int s = 0; s < kPackSlots; ++s)
             mbar_init(bars + 8 * s, 1);
@@ -719,6 +943,7 @@ __device__ __forceinline__ void run_warp(const DevTable &t, const DevState &st, 
         asm volatile("griddepcontrol.wait;" ::: "memory");
     Ctx<NW> c;
     reset(c);
+    c.groups = smem + pack_warp_bytes(NW);
     int at = 0;                  // slot of the step to be screened
     uint32_t phases = 0;         // parity of each slot's next completion
     // the step in slot `at` has landed (bounded; warp-uniform)
@@ -743,24 +968,24 @@ __device__ __forceinline__ void run_warp(const DevTable &t, const DevState &st, 
             issue();             // a tile of one step left the copies waiting for this tile's successor
         const PackShape sh = pack_shape(T);
         if (PERSIST) {
-            leave<NW, true>(ps, c);
+            leave<NW, G, true>(ps, c);
             c.s = -1;
             if (!wait_version(st.ver, (int)T.scenario, rt, st.err, a.wait_ms, st.stats)) {
                 ok = false;
                 break;
             }
             ps.round = rt;
-            enter(ps, c, (int)T.scenario);
+            enter<NW, G>(ps, c, (int)T.scenario);
         } else if ((int)T.scenario != c.s) {
-            leave<NW, false>(ps, c);
-            enter(ps, c, (int)T.scenario);
+            leave<NW, G, false>(ps, c);
+            enter<NW, G>(ps, c, (int)T.scenario);
         }
         if (__any_sync(FULL, (gave_up & DEV_ERR_TIMEOUT) != 0u)) {
             ok = false;
             break;
         }
         if (c.wins >= kPackSpill)
-            add_demand(ps, c);
+            add_demand<NW, G>(ps, c);
         const int n_job = (int)T.n_job, steps = sh.steps;
         if (sh.code < (int)kPackTiny) {
             const int code = sh.code, sub = lane & ((1 << code) - 1), jl = lane >> code;
@@ -770,8 +995,8 @@ __device__ __forceinline__ void run_warp(const DevTable &t, const DevState &st, 
                 if (!(ok = landed()))
                     break;
                 if (!c.skip)
-                    step_jobs<NW, PLAIN>(ps, c, reinterpret_cast<const uint4 *>(smem + at * kSlot), sh.v, ia, ib, has_a, has_b,
-                                         any_b, code, sh.narrow ? 2 : 3, kt, st_i * sh.per_step + jl, n_job);
+                    step_jobs<NW, G, PLAIN>(ps, c, reinterpret_cast<const uint4 *>(smem + at * kSlot), sh.v, ia, ib, has_a, has_b,
+                                         any_b, code, sh.narrow ? 2 : 3, job0, st_i * sh.per_step + jl, n_job);
                 release();
             }
             c.wins += steps;
@@ -793,7 +1018,7 @@ __device__ __forceinline__ void run_warp(const DevTable &t, const DevState &st, 
                         if (lane >= (h ? sh.cb : sh.ca))
                             break;
                         float q[4], r1, r2;
-                        screen4<NW>(slot + (h ? sh.ca : 0) + lane, sh.v, pk.fmt, c, q);
+                        screen4<NW, G>(slot + (h ? sh.ca : 0) + lane, sh.v, pk.fmt, c, q);
                         two_smallest(q, r1, r2);
                         if (r1 < big.m1) {   // increasing index: earlier options keep ties
                             big.m2 = fminf(big.m1, r2);
@@ -805,8 +1030,8 @@ __device__ __forceinline__ void run_warp(const DevTable &t, const DevState &st, 
                     }
                     __syncwarp();
                     if (++ch == sh.nch) {
-                        close_large<NW, PLAIN>(ps, c,
-                                               pk.data + ((uint64_t)T.base + (uint64_t)job * sh.nch * sh.v) * (NW + 1), sh, kt,
+                        close_large<NW, G, PLAIN>(ps, c,
+                                               pk.data + ((uint64_t)T.base + (uint64_t)job * sh.nch * sh.v) * (NW + 1), sh, job0,
                                                job, big);
                         ch = 0;
                         ++job;
@@ -814,7 +1039,7 @@ __device__ __forceinline__ void run_warp(const DevTable &t, const DevState &st, 
                 }
                 release();
             }
-            add_pending(c, pk.fmt, big);
+            add_pending<NW, G>(ps, c, big);
             c.wins += n_job;
         } else {
             for (int st_i = 0; st_i < steps; ++st_i) {
@@ -826,7 +1051,7 @@ __device__ __forceinline__ void run_warp(const DevTable &t, const DevState &st, 
                     for (int h = 0; h < 2; ++h) {
                         const int o0 = 4 * (64 * st_i + 32 * h + lane), j0 = o0 / sh.m;   // m = 1 or 2
                         if (j0 < n_job)
-                            step_tiny<NW, PLAIN>(ps, c, slot + 32 * h + lane, 64, sh.m, kt, j0, n_job - j0);
+                            step_tiny<NW, G, PLAIN>(ps, c, slot + 32 * h + lane, 64, sh.m, job0, j0, n_job - j0);
                     }
                 }
                 release();
@@ -837,16 +1062,18 @@ __device__ __forceinline__ void run_warp(const DevTable &t, const DevState &st, 
             break;
         ++c.tiles;
         if (kn < 0) {
-            leave<NW, PERSIST>(ps, c);
+            leave<NW, G, PERSIST>(ps, c);
             break;
         }
         T = N;
-        kt = kn;
+        job0 = jobn;
         rt = rn;
         in_next = false;
         kn = next(&rn);
-        if (kn >= 0)
+        if (kn >= 0) {
             N = load(kn);
+            jobn = __ldg(pk.job_begin + kn);
+        }
     }
     if (!ok) {   // a wait gave up: wait (bounded) for every copy still in flight, then leave
         for (; flying > 0; --flying, at ^= 1) {
@@ -859,9 +1086,10 @@ __device__ __forceinline__ void run_warp(const DevTable &t, const DevState &st, 
         atomicAdd(st.stats, (unsigned long long)n);
 }
 
-// One pass: warp w evaluates the tiles of its range. PLAIN: a round pass without traces.
-template <int NW, bool PLAIN>
-__global__ void __launch_bounds__(kPackWarps * 32, pack_min_ctas(NW))
+// One pass: warp w evaluates the tiles of its range. PLAIN: a round pass without traces. G: a table with a
+// group column.
+template <int NW, bool G, bool PLAIN>
+__global__ void __launch_bounds__(kPackWarps * 32, pack_min_ctas(NW, G))
     k_packed(const __grid_constant__ DevTable t, const __grid_constant__ DevState st, const __grid_constant__ DevPack pk,
              const __grid_constant__ SolveArgs a, int round, int kind)
 {
@@ -877,7 +1105,8 @@ __global__ void __launch_bounds__(kPackWarps * 32, pack_min_ctas(NW))
         k = __ldg(pk.warp_begin + w);
         end = __ldg(pk.warp_begin + w + 1);
     }
-    run_warp<NW, PLAIN, false>(t, st, pk, a, round, kind, smem + (size_t)wid * pack_warp_bytes(NW),
+    run_warp<NW, G, PLAIN, false>(t, st, pk, a, round, kind,
+                               smem + (size_t)wid * (pack_warp_bytes(NW) + (G ? pk.fmt.g_bytes : 0)),
                                (w == 0 && round == 0 && kind == PASS_ROUND) ? a.hold_tx : 0u,
                                [&](int *) { return k < end ? k++ : -1; });
 }
@@ -905,7 +1134,7 @@ __global__ void __launch_bounds__(kPackWarps * 32, pack_min_ctas(NW))
     unsigned int pend = 0;
     if (lane == 0)
         pend = atomicAdd(st.work, 1u);
-    run_warp<NW, true, true>(t, st, pk, a, 0, (int)PASS_ROUND, smem + (size_t)wid * pack_warp_bytes(NW),
+    run_warp<NW, false, true, true>(t, st, pk, a, 0, (int)PASS_ROUND, smem + (size_t)wid * pack_warp_bytes(NW),
                              blockIdx.x == 0 && wid == 0 ? a.hold_tx : 0u,
                              [&](int *round) {
                                  const unsigned int q = __shfl_sync(FULL, pend, 0);
@@ -956,6 +1185,8 @@ __global__ void __launch_bounds__(4 * kPackStepVecs) k_pack(DevTable t, const __
         if (jl < n_job) {
             const int64_t job = pk.job ? pk.job[j0 + jl] : j0 + jl;
             const int64_t a = t.job_off[job];
+            if (opt == 0 && pk.opt0)
+                pk.opt0[j0 + jl] = a;
             if (opt < t.job_off[job + 1] - a) {
                 const int32_t *u = t.units + (a + opt) * R;
                 if (u[0] >= 0) {   // not a duplicate
@@ -969,6 +1200,8 @@ __global__ void __launch_bounds__(4 * kPackStepVecs) k_pack(DevTable t, const __
                         f[k] = (uint32_t)(u[pk.fmt.col_lo[k]] & 0x7fffffff);
                     if (k < pk.fmt.nw && pk.fmt.col_hi[k] >= 0)
                         f[k] |= (uint32_t)(u[pk.fmt.col_hi[k]] & 0x7fffffff) << pk.fmt.shift[k];
+                    if (pk.fmt.g_mask != 0u && k == pk.fmt.g_word)
+                        f[k] |= pack_slot(t.group[a + opt]) << pk.fmt.g_shift;
                 }
             }
         }
@@ -981,38 +1214,54 @@ __global__ void __launch_bounds__(4 * kPackStepVecs) k_pack(DevTable t, const __
     }
 }
 
-template <int NW>
+template <int NW, bool G>
 struct PackKernels {
+    static constexpr int kKernels = G ? 2 : 3;
     static const void *fn(int which)
     {
-        return which == 0   ? reinterpret_cast<const void *>(&k_packed<NW, true>)
-               : which == 1 ? reinterpret_cast<const void *>(&k_packed<NW, false>)
-                            : reinterpret_cast<const void *>(&k_packed_persist<NW>);
+        if constexpr (!G)
+            if (which == 2)
+                return reinterpret_cast<const void *>(&k_packed_persist<NW>);
+        return which == 0 ? reinterpret_cast<const void *>(&k_packed<NW, G, true>)
+                          : reinterpret_cast<const void *>(&k_packed<NW, G, false>);
     }
 };
 
 template <typename F>
-auto pack_dispatch(int nw, F &&f)
+auto pack_dispatch(int nw, bool grouped, F &&f)
 {
+    if (grouped)
+        switch (nw) {
+        case 3: return f(PackKernels<3, true>());
+        case 4: return f(PackKernels<4, true>());
+        default: return f(PackKernels<6, true>());
+        }
     switch (nw) {
-    case 2: return f(PackKernels<2>());
-    case 3: return f(PackKernels<3>());
-    case 4: return f(PackKernels<4>());
-    case 6: return f(PackKernels<6>());
-    default: return f(PackKernels<8>());
+    case 2: return f(PackKernels<2, false>());
+    case 3: return f(PackKernels<3, false>());
+    case 4: return f(PackKernels<4, false>());
+    case 6: return f(PackKernels<6, false>());
+    default: return f(PackKernels<8, false>());
     }
+}
+
+int pack_smem(int nw, int group_bytes)
+{
+    return kPackWarps * (pack_warp_bytes(nw) + group_bytes);
 }
 
 }  // namespace
 
-int packed_ctas_per_sm(int nw)
+int packed_ctas_per_sm(int nw, int group_bytes)
 {
-    return pack_dispatch(nw, [&](auto k) -> int {
+    return pack_dispatch(nw, group_bytes > 0, [&](auto k) -> int {
         int best = 0;
-        const int smem = kPackWarps * pack_warp_bytes(nw);
-        for (int i = 0; i < 3; ++i) {
+        // the limit is the kernel's, not the table's: the largest price table's for every one
+        const int smem = pack_smem(nw, group_bytes);
+        const int limit = pack_smem(nw, group_bytes > 0 ? pack_group_bytes(kPackMaxPrices, kPackMaxPrices) : 0);
+        for (int i = 0; i < decltype(k)::kKernels; ++i) {
             int n = 0;
-            if (cudaFuncSetAttribute(decltype(k)::fn(i), cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
+            if (cudaFuncSetAttribute(decltype(k)::fn(i), cudaFuncAttributeMaxDynamicSharedMemorySize, limit) != cudaSuccess ||
                 cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, decltype(k)::fn(i), kPackWarps * 32, smem) !=
                     cudaSuccess) {
                 cudaGetLastError();
@@ -1039,7 +1288,8 @@ cudaError_t launch_packed(const DevTable &t, const DevState &st, const DevPack &
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)((pk.n_warps + kPackWarps - 1) / kPackWarps));
     cfg.blockDim = dim3(kPackWarps * 32);
-    cfg.dynamicSmemBytes = (size_t)(kPackWarps * pack_warp_bytes(pk.fmt.nw));
+    const int group_bytes = t.group ? pk.fmt.g_bytes : 0;
+    cfg.dynamicSmemBytes = (size_t)pack_smem(pk.fmt.nw, group_bytes);
     cfg.stream = stream;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -1048,7 +1298,8 @@ cudaError_t launch_packed(const DevTable &t, const DevState &st, const DevPack &
     cfg.numAttrs = pdl ? 1 : 0;
     int k = kind;
     void *args[] = {(void *)&t, (void *)&st, (void *)&pk, (void *)&a, (void *)&round, (void *)&k};
-    return pack_dispatch(pk.fmt.nw, [&](auto kk) { return cudaLaunchKernelExC(&cfg, decltype(kk)::fn(plain ? 0 : 1), args); });
+    return pack_dispatch(pk.fmt.nw, group_bytes > 0,
+                         [&](auto kk) { return cudaLaunchKernelExC(&cfg, decltype(kk)::fn(plain ? 0 : 1), args); });
 }
 
 cudaError_t launch_packed_persist(const DevTable &t, const DevState &st, const DevPack &pk, const SolveArgs &a,
@@ -1057,7 +1308,7 @@ cudaError_t launch_packed_persist(const DevTable &t, const DevState &st, const D
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)grid);
     cfg.blockDim = dim3(kPackWarps * 32);
-    cfg.dynamicSmemBytes = (size_t)(kPackWarps * pack_warp_bytes(pk.fmt.nw));
+    cfg.dynamicSmemBytes = (size_t)pack_smem(pk.fmt.nw, 0);
     cfg.stream = stream;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeCooperative;   // every CTA co-resident: the version waits can end
@@ -1065,7 +1316,7 @@ cudaError_t launch_packed_persist(const DevTable &t, const DevState &st, const D
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     void *args[] = {(void *)&t, (void *)&st, (void *)&pk, (void *)&a, (void *)&n_rounds};
-    return pack_dispatch(pk.fmt.nw, [&](auto kk) { return cudaLaunchKernelExC(&cfg, decltype(kk)::fn(2), args); });
+    return pack_dispatch(pk.fmt.nw, false, [&](auto kk) { return cudaLaunchKernelExC(&cfg, decltype(kk)::fn(2), args); });
 }
 
 }  // namespace esp

@@ -1,4 +1,4 @@
-// The packed screen copy of an option table without a group column (internal): what the fp32 screen of
+// The packed screen copy of an option table (internal): what the fp32 screen of
 // the evaluation pass reads, bit for bit, in fewer bytes, and the tiles of the packed passes over it.
 //
 // Per option: one word -v32 (v truncated to fp32 as the screen takes it, negated; +inf for a load-time
@@ -28,7 +28,37 @@ struct PackFormat {
     // with f = funnelshift_r(w, magic[k], shift[k]): the bits of the float 2^23 + high field
     uint32_t magic[kPackMaxWords];
     int8_t col_lo[kPackMaxWords], col_hi[kPackMaxWords];   // table column of each field, -1: none
+    // tables with a group column: the last word holds the columns that are priced per group; word g_word
+    // also holds, from bit g_shift on, the option's group slot (pack_slot)
+    int32_t g_word, g_shift;
+    uint32_t g_mask;                     // 0: no group column
+    int32_t g_bytes;                     // a warp's shared memory for the groups' prices (pack_group_bytes)
 };
+
+// The slot of group g in the warp's table of group prices: every ninth slot is left out, so that the groups
+// 8 apart that neighbouring lanes look up lie in different banks.
+ESP_HD uint32_t pack_slot(uint32_t g)
+{
+    return g + (g >> 3);
+}
+ESP_HD uint32_t pack_slot_group(uint32_t slot)
+{
+    return slot - slot / 9;
+}
+
+// Grouped tables that the packed passes take: one or two columns priced per group (one word), and at
+// most kPackMaxPrices prices (the price table is held per warp; more would cost resident CTAs).
+constexpr int kPackMaxPrices = 1024;
+ESP_HD bool pack_groups_fit(int R, int r_global, int P)
+{
+    return R - r_global <= 2 && P <= kPackMaxPrices;
+}
+// Bytes of that table: two fp32 prices per slot; the price update puts P new prices there.
+ESP_HD int pack_group_bytes(int P, int n_groups)
+{
+    const int a = 8 * ((int)pack_slot((uint32_t)n_groups) + 1), b = 8 * P;
+    return ((a > b ? a : b) + 15) & ~15;
+}
 
 // Steps. A warp screens up to 256 options at once, eight consecutive options of a job per lane as two
 // vectors of four (one 16-byte vector per word plane holds four options' words). A step's data are

@@ -1,6 +1,7 @@
 // The staged evaluation-pass kernel of the ESP tatonnement (Sec. 3.2.2; Eq. esp_score without Gamma) for
 // sm_103a, instantiated by esp_kernels.cu: the tables that the packed passes (esp_packed.cu) do not take,
-// which are grouped ones and those with units of 2^23 or more. The exactness argument and the
+// which are those with units of 2^23 or more, more unit words than eight, or a group column beyond
+// pack_groups_fit. The exactness argument and the
 // aggregation are stated in esp_kernels.cu.
 #pragma once
 

@@ -280,11 +280,12 @@ bool sort_layout(const int64_t *off, int32_t S, int32_t J, SortedLayout &out, in
     return (int64_t)out.jmap.size() == n_jobs;
 }
 
-bool pack_format(const int32_t *umax, int32_t R, PackFormat &out)
+bool pack_format(const int32_t *umax, int32_t R, PackFormat &out, int32_t r_global, int32_t n_groups)
 {
     out = PackFormat{};
     if (R < 1 || R > kMaxR)
         return false;
+    const int32_t flat = n_groups > 0 ? r_global : R;   // columns priced alike for every option
     struct Col {
         int bits, col;
     };
@@ -297,37 +298,74 @@ bool pack_format(const int32_t *umax, int32_t R, PackFormat &out)
             return false;
         cols.push_back({std::max(b, 1), r});
     }
-    std::stable_sort(cols.begin(), cols.end(), [](const Col &x, const Col &y) { return x.bits > y.bits; });
+    std::stable_sort(cols.begin(), cols.begin() + flat, [](const Col &x, const Col &y) { return x.bits > y.bits; });
     std::vector<char> used(cols.size(), 0);
-    int nw = 0;
+    int nw = 0, taken[kPackMaxWords] = {}, high[kPackMaxWords] = {};   // bits of a word's low and high field
     for (int k = 0; k < kPackMaxWords; ++k) {   // empty words: nothing low, one bit high
         out.mask[k] = 0u;
         out.shift[k] = 31;
         out.magic[k] = 0x4b000000u >> 1;
         out.col_lo[k] = out.col_hi[k] = -1;
     }
-    for (size_t i = 0; i < cols.size(); ++i) {
+    auto put = [&](int k, const Col &lo, const Col *hi) {
+        taken[k] = lo.bits;
+        out.mask[k] = (1u << lo.bits) - 1u;
+        out.col_lo[k] = (int8_t)lo.col;
+        if (hi) {
+            high[k] = hi->bits;
+            out.shift[k] = 32 - hi->bits;
+            out.magic[k] = 0x4b000000u >> hi->bits;   // exact: its low 24 bits are zero
+            out.col_hi[k] = (int8_t)hi->col;
+        }
+    };
+    for (int32_t i = 0; i < flat; ++i) {
         if (used[i])
             continue;
         if (nw == kPackMaxWords)
             return false;
-        out.mask[nw] = (1u << cols[i].bits) - 1u;
-        out.col_lo[nw] = (int8_t)cols[i].col;
-        for (size_t j = i + 1; j < cols.size(); ++j)
+        const Col *hi = nullptr;
+        for (int32_t j = i + 1; j < flat; ++j)
             if (!used[j] && cols[i].bits + cols[j].bits <= 32) {
                 used[j] = 1;
-                out.shift[nw] = 32 - cols[j].bits;
-                out.magic[nw] = 0x4b000000u >> cols[j].bits;   // exact: its low 24 bits are zero
-                out.col_hi[nw] = (int8_t)cols[j].col;
+                hi = &cols[j];
                 break;
             }
-        ++nw;
+        put(nw++, cols[i], hi);
     }
-    for (int n : {2, 3, 4, 6, 8})
-        if (nw <= n) {
-            out.nw = n;
-            return true;
+    if (n_groups <= 0) {
+        for (int n : {2, 3, 4, 6, 8})
+            if (nw <= n) {
+                out.nw = n;
+                return true;
+            }
+        return false;
+    }
+    const Col *hi = R - flat == 2 ? &cols[flat + 1] : nullptr;
+    if (R - flat < 1 || R - flat > 2 || cols[flat].bits + (hi ? hi->bits : 0) > 32)
+        return false;
+    int slot_bits = 1;
+    while ((pack_slot((uint32_t)(n_groups - 1)) >> slot_bits) != 0)
+        ++slot_bits;
+    for (int n : {3, 4, 6}) {
+        if (nw + 1 > n)
+            continue;
+        put(n - 1, cols[flat], hi);
+        for (int k = 0; k < n; ++k) {
+            // an empty word's high field is a zero bit of no column
+            if (taken[k] + std::max(high[k], out.col_hi[k] < 0 ? 1 : 0) + slot_bits <= 32) {
+                out.nw = n;
+                out.g_word = k;
+                out.g_shift = taken[k];
+                out.g_mask = (1u << slot_bits) - 1u;
+                return true;
+            }
         }
+        out.mask[n - 1] = 0u;   // no room for the slot: one more word
+        out.shift[n - 1] = 31;
+        out.magic[n - 1] = 0x4b000000u >> 1;
+        out.col_lo[n - 1] = out.col_hi[n - 1] = -1;
+        taken[n - 1] = high[n - 1] = 0;
+    }
     return false;
 }
 

@@ -65,8 +65,10 @@ struct PackPlan {
 
 // Word layout of the unit fields for the largest unit of each column over the table (each below
 // 2^23): columns paired so that two fit 32 bits, the widest with the widest that still fits. False when
-// the table needs more words than the passes have (kPackMaxWords) or a unit is 2^23 or more.
-bool pack_format(const int32_t *umax, int32_t R, PackFormat &out);
+// the table needs more words than the passes have (kPackMaxWords) or a unit is 2^23 or more. n_groups > 0:
+// columns r_global .. R - 1 (one or two) are priced per group and share the last word; the option's group
+// slot takes bits that a word leaves free, or a word of its own (3, 4 or 6 words).
+bool pack_format(const int32_t *umax, int32_t R, PackFormat &out, int32_t r_global = 0, int32_t n_groups = 0);
 
 // Packed order (per scenario, jobs of the same kind and vector count together), tiles of at most
 // kPackTileSteps steps (fewer where the table is small, so that every warp has work; a job of more steps
