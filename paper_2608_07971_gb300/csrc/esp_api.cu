@@ -1894,23 +1894,21 @@ esp_status esp_load_placement(esp_ctx *ctx, int32_t S, int32_t J, int32_t KC, in
         return st;
     }
     // the grid-resident solve (ESP_FLAG_RESIDENT): one CTA per SM holds the price state of every
-    // scenario and each warp at most kPlaceResJobs jobs, all in shared memory
-    if ((int64_t)S * P <= kPlaceResMaxPrices &&
-        n_jobs <= (int64_t)kPlaceResJobs * kPlaceResWarps * ctx->sm_count &&
-        place_res_smem_bytes(S, P, KC, R) <= optin && place_res_ctas_per_sm(S, P, KC, R) >= 1) {
+    // scenario and each warp a job, all in shared memory; as many warps per CTA as that takes, since the round
+    // is a chain, and fewer warps meet at a CTA's barriers sooner (us per round with at least 8,
+    // 16 and 32 warps: 1000 jobs x 8 x 30 6.87, 7.15 and 8.27; 100 jobs x 4 x 10 5.37, 5.62 and 6.40; two scenarios of
+    // 500 x 12 x 64 9.14, 8.69 and 10.1)
+    int32_t rw = 8;
+    while (rw < kPlaceResMaxWarps && n_jobs > (int64_t)rw * ctx->sm_count)
+        rw *= 2;
+    if ((int64_t)S * P <= kPlaceResMaxPrices && n_jobs <= (int64_t)rw * ctx->sm_count &&
+        place_res_smem_bytes(S, P, KC, R, rw) <= optin && place_res_ctas_per_sm(S, P, KC, R, rw) >= 1) {
         PlaceRes &pr = ctx->place_res;
-        const int32_t Wr = (int32_t)std::min<int64_t>(n_jobs, (int64_t)kPlaceResWarps * ctx->sm_count);
-        std::vector<int32_t> wr((size_t)Wr + 1);
-        for (int32_t w = 0; w <= Wr; ++w)
-            wr[(size_t)w] = (int32_t)((__int128)n_jobs * w / Wr);
-        int32_t *d_wr = nullptr;
         PALLOC(pr.U3, 3 * (size_t)S * P);
         PALLOC(pr.bar, 2);
-        PALLOC(d_wr, (size_t)Wr + 1);
-        ESP_CUDA(h2d(d_wr, wr.data(), wr.size() * sizeof(int32_t)));
-        pr.warp_job = d_wr;
-        pr.n_warps = Wr;
-        pr.grid = (Wr + kPlaceResWarps - 1) / kPlaceResWarps;
+        pr.n_jobs = (int32_t)n_jobs;
+        pr.warps = rw;
+        pr.grid = (int32_t)((n_jobs + rw - 1) / rw);
         ctx->place_res_ok = true;
     }
 #undef PALLOC

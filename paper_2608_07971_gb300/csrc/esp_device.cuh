@@ -76,6 +76,14 @@ __device__ __forceinline__ double key_value(long long k)
     return __longlong_as_double(k ^ ((k >> 63) & 0x7fffffffffffffffLL));
 }
 
+// Smallest value over the warp (one hardware reduction).
+__device__ __forceinline__ float warp_min_f32(float x)
+{
+    float r;
+    asm volatile("redux.sync.min.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(x));
+    return r;
+}
+
 __device__ __forceinline__ double warp_sum_fixed(double x)
 {
 #pragma unroll

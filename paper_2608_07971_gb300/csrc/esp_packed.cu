@@ -95,14 +95,6 @@ __device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigne
     return r;
 }
 
-// Smallest value over the warp (one hardware reduction).
-__device__ __forceinline__ float warp_min_f32(float x)
-{
-    float r;
-    asm volatile("redux.sync.min.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(x));
-    return r;
-}
-
 // The warp's state for the scenario it is in.
 template <int NW>
 struct Ctx {

@@ -37,15 +37,16 @@ __host__ __device__ inline int place_warp_bytes(int R, int P, int KC)
     return round16(KC * R * 4) + round16(KC * 8) + round16(KC * 4) + round16(KC * R * 4) + round16(P * 4);
 }
 
-template <int RT>
-__device__ __forceinline__ float place_global_part(const int32_t *u, double v, const ScenarioPrices &sp, int rg)
+// u: int32 units, or the same already converted (__int2float_rn)
+template <int RT, typename U>
+__device__ __forceinline__ float place_global_part(const U *u, double v, const ScenarioPrices &sp, int rg)
 {
     float g = -screen_value(v);
 #pragma unroll
     for (int r = 0; r < Cols<RT>::N; ++r) {
         if (r >= rg)
             break;
-        g = __fmaf_rn(sp.pf[r], __int2float_rn(u[r]), g);
+        g = __fmaf_rn(sp.pf[r], (float)u[r], g);
     }
     return g;
 }
@@ -250,14 +251,14 @@ __device__ bool grid_barrier(unsigned int *bar, unsigned int target, unsigned in
         asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t0));
         bool ok = false;
         for (uint32_t it = 0;; ++it) {
-            unsigned int v, ab;
-            asm volatile("ld.acquire.gpu.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
-            if ((int)(v - target) >= 0) {
+            // both words in one trip to L2 (they are one aligned 8-byte word)
+            unsigned long long v;
+            asm volatile("ld.acquire.gpu.u64 %0, [%1];" : "=l"(v) : "l"(bar) : "memory");
+            if ((int)((unsigned int)v - target) >= 0) {
                 ok = true;
                 break;
             }
-            asm volatile("ld.relaxed.gpu.u32 %0, [%1];" : "=r"(ab) : "l"(bar + 1) : "memory");
-            if (ab != 0u)
+            if ((unsigned int)(v >> 32) != 0u)
                 break;
             if (it > 64) {
                 uint64_t t1;
@@ -292,19 +293,23 @@ __device__ __forceinline__ double exact_score_shared(const int32_t *u, double v,
     return s;
 }
 
-// All T rounds of a placement solve in one cooperative launch of one CTA (kPlaceResWarps warps)
-// per SM. Each warp holds its (at most kPlaceResJobs) jobs in shared memory for the whole solve:
+// All T rounds of a placement solve in one cooperative launch of one CTA (W warps) per SM. Each warp
+// holds one job in shared memory for the whole solve:
 // configuration units (int32 and fp32), values, and per lane the penalties of its two nodes. Each
 // CTA holds the whole price state of every scenario in shared memory (S * P <= kPlaceResMaxPrices).
 // A round: best responses of the CTA's jobs (the arithmetic of k_place), their demand summed in
 // shared memory and added to buffer round % 3 of U3 with one atomic per column, a grid barrier,
 // then Eq. price_update by the whole CTA from the same totals (one price per thread; per-scenario
 // maxima and flags through shared atomics, which are order-independent), identical in every CTA.
+// What bounds it is the chain of a round: best response, shared sums, atomics, grid barrier, update, bound. One
+// job per warp: 9.8 us per round of 4096 jobs x 12 x 64, where two jobs one after the other in each of 16 warps,
+// the sums as 64-bit shared atomics, two trips to L2 per poll of the barrier, two fp64 divides per price and the
+// bound in fp64 took 15.0 (all but the first of these: 12.1).
 // CTA 0 writes the price and demand trajectories, clears the buffer that was last read before this
 // round's barrier, and publishes the final state for the final pass. Hash and dual traces are not
 // supported here (the host keeps the per-round launches for them).
-template <int RT>
-__global__ void __launch_bounds__(kPlaceResWarps * 32, 1) k_place_res(DevTable t, DevState st, DevPlace pl,
+template <int RT, int W>
+__global__ void __launch_bounds__(W * 32, 1) k_place_res(DevTable t, DevState st, DevPlace pl,
                                                                    SolveArgs a, PlaceRes pr)
 {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -313,18 +318,22 @@ __global__ void __launch_bounds__(kPlaceResWarps * 32, 1) k_place_res(DevTable t
     const int R = RT ? RT : t.R, rg = t.r_global;
     const int S = t.S, P = t.P, SP = S * P, T = a.T;
     const int KC = pl.KC, N = pl.N, NT = pl.NT;
-    const PlaceResLayout L = place_res_layout(S, P, KC, R);
+    const PlaceResLayout L = place_res_layout(S, P, KC, R, W);
 
-    unsigned long long *Uc = reinterpret_cast<unsigned long long *>(smem + L.u);
+    // the CTA's demand of each price as two 32-bit sums, of the low 16 bits and of the rest of its winners' units:
+    // an atomic add of 64 bits in shared memory is a loop of compare-and-swaps, which the columns that all
+    // jobs share kept repeating
+    uint32_t *Uc = reinterpret_cast<uint32_t *>(smem + L.u);
+    static_assert(W <= 65536, "a sum of 16-bit parts fits 32 bits");
     double *lam_s = reinterpret_cast<double *>(smem + L.lam);
     double *p64_s = reinterpret_cast<double *>(smem + L.p64);
-    double *capd_s = reinterpret_cast<double *>(smem + L.capd);
+    double *rcp_s = reinterpret_cast<double *>(smem + L.rcp);
     long long *cap_s = reinterpret_cast<long long *>(smem + L.cap);
     float *p32_s = reinterpret_cast<float *>(smem + L.p32);
     float *eb_s = reinterpret_cast<float *>(smem + L.eb);
     int *frozen_s = reinterpret_cast<int *>(smem + L.flags);
     int *status_s = frozen_s + S, *conv_s = frozen_s + 2 * S, *rounds_s = frozen_s + 3 * S;
-    int *bad_s = frozen_s + 4 * S, *huge_s = frozen_s + 5 * S;
+    int *bad_s = frozen_s + 4 * S;
     unsigned long long *dmax_s = reinterpret_cast<unsigned long long *>(smem + L.maxes);
     unsigned long long *amax_s = dmax_s + S;
     unsigned char *wb = smem + L.warps + (size_t)wid * L.warp_bytes;
@@ -336,8 +345,8 @@ __global__ void __launch_bounds__(kPlaceResWarps * 32, 1) k_place_res(DevTable t
         p64_s[i] = st.p64[i];
         p32_s[i] = st.p32[i];
         cap_s[i] = t.cap[i];
-        capd_s[i] = (double)t.cap[i];
-        Uc[i] = 0ull;
+        rcp_s[i] = st.rcp[i];
+        Uc[2 * i] = Uc[2 * i + 1] = 0u;
     }
     for (int i = tid; i < S; i += blockDim.x) {
         eb_s[i] = st.ebound[i];
@@ -346,62 +355,47 @@ __global__ void __launch_bounds__(kPlaceResWarps * 32, 1) k_place_res(DevTable t
         conv_s[i] = 0;
         rounds_s[i] = 0;
         bad_s[i] = 0;
-        huge_s[i] = 0;
         dmax_s[i] = 0ull;
         amax_s[i] = 0ull;
     }
-    const int w = blockIdx.x * kPlaceResWarps + wid;
-    const int64_t j0 = (w < pr.n_warps) ? pr.warp_job[w] : 0;
-    const int nj = (w < pr.n_warps) ? (int)(pr.warp_job[w + 1] - j0) : 0;
+    // of the scenario whose bound this warp computes (the first, when there are more scenarios than warps)
+    const float own_umax = wid < S && lane < R ? __int2float_ru(st.umax[(size_t)wid * R + lane]) : 0.0f;
+    const float own_vmax = wid < S ? __double2float_ru(st.vmax[wid]) : 0.0f;
+    const int64_t j = (int64_t)blockIdx.x * W + wid;
+    const bool has_job = j < pr.n_jobs;
     const int n0 = lane, n1 = lane + 32;
     const bool h0 = n0 < N, h1 = n1 < N;
-    float pen0[kPlaceResJobs], pen1[kPlaceResJobs];
-    uint32_t dup[kPlaceResJobs];
-    int scen[kPlaceResJobs];
-#pragma unroll
-    for (int q = 0; q < kPlaceResJobs; ++q) {
-        pen0[q] = pen1[q] = 0.0f;
-        dup[q] = 0u;
-        scen[q] = 0;
-        if (q < nj) {
-            const int64_t j = j0 + q;
-            scen[q] = (int)(j / t.J);
-            int32_t *us = reinterpret_cast<int32_t *>(wb + L.job_units + q * L.job_bytes);
-            float *ufs = reinterpret_cast<float *>(wb + L.job_ufs + q * L.job_bytes);
-            double *vs = reinterpret_cast<double *>(wb + L.job_vals + q * L.job_bytes);
-            for (int i = lane; i < KC * R; i += 32) {
-                const int32_t u = __ldg(pl.cfg_units + j * KC * R + i);
-                us[i] = u;
-                ufs[i] = __int2float_rn(u);
-            }
-            for (int k = lane; k < KC; k += 32)
-                vs[k] = __ldg(pl.cfg_values + j * KC + k);
-            const float sens = __ldg(pl.sens + j);
-            const int aj = __ldg(pl.job_type + j);
-            dup[q] = __ldg(pl.cfg_dup + j);
-            pen0[q] = h0 ? __fmul_rn(sens, __ldg(pl.D + aj * NT + __ldg(pl.node_type + n0))) : 0.0f;
-            pen1[q] = h1 ? __fmul_rn(sens, __ldg(pl.D + aj * NT + __ldg(pl.node_type + n1))) : 0.0f;
-            float *pens = reinterpret_cast<float *>(wb + L.job_pens + q * L.job_bytes);
-            pens[n0] = pen0[q];
-            pens[n1] = pen1[q];
+    float pa = 0.0f, pb = 0.0f;   // penalties of the lane's nodes
+    uint32_t dup = 0u;
+    int sc = 0;
+    int32_t *us = reinterpret_cast<int32_t *>(wb + L.job_units);
+    float *ufs = reinterpret_cast<float *>(wb + L.job_ufs);
+    double *vs = reinterpret_cast<double *>(wb + L.job_vals);
+    float *pens = reinterpret_cast<float *>(wb + L.job_pens);
+    if (has_job) {
+        sc = (int)(j / t.J);
+        for (int i = lane; i < KC * R; i += 32) {
+            const int32_t u = __ldg(pl.cfg_units + j * KC * R + i);
+            us[i] = u;
+            ufs[i] = __int2float_rn(u);
         }
+        for (int k = lane; k < KC; k += 32)
+            vs[k] = __ldg(pl.cfg_values + j * KC + k);
+        const float sens = __ldg(pl.sens + j);
+        const int aj = __ldg(pl.job_type + j);
+        dup = __ldg(pl.cfg_dup + j);
+        pa = h0 ? __fmul_rn(sens, __ldg(pl.D + aj * NT + __ldg(pl.node_type + n0))) : 0.0f;
+        pb = h1 ? __fmul_rn(sens, __ldg(pl.D + aj * NT + __ldg(pl.node_type + n1))) : 0.0f;
+        pens[n0] = pa;
+        pens[n1] = pb;
     }
     __syncthreads();
 
     for (int round = 0; round < T; ++round) {
         unsigned long long *Ub = pr.U3 + (size_t)(round % 3) * SP;
 
-        // ---- best responses of this warp's jobs at the CTA's prices
-#pragma unroll
-        for (int q = 0; q < kPlaceResJobs; ++q) {
-            if (q >= nj)
-                break;
-            const int sc = scen[q];
-            if (frozen_s[sc])
-                continue;
-            const int32_t *us = reinterpret_cast<const int32_t *>(wb + L.job_units + q * L.job_bytes);
-            const float *ufs = reinterpret_cast<const float *>(wb + L.job_ufs + q * L.job_bytes);
-            const double *vs = reinterpret_cast<const double *>(wb + L.job_vals + q * L.job_bytes);
+        // ---- best response of this warp's job at the CTA's prices
+        if (has_job && !frozen_s[sc]) {
             const float *p32s = p32_s + (size_t)sc * P;
             const double *p64s = p64_s + (size_t)sc * P;
             ScenarioPrices sp;
@@ -413,10 +407,8 @@ __global__ void __launch_bounds__(kPlaceResWarps * 32, 1) k_place_res(DevTable t
             sp.e2 = sp.exact ? INFINITY : 2.0f * e;
             __syncwarp();
             for (int k = lane; k < KC; k += 32)
-                gs[k] = ((dup[q] >> k) & 1u) ? INFINITY : place_global_part<RT>(us + k * R, vs[k], sp, rg);
+                gs[k] = ((dup >> k) & 1u) ? INFINITY : place_global_part<RT>(ufs + k * R, vs[k], sp, rg);
             __syncwarp();
-            const float pa = pen0[q], pb = pen1[q];
-            const float *pens = reinterpret_cast<const float *>(wb + L.job_pens + q * L.job_bytes);
             // this lane's node prices (columns r >= rg of nodes n0, n1) in registers
             const int nc = R - rg;
             float pn0[Cols<RT>::N], pn1[Cols<RT>::N];
@@ -457,16 +449,21 @@ __global__ void __launch_bounds__(kPlaceResWarps * 32, 1) k_place_res(DevTable t
                 if (h1)
                     fold(q1, k * N + n1);
             }
-            const Best x = allreduce_best(Best{m1, i1, m2});
-            const float thr = __fadd_ru(x.m1, sp.e2);
-            int win = x.idx;
-            if (sp.exact || !(x.m2 > thr)) {
+            // smallest, second smallest and holder over the warp by hardware reductions: the holder offers its
+            // second smallest, the others their smallest; two holders make both equal (and the job ambiguous)
+            const float g1 = warp_min_f32(m1);
+            const unsigned holders = __ballot_sync(FULL, m1 == g1);
+            const float o2 = warp_min_f32(m1 == g1 ? m2 : m1);
+            const float g2 = (holders & (holders - 1u)) ? g1 : o2;
+            const float thr = __fadd_ru(g1, sp.e2);
+            int win = __shfl_sync(FULL, i1, __ffs((int)holders) - 1);
+            if (sp.exact || !(g2 > thr)) {
                 // survivors (q <= thr; all in exact mode; repeated configurations never), listed in
                 // (k, node half, lane) order; up to 32 are rescored in fp64 one per lane
                 int *cand = reinterpret_cast<int *>(wb + L.cand);
                 int total = 0;
                 for (int k = 0; k < KC && total <= 32; ++k) {
-                    if ((dup[q] >> k) & 1u)
+                    if ((dup >> k) & 1u)
                         continue;
                     float q0, q1;
                     node_q(k, q0, q1);
@@ -498,7 +495,7 @@ __global__ void __launch_bounds__(kPlaceResWarps * 32, 1) k_place_res(DevTable t
                 } else {
                     // many survivors: each lane rescores its own
                     for (int k = 0; k < KC; ++k) {
-                        if ((dup[q] >> k) & 1u)
+                        if ((dup >> k) & 1u)
                             continue;
                         float q0, q1;
                         node_q(k, q0, q1);
@@ -540,24 +537,26 @@ __global__ void __launch_bounds__(kPlaceResWarps * 32, 1) k_place_res(DevTable t
             // the winner's units into the CTA's demand (lane r: column r)
             const int kw = win / N, nw = win - kw * N;
             if (lane < R) {
-                const long long u = us[kw * R + lane];
+                const uint32_t u = (uint32_t)us[kw * R + lane];
                 const int col = lane >= rg ? rg + (R - rg) * nw + (lane - rg) : lane;
-                if (u != 0)
-                    atomicAdd(Uc + (size_t)sc * P + col, (unsigned long long)u);
+                uint32_t *dst = Uc + 2 * ((size_t)sc * P + col);
+                if (u & 0xffffu)
+                    atomicAdd(dst, u & 0xffffu);
+                if (u >> 16)
+                    atomicAdd(dst + 1, u >> 16);
             }
         }
         __syncthreads();
         // ---- the CTA's demand into the round's buffer; per-scenario reductions reset
         for (int i = tid; i < SP; i += blockDim.x) {
-            const unsigned long long v = Uc[i];
-            if (v != 0ull) {
-                atomicAdd(Ub + i, v);
-                Uc[i] = 0ull;
+            const uint2 v = *reinterpret_cast<const uint2 *>(Uc + 2 * i);
+            if ((v.x | v.y) != 0u) {
+                atomicAdd(Ub + i, (unsigned long long)v.x + ((unsigned long long)v.y << 16));
+                Uc[2 * i] = Uc[2 * i + 1] = 0u;
             }
         }
         for (int i = tid; i < S; i += blockDim.x) {
             bad_s[i] = 0;
-            huge_s[i] = 0;
             dmax_s[i] = 0ull;
             amax_s[i] = 0ull;
         }
@@ -568,10 +567,11 @@ __global__ void __launch_bounds__(kPlaceResWarps * 32, 1) k_place_res(DevTable t
         // into registers, and written once no price of the scenario became non-finite
         const double eta = step_size(a.eta0, a.step, round);
         const bool lead = blockIdx.x == 0;
-        double nl_r[kPlaceResPricesPerThread], pe_r[kPlaceResPricesPerThread];
+        constexpr int kPrices = (kPlaceResMaxPrices + W * 32 - 1) / (W * 32);   // per thread
+        double nl_r[kPrices], pe_r[kPrices];
 #pragma unroll
-        for (int m = 0; m < kPlaceResPricesPerThread; ++m) {
-            const int i = tid + m * kPlaceResWarps * 32;
+        for (int m = 0; m < kPrices; ++m) {
+            const int i = tid + m * W * 32;
             nl_r[m] = pe_r[m] = 0.0;
             if (i >= SP)
                 break;
@@ -582,9 +582,10 @@ __global__ void __launch_bounds__(kPlaceResWarps * 32, 1) k_place_res(DevTable t
             if (lead && st.dem_trace)
                 st.dem_trace[((size_t)sc * T + round) * P + (i - sc * P)] = U;
             const double lam = lam_s[i];
-            const double nl = price_step(lam, U, cap_s[i], capd_s[i], eta, a.mode);
+            const double capd = (double)cap_s[i], rcp = rcp_s[i];
+            const double nl = price_step_rcp(lam, U, cap_s[i], capd, rcp, eta, a.mode);
             nl_r[m] = nl;
-            pe_r[m] = effective_price(nl, capd_s[i], a.mode);
+            pe_r[m] = effective_price_rcp(nl, capd, rcp, a.mode);
             if (!isfinite(nl))
                 atomicOr(bad_s + sc, 1);
             if (a.tol > 0.0) {   // maxima of the stopping rule (non-negative doubles order as integers)
@@ -594,8 +595,8 @@ __global__ void __launch_bounds__(kPlaceResWarps * 32, 1) k_place_res(DevTable t
         }
         __syncthreads();
 #pragma unroll
-        for (int m = 0; m < kPlaceResPricesPerThread; ++m) {
-            const int i = tid + m * kPlaceResWarps * 32;
+        for (int m = 0; m < kPrices; ++m) {
+            const int i = tid + m * W * 32;
             if (i >= SP)
                 break;
             const int sc = i / P;
@@ -606,12 +607,12 @@ __global__ void __launch_bounds__(kPlaceResWarps * 32, 1) k_place_res(DevTable t
                 st.lam_trace[((size_t)sc * (T + 1) + round + 1) * P + (i - sc * P)] = nl_r[m];
             p64_s[i] = pe_r[m];
             p32_s[i] = __double2float_rn(pe_r[m]);
-            if (!(pe_r[m] <= 0x1p100))
-                atomicOr(huge_s + sc, 1);
         }
         __syncthreads();
-        // stopping rule and screen bound, one warp per scenario (the summation order of set_prices)
-        for (int sc = wid; sc < S; sc += kPlaceResWarps) {
+        // stopping rule and screen bound, one warp per scenario. E only has to bound the screen's error from
+        // above: it is computed in fp32 with every operation rounded up, from p <= p32 (1 + 2^-23) + 2^-149 and
+        // M = max|v| + sum_r (largest p_r) max u_r; no fp64 operation, and one reduction per node column
+        for (int sc = wid; sc < S; sc += W) {
             if (frozen_s[sc])
                 continue;
             if (bad_s[sc]) {
@@ -624,20 +625,24 @@ __global__ void __launch_bounds__(kPlaceResWarps * 32, 1) k_place_res(DevTable t
             const double dmax = __longlong_as_double((long long)dmax_s[sc]);
             const double amax = __longlong_as_double((long long)amax_s[sc]);
             const bool conv = (a.tol > 0.0) && (dmax <= a.tol * fmax(1.0, amax));
-            const double *p64s = p64_s + (size_t)sc * P;
-            double term = 0.0;
-            const int rgm = (t.n_groups == 0) ? R : rg;
-            if (lane < rgm)
-                term = p64s[lane] * (double)st.umax[(size_t)sc * R + lane];
-            for (int c2 = 0; c2 < R - rgm; ++c2) {
-                double pm = 0.0;
+            const float *p32s = p32_s + (size_t)sc * P;
+            const float umax_up = sc == wid ? own_umax : lane < R ? __int2float_ru(st.umax[(size_t)sc * R + lane]) : 0.0f;
+            const float vmax_up = sc == wid ? own_vmax : __double2float_ru(st.vmax[sc]);
+            float p = lane < rg ? p32s[lane] : 0.0f;   // lane r: the largest price of column r
+            for (int c2 = 0; c2 < R - rg; ++c2) {
+                uint32_t pm = 0u;                      // prices are not negative: their bits order as they do
                 for (int gi = lane; gi < t.n_groups; gi += 32)
-                    pm = fmax(pm, p64s[rgm + (R - rgm) * gi + c2]);
-                pm = warp_max(pm);
-                if (lane == rgm + c2)
-                    term = pm * (double)st.umax[(size_t)sc * R + lane];
+                    pm = max(pm, __float_as_uint(p32s[rg + (R - rg) * gi + c2]));
+                pm = __reduce_max_sync(FULL, pm);
+                p = lane == rg + c2 ? __uint_as_float(pm) : p;
             }
-            const double M = st.vmax[sc] + warp_sum_fixed(term);
+            const float p_up = __fadd_ru(__fmul_ru(p, 1.0f + 0x1p-23f), 0x1p-149f);
+            const bool huge = __any_sync(FULL, lane < R && !(p_up <= 0x1p100f));
+            float term = lane < R ? __fmul_ru(p_up, umax_up) : 0.0f;
+#pragma unroll
+            for (int d = 8; d >= 1; d >>= 1)           // lanes 0 .. 15 hold the terms
+                term = __fadd_ru(term, __shfl_xor_sync(FULL, term, d));
+            const float M = __fadd_ru(vmax_up, term);
             if (lane == 0) {
                 if (lead && st.time_trace)
                     st.time_trace[(size_t)sc * T + round] = global_ns();
@@ -646,7 +651,9 @@ __global__ void __launch_bounds__(kPlaceResWarps * 32, 1) k_place_res(DevTable t
                     conv_s[sc] = 1;
                     frozen_s[sc] = 1;
                 }
-                eb_s[sc] = screen_bound(M, R, a.exact_only || huge_s[sc] != 0);
+                eb_s[sc] = a.exact_only || huge || !(M <= 0x1p100f)
+                               ? INFINITY
+                               : __fadd_ru(__fmul_ru(M, (4.0f * R + 16.0f) * 0x1p-24f), 0x1p-99f);
             }
         }
         if (lead) {   // buffer (round + 2) % 3 was last read before this round's barrier
@@ -727,19 +734,32 @@ cudaError_t launch_place(const DevTable &t, const DevState &st, const DevPlace &
     return cudaGetLastError();
 }
 
-int place_res_smem_bytes(int S, int P, int KC, int R)
+int place_res_smem_bytes(int S, int P, int KC, int R, int warps)
 {
-    return place_res_layout(S, P, KC, R).total;
+    return place_res_layout(S, P, KC, R, warps).total;
 }
 
-int place_res_ctas_per_sm(int S, int P, int KC, int R)
+static const void *place_res_kernel(int R, int warps)
 {
-    const int smem = place_res_smem_bytes(S, P, KC, R);
-    const void *fn = R == 8 ? reinterpret_cast<const void *>(&k_place_res<8>)
-                            : reinterpret_cast<const void *>(&k_place_res<0>);
-    int m = 0;
-    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&m, fn, kPlaceResWarps * 32, smem) != cudaSuccess) {
+    if (R == 8)
+        return warps == 8    ? reinterpret_cast<const void *>(&k_place_res<8, 8>)
+               : warps == 16 ? reinterpret_cast<const void *>(&k_place_res<8, 16>)
+                             : reinterpret_cast<const void *>(&k_place_res<8, 32>);
+    return warps == 8    ? reinterpret_cast<const void *>(&k_place_res<0, 8>)
+           : warps == 16 ? reinterpret_cast<const void *>(&k_place_res<0, 16>)
+                         : reinterpret_cast<const void *>(&k_place_res<0, 32>);
+}
+
+int place_res_ctas_per_sm(int S, int P, int KC, int R, int warps)
+{
+    const void *fn = place_res_kernel(R, warps);
+    // the limit is the kernel's, not the table's: the device's largest for every one
+    int m = 0, dev = 0, optin = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess ||
+        cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - 1024) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&m, fn, warps * 32, place_res_smem_bytes(S, P, KC, R, warps)) !=
+            cudaSuccess) {
         cudaGetLastError();
         return 0;
     }
@@ -758,17 +778,16 @@ static cudaError_t place_res_launch(const DevTable &t, const DevState &st, const
         return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)pr.grid);
-    cfg.blockDim = dim3(kPlaceResWarps * 32);
-    cfg.dynamicSmemBytes = (size_t)place_res_smem_bytes(t.S, t.P, pl.KC, t.R);
+    cfg.blockDim = dim3((unsigned)pr.warps * 32);
+    cfg.dynamicSmemBytes = (size_t)place_res_smem_bytes(t.S, t.P, pl.KC, t.R, pr.warps);
     cfg.stream = stream;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeCooperative;   // every CTA co-resident: the grid barrier can complete
     attr[0].val.cooperative = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    if (t.R == 8)
-        return cudaLaunchKernelEx(&cfg, k_place_res<8>, t, st, pl, a, pr);
-    return cudaLaunchKernelEx(&cfg, k_place_res<0>, t, st, pl, a, pr);
+    void *args[] = {(void *)&t, (void *)&st, (void *)&pl, (void *)&a, (void *)&pr};
+    return cudaLaunchKernelExC(&cfg, place_res_kernel(t.R, pr.warps), args);
 }
 
 cudaError_t launch_place_res(const DevTable &t, const DevState &st, const DevPlace &pl, const SolveArgs &a,
