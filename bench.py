@@ -116,7 +116,7 @@ def measured_peak():
         return 6800.0, "fallback"
 
 
-PASS_KERNEL_SOURCES = ("esp_packed.cu", "esp_packed.h", "esp_kernels.cu", "esp_pass.cuh", "esp_tile.cuh", "esp_ptx.cuh", "esp_warp.cuh",
+PASS_KERNEL_SOURCES = ("esp_packed.cu", "esp_packed.h", "esp_div.h", "esp_kernels.cu", "esp_pass.cuh", "esp_tile.cuh", "esp_ptx.cuh", "esp_warp.cuh",
                        "esp_device.cuh", "esp_common.h", "esp_kernels.h")
 
 
@@ -142,6 +142,23 @@ def kernel_traffic(workload: str, n_opt_launch: int):
         return float(rec["dram_bytes_per_launch"]) / float(rec["options_per_launch"]) * n_opt_launch
     except Exception:
         return None
+
+
+def pass_bytes(t, kernel: int) -> int:
+    """Bytes of the table that one evaluation pass has to read: 4 bytes per option and per unit word of the
+    packed copy (columns paired, the widest with the widest that fits 32 bits, rounded up to a kernel's word
+    count) where the packed passes run, else the table itself."""
+    if kernel not in (1, 3) or t.group is not None or int(t.units.max(initial=0)) >= 1 << 23:
+        return t.table_bytes()
+    bits = sorted((max(1, int(u).bit_length()) for u in t.units.max(axis=0)), reverse=True)
+    words = 0
+    while bits:
+        lo = bits.pop(0)
+        hi = next((i for i, b in enumerate(bits) if lo + b <= 32), None)
+        if hi is not None:
+            bits.pop(hi)
+        words += 1
+    return t.n_opt * 4 * (1 + next((n for n in (2, 3, 4, 6, 8) if words <= n), 8))
 
 
 # fp32 FMA units of a GB300 (152 SMs x 128 lanes) at the maximum SM clock, 2 flops per FMA
@@ -408,7 +425,7 @@ def time_streaming(esp, solver, w, T, args, dist, barrier, stream, clk=None):
     # between launches are charged to the passes, so this understates the kernel slightly)
     other_ms = max(0.0, ms_ev - pass_ms)
     avg_ms = max(1e-9, ms / (T + 1))
-    bytes_pass = t.table_bytes()
+    bytes_pass = pass_bytes(t, esp.esp_debug_pass_kernel(ctx))
     achieved = bytes_pass / (avg_ms / 1e3) / 1e9
     ev_avg_ms = pass_ms / max(n_pass, 1)
     ev_achieved = bytes_pass / (ev_avg_ms / 1e3) / 1e9 if n_pass else None
@@ -425,7 +442,7 @@ def time_streaming(esp, solver, w, T, args, dist, barrier, stream, clk=None):
                 "traffic": kernel_traffic(w.name, t.n_opt),
                 "peak_kind": f"{peak_kind} hbm_gbs (copy)",
                 "frac_of_nominal_8tbs": achieved / 8000.0,
-                "bytes_per_launch": bytes_pass, "avg_launch_ms": avg_ms,
+                "bytes_per_launch": bytes_pass, "table_bytes": t.table_bytes(), "avg_launch_ms": avg_ms,
                 "launches_per_step": T + 1,
                 "persistent": persist,
                 "per_round_note": ("the T rounds run in one launch: bytes_per_launch and avg_launch_ms are per "

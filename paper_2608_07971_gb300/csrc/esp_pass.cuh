@@ -20,8 +20,6 @@ namespace esp {
 
 namespace {
 
-// Data of tile-local option o (stage) or of job option o (global, gfirst = the job's first option).
-
 // Asks L2 for the option bytes of tile d (lane 0 only), a few tiles before the stage copy of the
 // same bytes is issued: the DRAM latency is then hidden by L2 rather than by shared memory.
 __device__ __forceinline__ void prefetch_tile(const DevTable &t, const TileDesc &d)
@@ -34,9 +32,6 @@ __device__ __forceinline__ void prefetch_tile(const DevTable &t, const TileDesc 
     prefetch_l2(reinterpret_cast<const unsigned char *>(t.units) + ulo, (uint32_t)(uhi - ulo));
     prefetch_l2(reinterpret_cast<const unsigned char *>(t.values) + vlo, (uint32_t)(vhi - vlo));
 }
-
-// Chunk tile of a job larger than a tile: all its options belong to one job, so no segmentation is
-
 
 // Issues the bulk copies of tile d into a stage; lane 0 only (issuing the copies from several lanes
 // at once measured slower). Uniform tables and runs of the sorted layout need no job offsets.

@@ -49,12 +49,6 @@ __device__ __forceinline__ void fence_proxy_async()
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
 
-// Plain arrival (one count) on a barrier.
-__device__ __forceinline__ void mbar_arrive(uint32_t bar)
-{
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
-
 // Waits on the phase of the given parity without a time hint: the thread may be suspended for a short,
 // system-dependent time and resumes when the phase completes.
 __device__ __forceinline__ bool mbar_try_wait_nohint(uint32_t bar, uint32_t parity)
@@ -89,25 +83,6 @@ __device__ __forceinline__ bool wait_stage(uint32_t bar, uint32_t parity, unsign
     const uint64_t limit = (uint64_t)limit_ms * 1000000ull;
     for (;;) {
         if (mbar_try_wait_nohint(bar, parity))
-            return true;
-        if (global_ns() - t0 > limit)
-            break;
-    }
-    atomicOr(err, DEV_ERR_TIMEOUT);
-    return false;
-}
-
-// Bounded wait until a shared word holds `want` (a stage's sequence word): polls it and gives up after
-// `limit_ms` milliseconds of the global timer, flagging a timeout.
-__device__ __forceinline__ bool wait_word(const volatile int *w, int want, unsigned int *err, uint32_t limit_ms)
-{
-    if (*w == want)
-        return true;
-    const uint64_t t0 = global_ns();
-    const uint64_t limit = (uint64_t)limit_ms * 1000000ull;
-    for (;;) {
-        __nanosleep(32);
-        if (*w == want)
             return true;
         if (global_ns() - t0 > limit)
             break;
