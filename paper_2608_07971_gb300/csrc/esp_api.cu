@@ -1905,7 +1905,7 @@ esp_status esp_load_placement(esp_ctx *ctx, int32_t S, int32_t J, int32_t KC, in
         place_res_smem_bytes(S, P, KC, R, rw) <= optin && place_res_ctas_per_sm(S, P, KC, R, rw) >= 1) {
         PlaceRes &pr = ctx->place_res;
         PALLOC(pr.U3, 3 * (size_t)S * P);
-        PALLOC(pr.bar, 2);
+        PALLOC(pr.bar, 1);
         pr.n_jobs = (int32_t)n_jobs;
         pr.warps = rw;
         pr.grid = (int32_t)((n_jobs + rw - 1) / rw);

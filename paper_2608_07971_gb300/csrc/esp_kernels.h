@@ -137,7 +137,7 @@ constexpr int kPlaceResMaxWarps = 32;      // warps per CTA of the grid-resident
 // the grid holding job w.
 struct PlaceRes {
     unsigned long long *U3;     // 3 * S * P: the demand of round r in buffer r % 3
-    unsigned int *bar;          // [0] barrier arrivals, [1] abort; zeroed before each launch
+    unsigned long long *bar;    // the grid barrier's word (esp_barrier.h); zeroed before each launch
     int32_t n_jobs, grid, warps;
 };
 

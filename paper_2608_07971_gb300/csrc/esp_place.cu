@@ -7,6 +7,7 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
+#include "esp_barrier.h"
 #include "esp_device.cuh"
 #include "esp_kernels.h"
 #include "esp_place.h"
@@ -237,28 +238,27 @@ __global__ void __launch_bounds__(kPlaceWarps * 32, 4) k_place(DevTable t, DevSt
     place_jobs<RT>(c, pl, ws, pl.warp_job[w], pl.warp_job[w + 1], lane);
 }
 
-// Grid-wide barrier of a cooperative launch: every CTA adds 1 to *bar and waits until it reaches
-// target (= CTAs x barriers so far). Thread 0 waits, bounded (about 4 s); on expiry, or when
-// another CTA gave up (bar[1] != 0), the barrier fails for the whole CTA, the device error word is
-// flagged and bar[1] set so that no CTA waits for it any longer.
-__device__ bool grid_barrier(unsigned int *bar, unsigned int target, unsigned int *err, int *ok_s)
+// Grid-wide barrier of a cooperative launch: every CTA adds 1 to the count of *bar (esp_barrier.h) and waits
+// until it reaches target (= CTAs x barriers so far). Thread 0 waits, bounded (about 4 s); on expiry, or
+// when another CTA gave up, the barrier fails for the whole CTA, the device error word is flagged and the word's
+// abort bit set so that no CTA waits for it any longer. Every access of the word is 64 bits wide; the arrival
+// releases (cumulatively, after the CTA barrier) what every thread of the CTA did before it.
+__device__ bool grid_barrier(unsigned long long *bar, unsigned long long target, unsigned int *err, int *ok_s)
 {
-    __threadfence();
     __syncthreads();
     if (threadIdx.x == 0) {
-        atomicAdd(bar, 1u);
+        asm volatile("red.release.gpu.global.add.u64 [%0], %1;" ::"l"(bar), "l"(1ull) : "memory");
         uint64_t t0;
         asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t0));
         bool ok = false;
         for (uint32_t it = 0;; ++it) {
-            // both words in one trip to L2 (they are one aligned 8-byte word)
             unsigned long long v;
             asm volatile("ld.acquire.gpu.u64 %0, [%1];" : "=l"(v) : "l"(bar) : "memory");
-            if ((int)((unsigned int)v - target) >= 0) {
+            if (bar_reached(v, target)) {
                 ok = true;
                 break;
             }
-            if ((unsigned int)(v >> 32) != 0u)
+            if (bar_aborted(v))
                 break;
             if (it > 64) {
                 uint64_t t1;
@@ -270,7 +270,7 @@ __device__ bool grid_barrier(unsigned int *bar, unsigned int target, unsigned in
         }
         if (!ok) {
             atomicOr(err, DEV_ERR_TIMEOUT);
-            atomicExch(bar + 1, 1u);
+            atomicOr(bar, kBarAbort);
         }
         *ok_s = ok ? 1 : 0;
     }
@@ -560,7 +560,7 @@ __global__ void __launch_bounds__(W * 32, 1) k_place_res(DevTable t, DevState st
             dmax_s[i] = 0ull;
             amax_s[i] = 0ull;
         }
-        if (!grid_barrier(pr.bar, (unsigned int)(round + 1) * gridDim.x, st.err, &ok_s))
+        if (!grid_barrier(pr.bar, (unsigned long long)(round + 1) * gridDim.x, st.err, &ok_s))
             break;
 
         // ---- Eq. price_update of every scenario, one price per thread: the new prices are computed
@@ -769,9 +769,7 @@ int place_res_ctas_per_sm(int S, int P, int KC, int R, int warps)
 static cudaError_t place_res_launch(const DevTable &t, const DevState &st, const DevPlace &pl, const SolveArgs &a,
                                     const PlaceRes &pr, cudaStream_t stream, bool hold_barrier)
 {
-    cudaError_t e = cudaMemsetAsync(pr.bar, 0, 2 * sizeof(unsigned int), stream);
-    if (e == cudaSuccess && hold_barrier)   // every byte 0xC0: the counter far short of its targets
-        e = cudaMemsetAsync(pr.bar, 0xC0, sizeof(unsigned int), stream);
+    cudaError_t e = cudaMemsetAsync(pr.bar, hold_barrier ? kBarHeldByte : 0, sizeof(*pr.bar), stream);
     if (e == cudaSuccess)   // the last rounds of the previous solve leave demand in two buffers
         e = cudaMemsetAsync(pr.U3, 0, 3 * (size_t)t.S * t.P * sizeof(unsigned long long), stream);
     if (e != cudaSuccess)
