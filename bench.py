@@ -144,21 +144,10 @@ def kernel_traffic(workload: str, n_opt_launch: int):
         return None
 
 
-def pass_bytes(t, kernel: int) -> int:
-    """Bytes of the table that one evaluation pass has to read: 4 bytes per option and per unit word of the
-    packed copy (columns paired, the widest with the widest that fits 32 bits, rounded up to a kernel's word
-    count) where the packed passes run, else the table itself."""
-    if kernel not in (1, 3) or t.group is not None or int(t.units.max(initial=0)) >= 1 << 23:
-        return t.table_bytes()
-    bits = sorted((max(1, int(u).bit_length()) for u in t.units.max(axis=0)), reverse=True)
-    words = 0
-    while bits:
-        lo = bits.pop(0)
-        hi = next((i for i, b in enumerate(bits) if lo + b <= 32), None)
-        if hi is not None:
-            bits.pop(hi)
-        words += 1
-    return t.n_opt * 4 * (1 + next((n for n in (2, 3, 4, 6, 8) if words <= n), 8))
+def pass_bytes(t, words: int) -> int:
+    """Bytes of the table that one evaluation pass has to read: a 4-byte value and `words` unit words per option of
+    the packed copy where the packed passes run, else (0 words) the table itself."""
+    return t.n_opt * 4 * (1 + words) if words else t.table_bytes()
 
 
 # fp32 FMA units of a GB300 (152 SMs x 128 lanes) at the maximum SM clock, 2 flops per FMA
@@ -425,12 +414,13 @@ def time_streaming(esp, solver, w, T, args, dist, barrier, stream, clk=None):
     # between launches are charged to the passes, so this understates the kernel slightly)
     other_ms = max(0.0, ms_ev - pass_ms)
     avg_ms = max(1e-9, ms / (T + 1))
-    bytes_pass = pass_bytes(t, esp.esp_debug_pass_kernel(ctx))
+    bytes_pass = pass_bytes(t, esp.esp_debug_packed_words(ctx))
     achieved = bytes_pass / (avg_ms / 1e3) / 1e9
     ev_avg_ms = pass_ms / max(n_pass, 1)
     ev_achieved = bytes_pass / (ev_avg_ms / 1e3) / 1e9 if n_pass else None
     kind = {0: "k_pass (per-warp pass, two bulk copies per tile)",
-            1: "k_packed or k_pass (a private copy in the order of its tiles, one bulk copy per step or tile)",
+            1: "k_packed (packed screen copy, one bulk copy per 256 options)" if esp.esp_debug_packed_words(ctx)
+            else "k_pass (per-warp pass, one bulk copy per tile from the tile-interleaved table)",
             3: "k_packed (packed screen copy, one bulk copy per 256 options)"}.get(
         esp.esp_debug_pass_kernel(ctx), "k_place (factored placement pass)")
     persist = esp.esp_debug_persistent(ctx) > 0

@@ -63,7 +63,7 @@ esp_status esp_debug_set_sorted_layout(esp_ctx *ctx, int32_t enable);
 esp_status esp_debug_set_pdl(esp_ctx *ctx, int32_t mode);
 
 /* Warps of the evaluation pass planned by later loads, as a number of waves of resident CTAs
- * (1..8; 0 = the library's choice, two waves): more waves give smaller warp ranges that the hardware
+ * (1..8; 0 = the library's choice: one wave for packed tables and sorted layouts, else two): more waves give smaller warp ranges that the hardware
  * schedules as CTAs finish. Results are the same for any setting. */
 esp_status esp_debug_set_plan_waves(esp_ctx *ctx, int32_t waves);
 
@@ -102,6 +102,10 @@ esp_status esp_debug_fail_alloc(esp_ctx *ctx, int64_t n);
  * the packed screen copy where the persistent pass is available too. */
 esp_status esp_debug_pass_kernel(esp_ctx *ctx, int32_t *kind);
 
+/* *words receives the unit words per option of the loaded table's packed screen copy (an evaluation pass then reads
+ * 4 bytes more than these per option), 0 when the table is evaluated by another pass. */
+esp_status esp_debug_packed_words(esp_ctx *ctx, int32_t *words);
+
 /* Persistent pass: every round of a solve in one cooperative launch, each scenario's next round
  * released by its price update instead of a kernel boundary (packed tables of R = 4, 6 or 8, or large
  * enough to use it by default; solves without per-pass events, fingerprint or dual trace). mode -1 (the
@@ -119,15 +123,16 @@ esp_status esp_debug_persist_waits(esp_ctx *ctx, int64_t *ns, int64_t *waits, in
 
 /* Profile of the last esp_load_options / esp_load_options_device of this context: ms[0..6] the host
  * milliseconds from its start until its uploads and validation were queued, until the duplicate marks
- * were queued, until the packed passes were planned, until that plan was stored, until the uploads,
- * validation and duplicate marks were done, until the private copy of the table and the solve
+ * were queued, until the packed passes were planned, until the staged pass was (where that one is expected to
+ * run), until the uploads, validation and duplicate marks were done, until the private copy of the table and the solve
  * state were queued, and until it returned; *mallocs and *frees the cudaMalloc and cudaFree calls it
  * made (a reload of a table of the same shape makes none). */
 esp_status esp_debug_load_profile(esp_ctx *ctx, double *ms, int64_t *mallocs, int64_t *frees);
 
 /* enable = 0 makes later loads use the staged pass (integer units in the tile-interleaved table); 1
- * restores the default, the packed passes where every unit is below 2^23, the table has no group column
- * and its unit fields fit 8 words per option. Results are identical either way. */
+ * restores the default, the packed passes where every unit is below 2^23 and the unit fields fit 8 words per
+ * option (with a group column: one or two columns per group in one word of at most 6, and at most 1024 prices).
+ * Results are identical either way. (The name is that of an earlier form of the switch.) */
 esp_status esp_debug_set_stage_f32(esp_ctx *ctx, int32_t enable);
 
 /* enable = 0 makes later loads use the staged pass with separate unit and value arrays (two bulk copies

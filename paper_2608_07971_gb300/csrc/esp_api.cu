@@ -589,7 +589,8 @@ esp_status load_packed(esp_ctx *ctx, const PackFormat &fmt)
     // steps per warp) 23.6 / 34.2 / 55.1 / 144 us against 33.0 / 30.9 / 41.0 / 90.2, heavy-tailed table at
     // 2 / 4 / 16 scenarios 50 / 91 / 247 against 48 / 63 / 170: below, the waits for prices cost more than
     // the launches; above, static tile ranges leave the GPU waiting for its slowest warps. Smaller
-    // tables of R = 4, 6, 8 take it on request.
+    // tables take it on request where R is 4, 6 or 8, the widths that the request has always been granted for
+    // (the kernel itself depends on the word count only).
     // A table with a group column has no persistent pass.
     const int per_sm = packed_ctas_per_sm(fmt.nw, fmt.g_bytes);
     if (per_sm > 0 && d.n_tiles > 0 && !ctx->group) {
@@ -2330,6 +2331,16 @@ esp_status esp_debug_persistent(esp_ctx *ctx, int32_t *grid)
     *grid = (ctx->persist_mode > 0 || (ctx->persist_mode < 0 && ctx->persist_auto)) ? ctx->persist_grid : 0;
     return ESP_OK;
 }
+esp_status esp_debug_packed_words(esp_ctx *ctx, int32_t *words)
+{
+    if (!ctx || !words)
+        return ESP_ERR_INVALID_ARG;
+    if (!ctx->loaded)
+        return ESP_ERR_NOT_LOADED;
+    *words = ctx->packed ? ctx->pack.fmt.nw : 0;
+    return ESP_OK;
+}
+
 
 esp_status esp_debug_set_stage_f32(esp_ctx *ctx, int32_t enable)
 {

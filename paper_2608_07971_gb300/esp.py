@@ -32,7 +32,7 @@ EXPORTED = [
     "esp_debug_hold_barrier", "esp_debug_set_wait_limit", "esp_debug_hold_stage", "esp_debug_fail_alloc",
     "esp_debug_pass_kernel", "esp_debug_set_interleave", "esp_debug_set_stage_f32",
     "esp_debug_set_persistent", "esp_debug_persistent", "esp_debug_persist_waits",
-    "esp_debug_load_profile",
+    "esp_debug_load_profile", "esp_debug_packed_words",
     "esp_evaluate_noalloc",
     "esp_set_penalties", "esp_adaptive_threshold", "esp_effective_capacity", "esp_load_placement",
     "esp_iac_create", "esp_iac_set_stream", "esp_iac_load_model", "esp_iac_predict", "esp_iac_predict_host",
@@ -107,6 +107,7 @@ def load_library(path: Optional[str] = None):
         "esp_debug_hold_stage": ([vp], st),
         "esp_debug_fail_alloc": ([vp, i64], st),
         "esp_debug_pass_kernel": ([vp, ctypes.POINTER(i32)], st),
+        "esp_debug_packed_words": ([vp, ctypes.POINTER(i32)], st),
         "esp_debug_set_interleave": ([vp, i32], st),
         "esp_debug_set_stage_f32": ([vp, i32], st),
         "esp_debug_set_persistent": ([vp, i32], st),
@@ -536,6 +537,13 @@ def esp_debug_pass_kernel(ctx: int) -> int:
     its tiles, one launch per round; 2 factored placement; 3 packed, persistent pass available."""
     k = ctypes.c_int32()
     _check(load_library().esp_debug_pass_kernel(ctx, ctypes.byref(k)), "esp_debug_pass_kernel")
+    return k.value
+
+
+def esp_debug_packed_words(ctx: int) -> int:
+    """Unit words per option of the loaded table's packed copy; 0: another pass evaluates it."""
+    k = ctypes.c_int32()
+    _check(load_library().esp_debug_packed_words(ctx, ctypes.byref(k)), "esp_debug_packed_words")
     return k.value
 
 

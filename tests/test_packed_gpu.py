@@ -48,7 +48,7 @@ def mixed(ks, J, R, seed, umax=5000, S=2):
 
 def run_all(t, T=12, persist=True, packed=True):
     a = esp.Solver(t)
-    assert not packed or esp.esp_debug_pass_kernel(a.ctx) in (1, 3)
+    assert (esp.esp_debug_packed_words(a.ctx) > 0) == packed
     traced = a.solve(0.3, T, traces=True)
     check_solution(t, traced, list(range(t.S)), 0.3, T, esp.ESP_PRICE_NORMALIZED, esp.ESP_STEP_FIXED)
     plain = a.solve(0.3, T)
@@ -88,6 +88,21 @@ def test_unit_words(R, umax):
     """2 to 8 unit words (over eight columns of 23 bits need more: the staged pass takes those)."""
     run_all(mixed([16, 3, 130, 1], 40, R, 100 * R + 1, umax=umax), T=6, persist=R == 8,
             packed=R <= 8 or umax <= 65535)
+
+
+@pytest.mark.parametrize("R,words", [(4, 2), (6, 3), (8, 4), (12, 6), (16, 8)])
+def test_every_word_count_of_the_persistent_pass(R, words):
+    """Tables that take the persistent pass by default, for each instantiation of it."""
+    t = mixed([32], 16384, R, R, umax=65535, S=8)
+    s = esp.Solver(t)
+    assert esp.esp_debug_packed_words(s.ctx) == words and esp.esp_debug_persistent(s.ctx) > 0
+    a = s.solve(0.3, 3)
+    assert s.launches() == 4
+    esp.esp_debug_set_persistent(s.ctx, 0)
+    b = s.solve(0.3, 3)
+    assert s.launches() == 3 + 3
+    assert np.array_equal(a.lam, b.lam) and np.array_equal(a.sel, b.sel) and np.array_equal(a.demand, b.demand)
+    s.close()
 
 
 def test_large_table_of_other_widths_takes_the_persistent_pass():

@@ -24,7 +24,7 @@ def _lib():
 
 def run_all(t, T=10, kind=1):
     a = esp.Solver(t)
-    assert esp.esp_debug_pass_kernel(a.ctx) == kind
+    assert esp.esp_debug_pass_kernel(a.ctx) == kind and (esp.esp_debug_packed_words(a.ctx) > 0) == (kind == 1)
     b = esp.Solver()
     esp.esp_debug_set_interleave(b.ctx, False)      # the staged pass
     b.load(t)
