@@ -55,6 +55,10 @@ OUT_OF_BOUNDS = {
     ("for (int32_t k = 0; k < P; ++k) {", "for (int32_t k = 0; k <= P; ++k) {"),
     ("for (int32_t j = 0; j < J; ++j)", "for (int32_t j = 0; j <= J; ++j)"),
     ("for (int32_t r = 0; r < R; ++r) {", "for (int32_t r = 0; r <= R; ++r) {"),
+    # one option too many: caught or not by what the memory behind the last job's options holds
+    ("for (int64_t o = first + 1; o < last; ++o) {", "for (int64_t o = first + 1; o <= last; ++o) {"),
+    ("for (int64_t o = t->job_off[j]; o < t->job_off[j + 1]; ++o) {", "for (int64_t o = t->job_off[j]; o <= t->job_off[j + 1]; ++o) {"),
+    ("for (int64_t o = q_off[q] + 1; o < q_off[q + 1]; ++o)", "for (int64_t o = q_off[q] + 1; o <= q_off[q + 1]; ++o)"),
 }
 
 
