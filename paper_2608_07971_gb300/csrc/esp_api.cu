@@ -1067,16 +1067,16 @@ esp_status plan_resident_options(esp_ctx *ctx)
             esp_ctx::ResOption o;
             o.plan.cs = cs;
             o.plan.k = rk;
-            // lanes per job: as many as the CTA has for its jobs, up to one per option. The lanes of one
-            // option read 32 / lanes consecutive jobs; an odd multiple of that as the pitch keeps the
-            // options of a warp's lanes in different banks
+            // lanes per job: as many as the CTA has for its jobs, up to one per option
             o.plan.lanes = 1;
             while (o.plan.lanes < 8 && 2 * o.plan.lanes * sh.m_max <= kResWarps * 32 && 2 * o.plan.lanes <= ctx->pc.max_k)
                 o.plan.lanes *= 2;
             const int32_t unit = 32 / o.plan.lanes;
-            o.plan.m_pad = std::max(1, (sh.m_max + unit - 1) / unit) * unit;
-            if (o.plan.lanes > 1 && (o.plan.m_pad / unit) % 2 == 0)
-                o.plan.m_pad += unit;
+            int32_t pitch = unit;
+            while (pitch < sh.m_max && pitch < 32)
+                pitch *= 2;
+            o.plan.m_pad = std::max(pitch, (sh.m_max + pitch - 1) / pitch * pitch);
+            o.plan.spread = std::min(o.plan.lanes, pitch / unit) - 1;
             o.plan.n_cap = (sh.n_max + 1) & ~1LL;
             o.smem = res_smem_bytes(R, o.plan);
             o.n_max = sh.n_max;
@@ -1131,6 +1131,8 @@ esp_status plan_resident_options(esp_ctx *ctx)
             // the automatic choice runs only where it is predicted faster than streaming: S scenarios take
             // ceil(S / clusters) waves of clusters; a streaming round takes about 12 us plus its table (half of
             // it, packed) at 6 TB/s, and 6.5 us (launch and update latency) where it is a few steps
+            // the pitch, a power of two up to 16 or a multiple of 32; the kernel's exclusive or spreads the job slots of
+            // the lanes that read one job's options over it
             if (ctx->res_auto >= 0) {
                 const esp_ctx::ResOption &o = ctx->res[ctx->res_auto];
                 const double waves = std::ceil((double)S / (double)o.clusters);

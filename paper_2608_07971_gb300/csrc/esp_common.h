@@ -79,8 +79,8 @@ constexpr int kResMaxCluster = 16;   // CTAs per cluster of the resident kernel 
 constexpr int kResCols = kMaxR + 2;  // words of a demand partial: R columns, fingerprint, dual sum
 
 // Shared-memory layout of one CTA of the resident kernel: the CTA's slice of a scenario's table
-// (uniform K: option k of slice job jj at slot k * m_pad + jj, so a warp reading one option of 32
-// consecutive jobs touches 32 consecutive words; general: CSR order with local job offsets), the
+// (uniform K: option k of slice job jj at slot k * m_pad + jj, the jobs of an option spread by an exclusive or where
+// several lanes read a job's options (ResSlice::slot); general: CSR order with local job offsets), the
 // per-warp and per-cluster demand partials, and the prices of the current round.
 struct ResLayout {
     int64_t vals, units, loff, wpart, cpart, prices, bytes;

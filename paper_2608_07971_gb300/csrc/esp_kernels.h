@@ -199,7 +199,8 @@ struct ResPlan {
     int32_t cs;
     int32_t k;          // > 0: every job has k options (interleaved layout); 0: CSR layout
     int32_t lanes;      // lanes per job (1, 2, 4 or 8)
-    int32_t m_pad;      // job slots of a slice: an odd multiple of 32 / lanes
+    int32_t m_pad;      // job slots of a slice: a power of two from 32 / lanes up to 16, or a multiple of 32
+    int32_t spread;     // the lanes whose options the exclusive or tells apart, less 1: as many as m_pad has room for
     int64_t n_cap;      // option slots of a slice (CSR layout)
 };
 

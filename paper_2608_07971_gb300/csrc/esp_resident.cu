@@ -128,6 +128,7 @@ struct ResSlice {
     int stride;             // distance between the columns of one option (m_pad, or 1)
     int K;                  // uniform layout: options per job
     int lanes, log2_jobs;   // lanes per job; log2 of the jobs a warp takes at once (32 / lanes)
+    int spread;             // ResPlan::spread
     int jloc0;              // scenario-local index of the slice's first job
     int64_t gj0;            // global index of the slice's first job
     int R;
@@ -136,11 +137,16 @@ struct ResSlice {
     float e2;                   // 2E, +inf in exact mode
     bool exact;
 
-    __device__ __forceinline__ int ucol0(int jj, int ob, int k) const
+    // Slot of job jj in the columns of option k (uniform layout). The lanes of one load read consecutive options of the
+    // same 32 / lanes jobs, R pitches apart, so a pitch alone cannot keep them in different banks for even R: this
+    // exclusive or does, for any R and without padding the slice beyond a multiple of 32 jobs.
+    __device__ __forceinline__ int slot(int jj, int k) const { return UNI ? jj ^ ((k & spread) << log2_jobs) : jj; }
+    // First unit word and value of option k of the job at slot js
+    __device__ __forceinline__ int ucol0(int js, int ob, int k) const
     {
-        return UNI ? k * R * stride + jj : (ob + k) * R;
+        return UNI ? k * R * stride + js : (ob + k) * R;
     }
-    __device__ __forceinline__ int vslot(int jj, int ob, int k) const { return UNI ? k * stride + jj : ob + k; }
+    __device__ __forceinline__ int vslot(int js, int ob, int k) const { return UNI ? k * stride + js : ob + k; }
 };
 
 template <int RT, bool UNI, bool SMALL>
@@ -197,8 +203,8 @@ __device__ __forceinline__ int res_resolve_lane(const ResSlice<RT, UNI> &sl, int
     int bi = kIdxNone;
     double bs = 0.0;
     for (int k = 0; k < K; ++k) {
-        const int bu = sl.ucol0(jj, ob, k);
-        const double v = sl.V[sl.vslot(jj, ob, k)];
+        const int js = sl.slot(jj, k), bu = sl.ucol0(js, ob, k);
+        const double v = sl.V[sl.vslot(js, ob, k)];
         bool dup;
         const float q = res_screen<RT, UNI, SMALL>(sl, bu, v, dup);
         if (dup || (!sl.exact && q > thr))
@@ -225,8 +231,8 @@ __device__ __forceinline__ int res_resolve_warp(const ResSlice<RT, UNI> &sl, int
     int bi = kIdxNone;
     double bs = 0.0;
     for (int k = lane; k < K; k += 32) {
-        const int bu = sl.ucol0(jj, ob, k);
-        const double v = sl.V[sl.vslot(jj, ob, k)];
+        const int js = sl.slot(jj, k), bu = sl.ucol0(js, ob, k);
+        const double v = sl.V[sl.vslot(js, ob, k)];
         bool dup;
         const float q = res_screen<RT, UNI, SMALL>(sl, bu, v, dup);
         if (dup || (!sl.exact && q > thr))
@@ -274,6 +280,7 @@ __device__ __forceinline__ void res_evaluate(const DevState &st, const ResSlice<
         }
         float m1 = INFINITY, m2 = INFINITY;
         int i1 = 0;
+        const int js = sl.slot(jj, sub);   // every option of the lane is sub modulo lanes
         // four options at a time, so that their loads are in flight together (one after the other, an
         // option took 119 cycles)
         for (int k0 = sub; k0 < K; k0 += 4 * sl.lanes) {
@@ -282,7 +289,7 @@ __device__ __forceinline__ void res_evaluate(const DevState &st, const ResSlice<
             for (int i = 0; i < 4; ++i) {
                 const int k = k0 + i * sl.lanes, kk = k < K ? k : k0;
                 bool dup;
-                q[i] = res_screen<RT, UNI, SMALL>(sl, sl.ucol0(jj, ob, kk), sl.V[sl.vslot(jj, ob, kk)], dup);
+                q[i] = res_screen<RT, UNI, SMALL>(sl, sl.ucol0(js, ob, kk), sl.V[sl.vslot(js, ob, kk)], dup);
                 q[i] = (dup || k >= K) ? INFINITY : q[i];
             }
 #pragma unroll
@@ -333,7 +340,7 @@ __device__ __forceinline__ void res_evaluate(const DevState &st, const ResSlice<
         }
         if (!act || sub != 0)
             continue;
-        const int bw = sl.ucol0(jj, ob, w);
+        const int jw = sl.slot(jj, w), bw = sl.ucol0(jw, ob, w);
 #pragma unroll
         for (int r = 0; r < ResCols<RT>::N; ++r) {
             if (RT == 0 && r >= R)
@@ -346,7 +353,7 @@ __device__ __forceinline__ void res_evaluate(const DevState &st, const ResSlice<
         if (want_hash)
             acc.hash += splitmix64_mix(((uint64_t)(uint32_t)(sl.jloc0 + jj) << 32) | (uint32_t)w);
         if (FINAL || want_min) {
-            const double vw = sl.V[sl.vslot(jj, ob, w)];
+            const double vw = sl.V[sl.vslot(jw, ob, w)];
             if (!have_s)
                 s_w = res_exact<RT, UNI, SMALL>(sl, bw, vw);
             if (FINAL) {
@@ -440,18 +447,20 @@ __global__ void __launch_bounds__(kResThreads, ESP_RES_MIN_CTAS) k_resident(DevT
     const int n = (int)(t.job_off[gj0 + m] - o0);
     {
         const int32_t *gu = t.units + o0 * R;
+        const int log2_jobs = 5 - (__ffs(rp.lanes) - 1);
+        auto column = [&](int o) { return (o / rp.k) ^ (((o % rp.k) & rp.spread) << log2_jobs); };   // ResSlice::slot
         for (int i = threadIdx.x; i < n * R; i += kResThreads) {
             const int o = i / R, r = i - o * R;
             const uint32_t w = stored_unit<SMALL>(__ldg(gu + i));
             if (UNI)
-                Us[((o % rp.k) * R + r) * rp.m_pad + o / rp.k] = w;
+                Us[((o % rp.k) * R + r) * rp.m_pad + column(o)] = w;
             else
                 Us[i] = w;
         }
         for (int o = threadIdx.x; o < n; o += kResThreads) {
             const double v = __ldg(t.values + o0 + o);
             if (UNI)
-                Vs[(o % rp.k) * rp.m_pad + o / rp.k] = v;
+                Vs[(o % rp.k) * rp.m_pad + column(o)] = v;
             else
                 Vs[o] = v;
         }
@@ -491,6 +500,7 @@ __global__ void __launch_bounds__(kResThreads, ESP_RES_MIN_CTAS) k_resident(DevT
     sl.K = rp.k;
     sl.lanes = rp.lanes;
     sl.log2_jobs = 5 - (__ffs(rp.lanes) - 1);
+    sl.spread = rp.spread;
     sl.jloc0 = j0;
     sl.gj0 = gj0;
     sl.R = R;
