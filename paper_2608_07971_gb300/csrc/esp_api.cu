@@ -1107,39 +1107,14 @@ esp_status plan_resident_options(esp_ctx *ctx)
                 at += shapes[i].cuts.size();
             }
             ESP_CUDA(cudaStreamSynchronize(ctx->stream));
-            // automatic size: most scenario-rounds per microsecond under a simple cost model, fitted to
-            // rounds measured on GB300: 2.0 us (prices and barriers), 0.3 + 0.02 cs us for the exchange in a
-            // cluster, and 0.09 us per option a lane screens one after the other (a 2048-job cluster
-            // of 16 options per job: 3.60 us with 16 CTAs, 4.0 with 8; 500 jobs of 8: 3.07, 2.77, 2.66
-            // and 2.77 with 1, 2, 4 and 16; tiny cluster: 2.16 with 1, 2.4 with 16). Slices in CSR order
-            // and widths without an instantiation cost about twice that per option, each (seven ragged
-            // 1777-job clusters of 5 columns: 19.5 us). Ties keep the smaller cluster
-            const double per_option = 0.09 * (ctx->pc.min_k == ctx->pc.max_k ? 1.0 : 2.0) *
-                                      (R == 4 || R == 6 || R == 8 ? 1.0 : 2.0);
-            auto round_us = [&](const esp_ctx::ResOption &o) {
-                const double serial = std::max((double)o.n_max / (kResWarps * 32), (double)ctx->pc.max_k / o.plan.lanes);
-                return 2.0 + (o.plan.cs == 1 ? 0.0 : 0.3 + 0.02 * o.plan.cs) + per_option * serial;
-            };
-            double best = -1.0;
-            for (size_t i = 0; i < ctx->res.size(); ++i) {
-                const double rate = (double)std::min<int64_t>(S, ctx->res[i].clusters) / round_us(ctx->res[i]);
-                if (rate > best * 1.02) {
-                    best = rate;
-                    ctx->res_auto = (int)i;
-                }
-            }
-            // the automatic choice runs only where it is predicted faster than streaming: S scenarios take
-            // ceil(S / clusters) waves of clusters; a streaming round takes about 12 us plus its table (half of
-            // it, packed) at 6 TB/s, and 6.5 us (launch and update latency) where it is a few steps
-            // the pitch, a power of two up to 16 or a multiple of 32; the kernel's exclusive or spreads the job slots of
-            // the lanes that read one job's options over it
-            if (ctx->res_auto >= 0) {
-                const esp_ctx::ResOption &o = ctx->res[ctx->res_auto];
-                const double waves = std::ceil((double)S / (double)o.clusters);
-                const double bytes = (double)ctx->n_opt * (4.0 * R + 8.0);
-                const double stream_us = bytes < 1e5 ? 6.5 : 12.0 + bytes / 12e6;
-                ctx->res_slower = waves * round_us(o) > stream_us;
-            }
+            // automatic size: the shortest predicted round; where streaming is predicted shorter, that runs instead
+            std::vector<ResSize> sizes;
+            for (size_t i = 0; i < ctx->res.size(); ++i)
+                sizes.push_back({ctx->res[i].plan.cs, ctx->res[i].plan.lanes, shapes[i].m_max, ctx->res[i].clusters, ctx->res[i].n_max});
+            ctx->res_auto = resident_choice(S, R, ctx->pc.min_k, ctx->pc.max_k, ctx->sm_count, sizes);
+            if (ctx->res_auto >= 0)
+                ctx->res_slower = resident_round_us(S, R, ctx->pc.min_k, ctx->pc.max_k, ctx->sm_count, sizes[(size_t)ctx->res_auto]) >
+                                  streaming_round_us(ctx->n_opt, R, ctx->packed ? ctx->pack.fmt.nw : 0, ctx->sm_count);
         }
     }
 
