@@ -93,7 +93,6 @@ struct ResShape {
 // Fills out for cs CTAs per scenario. Returns false on inconsistent offsets.
 bool plan_resident(const int64_t *job_off, int32_t S, int32_t J, int32_t cs, ResShape &out);
 
-}  // namespace esp
 // One cluster size that fits: its lanes per job, largest slice (jobs, options) and co-resident clusters.
 struct ResSize {
     int32_t cs, lanes, m_max, clusters;
@@ -108,3 +107,4 @@ double streaming_round_us(int64_t n_opt, int32_t R, int32_t words, int32_t sms);
 // The size with the shortest predicted round (-1: none in sizes); ties keep the smaller cluster.
 int resident_choice(int32_t S, int32_t R, int64_t min_k, int64_t max_k, int32_t sms, const std::vector<ResSize> &sizes);
 
+}  // namespace esp
