@@ -23,9 +23,9 @@
 // per round where the staged pass took 77.4; of the 29, 19 are the screen (63 MB, which L2 holds), the rest the
 // chain of the slowest ambiguous job and of the update of 134 prices.
 //
-// The winner's units come from the words in the slot. Values in fp64 and int32 units are read from
-// the table itself, only to rescore the survivors of ambiguous jobs and for the outputs of the final
-// pass.
+// The winner's units come from the words in the slot, and so do those of options that are scored exactly (the
+// survivors of ambiguous jobs, every option in exact mode, the winners of the final pass): of the table itself only
+// their fp64 values are read.
 
 #include <algorithm>
 #include <cmath>
@@ -57,14 +57,15 @@ constexpr int pack_min_ctas(int nw, bool grouped = false)
     return grouped ? 4 : nw <= 3 ? ESP_PACK_CTAS : nw == 4 ? 5 : 4;
 }
 
-// Shared memory of a warp: the slots, then their barriers.
+// Shared memory of a warp: the slots, their barriers, then the fp64 prices of the columns that every option shares.
+constexpr int kPackPriceBytes = kMaxR * 8;
 __host__ __device__ constexpr int pack_slot_bytes(int nw)
 {
     return (nw + 1) * kPackStepVecs * 16;
 }
 __host__ __device__ constexpr int pack_warp_bytes(int nw)
 {
-    return kPackSlots * pack_slot_bytes(nw) + 16;
+    return kPackSlots * pack_slot_bytes(nw) + 16 + kPackPriceBytes;
 }
 
 __device__ __forceinline__ unsigned long long pack2(float lo, float hi)
@@ -103,7 +104,8 @@ struct Ctx {
     uint32_t wins;                  // upper bound of the winners in them
     unsigned long long hash;
     const double *p64;              // fp64 prices of the scenario
-    unsigned char *groups;          // grouped tables: shared memory, the two fp32 prices of each group slot
+    unsigned char *groups;          // shared memory behind the prices; grouped tables: two fp32 prices of each slot
+    bool have64;                    // the fp64 prices below `groups` are this scenario's (fetch_prices)
     float e2;                       // 2E, +inf: exact evaluation
     bool exact, skip;
     int s;                          // scenario, -1: none
@@ -202,37 +204,59 @@ __device__ __forceinline__ void add_option(const Pass &ps, Ctx<NW> &c, const uin
         add_group(ps, c, w[NW * plane * 4], w[(f.g_word + 1) * plane * 4]);
 }
 
-// The exact score of option o of the pass table (the chain of Eq. esp_score in column order).
-template <bool G>
-__device__ __forceinline__ double exact_option(const DevTable &t, const double *p64, int64_t o)
+// The scenario's fp64 prices into the warp's shared memory, once per scenario (the whole warp calls it). A pass of one
+// round fetches them with the scenario's other prices; the persistent pass, which comes to a scenario for each tile,
+// only before something is scored exactly.
+template <int NW, bool G>
+__device__ __forceinline__ void fetch_prices(const Pass &ps, Ctx<NW> &c)
 {
-    const int R = t.R, rg = t.r_global;
-    const int32_t *u = t.units + o * R;
-    double s = -__ldg(t.values + o);
-    if (!G) {
-        for (int r = 0; r < R; ++r) {
-            const int32_t x = __ldg(u + r);
-            // prices through L2: a persistent pass sees them change between rounds
-            s = __fma_rn(__ldcg(p64 + r), __int2double_rn(r == 0 ? (x & 0x7fffffff) : x), s);
-        }
-        return s;
+    if (c.have64)
+        return;
+    c.have64 = true;
+    if (ps.lane < (G ? ps.t.r_global : ps.t.R))   // through L2: a persistent pass sees them change between rounds
+        reinterpret_cast<double *>(c.groups - kPackPriceBytes)[ps.lane] = __ldcg(c.p64 + ps.lane);
+    __syncwarp();
+}
+
+// A whole number below 2^23 in fp64, by way of its fp32 bits: integer operations instead of a conversion, which would
+// take as long a turn of the fp64 unit as the multiply-add that the number is for.
+__device__ __forceinline__ double whole_f64(uint32_t u)
+{
+    const uint32_t b = __float_as_uint(__uint_as_float(0x4b000000u | u) - 8388608.0f);
+    return __hiloint2double(b != 0u ? (int)((b >> 3) + (896u << 20)) : 0, (int)(b << 29));   // exponent bias 127 -> 1023
+}
+
+// The exact score (the chain of Eq. esp_score in column order) of the option of value v whose words are at w (plane
+// 0). The units are whole numbers in the words, so only v is read from the table. (With units and prices read from the
+// table and L2 column by column, exact mode took 254 us per round on 256 scenarios of 2048 x 16, R = 6, where the staged
+// pass took 204 and this takes 130; the slowest ambiguous job is the end of every round, so a 2048-job cluster went
+// from 10.0 to 8.7 us too, the what-if batch from 85 to 81 and the heavy-tailed table from 158 to 153.)
+template <int NW, bool G>
+__device__ __forceinline__ double exact_words(const Pass &ps, const Ctx<NW> &c, const uint32_t *w, int plane, double v)
+{
+    const PackFormat &f = ps.pk.fmt;
+    const int R = ps.t.R, rg = G ? ps.t.r_global : R;
+    const double *p = reinterpret_cast<const double *>(c.groups - kPackPriceBytes);
+    double s = -v;
+    auto unit = [&](int r) {
+        const int at = f.field[r], k = at >> 1;
+        const uint32_t x = w[(k + 1) * plane * 4];
+        return whole_f64((at & 1) ? x >> f.shift[k] : x & f.mask[k]);
+    };
+    double pg[2] = {0.0, 0.0};
+    if (G) {
+        const double *own = c.p64 + rg + (R - rg) * (int)pack_slot_group((w[(f.g_word + 1) * plane * 4] >> f.g_shift) & f.g_mask);
+        pg[0] = __ldcg(own);
+        if (R - rg == 2)
+            pg[1] = __ldcg(own + 1);
     }
-    // four columns' units and prices on their way together (placement table of 4096 jobs: 38.7 -> 37.0 us per
-    // round; without groups the plain loop is the faster one, 10.3 against 10.7 on a 2048-job cluster)
-    const int own = (R - rg) * (int)__ldg(t.group + o);
-    for (int r0 = 0; r0 < R; r0 += 4) {
-        double p[4];
-        int32_t x[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int r = r0 + i < R ? r0 + i : r0;
-            x[i] = __ldg(u + r);
-            p[i] = __ldcg(p64 + (r >= rg ? r + own : r));
-        }
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-            if (r0 + i < R)
-                s = __fma_rn(p[i], __int2double_rn(x[i] & 0x7fffffff), s);
+#pragma unroll 4
+    for (int r = 0; r < rg; ++r)
+        s = __fma_rn(p[r], unit(r), s);
+    if (G) {
+        s = __fma_rn(pg[0], unit(rg), s);
+        if (R - rg == 2)
+            s = __fma_rn(pg[1], unit(rg + 1), s);
     }
     return s;
 }
@@ -242,16 +266,27 @@ struct Exact {
     int idx;
 };
 
-// The lexicographic minimum of (s, index) over the options first + i, i in the bits of `mask`, in fp64;
-// their indices are loc + i. (Ambiguous jobs only; out of line it made the row loops spill around the call.)
-template <bool G>
-__device__ __forceinline__ Exact rescore(const DevTable &t, const double *p64, int64_t first, uint32_t mask, int loc)
+// The value of the first option in `mask` (rescore's first one; loaded ahead of the prices, so that one trip to memory
+// covers both).
+__device__ __forceinline__ double first_value(const Pass &ps, int64_t first, uint32_t mask)
+{
+    return mask != 0u ? __ldg(ps.t.values + first + (__ffs((int)mask) - 1)) : 0.0;
+}
+
+// The lexicographic minimum of (s, index) in fp64 over the options first + i, i in the bits of `mask`: the words of
+// options 0 .. 3 start at wa, those of 4 .. 7 at wb; v: the first one's value. Their indices are loc + i.
+// (Ambiguous jobs only; out of line it made the row loops spill around the call.)
+template <int NW, bool G>
+__device__ __forceinline__ Exact rescore(const Pass &ps, const Ctx<NW> &c, const uint32_t *wa, const uint32_t *wb, int plane,
+                                         int64_t first, uint32_t mask, int loc, double v)
 {
     Exact x{0x7fffffffffffffffLL, kIdxNone};
     while (mask != 0u) {
         const int i = __ffs((int)mask) - 1;
         mask &= mask - 1;
-        const long long k = order_key(exact_option<G>(t, p64, first + i));
+        const double next = G ? first_value(ps, first, mask) : 0.0;   // (ungrouped: the registers it takes cost more)
+        const long long k = order_key(exact_words<NW, G>(ps, c, (i < 4 ? wa : wb) + (i & 3), plane, v));
+        v = G ? next : first_value(ps, first, mask);
         if (k < x.key) {   // increasing index: the first of equal scores stays
             x.key = k;
             x.idx = loc + i;
@@ -291,19 +326,21 @@ __device__ __forceinline__ int64_t first_option(const Pass &ps, int i)
     return ps.pk.all_k > 0 ? (int64_t)i * ps.pk.all_k : __ldg(ps.pk.opt0 + i);
 }
 
-// Outputs of a winner beyond its demand: its packed job, local index and, when known, exact score.
+// Outputs of a winner beyond its demand: its packed job i, local index, value (read where it is wanted), words and,
+// when known, exact score.
 template <int NW, bool G>
-__device__ __forceinline__ void extras(const Pass &ps, Ctx<NW> &c, int i, int local, bool have_s, long long key)
+__device__ __forceinline__ void extras(const Pass &ps, Ctx<NW> &c, int i, int local, double v, const uint32_t *w, int plane,
+                                       bool have_s, long long key)
 {
     const int64_t job = ps.pk.job ? __ldg(ps.pk.job + i) : i;
     if (ps.want_hash)
         c.hash += splitmix64_mix(((uint64_t)(uint32_t)(job - (int64_t)c.s * ps.t.J) << 32) | (uint32_t)local);
     if (ps.kind == PASS_FINAL) {
         ps.st.sel[job] = local;
-        ps.st.job_val[job] = __ldg(ps.t.values + first_option(ps, i) + local);
+        ps.st.job_val[job] = v;
     }
     if (ps.want_min)
-        ps.st.job_min[job] = have_s ? key_value(key) : exact_option<G>(ps.t, c.p64, first_option(ps, i) + local);
+        ps.st.job_min[job] = have_s ? key_value(key) : exact_words<NW, G>(ps, c, w, plane, v);
 }
 
 // Adds the lane's demand to the scenario's totals: every sum across the warp by two hardware reductions
@@ -586,7 +623,7 @@ __device__ __forceinline__ void leave(const Pass &ps, Ctx<NW> &c)
 }
 
 // Prices, bound and state of scenario s (through L2: another warp of this launch may have written them).
-template <int NW, bool G>
+template <int NW, bool G, bool PERSIST>
 __device__ __forceinline__ void enter(const Pass &ps, Ctx<NW> &c, int s)
 {
     const DevState &st = ps.st;
@@ -596,6 +633,11 @@ __device__ __forceinline__ void enter(const Pass &ps, Ctx<NW> &c, int s)
     c.tiles = 0;
     const int frozen = __ldcg(st.frozen + s);
     const float e = __ldcg(st.ebound + s);
+    c.p64 = st.p64 + sp;
+    c.have64 = !PERSIST;
+    double *const prices = reinterpret_cast<double *>(c.groups - kPackPriceBytes);
+    const bool mine = !PERSIST && ps.lane < (G ? ps.t.r_global : ps.t.R);
+    const double p64 = mine ? __ldcg(c.p64 + ps.lane) : 0.0;
 #pragma unroll
     for (int k = 0; k < (G ? NW - 1 : NW); ++k) {
         const float pl = f.col_lo[k] >= 0 ? __ldcg(st.p32 + sp + f.col_lo[k]) : 0.0f;
@@ -615,7 +657,9 @@ __device__ __forceinline__ void enter(const Pass &ps, Ctx<NW> &c, int s)
     c.skip = ps.kind == PASS_ROUND && frozen != 0;
     c.exact = !(e < INFINITY);
     c.e2 = c.exact ? INFINITY : 2.0f * e;
-    c.p64 = st.p64 + sp;
+    if (mine)
+        prices[ps.lane] = p64;
+    __syncwarp();
 }
 
 // A step of whole jobs of 3 .. 256 options: each job has 2^code lanes, its lane sub the options
@@ -665,12 +709,17 @@ __device__ __forceinline__ void step_jobs(const Pass &ps, Ctx<NW> &c, const uint
     if (__any_sync(FULL, amb)) {
         const int loc = (ps.lane & ((1 << code) - 1)) << per;
         Exact x{0x7fffffffffffffffLL, kIdxNone};
+        uint32_t sv = 0u;
+        int64_t first = 0;
         if (amb) {
-            const uint32_t sv = (has_a ? survivors(slot[ia], qa, c.exact, thr) : 0u) |
-                                (has_b ? survivors(slot[ib], qb, c.exact, thr) << 4 : 0u);
-            if (sv != 0u)
-                x = rescore<G>(ps.t, c.p64, first_option(ps, job0 + jl) + loc, sv, loc);
+            sv = (has_a ? survivors(slot[ia], qa, c.exact, thr) : 0u) | (has_b ? survivors(slot[ib], qb, c.exact, thr) << 4 : 0u);
+            first = first_option(ps, job0 + jl) + loc;
         }
+        const double v = first_value(ps, first, sv);
+        fetch_prices<NW, G>(ps, c);
+        if (sv != 0u)
+            x = rescore<NW, G>(ps, c, reinterpret_cast<const uint32_t *>(slot + ia), reinterpret_cast<const uint32_t *>(slot + ib), V,
+                               first, sv, loc, v);
         x = group_min(x, 1 << code);
         if (amb && x.idx >= loc && x.idx < loc + (1 << per)) {
             mine = have_s = true;
@@ -680,46 +729,71 @@ __device__ __forceinline__ void step_jobs(const Pass &ps, Ctx<NW> &c, const uint
         }
     }
     if (mine) {
-        add_option<NW, G>(ps, c, reinterpret_cast<const uint32_t *>(slot + (o < 4 ? ia : ib)) + (o & 3), V);
-        if (!PLAIN)
-            extras<NW, G>(ps, c, job0 + jl, ((ps.lane & ((1 << code) - 1)) << per) + o, have_s, key);
+        const uint32_t *w = reinterpret_cast<const uint32_t *>(slot + (o < 4 ? ia : ib)) + (o & 3);
+        add_option<NW, G>(ps, c, w, V);
+        if (!PLAIN) {
+            const int local = ((ps.lane & ((1 << code) - 1)) << per) + o;
+            const double v = ps.want_min ? __ldg(ps.t.values + first_option(ps, job0 + jl) + local) : 0.0;
+            extras<NW, G>(ps, c, job0 + jl, local, v, w, V, have_s, key);
+        }
     }
 }
 
 // Four consecutive options of a tile whose jobs have one or two: jobs job0 + j0 .., `n` of them left in
-// it. v: the vector.
+// it (none or less: the lane has no job). v: the vector. The whole warp calls it.
 template <int NW, bool G, bool PLAIN>
 __device__ __forceinline__ void step_tiny(const Pass &ps, Ctx<NW> &c, const uint4 *v, int V, int K, int job0, int j0, int n)
 {
-    float q[4];
-    screen4<NW, G>(v, V, ps.pk.fmt, c, q);
     const uint32_t *w = reinterpret_cast<const uint32_t *>(v);
+    float q[4], thr[2] = {INFINITY, INFINITY};
+    uint32_t amb = 0u, win = 0u;   // per pair of options: ambiguous; the second one wins
+    if (K == 2) {
+        screen4<NW, G>(v, V, ps.pk.fmt, c, q);
 #pragma unroll
-    for (int h = 0; h < 4; ++h) {
-        if (K == 2 && (h & 1))
+        for (int p = 0; p < 2; ++p) {
+            const float qa = q[2 * p], qb = q[2 * p + 1];
+            thr[p] = __fadd_ru(fminf(qa, qb), c.e2);
+            win |= qb < qa ? 1u << p : 0u;
+            amb |= p < n && (c.exact || !(fmaxf(qa, qb) > thr[p])) ? 1u << p : 0u;
+        }
+        if (__any_sync(FULL, amb != 0u))
+            fetch_prices<NW, G>(ps, c);
+    }
+    // the jobs' values on their way together (one after the other, a trip to memory each, made the final pass of a
+    // table with many such jobs several times as long as a round)
+    int64_t first[4] = {0, 0, 0, 0};
+    double val[4] = {0.0, 0.0, 0.0, 0.0};
+    if (!PLAIN && ps.want_min) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            if (j < n && j * K < 4)
+                first[j] = first_option(ps, job0 + j0 + j);
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            if (j < n && j * K < 4 && !((amb >> j) & 1u))
+                val[j] = __ldg(ps.t.values + first[j] + ((win >> j) & 1u));
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        if (j >= n || j * K >= 4)
             continue;
-        const int jl = K == 2 ? h >> 1 : h;
-        if (jl >= n)
-            continue;
-        int o = h;
+        int o = j * K + (int)((win >> j) & 1u);
         bool have_s = false;
         long long key = 0;
-        if (K == 2) {
-            const float qa = q[h], qb = q[(h + 1) & 3];
-            const float thr = __fadd_ru(fminf(qa, qb), c.e2);
-            o = qb < qa ? h + 1 : h;
-            if (c.exact || !(fmaxf(qa, qb) > thr)) {   // ambiguous
-                const uint32_t sv = (survivors(v[0], q, c.exact, thr) >> h) & 3u;
-                const Exact x = rescore<G>(ps.t, c.p64, first_option(ps, job0 + j0 + jl), sv, h);
-                o = x.idx;
-                key = x.key;
-                have_s = true;
-                ++c.resolved;
-            }
+        if (j < 2 && ((amb >> j) & 1u)) {
+            const uint32_t sv = (survivors(v[0], q, c.exact, thr[j]) >> (2 * j)) & 3u;
+            const int64_t f = first_option(ps, job0 + j0 + j);
+            const Exact x = rescore<NW, G>(ps, c, w + 2 * j, w, V, f, sv, 2 * j, first_value(ps, f, sv));
+            o = x.idx;
+            key = x.key;
+            have_s = true;
+            ++c.resolved;
+            if (!PLAIN && ps.want_min)
+                val[j] = __ldg(ps.t.values + first[j] + o - 2 * j);
         }
         add_option<NW, G>(ps, c, w + o, V);
         if (!PLAIN)
-            extras<NW, G>(ps, c, job0 + j0 + jl, o - h, have_s, key);
+            extras<NW, G>(ps, c, job0 + j0 + j, o - j * K, val[j], w + o, V, have_s, key);
     }
 }
 
@@ -769,7 +843,9 @@ __device__ __forceinline__ Exact rescan_large(const Pass &ps, const Ctx<NW> &c, 
         const uint4 *v = large_vec<NW>(base, sh, g);
         float q[4];
         screen4<NW, G>(v, sh.v, ps.pk.fmt, c, q);
-        const Exact y = rescore<G>(ps.t, c.p64, opt0 + 4 * g, survivors(v[0], q, c.exact, thr), 4 * g);
+        const uint32_t *w = reinterpret_cast<const uint32_t *>(v);
+        const uint32_t sv = survivors(v[0], q, c.exact, thr);
+        const Exact y = rescore<NW, G>(ps, c, w, w, sh.v, opt0 + 4 * g, sv, 4 * g, first_value(ps, opt0 + 4 * g, sv));
         if (y.key < x.key)
             x = y;
     }
@@ -789,7 +865,9 @@ __device__ __forceinline__ void rescan_lane(const Pass &ps, const Ctx<NW> &c, co
         const uint4 *v = large_vec<NW>(base, sh, g);
         float q[4];
         screen4<NW, G>(v, sh.v, ps.pk.fmt, c, q);
-        const Exact y = rescore<G>(ps.t, c.p64, opt0 + 4 * g, survivors(v[0], q, c.exact, thr), 4 * g);
+        const uint32_t *w = reinterpret_cast<const uint32_t *>(v);
+        const uint32_t sv = survivors(v[0], q, c.exact, thr);
+        const Exact y = rescore<NW, G>(ps, c, w, w, sh.v, opt0 + 4 * g, sv, 4 * g, first_value(ps, opt0 + 4 * g, sv));
         if (y.key < x.key || (y.key == x.key && y.idx < x.idx))
             x = y;
     }
@@ -809,17 +887,25 @@ __device__ __forceinline__ void close_large(const Pass &ps, Ctx<NW> &c, const ui
     bool mine = first, have_s = false;
     int win = b.idx;
     long long key = 0;
+    // words of option o of the job
+    auto words = [&](int o) { return reinterpret_cast<const uint32_t *>(large_vec<NW>(base, sh, o >> 2)) + (o & 3); };
     if (c.exact || !(m2 > thr)) {
         const int64_t opt0 = first_option(ps, job0 + jl);
         Exact x{0x7fffffffffffffffLL, kIdxNone};
+        const double own_value = first_value(ps, opt0 + b.idx, b.m1 <= thr && !c.exact ? 1u : 0u);
+        auto own_best = [&]() {
+            const uint32_t *w = words(b.idx);
+            x = rescore<NW, G>(ps, c, w, w, sh.v, opt0 + b.idx, 1u, b.idx, own_value);
+        };
+        fetch_prices<NW, G>(ps, c);
         if (!c.exact && !__any_sync(FULL, b.m2 <= thr)) {   // every lane's own best at most
             if (b.m1 <= thr)
-                x = rescore<G>(ps.t, c.p64, opt0 + b.idx, 1u, b.idx);
+                own_best();
         } else {
             const uint32_t several = __ballot_sync(FULL, b.m2 <= thr);   // lanes with more than their own best
             if (!c.exact && __popc(several) <= sh.nch) {
                 if (b.m1 <= thr && !(b.m2 <= thr))
-                    x = rescore<G>(ps.t, c.p64, opt0 + b.idx, 1u, b.idx);
+                    own_best();
                 for (uint32_t l = several; l != 0u; l &= l - 1u)
                     rescan_lane<NW, G>(ps, c, base, sh, opt0, thr, __ffs((int)l) - 1, x);
             } else {
@@ -836,14 +922,16 @@ __device__ __forceinline__ void close_large(const Pass &ps, Ctx<NW> &c, const ui
             ++c.resolved;
     }
     if (mine) {
-        const uint32_t *w = reinterpret_cast<const uint32_t *>(large_vec<NW>(base, sh, win >> 2)) + (win & 3);
+        const uint32_t *w = words(win);
 #pragma unroll
         for (int i = 0; i < NW; ++i)
             b.x[i] = __ldg(w + (i + 1) * sh.v * 4);
         if (G)
             b.slot = __ldg(w + (ps.pk.fmt.g_word + 1) * sh.v * 4);
-        if (!PLAIN)
-            extras<NW, G>(ps, c, job0 + jl, win, have_s, key);
+        if (!PLAIN) {
+            const double v = ps.want_min ? __ldg(ps.t.values + first_option(ps, job0 + jl) + win) : 0.0;
+            extras<NW, G>(ps, c, job0 + jl, win, v, w, sh.v, have_s, key);
+        }
     }
     b.m1 = b.m2 = INFINITY;
     b.idx = kIdxNone;
@@ -935,6 +1023,7 @@ __device__ __forceinline__ void run_warp(const DevTable &t, const DevState &st, 
         asm volatile("griddepcontrol.wait;" ::: "memory");
     Ctx<NW> c;
     reset(c);
+    c.have64 = !PERSIST;
     c.groups = smem + pack_warp_bytes(NW);
     int at = 0;                  // slot of the step to be screened
     uint32_t phases = 0;         // parity of each slot's next completion
@@ -967,10 +1056,10 @@ __device__ __forceinline__ void run_warp(const DevTable &t, const DevState &st, 
                 break;
             }
             ps.round = rt;
-            enter<NW, G>(ps, c, (int)T.scenario);
+            enter<NW, G, true>(ps, c, (int)T.scenario);
         } else if ((int)T.scenario != c.s) {
             leave<NW, G, false>(ps, c);
-            enter<NW, G>(ps, c, (int)T.scenario);
+            enter<NW, G, false>(ps, c, (int)T.scenario);
         }
         if (__any_sync(FULL, (gave_up & DEV_ERR_TIMEOUT) != 0u)) {
             ok = false;
@@ -1042,8 +1131,7 @@ __device__ __forceinline__ void run_warp(const DevTable &t, const DevState &st, 
 #pragma unroll 1
                     for (int h = 0; h < 2; ++h) {
                         const int o0 = 4 * (64 * st_i + 32 * h + lane), j0 = o0 / sh.m;   // m = 1 or 2
-                        if (j0 < n_job)
-                            step_tiny<NW, G, PLAIN>(ps, c, slot + 32 * h + lane, 64, sh.m, job0, j0, n_job - j0);
+                        step_tiny<NW, G, PLAIN>(ps, c, slot + 32 * h + lane, 64, sh.m, job0, j0, n_job - j0);
                     }
                 }
                 release();

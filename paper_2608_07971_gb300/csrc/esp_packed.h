@@ -8,8 +8,8 @@
 //
 // Why: the pass over a table larger than L2 streams it every round, and at 4R + 8 bytes per option it
 // ran at 0.91-0.995 of the copy bandwidth. R = 6 columns of the cluster workloads hold 86 unit bits: three
-// words, 16 bytes per option with -v32 instead of 32. The fp64 values and the int32 units stay in
-// the table for the exact rescoring of ambiguous jobs and for the final pass.
+// words, 16 bytes per option with -v32 instead of 32. The fp64 values stay in the table for exact scores
+// (the units of which come from the words) and for the final pass.
 #pragma once
 
 #include <cstdint>
@@ -28,6 +28,7 @@ struct PackFormat {
     // with f = funnelshift_r(w, magic[k], shift[k]): the bits of the float 2^23 + high field
     uint32_t magic[kPackMaxWords];
     int8_t col_lo[kPackMaxWords], col_hi[kPackMaxWords];   // table column of each field, -1: none
+    int8_t field[kMaxR];                 // of each column: 2 x its word, + 1 for the high field
     // tables with a group column: the last word holds the columns that are priced per group; word g_word
     // also holds, from bit g_shift on, the option's group slot (pack_slot)
     int32_t g_word, g_shift;

@@ -358,11 +358,13 @@ bool pack_format(const int32_t *umax, int32_t R, PackFormat &out, int32_t r_glob
         taken[k] = lo.bits;
         out.mask[k] = (1u << lo.bits) - 1u;
         out.col_lo[k] = (int8_t)lo.col;
+        out.field[lo.col] = (int8_t)(2 * k);
         if (hi) {
             high[k] = hi->bits;
             out.shift[k] = 32 - hi->bits;
             out.magic[k] = 0x4b000000u >> hi->bits;   // exact: its low 24 bits are zero
             out.col_hi[k] = (int8_t)hi->col;
+            out.field[hi->col] = (int8_t)(2 * k + 1);
         }
     };
     for (int32_t i = 0; i < flat; ++i) {
