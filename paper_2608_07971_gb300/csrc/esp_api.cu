@@ -548,7 +548,7 @@ esp_status load_packed(esp_ctx *ctx, const PackFormat &fmt)
 {
     const PackPlan &p = ctx->pc.pack;
     PackTile *tiles = nullptr;
-    int32_t *jb = nullptr, *job = nullptr, *wb = nullptr, *scen_tiles = nullptr;
+    int32_t *jb = nullptr, *job = nullptr, *wb = nullptr, *fb = nullptr, *scen_tiles = nullptr;
     esp_status st = ESP_OK;
     auto up = [&](auto **ptr, const auto &src) {   // the host arrays stay in the plan cache
         if (st == ESP_OK)
@@ -562,6 +562,8 @@ esp_status load_packed(esp_ctx *ctx, const PackFormat &fmt)
     if (!p.job.empty())
         up(&job, p.job);
     up(&wb, p.warp_begin);
+    if (p.n_warps != (int32_t)p.tiles.size())   // else warp w has tile w
+        up(&fb, p.final_begin);
     up(&scen_tiles, p.scen_tiles);
     if (st == ESP_OK)
         st = dev_alloc(ctx, &ctx->pk_data, (size_t)p.vecs * (size_t)(fmt.nw + 1), 64, false);
@@ -576,6 +578,7 @@ esp_status load_packed(esp_ctx *ctx, const PackFormat &fmt)
     d.job_begin = jb;
     d.job = job;
     d.warp_begin = wb;
+    d.final_begin = fb;
     d.scen_tiles = scen_tiles;
     d.n_tiles = (int32_t)p.tiles.size();
     d.n_warps = p.n_warps;
@@ -1005,7 +1008,8 @@ bool state_ready(const esp_ctx *c)
                c->place.node_type && c->place.D && c->place.cfg_dup && c->place.warp_job && c->place.n_warps > 0 &&
                c->scen_warps;
     if (c->packed)
-        return c->pack.data && (c->pack.all_k > 0 || c->pack.opt0) && c->pack.tiles && c->pack.job_begin && c->pack.warp_begin && c->pack.scen_tiles && c->units &&
+        return c->pack.data && (c->pack.all_k > 0 || c->pack.opt0) && c->pack.tiles && c->pack.job_begin && c->pack.warp_begin &&
+               (c->pack.final_begin || c->pack.n_warps == c->pack.n_tiles) && c->pack.scen_tiles && c->units &&
                c->values && c->off;
     return c->grid == 0 || (c->scen_warps && c->tiles && c->warp_begin && c->units && c->values && c->off);
 }

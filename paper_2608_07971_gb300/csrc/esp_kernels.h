@@ -89,6 +89,7 @@ struct DevPack {
     const int32_t *job;          // table job of each job in the packed order; nullptr: the same
     int64_t *opt0;               // first option of each job in the packed order (k_pack); nullptr when all_k > 0
     const int32_t *warp_begin;   // n_warps + 1: the round pass's tile ranges
+    const int32_t *final_begin;  // n_warps + 1: the final pass's (nullptr where every warp has one tile)
     const int32_t *scen_tiles;   // S: tiles of each scenario (arrivals count tiles)
     int32_t n_tiles, n_warps;
     int32_t all_k;               // options of every job where all have the same, in the table's order; else 0

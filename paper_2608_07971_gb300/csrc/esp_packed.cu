@@ -1182,8 +1182,9 @@ __global__ void __launch_bounds__(kPackWarps * 32, pack_min_ctas(NW, G))
         return;
     int k = w, end = w + 1;
     if (pk.n_warps != pk.n_tiles) {
-        k = __ldg(pk.warp_begin + w);
-        end = __ldg(pk.warp_begin + w + 1);
+        const int32_t *begin = !PLAIN && kind == PASS_FINAL ? pk.final_begin : pk.warp_begin;
+        k = __ldg(begin + w);
+        end = __ldg(begin + w + 1);
     }
     run_warp<NW, G, PLAIN, false>(t, st, pk, a, round, kind,
                                smem + (size_t)wid * (pack_warp_bytes(NW) + (G ? pk.fmt.g_bytes : 0)),

@@ -360,11 +360,11 @@ bool pack_format(const int32_t *umax, int32_t R, PackFormat &out, int32_t r_glob
         out.col_lo[k] = (int8_t)lo.col;
         out.field[lo.col] = (int8_t)(2 * k);
         if (hi) {
+            out.field[hi->col] = (int8_t)(2 * k + 1);
             high[k] = hi->bits;
             out.shift[k] = 32 - hi->bits;
             out.magic[k] = 0x4b000000u >> hi->bits;   // exact: its low 24 bits are zero
             out.col_hi[k] = (int8_t)hi->col;
-            out.field[hi->col] = (int8_t)(2 * k + 1);
         }
     };
     for (int32_t i = 0; i < flat; ++i) {
@@ -532,22 +532,29 @@ bool plan_packed(const int64_t *off, int32_t S, int32_t J, int32_t max_warps, Pa
     out.job_begin.push_back((int32_t)n_jobs);
     if (out.tiles.size() >= (size_t)INT32_MAX)
         return false;
-    // 3. the round pass's ranges: contiguous tiles of about equal cost (in tenths of a step)
+    // 3. the passes' ranges: contiguous tiles of about equal cost (in tenths of a step). In the final pass a lane of
+    //    a step of one- and two-option jobs writes the outputs of up to eight winners, others of one at most.
     const int64_t n_tiles = (int64_t)out.tiles.size();
-    std::vector<int64_t> pre((size_t)n_tiles + 1, 0);
-    for (int64_t i = 0; i < n_tiles; ++i)
-        pre[i + 1] = pre[i] + 5 + 10LL * pack_shape(out.tiles[i]).steps;
     const int32_t W = (int32_t)std::min<int64_t>(max_warps, n_tiles);
     out.n_warps = W;
-    out.warp_begin.assign((size_t)W + 1, 0);
-    for (int32_t w = 1; w < W; ++w) {
-        const int64_t target = (int64_t)((__int128)pre[n_tiles] * w / W);
-        int64_t i = std::lower_bound(pre.begin(), pre.end(), target) - pre.begin();
-        if (i > 0 && target - pre[i - 1] < pre[i] - target)
-            --i;
-        out.warp_begin[w] = (int32_t)std::min<int64_t>(std::max<int64_t>(i, out.warp_begin[w - 1]), n_tiles);
-    }
-    out.warp_begin[W] = (int32_t)n_tiles;
+    std::vector<int64_t> pre((size_t)n_tiles + 1, 0);
+    auto split = [&](int64_t tiny_step, std::vector<int32_t> &begin) {
+        for (int64_t i = 0; i < n_tiles; ++i) {
+            const PackShape sh = pack_shape(out.tiles[i]);
+            pre[i + 1] = pre[i] + 5 + (sh.code == (int)kPackTiny ? tiny_step : 10) * sh.steps;
+        }
+        begin.assign((size_t)W + 1, 0);
+        for (int32_t w = 1; w < W; ++w) {
+            const int64_t target = (int64_t)((__int128)pre[n_tiles] * w / W);
+            int64_t i = std::lower_bound(pre.begin(), pre.end(), target) - pre.begin();
+            if (i > 0 && target - pre[i - 1] < pre[i] - target)
+                --i;
+            begin[w] = (int32_t)std::min<int64_t>(std::max<int64_t>(i, begin[w - 1]), n_tiles);
+        }
+        begin[W] = (int32_t)n_tiles;
+    };
+    split(10, out.warp_begin);
+    split(kPackFinalTiny, out.final_begin);
     return true;
 }
 
@@ -591,11 +598,13 @@ bool check_packed(const int64_t *off, int32_t S, int32_t J, const PackPlan &p, i
     }
     if (vecs != p.vecs || count != p.scen_tiles)
         return false;
-    if ((int32_t)p.warp_begin.size() != p.n_warps + 1 || p.warp_begin.front() != 0 || p.warp_begin.back() != n_tiles)
-        return false;
-    for (int32_t w = 0; w < p.n_warps; ++w)
-        if (p.warp_begin[w] > p.warp_begin[w + 1])
+    for (const std::vector<int32_t> *b : {&p.warp_begin, &p.final_begin}) {
+        if ((int32_t)b->size() != p.n_warps + 1 || b->front() != 0 || b->back() != n_tiles)
             return false;
+        for (int32_t w = 0; w < p.n_warps; ++w)
+            if ((*b)[w] > (*b)[w + 1])
+                return false;
+    }
     return true;
 }
 

@@ -50,12 +50,18 @@ struct SortedLayout {
 bool sort_layout(const int64_t *job_off, int32_t S, int32_t J, SortedLayout &out, int32_t run_max_k = kRunMaxK);
 
 
+// Cost of a step of one- and two-option jobs in the final pass, in tenths of another step's: up to eight winners per
+// lane, each with outputs to write and an exact score. (With the round pass's ranges, a few warps held all of them: a
+// one-round solve of the heavy-tailed table at 16 scenarios took 1.61 ms, 1.02 with these; 1.43 staged.)
+constexpr int64_t kPackFinalTiny = 40;
+
 // Plan of the packed passes over a table (esp_packed.h).
 struct PackPlan {
     std::vector<int32_t> job;          // table job of each job in the packed order; empty: the same order
     std::vector<int32_t> job_begin;    // n_tiles + 1: first job (packed order) of each tile
     std::vector<PackTile> tiles;       // by scenario
     std::vector<int32_t> warp_begin;   // n_warps + 1: the round pass's ranges of about equal cost
+    std::vector<int32_t> final_begin;  // n_warps + 1: the final pass's
     std::vector<int32_t> scen_tiles;   // S: tiles of each scenario
     int64_t vecs = 0;                  // vectors per plane of the whole copy
     int64_t steps = 0;

@@ -44,3 +44,10 @@ def test_exact_mode(S, J, K, R):
     t = table(S, J, K, R)
     packed, staged = (best_ms(t, 10, esp.ESP_FLAG_EXACT_ONLY, p) for p in (True, False))
     assert packed <= staged, (packed, staged)
+
+
+@pytest.mark.parametrize("S,J", [(8, 65536), (4, 16384)])
+def test_final_pass_of_short_solves(S, J):
+    t = table(S, J, -256, 6)
+    packed, staged = (best_ms(t, 1, 0, p) for p in (True, False))
+    assert packed <= 0.95 * staged, (packed, staged)
