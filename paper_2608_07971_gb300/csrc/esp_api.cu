@@ -1876,13 +1876,13 @@ esp_status esp_load_placement(esp_ctx *ctx, int32_t S, int32_t J, int32_t KC, in
         return st;
     }
     // the grid-resident solve (ESP_FLAG_RESIDENT): one CTA per SM holds the price state of every
-    // scenario and each warp a job, all in shared memory; as many warps per CTA as that takes, since the round
-    // is a chain, and fewer warps meet at a CTA's barriers sooner (us per round with at least 8,
-    // 16 and 32 warps: 1000 jobs x 8 x 30 6.87, 7.15 and 8.27; 100 jobs x 4 x 10 5.37, 5.62 and 6.40; two scenarios of
-    // 500 x 12 x 64 9.14, 8.69 and 10.1)
-    int32_t rw = 8;
-    while (rw < kPlaceResMaxWarps && n_jobs > (int64_t)rw * ctx->sm_count)
-        rw *= 2;
+    // scenario and each warp a job, all in shared memory. As few warps per CTA as hold every job, at least 8: the
+    // round is a chain, and fewer warps meet at a CTA's barriers sooner (us per round with 8, 10, 16 and 24 warps,
+    // R = 8: 1000 jobs x 8 x 30 7.16, 7.24, 7.50 and 8.19; 100 jobs x 4 x 10 5.46, 5.39, 5.55 and 6.06; only two
+    // scenarios of 500 x 12 x 64, whose 268 prices are more than 8 warps' threads, would gain: 9.62, 8.84, 9.12 and
+    // 9.87), and more SMs share the work (2433 jobs x 12 x 64, 17 warps on every SM against 32 on every second:
+    // R = 3 11.4 against 13.1, R = 8 9.50 against 10.9, R = 16 13.3 against 16.3).
+    const int32_t rw = (int32_t)std::min<int64_t>(kPlaceResMaxWarps, std::max<int64_t>(8, (n_jobs + ctx->sm_count - 1) / ctx->sm_count));
     if ((int64_t)S * P <= kPlaceResMaxPrices && n_jobs <= (int64_t)rw * ctx->sm_count &&
         place_res_smem_bytes(S, P, KC, R, rw) <= optin && place_res_ctas_per_sm(S, P, KC, R, rw) >= 1) {
         PlaceRes &pr = ctx->place_res;

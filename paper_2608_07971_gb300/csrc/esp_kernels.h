@@ -134,8 +134,13 @@ constexpr int kPlaceWarps = 4;
 constexpr int kPlaceResMaxPrices = 1024;   // S * P limit of the grid-resident placement solve
 constexpr int kPlaceResMaxWarps = 32;      // warps per CTA of the grid-resident placement solve, one job each
 
-// The grid-resident placement solve (k_place_res): one CTA of `warps` warps (8, 16 or 32) per SM at most, warp w of
-// the grid holding job w.
+// The grid-resident placement solve (k_place_res): one CTA of `warps` warps (8 to 32) per SM at most, warp w of
+// the grid holding job w. Instantiated for at most 8, 16 and 32 warps (their register budgets); the fewest warps
+// that each is launched with:
+ESP_HD constexpr int place_res_min_warps(int bound)
+{
+    return bound == 8 ? 8 : bound / 2 + 1;
+}
 struct PlaceRes {
     unsigned long long *U3;     // 3 * S * P: the demand of round r in buffer r % 3
     unsigned long long *bar;    // the grid barrier's word (esp_barrier.h); zeroed before each launch

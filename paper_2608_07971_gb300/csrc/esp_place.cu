@@ -293,7 +293,7 @@ __device__ __forceinline__ double exact_score_shared(const int32_t *u, double v,
     return s;
 }
 
-// All T rounds of a placement solve in one cooperative launch of one CTA (W warps) per SM. Each warp
+// All T rounds of a placement solve in one cooperative launch of one CTA (pr.warps warps, at most W) per SM. Each warp
 // holds one job in shared memory for the whole solve:
 // configuration units (int32 and fp32), values, and per lane the penalties of its two nodes. Each
 // CTA holds the whole price state of every scenario in shared memory (S * P <= kPlaceResMaxPrices).
@@ -304,7 +304,9 @@ __device__ __forceinline__ double exact_score_shared(const int32_t *u, double v,
 // What bounds it is the chain of a round: best response, shared sums, atomics, grid barrier, update, bound. One
 // job per warp: 9.8 us per round of 4096 jobs x 12 x 64, where two jobs one after the other in each of 16 warps,
 // the sums as 64-bit shared atomics, two trips to L2 per poll of the barrier, two fp64 divides per price and the
-// bound in fp64 took 15.0 (all but the first of these: 12.1).
+// bound in fp64 took 15.0 (all but the first of these: 12.1). The jobs are spread over every SM, so that no more
+// warps share one than they must; the bound W only sets the registers (64 per thread for 17 to 32 warps, which
+// spills for R other than 8: 4096 jobs of R = 16 16.2 us per round, 20.6 before).
 // CTA 0 writes the price and demand trajectories, clears the buffer that was last read before this
 // round's barrier, and publishes the final state for the final pass. Hash and dual traces are not
 // supported here (the host keeps the per-round launches for them).
@@ -318,7 +320,7 @@ __global__ void __launch_bounds__(W * 32, 1) k_place_res(DevTable t, DevState st
     const int R = RT ? RT : t.R, rg = t.r_global;
     const int S = t.S, P = t.P, SP = S * P, T = a.T;
     const int KC = pl.KC, N = pl.N, NT = pl.NT;
-    const PlaceResLayout L = place_res_layout(S, P, KC, R, W);
+    const PlaceResLayout L = place_res_layout(S, P, KC, R, pr.warps);
 
     // the CTA's demand of each price as two 32-bit sums, of the low 16 bits and of the rest of its winners' units:
     // an atomic add of 64 bits in shared memory is a loop of compare-and-swaps, which the columns that all
@@ -361,7 +363,7 @@ __global__ void __launch_bounds__(W * 32, 1) k_place_res(DevTable t, DevState st
     // of the scenario whose bound this warp computes (the first, when there are more scenarios than warps)
     const float own_umax = wid < S && lane < R ? __int2float_ru(st.umax[(size_t)wid * R + lane]) : 0.0f;
     const float own_vmax = wid < S ? __double2float_ru(st.vmax[wid]) : 0.0f;
-    const int64_t j = (int64_t)blockIdx.x * W + wid;
+    const int64_t j = (int64_t)blockIdx.x * pr.warps + wid;
     const bool has_job = j < pr.n_jobs;
     const int n0 = lane, n1 = lane + 32;
     const bool h0 = n0 < N, h1 = n1 < N;
@@ -567,11 +569,11 @@ __global__ void __launch_bounds__(W * 32, 1) k_place_res(DevTable t, DevState st
         // into registers, and written once no price of the scenario became non-finite
         const double eta = step_size(a.eta0, a.step, round);
         const bool lead = blockIdx.x == 0;
-        constexpr int kPrices = (kPlaceResMaxPrices + W * 32 - 1) / (W * 32);   // per thread
+        constexpr int kThreads = place_res_min_warps(W) * 32, kPrices = (kPlaceResMaxPrices + kThreads - 1) / kThreads;   // per thread
         double nl_r[kPrices], pe_r[kPrices];
 #pragma unroll
         for (int m = 0; m < kPrices; ++m) {
-            const int i = tid + m * W * 32;
+            const int i = tid + m * (int)blockDim.x;
             nl_r[m] = pe_r[m] = 0.0;
             if (i >= SP)
                 break;
@@ -596,7 +598,7 @@ __global__ void __launch_bounds__(W * 32, 1) k_place_res(DevTable t, DevState st
         __syncthreads();
 #pragma unroll
         for (int m = 0; m < kPrices; ++m) {
-            const int i = tid + m * W * 32;
+            const int i = tid + m * (int)blockDim.x;
             if (i >= SP)
                 break;
             const int sc = i / P;
@@ -612,7 +614,7 @@ __global__ void __launch_bounds__(W * 32, 1) k_place_res(DevTable t, DevState st
         // stopping rule and screen bound, one warp per scenario. E only has to bound the screen's error from
         // above: it is computed in fp32 with every operation rounded up, from p <= p32 (1 + 2^-23) + 2^-149 and
         // M = max|v| + sum_r (largest p_r) max u_r; no fp64 operation, and one reduction per node column
-        for (int sc = wid; sc < S; sc += W) {
+        for (int sc = wid; sc < S; sc += pr.warps) {
             if (frozen_s[sc])
                 continue;
             if (bad_s[sc]) {
@@ -742,11 +744,11 @@ int place_res_smem_bytes(int S, int P, int KC, int R, int warps)
 static const void *place_res_kernel(int R, int warps)
 {
     if (R == 8)
-        return warps == 8    ? reinterpret_cast<const void *>(&k_place_res<8, 8>)
-               : warps == 16 ? reinterpret_cast<const void *>(&k_place_res<8, 16>)
+        return warps <= 8    ? reinterpret_cast<const void *>(&k_place_res<8, 8>)
+               : warps <= 16 ? reinterpret_cast<const void *>(&k_place_res<8, 16>)
                              : reinterpret_cast<const void *>(&k_place_res<8, 32>);
-    return warps == 8    ? reinterpret_cast<const void *>(&k_place_res<0, 8>)
-           : warps == 16 ? reinterpret_cast<const void *>(&k_place_res<0, 16>)
+    return warps <= 8    ? reinterpret_cast<const void *>(&k_place_res<0, 8>)
+           : warps <= 16 ? reinterpret_cast<const void *>(&k_place_res<0, 16>)
                          : reinterpret_cast<const void *>(&k_place_res<0, 32>);
 }
 

@@ -32,3 +32,20 @@ def test_job_counts(warps, extra, big):
     assert s.launches() == (4 if fits else 12)
     same_solution(res, ref, fields=("lam", "sel", "demand"))
     s.close()
+
+
+@pytest.mark.parametrize("R", [6, 8, 16])
+def test_one_job_more_than_16_per_sm(R):
+    """The jobs are spread over every SM: one more than 16 warps per SM hold costs a round little (with the next power
+    of two of warps on half of the SMs, a round of R = 16 took 1.4 times as long). Device time, the shortest of
+    several solves."""
+    import torch
+    n = 16 * torch.cuda.get_device_properties(0).multi_processor_count
+    us = []
+    for jobs in (n, n + 1):
+        f = random_factors(R, S=1, J=jobs, KC=12, N=64, R=R, rg=R - 2)
+        s = esp.Solver()
+        s.load_placement(f)
+        us.append(min(float(s.solve(0.02, 60, flags=esp.ESP_FLAG_RESIDENT).result["device_ms"][0]) for _ in range(6)))
+        s.close()
+    assert us[1] <= 1.25 * us[0], us
