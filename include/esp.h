@@ -234,7 +234,9 @@ esp_status esp_load_placement(esp_ctx *ctx, int32_t S, int32_t J, int32_t KC, in
  *           no interference penalty
  *   tau     host, S*J fp64: tolerance thresholds tau_j(t) (esp_adaptive_threshold); required with
  *           s_hat, ignored without
- * gamma0 = 0 with s_hat = NULL restores the loaded values. Errors: ESP_ERR_NOT_LOADED,
+ * gamma0 = 0 with s_hat = NULL restores the loaded values. Device memory: the first call keeps a copy of the
+ * loaded values (8 bytes per option), the first with c_cur 4 bytes per job, the first with s_hat 8 bytes per option
+ * and per job, all until the table is replaced or the context destroyed. Errors: ESP_ERR_NOT_LOADED, ESP_ERR_OOM,
  * ESP_ERR_INVALID_ARG (bad weights, a c_cur at or beyond its job's option count, a non-finite
  * effective value; the context then holds the loaded values, without penalties). */
 esp_status esp_set_penalties(esp_ctx *ctx, double gamma0, const int32_t *c_cur, double alpha, const double *s_hat,

@@ -98,7 +98,8 @@ struct esp_ctx {
     int32_t *s_jmap = nullptr;
     // Gamma term (esp_set_penalties): the loaded values, kept once penalties are first set
     double *values0 = nullptr;
-    unsigned char *pen_in = nullptr;   // device copies of its inputs (current configurations, slowdowns, thresholds)
+    int32_t *pen_cur = nullptr;        // device copies of its inputs, from the first call that gives them:
+    double *pen_sh = nullptr;          // current configurations; slowdowns, then thresholds
     // the pass table tile by tile (units then values of each tile; one bulk copy per tile), when every
     // tile of the per-warp plan allows it; n_tiles: tiles of that plan
     unsigned char *il = nullptr;
@@ -306,7 +307,8 @@ void release_table(esp_ctx *ctx, bool keep = false)
     ctx->s_off = nullptr;
     ctx->s_jmap = nullptr;
     ctx->values0 = nullptr;
-    ctx->pen_in = nullptr;
+    ctx->pen_cur = nullptr;
+    ctx->pen_sh = nullptr;
     ctx->il = nullptr;
     ctx->packed = false;
     ctx->pack = DevPack{};
@@ -1942,11 +1944,9 @@ esp_status esp_set_penalties(esp_ctx *ctx, double gamma0, const int32_t *c_cur, 
         return ESP_ERR_INVALID_ARG;
     ESP_CUDA(cudaSetDevice(ctx->device));
     const size_t n_jobs = (size_t)ctx->S * ctx->J, n_opt = (size_t)ctx->n_opt;
-    // The loaded values and the inputs' device copies, allocated by the first call and kept with the table
-    // (a cudaMalloc and cudaFree per call took 60 to 180 us of a 0.5 ms outer round of the ESP-IAC loop,
-    // depending on whether the driver had to map memory for them).
-    const size_t cur_b = (n_jobs * sizeof(int32_t) + 255) & ~size_t(255), sh_b = (n_opt * sizeof(double) + 255) & ~size_t(255),
-                 tau_b = n_jobs * sizeof(double);
+    // The loaded values and the inputs' device copies, allocated by the first call that needs them and kept with
+    // the table (a cudaMalloc and cudaFree per call took 60 to 180 us of a 0.5 ms outer round of the ESP-IAC loop,
+    // depending on whether the driver had to map memory for them). Inputs that are never given take no memory.
     if (!ctx->values0) {
         double *v0 = nullptr;
         if ((st = dev_alloc(ctx, &v0, n_opt, 64, false)) != ESP_OK)
@@ -1954,17 +1954,18 @@ esp_status esp_set_penalties(esp_ctx *ctx, double gamma0, const int32_t *c_cur, 
         ESP_CUDA(cudaMemcpyAsync(v0, ctx->values, n_opt * sizeof(double), cudaMemcpyDeviceToDevice, ctx->stream));
         ctx->values0 = v0;
     }
-    if (!ctx->pen_in && (c_cur || s_hat) && (st = dev_alloc(ctx, &ctx->pen_in, cur_b + sh_b + tau_b, 64, false)) != ESP_OK)
+    if (c_cur && !ctx->pen_cur && (st = dev_alloc(ctx, &ctx->pen_cur, n_jobs, 64, false)) != ESP_OK)
         return st;
-    unsigned char *buf = ctx->pen_in;
-    int32_t *d_cur = c_cur ? reinterpret_cast<int32_t *>(buf) : nullptr;
-    double *d_sh = s_hat ? reinterpret_cast<double *>(buf + cur_b) : nullptr;
-    double *d_tau = s_hat ? reinterpret_cast<double *>(buf + cur_b + sh_b) : nullptr;
+    if (s_hat && !ctx->pen_sh && (st = dev_alloc(ctx, &ctx->pen_sh, n_opt + n_jobs, 64, false)) != ESP_OK)
+        return st;
+    int32_t *d_cur = c_cur ? ctx->pen_cur : nullptr;
+    double *d_sh = s_hat ? ctx->pen_sh : nullptr;
+    double *d_tau = s_hat ? ctx->pen_sh + n_opt : nullptr;
     if (c_cur)
         ESP_CUDA(cudaMemcpyAsync(d_cur, c_cur, n_jobs * sizeof(int32_t), cudaMemcpyHostToDevice, ctx->stream));
     if (s_hat) {
         ESP_CUDA(cudaMemcpyAsync(d_sh, s_hat, n_opt * sizeof(double), cudaMemcpyHostToDevice, ctx->stream));
-        ESP_CUDA(cudaMemcpyAsync(d_tau, tau, tau_b, cudaMemcpyHostToDevice, ctx->stream));
+        ESP_CUDA(cudaMemcpyAsync(d_tau, tau, n_jobs * sizeof(double), cudaMemcpyHostToDevice, ctx->stream));
     }
     ESP_CUDA(cudaMemsetAsync(ctx->valflags, 0, sizeof(unsigned int), ctx->stream));
     ESP_CUDA(launch_apply_penalties(dev_table(ctx), ctx->values0, d_cur, d_sh, d_tau, gamma0, alpha, ctx->values,
