@@ -936,13 +936,22 @@ esp_status load_common(esp_ctx *ctx, int32_t S, int32_t J, int32_t R, int32_t P,
     PackFormat fmt;
     if (pack_ok && pack_format(col_max.data(), R, fmt, rg, n_groups)) {
         fmt.g_bytes = group_bytes;
-        if ((st = load_packed(ctx, fmt)) != ESP_OK) {
+        const size_t held = ctx->table_bufs.size();
+        st = load_packed(ctx, fmt);
+        if (st == ESP_ERR_OOM && grouped) {   // no room for the copy: the staged pass reads the table itself
+            cudaStreamSynchronize(ctx->stream);
+            for (size_t i = held; i < ctx->table_bufs.size(); ++i)
+                cudaFree(ctx->table_bufs[i].first);
+            ctx->table_bufs.resize(held);
+            ctx->pack = DevPack{};
+            ctx->pk_data = nullptr;
+        } else if (st != ESP_OK) {
             release_table(ctx);
             return st;
         }
-    } else {
-        if (may_sort)
-            st = load_sorted(ctx);
+    }
+    if (!ctx->packed) {
+        st = may_sort ? load_sorted(ctx) : ESP_OK;
         if (st == ESP_OK)
             st = load_staged(ctx);
         if (st != ESP_OK) {
