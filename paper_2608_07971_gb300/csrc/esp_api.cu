@@ -60,6 +60,7 @@ struct PlanCache {
     esp::SortedLayout lay;
     bool has_plan = false;         // plan: the staged pass's tiles
     esp::Plan plan;
+    bool wide = false;             // units of 2^23 or more at the last load of these offsets
     bool has_pack = false;         // pack: the packed passes' tiles
     int32_t pack_warps = 0;
     esp::PackPlan pack;
@@ -126,7 +127,7 @@ struct esp_ctx {
     TileDesc *tiles = nullptr;
     int32_t *warp_begin = nullptr;
     bool il_enabled = true;          // later loads may pack or interleave the table (esp_debug_set_interleave)
-    bool il_f32_enabled = true;      // ... pack it (esp_debug_set_stage_f32)
+    bool pack_enabled = true;      // ... pack it (esp_debug_set_stage_f32)
     // failure-detection hooks (esp_debug.h): limit of a bounded wait of the evaluation passes in ms
     // (0: the default, 4 s), extra bytes announced on the next solve's first stage, allocations left
     // before an injected failure (-1: none)
@@ -607,6 +608,53 @@ esp_status load_packed(esp_ctx *ctx, const PackFormat &fmt)
     return ESP_OK;
 }
 
+// The sorted layout of a general table without a group column, into the plan cache.
+void plan_sorted(esp_ctx *ctx)
+{
+    PlanCache &pc = ctx->pc;
+    if (!pc.has_lay) {
+        pc.sorted = sort_layout(pc.off.data(), ctx->S, ctx->J, pc.lay, kRunMaxK);
+        pc.has_lay = true;
+    }
+}
+
+// The staged pass's tiles (of the sorted layout, or of the table's own order), into the plan cache.
+esp_status plan_staged(esp_ctx *ctx, bool sorted)
+{
+    PlanCache &pc = ctx->pc;
+    const int32_t S = ctx->S, J = ctx->J, R = ctx->R;
+    const bool grouped = ctx->group != nullptr;
+    const int64_t *plan_off = sorted ? pc.lay.off.data() : pc.off.data();
+    const int32_t *plan_scen = sorted ? pc.lay.scen.data() : nullptr;
+    const int32_t *plan_runk = sorted ? pc.lay.runk.data() : nullptr;
+    const int tile_opt = tile_options_for(R, grouped, ctx->max_k, ctx->uniform_k >= 4);
+    // a sorted layout's tiles are runs and chunks only (the sorted layout exists only without a group
+    // column): the runs-only instantiation
+    const int mode = ctx->uniform_k > 0 ? kModeUniform : (sorted && !grouped) ? kModeRuns : kModeGeneral;
+    const int per_sm = pass_ctas_per_sm(R, grouped, mode, ctx->P, tile_opt);
+    if (per_sm < 1)
+        return ESP_ERR_UNSUPPORTED;
+    // Ranges of the plan as waves of resident CTAs: two by default (CTAs that finish early take the
+    // second wave's ranges), one for a sorted layout (measured 2% faster there).
+    const int waves = ctx->plan_waves > 0 ? ctx->plan_waves : (mode == kModeRuns) ? 1 : 2;
+    const int max_warps = ctx->sm_count * per_sm * kWarpsPerCta * waves;
+    if (!(pc.has_plan && pc.max_warps == max_warps && pc.tile_opt == tile_opt)) {
+        pc.has_plan = false;
+        if (!plan_tiles(plan_off, S, J, tile_opt, max_warps, pc.plan, plan_scen, plan_runk) ||
+            !check_plan(plan_off, S, J, pc.plan, plan_scen, plan_runk))
+            return ESP_ERR_INVALID_ARG;
+        pc.has_plan = true;
+        pc.max_warps = max_warps;
+        pc.tile_opt = tile_opt;
+    }
+    // the runs-only instantiation has no path for a general tile
+    if (mode == kModeRuns)
+        for (const TileDesc &d : pc.plan.tiles)
+            if (!(d.flags & (TILE_RUN | TILE_BIG)))
+                return ESP_ERR_INVALID_ARG;
+    return ESP_OK;
+}
+
 // Builds the sorted layout of a general table without a group column for the staged pass (a table that
 // the packed passes do not take): runs of equal-size jobs take its uniform paths. Jobs keep their
 // option order, so the copy inherits the duplicate marks of the original; its padding is marked as it is
@@ -614,10 +662,7 @@ esp_status load_packed(esp_ctx *ctx, const PackFormat &fmt)
 esp_status load_sorted(esp_ctx *ctx)
 {
     PlanCache &pc = ctx->pc;
-    if (!pc.has_lay) {
-        pc.sorted = sort_layout(pc.off.data(), ctx->S, ctx->J, pc.lay, kRunMaxK);
-        pc.has_lay = true;
-    }
+    plan_sorted(ctx);
     if (!pc.sorted)
         return ESP_OK;
     const SortedLayout &lay = pc.lay;
@@ -648,39 +693,12 @@ esp_status load_sorted(esp_ctx *ctx)
 // and, where every tile allows it, the tile-interleaved copy.
 esp_status load_staged(esp_ctx *ctx)
 {
-    PlanCache &pc = ctx->pc;
-    const int32_t S = ctx->S, J = ctx->J, R = ctx->R;
+    const int32_t S = ctx->S, R = ctx->R;
     const bool grouped = ctx->group != nullptr;
-    const int64_t *plan_off = ctx->sorted ? pc.lay.off.data() : pc.off.data();
-    const int32_t *plan_scen = ctx->sorted ? pc.lay.scen.data() : nullptr;
-    const int32_t *plan_runk = ctx->sorted ? pc.lay.runk.data() : nullptr;
-    const int tile_opt = tile_options_for(R, grouped, ctx->max_k, ctx->uniform_k >= 4);
-    // a sorted layout's tiles are runs and chunks only (the sorted layout exists only without a group
-    // column): the runs-only instantiation
-    const int mode = ctx->uniform_k > 0 ? kModeUniform : (ctx->sorted && !grouped) ? kModeRuns : kModeGeneral;
-    const int per_sm = pass_ctas_per_sm(R, grouped, mode, ctx->P, tile_opt);
-    if (per_sm < 1)
-        return ESP_ERR_UNSUPPORTED;
-    // Ranges of the plan as waves of resident CTAs: two by default (CTAs that finish early take the
-    // second wave's ranges), one for a sorted layout (measured 2% faster there).
-    const int waves = ctx->plan_waves > 0 ? ctx->plan_waves : (mode == kModeRuns) ? 1 : 2;
-    const int max_warps = ctx->sm_count * per_sm * kWarpsPerCta * waves;
-    if (!(pc.has_plan && pc.max_warps == max_warps && pc.tile_opt == tile_opt)) {
-        pc.has_plan = false;
-        if (!plan_tiles(plan_off, S, J, tile_opt, max_warps, pc.plan, plan_scen, plan_runk) ||
-            !check_plan(plan_off, S, J, pc.plan, plan_scen, plan_runk))
-            return ESP_ERR_INVALID_ARG;
-        pc.has_plan = true;
-        pc.max_warps = max_warps;
-        pc.tile_opt = tile_opt;
-    }
-    const Plan &plan = pc.plan;
-    // the runs-only instantiation has no path for a general tile
-    if (mode == kModeRuns)
-        for (const TileDesc &d : plan.tiles)
-            if (!(d.flags & (TILE_RUN | TILE_BIG)))
-                return ESP_ERR_INVALID_ARG;
-    esp_status st = ESP_OK;
+    esp_status st = plan_staged(ctx, ctx->sorted);
+    if (st != ESP_OK)
+        return st;
+    const Plan &plan = ctx->pc.plan;
     auto al = [&](auto **ptr, size_t n) {
         if (st == ESP_OK)
             st = dev_alloc(ctx, ptr, n);
@@ -844,6 +862,7 @@ esp_status load_common(esp_ctx *ctx, int32_t S, int32_t J, int32_t R, int32_t P,
     ESP_CUDA(cudaMemcpyAsync(h_vflags, ctx->valflags, sizeof(unsigned int), cudaMemcpyDeviceToHost, ctx->stream));
     ESP_CUDA(cudaMemcpyAsync(ctx->h_stage + 16, ctx->umax, (size_t)S * R * sizeof(int32_t), cudaMemcpyDeviceToHost,
                              ctx->stream));
+    ESP_CUDA(cudaEventRecord(ctx->load_ev[0], ctx->stream));   // the validation's answer (LoadStreamScope is done with it)
     ctx->load_ms[0] = since();   // uploads and validation queued
     // the plan of the previous load serves when the shape and offsets are the same
     PlanCache &pc = ctx->pc;
@@ -874,32 +893,9 @@ esp_status load_common(esp_ctx *ctx, int32_t S, int32_t J, int32_t R, int32_t P,
     // plan the evaluation pass
     ctx->uniform_k = (!grouped && min_k == max_k && max_k <= 32 && (max_k & (max_k - 1)) == 0) ? (int32_t)max_k : 0;
 
-    // the packed passes (esp_packed.h) take a table whose units are below 2^23, grouped ones where
-    // pack_groups_fit; the first is known after the validation, so the plan for them is made meanwhile, for
-    // the unit words that pairs of columns need. Tables they do not take are evaluated by the staged pass,
-    // general ones without a group column in the sorted layout.
-    const bool may_sort = ctx->sorted_enabled && !grouped && ctx->uniform_k == 0 && J >= 1;
-    const bool may_pack = ctx->il_enabled && ctx->il_f32_enabled && n_jobs > 0 &&
-                          (grouped ? pack_groups_fit(R, rg, P) : ctx->uniform_k > 0 || may_sort);
-    const int group_bytes = grouped ? pack_group_bytes(P, n_groups) : 0;
-    ctx->load_ms[1] = since();
-    PackPlan pack_new;
-    int32_t pack_warps = 0;
-    bool pack_cached = false, pack_ok = false;
-    if (may_pack) {
-        const int per_sm = grouped ? packed_ctas_per_sm(R <= 6 ? 3 : R <= 8 ? 4 : 6, group_bytes)
-                                   : packed_ctas_per_sm(R <= 4 ? 2 : R <= 6 ? 3 : R <= 8 ? 4 : R <= 12 ? 6 : 8);
-        const int waves = ctx->plan_waves > 0 ? ctx->plan_waves : 1;
-        pack_warps = ctx->sm_count * std::max(per_sm, 1) * kWarpsPerCta * waves;
-        pack_cached = cached && pc.has_pack && pc.pack_warps == pack_warps;
-        const int64_t all_k = min_k == max_k ? max_k : 0;
-        pack_ok = per_sm > 0 && (pack_cached || (plan_packed(off_host, S, J, pack_warps, pack_new, all_k) &&
-                                                 check_packed(off_host, S, J, pack_new, all_k)));
-    }
-    ctx->load_ms[2] = since();   // packed passes planned
-    // keep this load's layout (and below its plan) for the next load of the same offsets
+    // keep this load's layout and plans for the next load of the same offsets
     if (!cached) {
-        pc.valid = true;
+        pc.valid = false;
         pc.S = S;
         pc.J = J;
         pc.R = R;
@@ -910,11 +906,55 @@ esp_status load_common(esp_ctx *ctx, int32_t S, int32_t J, int32_t R, int32_t P,
         pc.min_k = min_k;
         pc.max_k = max_k;
         pc.has_lay = pc.has_plan = pc.has_pack = false;
+        pc.valid = true;
     }
-    if (pack_ok && !pack_cached) {
-        pc.has_pack = true;
-        pc.pack_warps = pack_warps;
-        pc.pack = std::move(pack_new);
+    // the packed passes (esp_packed.h) take a table whose units are below 2^23, grouped ones where
+    // pack_groups_fit; the first is known after the validation. The host plans meanwhile, for the unit words that
+    // pairs of columns need. Tables they do not take are evaluated by the staged pass, general ones without a
+    // group column in the sorted layout.
+    const bool may_sort = ctx->sorted_enabled && !grouped && ctx->uniform_k == 0 && J >= 1;
+    const bool may_pack = ctx->il_enabled && ctx->pack_enabled && n_jobs > 0 &&
+                          (grouped ? pack_groups_fit(R, rg, P) : ctx->uniform_k > 0 || may_sort);
+    const int group_bytes = grouped ? pack_group_bytes(P, n_groups) : 0;
+    // A guess, so that a table of wide units is planned for the pass that takes it: what the last load of these
+    // offsets had, else the first rows of a host table, or the validation's answer where it is there by now (a
+    // table that was on the device already). Planned for the packed pass first, and for the staged one after
+    // the upload, the first load of 65536 ragged jobs with units up to 2^25 took 3.7 ms, 2.5 without.
+    bool wide = cached && pc.wide;
+    if (may_pack && !cached && !device_src) {
+        for (int64_t i = 0; i < std::min<int64_t>(n_opt, 256) * R; ++i)
+            wide = wide || units[i] >= (1 << 23);
+    } else if (may_pack && !cached) {
+        const cudaError_t e = cudaEventQuery(ctx->load_ev[0]);
+        if (e != cudaErrorNotReady)
+            ESP_CUDA(e);
+        else
+            cudaGetLastError();
+        for (size_t i = 0; i < (size_t)S * R && e == cudaSuccess; ++i)
+            wide = wide || h_umax[i] >= (1 << 23);
+    }
+    ctx->load_ms[1] = since();
+    bool pack_ok = false;
+    auto plan_pack = [&]() {
+        const int per_sm = grouped ? packed_ctas_per_sm(R <= 6 ? 3 : R <= 8 ? 4 : 6, group_bytes)
+                                   : packed_ctas_per_sm(R <= 4 ? 2 : R <= 6 ? 3 : R <= 8 ? 4 : R <= 12 ? 6 : 8);
+        const int waves = ctx->plan_waves > 0 ? ctx->plan_waves : 1;
+        const int32_t warps = ctx->sm_count * std::max(per_sm, 1) * kWarpsPerCta * waves;
+        const int64_t all_k = min_k == max_k ? max_k : 0;
+        if (!(pc.has_pack && pc.pack_warps == warps)) {
+            pc.has_pack = false;
+            pc.has_pack = plan_packed(off_host, S, J, warps, pc.pack, all_k) && check_packed(off_host, S, J, pc.pack, all_k);
+            pc.pack_warps = warps;
+        }
+        pack_ok = per_sm > 0 && pc.has_pack;
+    };
+    if (may_pack && !wide)
+        plan_pack();
+    ctx->load_ms[2] = since();   // packed passes planned
+    if (!may_pack || wide) {     // the staged pass's, for load_sorted and load_staged (which report a failure)
+        if (may_sort)
+            plan_sorted(ctx);
+        plan_staged(ctx, may_sort && pc.sorted);
     }
     ctx->load_ms[3] = since();   // planned
     // the validation result (the copies, validation and duplicate marking ran during the planning)
@@ -933,6 +973,9 @@ esp_status load_common(esp_ctx *ctx, int32_t S, int32_t J, int32_t R, int32_t P,
             ctx->small_units = 0;
     }
     ALLOC(ctx->arrive, (size_t)S);
+    pc.wide = ctx->small_units == 0;
+    if (may_pack && wide && !pc.wide)   // the guess was wrong
+        plan_pack();
     PackFormat fmt;
     if (pack_ok && pack_format(col_max.data(), R, fmt, rg, n_groups)) {
         fmt.g_bytes = group_bytes;
@@ -1086,6 +1129,8 @@ esp_status plan_resident_options(esp_ctx *ctx)
             o.plan.lanes = 1;
             while (o.plan.lanes < 8 && 2 * o.plan.lanes * sh.m_max <= kResWarps * 32 && 2 * o.plan.lanes <= ctx->pc.max_k)
                 o.plan.lanes *= 2;
+            // the pitch, a power of two up to 16 or a multiple of 32; the kernel's exclusive or spreads the job slots of
+            // the lanes that read one job's options over it
             const int32_t unit = 32 / o.plan.lanes;
             int32_t pitch = unit;
             while (pitch < sh.m_max && pitch < 32)
@@ -2286,6 +2331,16 @@ esp_status esp_debug_set_interleave(esp_ctx *ctx, int32_t enable)
     return ESP_OK;
 }
 
+esp_status esp_debug_packed_words(esp_ctx *ctx, int32_t *words)
+{
+    if (!ctx || !words)
+        return ESP_ERR_INVALID_ARG;
+    if (!ctx->loaded)
+        return ESP_ERR_NOT_LOADED;
+    *words = ctx->packed ? ctx->pack.fmt.nw : 0;
+    return ESP_OK;
+}
+
 esp_status esp_debug_pass_kernel(esp_ctx *ctx, int32_t *kind)
 {
     esp_status st = check_ctx(ctx);
@@ -2322,23 +2377,13 @@ esp_status esp_debug_persistent(esp_ctx *ctx, int32_t *grid)
     *grid = (ctx->persist_mode > 0 || (ctx->persist_mode < 0 && ctx->persist_auto)) ? ctx->persist_grid : 0;
     return ESP_OK;
 }
-esp_status esp_debug_packed_words(esp_ctx *ctx, int32_t *words)
-{
-    if (!ctx || !words)
-        return ESP_ERR_INVALID_ARG;
-    if (!ctx->loaded)
-        return ESP_ERR_NOT_LOADED;
-    *words = ctx->packed ? ctx->pack.fmt.nw : 0;
-    return ESP_OK;
-}
-
 
 esp_status esp_debug_set_stage_f32(esp_ctx *ctx, int32_t enable)
 {
     esp_status st = check_ctx(ctx);
     if (st != ESP_OK)
         return st;
-    ctx->il_f32_enabled = enable != 0;
+    ctx->pack_enabled = enable != 0;
     return ESP_OK;
 }
 
