@@ -871,17 +871,19 @@ esp_status load_common(esp_ctx *ctx, int32_t S, int32_t J, int32_t R, int32_t P,
                         std::memcmp(pc.off.data(), off_host, (size_t)(n_jobs + 1) * sizeof(int64_t)) == 0;
     // option counts, on the host meanwhile: every job non-empty makes the offsets strictly
     // increasing up to n_opt, so no kernel below can index outside the table
-    int64_t max_k = 1, min_k = n_jobs ? INT64_MAX : 1;
-    if (cached) {
-        max_k = pc.max_k;
-        min_k = pc.min_k;
-    } else {
+    auto count_range = [&]() -> std::pair<int64_t, int64_t> {
+        if (cached)
+            return {pc.min_k, pc.max_k};
+        int64_t lo = n_jobs ? INT64_MAX : 1, hi = 1;
         for (int64_t j = 0; j < n_jobs; ++j) {
             const int64_t k = off_host[j + 1] - off_host[j];
-            max_k = std::max<int64_t>(max_k, k);
-            min_k = std::min<int64_t>(min_k, k);
+            hi = std::max<int64_t>(hi, k);
+            lo = std::min<int64_t>(lo, k);
         }
-    }
+        return {lo, hi};
+    };
+    const auto range = count_range();
+    const int64_t min_k = range.first, max_k = range.second;
     if (min_k < 1) {
         cudaStreamSynchronize(ctx->stream);
         release_table(ctx);
@@ -895,18 +897,15 @@ esp_status load_common(esp_ctx *ctx, int32_t S, int32_t J, int32_t R, int32_t P,
 
     // keep this load's layout and plans for the next load of the same offsets
     if (!cached) {
-        pc.valid = false;
+        pc.valid = pc.has_lay = pc.has_plan = pc.has_pack = false;
         pc.S = S;
         pc.J = J;
         pc.R = R;
         pc.P = P;
         pc.grouped = grouped;
         pc.sorted_enabled = ctx->sorted_enabled;
-        pc.off.assign(off_host, off_host + n_jobs + 1);
         pc.min_k = min_k;
         pc.max_k = max_k;
-        pc.has_lay = pc.has_plan = pc.has_pack = false;
-        pc.valid = true;
     }
     // the packed passes (esp_packed.h) take a table whose units are below 2^23, grouped ones where
     // pack_groups_fit; the first is known after the validation. The host plans meanwhile, for the unit words that
@@ -917,15 +916,16 @@ esp_status load_common(esp_ctx *ctx, int32_t S, int32_t J, int32_t R, int32_t P,
                           (grouped ? pack_groups_fit(R, rg, P) : ctx->uniform_k > 0 || may_sort);
     const int group_bytes = grouped ? pack_group_bytes(P, n_groups) : 0;
     // A guess, so that a table of wide units is planned for the pass that takes it: what the last load of these
-    // offsets had, else the first rows of a host table, or the validation's answer where it is there by now (a
-    // table that was on the device already). Planned for the packed pass first, and for the staged one after
-    // the upload, the first load of 65536 ragged jobs with units up to 2^25 took 3.7 ms, 2.5 without.
+    // offsets had, else the first rows of a host table, or the validation's answer for a table that was on the
+    // device already: where it is there by now, and waited for where the plan is long. (65536 ragged jobs, first load
+    // in ms: units up to 2^25 2.4, 3.5 when planned for the packed pass first and for the staged one after the
+    // upload; small units 1.9, 1.8 without the wait.)
     bool wide = cached && pc.wide;
     if (may_pack && !cached && !device_src) {
         for (int64_t i = 0; i < std::min<int64_t>(n_opt, 256) * R; ++i)
             wide = wide || units[i] >= (1 << 23);
     } else if (may_pack && !cached) {
-        const cudaError_t e = cudaEventQuery(ctx->load_ev[0]);
+        const cudaError_t e = may_sort && n_jobs > 4096 ? cudaEventSynchronize(ctx->load_ev[0]) : cudaEventQuery(ctx->load_ev[0]);
         if (e != cudaErrorNotReady)
             ESP_CUDA(e);
         else
@@ -951,6 +951,10 @@ esp_status load_common(esp_ctx *ctx, int32_t S, int32_t J, int32_t R, int32_t P,
     if (may_pack && !wide)
         plan_pack();
     ctx->load_ms[2] = since();   // packed passes planned
+    if (!pc.valid) {
+        pc.off.assign(off_host, off_host + n_jobs + 1);
+        pc.valid = true;
+    }
     if (!may_pack || wide) {     // the staged pass's, for load_sorted and load_staged (which report a failure)
         if (may_sort)
             plan_sorted(ctx);

@@ -510,6 +510,7 @@ bool plan_packed(const int64_t *off, int32_t S, int32_t J, int32_t max_warps, Pa
             out.steps += pack_shape(PackTile{0, 0, g.mk, (uint32_t)g.n}).steps;
         }
     }
+    std::vector<int64_t> cost(1, 0), final_cost(1, 0);   // of the tiles so far, in tenths of a step
     const int64_t steps_max = std::min<int64_t>(kPackTileSteps, std::max<int64_t>(1, out.steps / (3LL * max_warps)));
     for (const Seg &g : segs) {
         const PackShape one = pack_shape(PackTile{0, 0, g.mk, 1});
@@ -527,22 +528,19 @@ bool plan_packed(const int64_t *off, int32_t S, int32_t J, int32_t max_warps, Pa
                 return false;
             ++out.scen_tiles[(size_t)g.scen];
             out.tiles.push_back(t);
+            cost.push_back(cost.back() + 5 + 10LL * sh.steps);
+            final_cost.push_back(final_cost.back() + 5 + (sh.code == (int)kPackTiny ? kPackFinalTiny : 10) * sh.steps);
         }
     }
     out.job_begin.push_back((int32_t)n_jobs);
     if (out.tiles.size() >= (size_t)INT32_MAX)
         return false;
-    // 3. the passes' ranges: contiguous tiles of about equal cost (in tenths of a step). In the final pass a lane of
-    //    a step of one- and two-option jobs writes the outputs of up to eight winners, others of one at most.
+    // 3. the passes' ranges: contiguous tiles of about equal cost. In the final pass a lane of a step of one- and
+    //    two-option jobs writes the outputs of up to eight winners, others of one at most.
     const int64_t n_tiles = (int64_t)out.tiles.size();
     const int32_t W = (int32_t)std::min<int64_t>(max_warps, n_tiles);
     out.n_warps = W;
-    std::vector<int64_t> pre((size_t)n_tiles + 1, 0);
-    auto split = [&](int64_t tiny_step, std::vector<int32_t> &begin) {
-        for (int64_t i = 0; i < n_tiles; ++i) {
-            const PackShape sh = pack_shape(out.tiles[i]);
-            pre[i + 1] = pre[i] + 5 + (sh.code == (int)kPackTiny ? tiny_step : 10) * sh.steps;
-        }
+    auto split = [&](const std::vector<int64_t> &pre, std::vector<int32_t> &begin) {
         begin.assign((size_t)W + 1, 0);
         for (int32_t w = 1; w < W; ++w) {
             const int64_t target = (int64_t)((__int128)pre[n_tiles] * w / W);
@@ -553,8 +551,8 @@ bool plan_packed(const int64_t *off, int32_t S, int32_t J, int32_t max_warps, Pa
         }
         begin[W] = (int32_t)n_tiles;
     };
-    split(10, out.warp_begin);
-    split(kPackFinalTiny, out.final_begin);
+    split(cost, out.warp_begin);
+    split(final_cost, out.final_begin);
     return true;
 }
 
