@@ -510,8 +510,13 @@ bool plan_packed(const int64_t *off, int32_t S, int32_t J, int32_t max_warps, Pa
             out.steps += pack_shape(PackTile{0, 0, g.mk, (uint32_t)g.n}).steps;
         }
     }
-    std::vector<int64_t> cost(1, 0), final_cost(1, 0);   // of the tiles so far, in tenths of a step
     const int64_t steps_max = std::min<int64_t>(kPackTileSteps, std::max<int64_t>(1, out.steps / (3LL * max_warps)));
+    const size_t tiles_max = segs.size() + (size_t)(out.steps / steps_max) + 1;   // about (jobs of many steps are rare)
+    out.tiles.reserve(tiles_max);
+    out.job_begin.reserve(tiles_max + 1);
+    std::vector<int64_t> cost(1, 0), final_cost(1, 0);   // of the tiles so far, in tenths of a step
+    cost.reserve(tiles_max + 1);
+    final_cost.reserve(tiles_max + 1);
     for (const Seg &g : segs) {
         const PackShape one = pack_shape(PackTile{0, 0, g.mk, 1});
         const int64_t jobs_max = std::max<int64_t>(1, steps_max / one.nch) * one.per_step;
@@ -542,9 +547,12 @@ bool plan_packed(const int64_t *off, int32_t S, int32_t J, int32_t max_warps, Pa
     out.n_warps = W;
     auto split = [&](const std::vector<int64_t> &pre, std::vector<int32_t> &begin) {
         begin.assign((size_t)W + 1, 0);
+        int64_t at = 0;   // first tile boundary at or beyond the target, which only grows
         for (int32_t w = 1; w < W; ++w) {
             const int64_t target = (int64_t)((__int128)pre[n_tiles] * w / W);
-            int64_t i = std::lower_bound(pre.begin(), pre.end(), target) - pre.begin();
+            while (pre[at] < target)
+                ++at;
+            int64_t i = at;
             if (i > 0 && target - pre[i - 1] < pre[i] - target)
                 --i;
             begin[w] = (int32_t)std::min<int64_t>(std::max<int64_t>(i, begin[w - 1]), n_tiles);
