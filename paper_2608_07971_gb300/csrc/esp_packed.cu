@@ -19,8 +19,8 @@
 //
 // Tables with a group column (G): the option's group slot is a field of one of its words, the columns priced
 // per group are its last word, and their two prices come from a table in the warp's shared memory. The
-// placement table of 4096 jobs x 768 options (R = 8, 64 groups; 20 bytes per option instead of 42) takes 29.1 us
-// per round where the staged pass took 77.4; of the 29, 19 are the screen (63 MB, which L2 holds), the rest the
+// placement table of 4096 jobs x 768 options (R = 8, 64 groups; 20 bytes per option instead of 42) takes 28.2 us
+// per round where the staged pass took 77.4; of the 28, 19 are the screen (63 MB, which L2 holds), the rest the
 // chain of the slowest ambiguous job and of the update of 134 prices.
 //
 // The winner's units come from the words in the slot, and so do those of options that are scored exactly (the

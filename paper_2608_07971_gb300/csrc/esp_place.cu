@@ -302,7 +302,7 @@ __device__ __forceinline__ double exact_score_shared(const int32_t *u, double v,
 // then Eq. price_update by the whole CTA from the same totals (one price per thread; per-scenario
 // maxima and flags through shared atomics, which are order-independent), identical in every CTA.
 // What bounds it is the chain of a round: best response, shared sums, atomics, grid barrier, update, bound. One
-// job per warp: 9.8 us per round of 4096 jobs x 12 x 64, where two jobs one after the other in each of 16 warps,
+// job per warp: 9.6 us per round of 4096 jobs x 12 x 64, where two jobs one after the other in each of 16 warps,
 // the sums as 64-bit shared atomics, two trips to L2 per poll of the barrier, two fp64 divides per price and the
 // bound in fp64 took 15.0 (all but the first of these: 12.1). The jobs are spread over every SM, so that no more
 // warps share one than they must; the bound W only sets the registers (64 per thread for 17 to 32 warps, which

@@ -16,8 +16,8 @@
 //      exchange; the arithmetic is the streaming path's (esp_device.cuh), so the prices are too.
 // What bounds it is the chain of one round, not a rate: of 7,400 cycles of a 2048-job cluster of 16
 // options in 16 CTAs, 1,800 are the screen, 400 the warp sums, 1,000 the sends, 2,100 the cluster
-// barrier, 500 the sum of the partials and 1,600 the update and the prices. Per round: 3.60 us, where one
-// lane per job, all sends from one warp and hardware division took 4.97; 2.1 and 3.0 on the tiny cluster.
+// barrier, 500 the sum of the partials and 1,600 the update and the prices. Per round: 3.5 us, where one
+// lane per job, all sends from one warp and hardware division took 4.97; 2.0 and 3.0 on the tiny cluster.
 // Sending the partials with an arrival on each peer's own barrier, so that no cluster barrier is needed, took
 // 4.4 to 5.2; 16 warps per CTA 3.95.
 // After the last round (or the stopping rule) the final evaluation at lambda^T writes the selection,
