@@ -592,8 +592,8 @@ esp_status load_packed(esp_ctx *ctx, const PackFormat &fmt)
     // The persistent pass: every CTA of its launch co-resident, no more warps than tiles. By default on
     // tables with at least kPersistMinSteps steps per warp of its launch. Measured per round (one launch
     // per round against persistent): what-if batch at 64 / 128 / 256 / 1024 scenarios (2.7 / 5.4 / 10.8 / 43
-    // steps per warp) 23.6 / 34.2 / 55.1 / 144 us against 33.0 / 30.9 / 41.0 / 90.2, heavy-tailed table at
-    // 2 / 4 / 16 scenarios 50 / 91 / 247 against 48 / 63 / 170: below, the waits for prices cost more than
+    // steps per warp) 17.6 / 24.8 / 39.0 / 108 us against 27.4 / 24.0 / 34.4 / 83.7, heavy-tailed table at
+    // 1 / 2 / 4 / 16 scenarios 27 / 41 / 64 / 186 against 40 / 39 / 49 / 158: below, the waits for prices cost more than
     // the launches; above, static tile ranges leave the GPU waiting for its slowest warps. Smaller
     // tables take it on request where R is 4, 6 or 8, the widths that the request has always been granted for
     // (the kernel itself depends on the word count only).
@@ -1187,9 +1187,9 @@ esp_status plan_resident_options(esp_ctx *ctx)
 
 // Whether the passes of this table are launched as programmatic dependents by default. Packed passes: where
 // every warp has one tile at most, so that its step is on chip before the pass before it ends (measured
-// per round: tiny cluster 7.9 -> 6.7 us, one 2048-job cluster 11.0 -> 10.7, a ragged batch of seven
-// 1777-job clusters 14.7 -> 13.4; with several tiles per warp, heavy-tailed at 1 and 16 scenarios, 28.3 ->
-// 29.0 and 232 -> 238). Staged passes: large uniform tables (what-if batch: -1.2% per solve; one 2048-job
+// per round: tiny cluster 7.9 -> 6.5 us, one 2048-job cluster 8.9 -> 8.6, a ragged batch of seven
+// 1777-job clusters 12.3 either way; with several tiles per warp no difference, heavy-tailed at 1 and 16 scenarios
+// 26.8 and 186). Staged passes: large uniform tables (what-if batch: -1.2% per solve; one 2048-job
 // scenario: +10%, the ragged 16-scenario table: +12%).
 bool pdl_default(const esp_ctx *c)
 {
