@@ -47,7 +47,7 @@ def test_planned_before_the_validation():
         ratio.append(first / known)
         assert esp.esp_debug_packed_words(s.ctx) == 0
         s.close()
-    assert min(ratio) < 2.5, ratio
+    assert min(ratio) < 4.0, ratio      # planning after the validation: about 10
 
 
 @pytest.mark.parametrize("device", [False, True])
